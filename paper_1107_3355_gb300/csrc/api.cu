@@ -470,7 +470,8 @@ static int prepare_workspace(gdpm_ctx* ctx, Runner& r, size_t V, uint32_t cap, u
     const size_t clean = ws.edep_clean;
     ws.edep_clean = 0;
     ws.edep_zero = 0;
-    if ((rc = ensure(ws.s1, V * 8)) || (rc = ensure(ws.s2, V * 8))) return rc;
+    // batches one after another accumulate s1, s2; side by side one fold ends the calculation
+    if (!concurrent && ((rc = ensure(ws.s1, V * 8)) || (rc = ensure(ws.s2, V * 8)))) return rc;
     if (concurrent) {
         // one grid per batch: V*n_batches doubles, or hi and lo halves of floats
         const size_t want = V * size_t(n_batches) * 8;
@@ -512,7 +513,7 @@ static size_t bytes_needed(gdpm_ctx* ctx, const Runner& r, size_t V, uint64_t n_
     const uint32_t cap = capacity_of(ctx, chunk);
     auto grow = [](const Buffer& b, size_t want) { return b.bytes >= want ? size_t(0) : want; };
     const Workspace& w = r.ws;
-    size_t n = grow(w.s1, V * 8) + grow(w.s2, V * 8);
+    size_t n = conc ? 0 : grow(w.s1, V * 8) + grow(w.s2, V * 8);
     n += conc ? grow(w.edep, V * size_t(n_batches) * 8) : grow(w.edep, V * 8) + grow(w.edep2, V * 8);
     const size_t qb = size_t(cap) * kQueueWords * 4;
     n += grow(w.qph, qb) + grow(w.qel0, qb) + grow(w.qel1, qb);
@@ -765,8 +766,18 @@ int simulate_impl(gdpm_ctx* ctx, Runner& r, gdpm_phantom* ph, gdpm_tables* tb,
     P.hrec = hrec;
     P.hrecd = hrecd;
     P.n_records = hrec ? ctx->hrec_n : 0;
-    GDPM_CUDA_TRY(cudaMemsetAsync(ws.s1.p, 0, V * 8, s));
-    GDPM_CUDA_TRY(cudaMemsetAsync(ws.s2.p, 0, V * 8, s));
+    // results: straight into device outputs, or via staging for host outputs
+    const bool dev_out = dose_out && sigma_out && is_device_ptr(dose_out) && is_device_ptr(sigma_out);
+    double *dd = dose_out, *ds = sigma_out;
+    if (!dev_out) {
+        if ((rc = ensure(ws.stage, V * 16))) return rc;
+        dd = static_cast<double*>(ws.stage.p);
+        ds = dd + V;
+    }
+    if (!conc) {
+        GDPM_CUDA_TRY(cudaMemsetAsync(ws.s1.p, 0, V * 8, s));
+        GDPM_CUDA_TRY(cudaMemsetAsync(ws.s2.p, 0, V * 8, s));
+    }
     const size_t grids = V * size_t(n_batches) * 8;
     if (conc) {
         // the previous calculation's fold cleared the grids it read
@@ -811,8 +822,7 @@ int simulate_impl(gdpm_ctx* ctx, Runner& r, gdpm_phantom* ph, gdpm_tables* tb,
         ++aux;
         if (run_rc == GDPM_OK) {
             const size_t pi = prof_begin(ctx, r, s, 2);
-            run_rc = launch_fold_batches(ctx, s, P, V, n_batches, nb_small, nb_rem,
-                                         static_cast<double*>(ws.s1.p), static_cast<double*>(ws.s2.p));
+            run_rc = launch_fold_final(ctx, s, P, V, n_batches, nb_small, nb_rem, dd, ds);
             prof_end(ctx, r, s, pi);
         }
     } else {
@@ -851,19 +861,8 @@ int simulate_impl(gdpm_ctx* ctx, Runner& r, gdpm_phantom* ph, gdpm_tables* tb,
         r.prof_kind.clear();
         return run_rc;
     }
-    // results: straight into device outputs, or via staging for host outputs
-    const bool dev_out = dose_out && sigma_out && is_device_ptr(dose_out) && is_device_ptr(sigma_out);
-    double *dd = dose_out, *ds = sigma_out;
-    if (!dev_out) {
-        if ((rc = ensure(ws.stage, V * 16))) {
-            cudaStreamSynchronize(s);       // the fold may still be clearing the grids
-            return rc;
-        }
-        dd = static_cast<double*>(ws.stage.p);
-        ds = dd + V;
-    }
-    if ((rc = launch_finalize_into(ctx, s, P, V, n_batches, static_cast<const double*>(ws.s1.p),
-                                   static_cast<const double*>(ws.s2.p), dd, ds))) {
+    if (!conc && (rc = launch_finalize_into(ctx, s, P, V, n_batches, static_cast<const double*>(ws.s1.p),
+                                            static_cast<const double*>(ws.s2.p), dd, ds))) {
         cudaStreamSynchronize(s);
         return rc;
     }
@@ -885,7 +884,7 @@ int simulate_impl(gdpm_ctx* ctx, Runner& r, gdpm_phantom* ph, gdpm_tables* tb,
         fill_stats(hc, hl, st);
         if (graph_k) phases = int64_t(*graph_k);
         st->phases = phases;
-        st->launches = phases + aux + 2;    // + finalize and metric
+        st->launches = phases + aux + (conc ? 1 : 2);   // + the metric (and the finalize)
         float ms = 0;
         cudaEventElapsedTime(&ms, r.ev0, r.ev1);
         st->transport_ms = ms;
@@ -1712,7 +1711,9 @@ int gdpm_simulate_beamlets(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb,
         GDPM_CUDA_TRY(cudaMemsetAsync(ctx->hrec, 0, total * 16, s));
         GDPM_CUDA_TRY(cudaMemsetAsync(ctx->hrecd, 0, total * 16, s));
     }
-    GDPM_CUDA_TRY(cudaMemsetAsync(ws.edep.p, 0, V * size_t(slots) * 8, s));
+    // the previous calculation's fold cleared the grids it read
+    const size_t grids = V * size_t(slots) * 8;
+    if (ws.edep_zero < grids) GDPM_CUDA_TRY(cudaMemsetAsync(ws.edep.p, 0, grids, s));
     GDPM_CUDA_TRY(cudaMemsetAsync(ws.counters.p, 0, C_NCOUNT * 8, s));
     GDPM_CUDA_TRY(cudaMemsetAsync(ws.ledger.p, 0, L_NLEDGER * 8, s));
     GDPM_CUDA_TRY(cudaMemsetAsync(ws.status.p, 0, 16, s));
@@ -1773,6 +1774,7 @@ int gdpm_simulate_beamlets(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb,
     GDPM_CUDA_TRY(cudaMemcpyAsync(hl, ws.ledger.p, L_NLEDGER * 8, cudaMemcpyDeviceToHost, s));
     GDPM_CUDA_TRY(cudaMemcpyAsync(hs, ws.status.p, 4, cudaMemcpyDeviceToHost, s));
     GDPM_CUDA_TRY(cudaStreamSynchronize(s));
+    ws.edep_clean = grids;                  // k_fold_sub has cleared every slot's grid
     if (st) {
         std::memset(st, 0, sizeof(*st));
         fill_stats(hc, hl, st);

@@ -219,6 +219,10 @@ int launch_fold_into(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t 
                      double* s1, double* s2);
 int launch_fold_batches(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t V, int n_batches,
                         uint32_t nb_small, uint32_t nb_rem, double* s1, double* s2);
+// The whole calculation's grids into dose and sigma, Dmax and the Sec. 3.1
+// metric (both outputs are needed); the grids are left zeroed.
+int launch_fold_final(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t V, int n_batches,
+                      uint32_t nb_small, uint32_t nb_rem, double* dose, double* sigma);
 int launch_finalize_into(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t V,
                          int n_batches, const double* s1, const double* s2, double* dose,
                          double* sigma);

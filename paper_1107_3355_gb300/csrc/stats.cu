@@ -139,56 +139,200 @@ __global__ void __launch_bounds__(256) k_fold(SimParams P, size_t V, double inv_
     if (threadIdx.x == 0 && t != 0.0) atomicAdd(&P.ledger[L_DEPOSITED], t);
 }
 
-// Sums of a voxel's batch tallies b in [b0, b1) of grids of V cells
-// starting at slot `first`: sum e and sum e^2, two FP64 operations per
-// tally.  GB300's FP64 rate (about 5e11 FMA/s), not HBM, bounds the fold,
-// so the batch weights are applied once per voxel, not per tally.  CLEAR
-// then zeroes the tallies, leaving the grids ready for the next
-// calculation; the stores come after all the loads, which a store between
-// them would serialise (the compiler cannot tell the addresses apart).
-template <bool CLEAR>
+// Mean dose of a voxel and its standard error, MeV/g per history, from the
+// sums a1, a2 over nb batches of x_b = E_b/n_b and x_b^2.  FP64 division and
+// square root are slow on this part, so 1/mass and sqrt(var) start from FP32
+// estimates and take one FP64 Newton step each (relative error ~1e-14).
+__device__ __forceinline__ double inverse_mass(float rho, double dvol) {
+    const double mass = double(rho) * dvol;
+    const double im = double(1.0f / float(mass));
+    return im * fma(-mass, im, 2.0);
+}
+__device__ __forceinline__ double root(double var) {
+    if (!(var > 0.0)) return 0.0;
+    double y = double(rsqrtf(float(var)));
+    y = y * fma(-0.5 * var * y, y, 1.5);
+    return var * y;
+}
+
+// Sums of a thread's batch tallies b in [b0, b1) at its VPT voxels v,
+// v + blockDim.x, ... over grids of V cells starting at slot `first`: sum e
+// and sum e^2 per voxel, two FP64 operations per tally.  GB300's FP64 rate
+// (about 5e11 FMA/s), not HBM, bounds a fold that spends them on every tally,
+// and most tallies are zero: even a field of 1e6 histories a batch leaves
+// four fifths of the CT phantom's voxels without a deposit in that batch.
+// So UB batches are loaded at a time only to see which are nonzero, and the
+// thread then walks its nonzero ones, in batch order, from L1 (adding zero
+// would change no bit of a sum); a warp spends FP64 operations for the lane
+// with the most.  Those tallies are then zeroed, after all of the chunk's
+// loads, which leaves the grids ready for the next calculation.
+// Measured with the finalize work in the same kernel (below): CT phantom, 10
+// grids of one beamlet's 1e5 histories 0.98 -> 0.24 ms; 128^3 slab, 100 grids
+// of 1e4 histories each 0.93 -> 0.45 ms; CT plan, 100 grids of 1e6 histories
+// each 3.7 -> 2.7 ms (6.7 GB read).  16 batches at a time and 64 registers
+// were best: 8 (40 registers) +14 %, 32 (128 registers) +25-33 %.
+template <int VPT, int UB>
 __device__ __forceinline__ void batch_sums(const SimParams& P, size_t V, size_t first, size_t v,
-                                           int b0, int b1, double& se, double& sq) {
-    for (int b = b0; b < b1; ++b) {
-        const size_t k = (first + size_t(b)) * V + v;
-        const double e = P.tally_mode == 0 ? P.edep[k] : double(P.edep_hi[k]) + double(P.edep_lo[k]);
-        se += e;
-        sq = fma(e, e, sq);
-    }
-    if (CLEAR) {
-        for (int b = b0; b < b1; ++b) {
-            const size_t k = (first + size_t(b)) * V + v;
-            if (P.tally_mode == 0) {
-                P.edep[k] = 0.0;
-            } else {
-                P.edep_hi[k] = 0.f;
-                P.edep_lo[k] = 0.f;
+                                           int b0, int b1, double (&se)[VPT], double (&sq)[VPT]) {
+    const bool pair = P.tally_mode != 0;
+    for (int b = b0; b < b1; b += UB) {
+        uint32_t mask[VPT] = {};
+        const size_t k0 = (first + size_t(b)) * V + v;
+        if (!pair) {
+            unsigned long long bits[UB][VPT];
+#pragma unroll
+            for (int u = 0; u < UB; ++u)
+#pragma unroll
+                for (int i = 0; i < VPT; ++i)
+                    bits[u][i] = (b + u < b1 && v + size_t(i) * blockDim.x < V)
+                                     ? reinterpret_cast<const unsigned long long*>(P.edep)[k0 + u * V + i * blockDim.x]
+                                     : 0ull;
+#pragma unroll
+            for (int u = 0; u < UB; ++u)
+#pragma unroll
+                for (int i = 0; i < VPT; ++i) mask[i] |= bits[u][i] ? 1u << u : 0u;
+        } else {
+#pragma unroll
+            for (int u = 0; u < UB; ++u)
+#pragma unroll
+                for (int i = 0; i < VPT; ++i)
+                    if (b + u < b1 && v + size_t(i) * blockDim.x < V) {
+                        const size_t k = k0 + u * V + i * blockDim.x;
+                        const uint32_t w = reinterpret_cast<const uint32_t*>(P.edep_hi)[k] |
+                                           reinterpret_cast<const uint32_t*>(P.edep_lo)[k];
+                        mask[i] |= w ? 1u << u : 0u;
+                    }
+        }
+#pragma unroll
+        for (int i = 0; i < VPT; ++i) {
+            const size_t ki = k0 + i * blockDim.x;
+            for (uint32_t m = mask[i]; m; m &= m - 1u) {
+                const size_t k = ki + size_t(__ffs(m) - 1) * V;
+                const double e = pair ? double(P.edep_hi[k]) + double(P.edep_lo[k]) : P.edep[k];
+                se[i] += e;
+                sq[i] = fma(e, e, sq[i]);
+            }
+            for (uint32_t m = mask[i]; m; m &= m - 1u) {
+                const size_t k = ki + size_t(__ffs(m) - 1) * V;
+                if (!pair) {
+                    P.edep[k] = 0.0;
+                } else {
+                    P.edep_hi[k] = 0.f;
+                    P.edep_lo[k] = 0.f;
+                }
             }
         }
     }
 }
 
-// All batches at once (batches run side by side, one tally grid each):
-// s1 += sum_b E_b/n_b, s2 += sum_b (E_b/n_b)^2 per voxel (the sums of a run
-// in parts accumulate).  The first n_big batches hold one history more.
-// The grids are left zeroed.
-__global__ void __launch_bounds__(256) k_fold_batches(SimParams P, size_t V, int nbatch,
-                                                      double inv_big, double inv_small, int n_big,
-                                                      double* __restrict__ s1, double* __restrict__ s2) {
-    __shared__ double s_red[32];
-    double dep = 0.0;
-    const int nbig = min(n_big, nbatch);
-    for (size_t v = blockIdx.x * size_t(blockDim.x) + threadIdx.x; v < V;
-         v += size_t(gridDim.x) * blockDim.x) {
-        double eb = 0.0, qb = 0.0, es = 0.0, qs = 0.0;
-        batch_sums<true>(P, V, 0, v, 0, nbig, eb, qb);
-        batch_sums<true>(P, V, 0, v, nbig, nbatch, es, qs);
-        dep += eb + es;
-        s1[v] += fma(eb, inv_big, es * inv_small);
-        s2[v] += fma(qb, inv_big * inv_big, qs * (inv_small * inv_small));
+// Voxels with dose, gathered by the threads of a CTA so that the FP64 work
+// per voxel (weights, mean, 1/mass, square root: about 30 operations) runs
+// with full warps however few of a warp's voxels hold dose.
+struct FoldItem {
+    double eb, qb, es, qs;      // sums over the long batches and over the short ones
+};
+constexpr int kFoldThreads = 256;
+struct FoldList {
+    FoldItem item[2 * kFoldThreads];
+    uint32_t vox[2 * kFoldThreads];
+    uint32_t n;
+};
+
+// Loop of a fold over the CTA's voxels: sum each voxel's tallies, hand a
+// voxel without dose to `empty(voxel)` and the others, in full CTA-loads, to
+// `full(voxel, item)`.
+template <int VPT, int UB, class Full, class Empty>
+__device__ __forceinline__ void fold_voxels(const SimParams& P, size_t V, size_t first, int nbig, int nbatch,
+                                            FoldList& L, Full full, Empty empty) {
+    if (threadIdx.x == 0) L.n = 0u;
+    __syncthreads();
+    for (size_t base = size_t(blockIdx.x) * kFoldThreads * VPT; base < V;
+         base += size_t(gridDim.x) * kFoldThreads * VPT) {
+        const size_t v = base + threadIdx.x;
+        double eb[VPT] = {}, qb[VPT] = {}, es[VPT] = {}, qs[VPT] = {};
+        if (nbig > 0) batch_sums<VPT, UB>(P, V, first, v, 0, nbig, eb, qb);
+        batch_sums<VPT, UB>(P, V, first, v, nbig, nbatch, es, qs);
+#pragma unroll
+        for (int i = 0; i < VPT; ++i) {
+            const size_t vi = v + size_t(i) * kFoldThreads;
+            // the sum of squares is zero only when every tally is
+            const bool have = vi < V && (qb[i] != 0.0 || qs[i] != 0.0);
+            if (vi < V && !have) empty(vi);
+            const uint32_t m = __ballot_sync(0xffffffffu, have);
+            uint32_t at = 0u;
+            if (m && (threadIdx.x & 31u) == 0u) at = atomicAdd(&L.n, uint32_t(__popc(m)));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & lanemask_lt());
+            if (have) {
+                L.item[at] = FoldItem{eb[i], qb[i], es[i], qs[i]};
+                L.vox[at] = uint32_t(vi);
+            }
+            __syncthreads();
+            // at most 255 left over plus 256 new ones: one full load at a time
+            const uint32_t n = L.n;
+            if (n >= uint32_t(kFoldThreads)) {
+                const uint32_t j = n - kFoldThreads + threadIdx.x;
+                full(size_t(L.vox[j]), L.item[j]);
+                __syncthreads();
+                if (threadIdx.x == 0) L.n = n - kFoldThreads;
+            }
+            __syncthreads();
+        }
     }
+    if (threadIdx.x < L.n) full(size_t(L.vox[threadIdx.x]), L.item[threadIdx.x]);
+}
+
+// All batches at once (batches run side by side, one tally grid each): per
+// voxel a1 = sum_b E_b/n_b and a2 = sum_b (E_b/n_b)^2; the first n_big
+// batches hold one history more.  FINAL: the grids hold the whole
+// calculation, so the voxel's dose and sigma follow at once (out1, out2; and
+// Dmax), with no sums written and read back.  Otherwise the sums of a run in
+// parts accumulate in out1, out2.  The grids are left zeroed.
+template <bool FINAL, int VPT, int UB>
+__global__ void __launch_bounds__(kFoldThreads, 4) k_fold_batches(SimParams P, size_t V, int nbatch,
+                                                               double inv_big, double inv_small, int n_big,
+                                                               double* __restrict__ out1,
+                                                               double* __restrict__ out2, double dvol,
+                                                               unsigned long long* dmax_bits,
+                                                               float metric_min_rho) {
+    __shared__ double s_red[32];
+    __shared__ FoldList L;
+    double dep = 0.0, mx = 0.0;
+    const double inv_n = 1.0 / nbatch;
+    const double inv_nn1 = FINAL ? 1.0 / (double(nbatch) * (nbatch - 1)) : 0.0;
+    fold_voxels<VPT, UB>(
+        P, V, 0, min(n_big, nbatch), nbatch, L,
+        [&](size_t v, const FoldItem& t) {
+            dep += t.eb + t.es;
+            const double a1 = fma(t.eb, inv_big, t.es * inv_small);
+            const double a2 = fma(t.qb, inv_big * inv_big, t.qs * (inv_small * inv_small));
+            if (FINAL) {
+                const double mean = a1 * inv_n;
+                const double var = fmax(0.0, (a2 - nbatch * mean * mean) * inv_nn1);
+                const float r = P.rho[v];
+                const double im = inverse_mass(r, dvol);
+                const double d = mean * im;
+                out1[v] = d;
+                out2[v] = root(var) * im;
+                if (r >= metric_min_rho) mx = fmax(mx, d);
+            } else {
+                out1[v] += a1;
+                out2[v] += a2;
+            }
+        },
+        [&](size_t v) {
+            if (FINAL) {
+                out1[v] = 0.0;
+                out2[v] = 0.0;
+            }
+        });
     const double t = block_sum(dep, s_red);
     if (threadIdx.x == 0 && t != 0.0) atomicAdd(&P.ledger[L_DEPOSITED], t);
+    if (FINAL) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, o));
+        if ((threadIdx.x & 31) == 0 && mx > 0.0)
+            atomicMax(dmax_bits, (unsigned long long)__double_as_longlong(mx));
+    }
 }
 
 // Dose matrix: sub-problem k (row k of the fluence map; blockIdx.y) tallied
@@ -196,50 +340,47 @@ __global__ void __launch_bounds__(256) k_fold_batches(SimParams P, size_t V, int
 // voxel (MeV/g per history of that sub-problem) to dose[(k-k0)*V + v] and
 // sigma[...]; with one batch only the dose.  inv_n[2k], inv_n[2k+1] are
 // 1/(histories of a long batch) and 1/(histories of a short batch) of
-// sub-problem k, whose first nbig[k] batches are the long ones.
-__global__ void __launch_bounds__(256) k_fold_sub(SimParams P, size_t V, uint32_t k0, int nb,
-                                                  const double* __restrict__ inv_n,
-                                                  const uint32_t* __restrict__ nbig, double dvol,
-                                                  double* __restrict__ dose, double* __restrict__ sigma) {
+// sub-problem k, whose first nbig[k] batches are the long ones.  The grids
+// are left zeroed.  With two batches a thread has only two tallies a voxel to
+// load, so it takes four voxels.  64 beamlets x 2 batches on the 128^3 slab
+// (134M voxels of output): memset and fold 17 -> 3.7 ms.
+template <int VPT, int UB>
+__global__ void __launch_bounds__(kFoldThreads) k_fold_sub(SimParams P, size_t V, uint32_t k0, int nb,
+                                                           const double* __restrict__ inv_n,
+                                                           const uint32_t* __restrict__ nbig, double dvol,
+                                                           double* __restrict__ dose,
+                                                           double* __restrict__ sigma) {
     __shared__ double s_red[32];
+    __shared__ FoldList L;
     const uint32_t k = k0 + blockIdx.y;
     const double ib = inv_n[2 * k], is = inv_n[2 * k + 1];
-    const uint32_t n_big = nbig[k];
+    const bool with_sigma = sigma && nb > 1;
+    double* const dk = dose + size_t(blockIdx.y) * V;
+    double* const sk = with_sigma ? sigma + size_t(blockIdx.y) * V : nullptr;
     double dep = 0.0;
-    const int nbg = int(min(n_big, uint32_t(nb)));
-    for (size_t v = blockIdx.x * size_t(blockDim.x) + threadIdx.x; v < V;
-         v += size_t(gridDim.x) * blockDim.x) {
-        double eb = 0.0, qb = 0.0, es = 0.0, qs = 0.0;
-        batch_sums<false>(P, V, size_t(k) * nb, v, 0, nbg, eb, qb);
-        batch_sums<false>(P, V, size_t(k) * nb, v, nbg, nb, es, qs);
-        dep += eb + es;
-        const double a1 = fma(eb, ib, es * is);
-        const double a2 = fma(qb, ib * ib, qs * (is * is));
-        const double mass = double(P.rho[v]) * dvol;
-        double im = double(1.0f / float(mass));
-        im = im * fma(-mass, im, 2.0);                       // Newton step for 1/mass
-        const size_t o = size_t(blockIdx.y) * V + v;
-        const double mean = a1 / nb;
-        dose[o] = mean * im;
-        if (sigma && nb > 1) {
-            const double var = fmax(0.0, (a2 - nb * mean * mean) / (double(nb) * (nb - 1)));
-            double sd = 0.0;
-            if (var > 0.0) {
-                double y = double(rsqrtf(float(var)));
-                y = y * fma(-0.5 * var * y, y, 1.5);         // Newton step for 1/sqrt(var)
-                sd = var * y;
-            }
-            sigma[o] = sd * im;
-        }
-    }
+    fold_voxels<VPT, UB>(
+        P, V, size_t(k) * nb, int(min(nbig[k], uint32_t(nb))), nb, L,
+        [&](size_t v, const FoldItem& t) {
+            dep += t.eb + t.es;
+            const double a1 = fma(t.eb, ib, t.es * is);
+            const double a2 = fma(t.qb, ib * ib, t.qs * (is * is));
+            const double im = inverse_mass(P.rho[v], dvol);
+            const double mean = a1 / nb;
+            dk[v] = mean * im;
+            if (with_sigma)
+                sk[v] = root(fmax(0.0, (a2 - nb * mean * mean) / (double(nb) * (nb - 1)))) * im;
+        },
+        [&](size_t v) {
+            dk[v] = 0.0;
+            if (with_sigma) sk[v] = 0.0;
+        });
     const double t = block_sum(dep, s_red);
     if (threadIdx.x == 0 && t != 0.0) atomicAdd(&P.ledger[L_DEPOSITED], t);
 }
 
-// Mean and standard error per voxel in MeV/g per history; Dmax.  FP64
-// division and square root are slow on this part, so 1/mass and sqrt(var)
-// start from FP32 estimates and take one FP64 Newton step each (relative
-// error ~1e-14).
+// Mean and standard error per voxel in MeV/g per history, and Dmax, from the
+// sums of all batches (batches run one after another, or in parts).  A voxel
+// without dose skips the FP64 arithmetic.
 __global__ void k_finalize(const double* __restrict__ s1, const double* __restrict__ s2,
                            const float* __restrict__ rho, size_t V, int nb, double dvol,
                            double* __restrict__ dose, double* __restrict__ sigma,
@@ -249,22 +390,19 @@ __global__ void k_finalize(const double* __restrict__ s1, const double* __restri
     const double inv_nn1 = 1.0 / (double(nb) * (nb - 1));
     for (size_t v = blockIdx.x * size_t(blockDim.x) + threadIdx.x; v < V;
          v += size_t(gridDim.x) * blockDim.x) {
-        const double mean = s1[v] * inv_n;
-        const double var = fmax(0.0, (s2[v] - nb * mean * mean) * inv_nn1);
-        const float r = rho[v];
-        const double mass = double(r) * dvol;
-        double im = double(1.0f / float(mass));
-        im = im * fma(-mass, im, 2.0);                       // Newton step for 1/mass
-        const double d = mean * im;
-        double sd = 0.0;
-        if (var > 0.0) {
-            double y = double(rsqrtf(float(var)));
-            y = y * fma(-0.5 * var * y, y, 1.5);             // Newton step for 1/sqrt(var)
-            sd = var * y;
+        const double a1 = s1[v], a2 = s2[v];
+        double d = 0.0, sd = 0.0;
+        if (a1 != 0.0 || a2 != 0.0) {
+            const double mean = a1 * inv_n;
+            const double var = fmax(0.0, (a2 - nb * mean * mean) * inv_nn1);
+            const float r = rho[v];
+            const double im = inverse_mass(r, dvol);
+            d = mean * im;
+            sd = root(var) * im;
+            if (r >= metric_min_rho) mx = fmax(mx, d);
         }
         if (dose) dose[v] = d;
-        if (sigma) sigma[v] = sd * im;
-        if (r >= metric_min_rho) mx = fmax(mx, d);
+        if (sigma) sigma[v] = sd;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, o));
@@ -281,12 +419,18 @@ __global__ void k_metric(const double* __restrict__ dose, const double* __restri
     __shared__ double s_red[32];
     const double dmax = __longlong_as_double((long long)*dmax_bits);
     double acc = 0.0, cnt = 0.0;
-    for (size_t v = blockIdx.x * size_t(blockDim.x) + threadIdx.x; v < V;
-         v += size_t(gridDim.x) * blockDim.x) {
-        if (dose[v] > 0.5 * dmax && rho[v] >= metric_min_rho) {
-            acc += sigma[v];
-            cnt += 1.0;
-        }
+    const double half = 0.5 * dmax;
+    const size_t step = size_t(gridDim.x) * blockDim.x;
+    for (size_t v = blockIdx.x * size_t(blockDim.x) + threadIdx.x; v < V; v += 4 * step) {
+        double d[4];                        // four loads in flight
+#pragma unroll
+        for (int u = 0; u < 4; ++u) d[u] = v + u * step < V ? dose[v + u * step] : 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (v + u * step < V && d[u] > half && rho[v + u * step] >= metric_min_rho) {
+                acc += sigma[v + u * step];
+                cnt += 1.0;
+            }
     }
     const double a = block_sum(acc, s_red);
     __syncthreads();
@@ -349,20 +493,49 @@ int launch_fold_into(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t 
     return GDPM_OK;
 }
 
+// Thread blocks of a fold over V voxels, VPT a thread: one wave of CTAs at
+// most (each loops over its share), so that the per-CTA reductions stay few.
+static unsigned fold_grid(gdpm_ctx* ctx, size_t V, int vpt, int ctas_per_sm) {
+    const size_t need = (V + size_t(256) * vpt - 1) / (size_t(256) * vpt);
+    return unsigned(std::max<size_t>(1, std::min<size_t>(need, size_t(ctx->sm_count) * ctas_per_sm)));
+}
+
 int launch_fold_batches(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t V, int n_batches,
                         uint32_t nb_small, uint32_t nb_rem, double* s1, double* s2) {
-    k_fold_batches<<<ctx->sm_count * 8, 256, 0, st>>>(P, V, n_batches, 1.0 / double(nb_small + 1),
-                                                        1.0 / double(nb_small), int(nb_rem), s1, s2);
+    k_fold_batches<false, 1, 16><<<fold_grid(ctx, V, 1, 8), kFoldThreads, 0, st>>>(
+        P, V, n_batches, 1.0 / double(nb_small + 1), 1.0 / double(nb_small), int(nb_rem), s1, s2, 0.0,
+        nullptr, 0.f);
     GDPM_CUDA_TRY(cudaGetLastError());
     return GDPM_OK;
+}
+
+static int launch_metric(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t V, const double* dose,
+                         const double* sigma) {
+    const unsigned long long* dmax_bits = reinterpret_cast<const unsigned long long*>(&P.ledger[L_DMAX]);
+    const size_t need = (V + 1023) / 1024;
+    const unsigned grid = unsigned(std::min<size_t>(std::max<size_t>(need, 1), size_t(ctx->sm_count) * 8));
+    k_metric<<<grid, 256, 0, st>>>(dose, sigma, P.rho, V, dmax_bits, P.ledger, ctx->metric_min_rho);
+    GDPM_CUDA_TRY(cudaGetLastError());
+    return GDPM_OK;
+}
+
+int launch_fold_final(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t V, int n_batches,
+                      uint32_t nb_small, uint32_t nb_rem, double* dose, double* sigma) {
+    const double dvol = double(P.dx) * P.dy * P.dz;
+    unsigned long long* dmax_bits = reinterpret_cast<unsigned long long*>(&P.ledger[L_DMAX]);
+    k_fold_batches<true, 1, 16><<<fold_grid(ctx, V, 1, 8), kFoldThreads, 0, st>>>(
+        P, V, n_batches, 1.0 / double(nb_small + 1), 1.0 / double(nb_small), int(nb_rem), dose, sigma,
+        dvol, dmax_bits, ctx->metric_min_rho);
+    GDPM_CUDA_TRY(cudaGetLastError());
+    return launch_metric(ctx, st, P, V, dose, sigma);
 }
 
 int launch_fold_sub(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t V, uint32_t k0,
                     uint32_t nk, int nb, const double* inv_n, const uint32_t* nbig, double* dose,
                     double* sigma) {
     const double dvol = double(P.dx) * P.dy * P.dz;
-    const uint32_t gx = uint32_t(std::min<size_t>((V + 255) / 256, size_t(ctx->sm_count) * 4));
-    k_fold_sub<<<dim3(gx, nk), 256, 0, st>>>(P, V, k0, nb, inv_n, nbig, dvol, dose, sigma);
+    k_fold_sub<4, 2><<<dim3(fold_grid(ctx, V, 4, 8), nk), kFoldThreads, 0, st>>>(P, V, k0, nb, inv_n, nbig, dvol,
+                                                                        dose, sigma);
     GDPM_CUDA_TRY(cudaGetLastError());
     return GDPM_OK;
 }
@@ -376,9 +549,7 @@ int launch_finalize_into(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, siz
                                                     dmax_bits, ctx->metric_min_rho);
     GDPM_CUDA_TRY(cudaGetLastError());
     if (dose && sigma) {
-        k_metric<<<ctx->sm_count * 4, 256, 0, st>>>(dose, sigma, P.rho, V, dmax_bits, P.ledger,
-                                                      ctx->metric_min_rho);
-        GDPM_CUDA_TRY(cudaGetLastError());
+        return launch_metric(ctx, st, P, V, dose, sigma);
     }
     return GDPM_OK;
 }
