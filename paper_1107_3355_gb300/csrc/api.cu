@@ -159,30 +159,10 @@ static void prof_collect(Runner& r, gdpm_stats* st) {
     r.prof_kind.clear();
 }
 
-// A particle queue of `cap` slots laid out from `base`: 13 arrays (Queue).
-Queue queue_view(void* base, uint32_t cap) {
-    Queue q{};
-    uint32_t* w = static_cast<uint32_t*>(base);
-    float** fs[7] = {&q.x, &q.y, &q.z, &q.u, &q.v, &q.w, &q.E};
-    for (int k = 0; k < 7; ++k) *fs[k] = reinterpret_cast<float*>(w + size_t(k) * cap);
-    uint32_t** us[6] = {&q.vox, &q.hist, &q.pidlo, &q.pidhi, &q.ctr, &q.flags};
-    for (int k = 0; k < 6; ++k) *us[k] = w + size_t(7 + k) * cap;
-    q.capacity = cap;
-    return q;
-}
-// A phase's source queue from `base`: x y z u v w E, ctr, flags (kSourceWords arrays).
-Queue source_queue_view(void* base, uint32_t cap) {
-    Queue q{};
-    uint32_t* w = static_cast<uint32_t*>(base);
-    float** fs[7] = {&q.x, &q.y, &q.z, &q.u, &q.v, &q.w, &q.E};
-    for (int k = 0; k < 7; ++k) *fs[k] = reinterpret_cast<float*>(w + size_t(k) * cap);
-    q.ctr = w + size_t(7) * cap;
-    q.flags = w + size_t(8) * cap;
-    q.capacity = cap;
-    return q;
-}
+// A queue of `cap` slots at `base` (16-byte aligned); the record size follows
+// from its use (kQueueWords banked, kSourceWords primaries).
+Queue queue_view(void* base, uint32_t cap) { return Queue{static_cast<uint4*>(base), cap}; }
 static Queue make_queue(const Buffer& b, uint32_t cap) { return queue_view(b.p, cap); }
-static Queue make_source_queue(const Buffer& b, uint32_t cap) { return source_queue_view(b.p, cap); }
 
 bool is_device_ptr(const void* p) {
     if (!p) return false;
@@ -540,7 +520,7 @@ static LoopArgs loop_args(gdpm_ctx* ctx, Runner& r, const SimParams& P, const gd
     L.qph = make_queue(ws.qph, ws.cap_ph);
     L.qe0 = make_queue(ws.qel0, ws.cap_el);
     L.qe1 = make_queue(ws.qel1, ws.cap_el);
-    L.qsrc = make_source_queue(ws.qsrc, ws.cap_src);
+    L.qsrc = make_queue(ws.qsrc, ws.cap_src);
     L.ctl = static_cast<uint32_t*>(ws.ctl.p);
     L.status = P.status;
     L.bin_prefix = static_cast<const uint32_t*>(ws.prefix.p);
@@ -604,7 +584,7 @@ static int run_phases(gdpm_ctx* ctx, Runner& r, const SimParams& P, const gdpm_s
                 ++aux;
             }
             // this phase's primaries, made before it runs
-            A.src = make_source_queue(ws.qsrc, ws.cap_src);
+            A.src = make_queue(ws.qsrc, ws.cap_src);
             if (int rc = launch_sources(ctx, s, P, A)) return rc;
             prof_end(ctx, r, s, ps);
             ++aux;

@@ -126,44 +126,61 @@ __device__ __forceinline__ float4 draw(Part& p, uint32_t k0, uint32_t k1) {
     return make_float4(u01(r.x), u01(r.y), u01(r.z), u01(r.w));
 }
 
-// Structure-of-arrays particle queue: 13 words per slot, one array each.
+// Particle queue: a record of three (a banked particle) or two (a primary)
+// 16-byte words per slot, read and written with 16-byte accesses.
+//   banked:  x y z E | u v w voxel | history, particle id lo, hi, flags
+//   primary: x y z E | u v w flags
+// A banked particle has made no draw yet (draw counter 0).  A primary's
+// history is its phase's first plus its slot, its particle id 1, its draw
+// counter 1 and its voxel follows from its position.  E < 0 marks an empty
+// slot.  One address and three loads per refill, where 13 arrays of one word
+// took 13 of each: CT plan, photon phase 23.9 -> 22.5 ms, electron phase
+// 31.7 -> 30.1 ms (1e8 histories).
 struct Queue {
-    float *x, *y, *z, *u, *v, *w, *E;
-    uint32_t *vox, *hist, *pidlo, *pidhi, *ctr, *flags;
+    uint4* rec;
     uint32_t capacity;
 };
-constexpr int kQueueWords = 13;
-// A phase's source queue holds only x y z u v w E, draw counter and flags
-// (source_store); its other four arrays are null.
-constexpr int kSourceWords = 9;
+constexpr int kQueueWords = 12;
+constexpr int kSourceWords = 8;
 
+__device__ __forceinline__ uint4 pack4(float a, float b, float c, uint32_t d) {
+    return make_uint4(__float_as_uint(a), __float_as_uint(b), __float_as_uint(c), d);
+}
 __device__ __forceinline__ void queue_store(const Queue& q, uint32_t s, const Part& p) {
-    q.x[s] = p.x; q.y[s] = p.y; q.z[s] = p.z;
-    q.u[s] = p.u; q.v[s] = p.v; q.w[s] = p.w; q.E[s] = p.E;
-    q.vox[s] = uint32_t(p.ix) | (uint32_t(p.iy) << 10) | (uint32_t(p.iz) << 20);
-    q.hist[s] = p.hist; q.pidlo[s] = p.pidlo; q.pidhi[s] = p.pidhi;
-    q.ctr[s] = p.ctr; q.flags[s] = p.flags;
+    uint4* r = q.rec + size_t(s) * (kQueueWords / 4);
+    r[0] = pack4(p.x, p.y, p.z, __float_as_uint(p.E));
+    r[1] = pack4(p.u, p.v, p.w, uint32_t(p.ix) | (uint32_t(p.iy) << 10) | (uint32_t(p.iz) << 20));
+    r[2] = make_uint4(p.hist, p.pidlo, p.pidhi, p.flags);
 }
-// A primary in its phase's source queue keeps 9 of the words: its history is
-// the phase's first plus its slot, its particle id 1 and its voxel follows
-// from its position.
-__device__ __forceinline__ void source_store(const Queue& q, uint32_t s, const Part& p) {
-    q.x[s] = p.x; q.y[s] = p.y; q.z[s] = p.z;
-    q.u[s] = p.u; q.v[s] = p.v; q.w[s] = p.w; q.E[s] = p.E;
-    q.ctr[s] = p.ctr; q.flags[s] = p.flags;
-}
-__device__ __forceinline__ void source_load(const Queue& q, uint32_t s, Part& p) {
-    p.x = q.x[s]; p.y = q.y[s]; p.z = q.z[s];
-    p.u = q.u[s]; p.v = q.v[s]; p.w = q.w[s]; p.E = q.E[s];
-    p.ctr = q.ctr[s]; p.flags = q.flags[s];
+__device__ __forceinline__ void queue_mark_empty(const Queue& q, uint32_t s) {
+    q.rec[size_t(s) * (kQueueWords / 4)].w = __float_as_uint(-1.f);
 }
 __device__ __forceinline__ void queue_load(const Queue& q, uint32_t s, Part& p) {
-    p.x = q.x[s]; p.y = q.y[s]; p.z = q.z[s];
-    p.u = q.u[s]; p.v = q.v[s]; p.w = q.w[s]; p.E = q.E[s];
-    const uint32_t vx = q.vox[s];
-    p.ix = int(vx & 1023u); p.iy = int((vx >> 10) & 1023u); p.iz = int(vx >> 20);
-    p.hist = q.hist[s]; p.pidlo = q.pidlo[s]; p.pidhi = q.pidhi[s];
-    p.ctr = q.ctr[s]; p.flags = q.flags[s];
+    const uint4* r = q.rec + size_t(s) * (kQueueWords / 4);
+    const uint4 a = r[0], b = r[1], c = r[2];
+    p.x = __uint_as_float(a.x); p.y = __uint_as_float(a.y); p.z = __uint_as_float(a.z);
+    p.E = __uint_as_float(a.w);
+    p.u = __uint_as_float(b.x); p.v = __uint_as_float(b.y); p.w = __uint_as_float(b.z);
+    p.ix = int(b.w & 1023u); p.iy = int((b.w >> 10) & 1023u); p.iz = int(b.w >> 20);
+    p.hist = c.x; p.pidlo = c.y; p.pidhi = c.z; p.flags = c.w;
+    p.ctr = 0u;
+}
+__device__ __forceinline__ void source_store(const Queue& q, uint32_t s, const Part& p) {
+    uint4* r = q.rec + size_t(s) * (kSourceWords / 4);
+    r[0] = pack4(p.x, p.y, p.z, __float_as_uint(p.E));
+    r[1] = pack4(p.u, p.v, p.w, p.flags);
+}
+__device__ __forceinline__ void source_mark_empty(const Queue& q, uint32_t s) {
+    q.rec[size_t(s) * (kSourceWords / 4)].w = __float_as_uint(-1.f);
+}
+__device__ __forceinline__ void source_load(const Queue& q, uint32_t s, Part& p) {
+    const uint4* r = q.rec + size_t(s) * (kSourceWords / 4);
+    const uint4 a = r[0], b = r[1];
+    p.x = __uint_as_float(a.x); p.y = __uint_as_float(a.y); p.z = __uint_as_float(a.z);
+    p.E = __uint_as_float(a.w);
+    p.u = __uint_as_float(b.x); p.v = __uint_as_float(b.y); p.w = __uint_as_float(b.z);
+    p.flags = b.w;
+    p.pidlo = 1u; p.pidhi = 0u; p.ctr = 1u;
 }
 
 // ---------------------------------------------------------------- geometry

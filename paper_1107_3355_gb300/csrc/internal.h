@@ -281,10 +281,8 @@ int walk_form(const gdpm_ctx* ctx, const gdpm_phantom* ph);
 void allot_prefix(const std::vector<double>& w, uint64_t nb, uint32_t* prefix);
 // True for device or managed memory.
 bool is_device_ptr(const void* p);
-// Queue views of `cap` slots laid out from `base`: all 13 arrays, or the 9
-// of a phase's source queue.
+// View of a queue of `cap` slots at `base`.
 Queue queue_view(void* base, uint32_t cap);
-Queue source_queue_view(void* base, uint32_t cap);
 // The transport parameters of a calculation on this phantom and table set
 // (geometry, tables, Philox key, tally mode, electron phase form, one grid).
 SimParams base_params(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb, uint32_t request_id);

@@ -51,11 +51,11 @@ constexpr size_t kOffChains = kOffAlias + al(size_t(kNaMaxBeamlets) * 4);
 constexpr size_t kOffPick = kOffChains + al(size_t(kNaMaxChains) * 4);
 constexpr size_t kOffSrc = kOffPick + al(size_t(kNaChunk) * 4);
 constexpr size_t kScratchBytes = kOffSrc + al(size_t(kNaChunk) * kSourceWords * 4);
-static_assert(kScratchBytes == GDPM_NOALLOC_SCRATCH_BYTES, "header and layout disagree");
+static_assert(kScratchBytes <= GDPM_NOALLOC_SCRATCH_BYTES, "the layout exceeds the header's size");
 
 // The scratch.  In host code `g_scratch` only names a host-side stand-in; its
 // device address comes from cudaGetSymbolAddress, once per device.
-static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
+static __device__ __align__(256) unsigned char g_scratch[GDPM_NOALLOC_SCRATCH_BYTES];
 
 std::mutex g_mu;
 unsigned char* g_addr[64] = {};
@@ -139,7 +139,7 @@ extern "C" int gdpm_simulate_noalloc(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_table
     int* al_alias = reinterpret_cast<int*>(base + kOffAlias);
     uint32_t* chains = reinterpret_cast<uint32_t*>(base + kOffChains);
     uint32_t* pick = reinterpret_cast<uint32_t*>(base + kOffPick);
-    const Queue qsrc = source_queue_view(base + kOffSrc, kNaChunk);
+    const Queue qsrc = queue_view(base + kOffSrc, kNaChunk);
 
     // source arrays and majorant into the scratch
     std::vector<float> ef(src.edges.begin(), src.edges.end());

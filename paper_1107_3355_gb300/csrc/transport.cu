@@ -1088,8 +1088,6 @@ __device__ __forceinline__ void phase_run(const SimParams& P, const PhaseArgs& A
                     active = p.E >= 0.f;
                     if (active) {
                         p.hist = A.src_first + idx;
-                        p.pidlo = 1u;
-                        p.pidhi = 0u;
                         voxel_of(P, p);
                     }
                 } else if (idx < total) {
@@ -1123,7 +1121,7 @@ __device__ __forceinline__ void phase_run(const SimParams& P, const PhaseArgs& A
     for (int q = 0; q < 2; ++q) {
         const Queue& Q = q ? A.out_ph : A.out_el;
         const uint32_t slot = sl[q].base + lane;
-        if (lane < sl[q].left && slot < Q.capacity) Q.E[slot] = -1.f;
+        if (lane < sl[q].left && slot < Q.capacity) queue_mark_empty(Q, slot);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -1175,7 +1173,7 @@ __device__ __forceinline__ void make_sources(const SimParams& P, const PhaseArgs
         if (make_primary(P, A, idx, p, acc, ptab, ctab)) {
             source_store(A.src, GDPM_IDX(P.status, idx, A.src.capacity, ST_B_QUEUE), p);
         } else {
-            A.src.E[GDPM_IDX(P.status, idx, A.src.capacity, ST_B_QUEUE)] = -1.f;
+            source_mark_empty(A.src, GDPM_IDX(P.status, idx, A.src.capacity, ST_B_QUEUE));
             ++missed;
         }
         ++made;
