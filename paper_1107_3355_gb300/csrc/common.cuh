@@ -61,25 +61,20 @@ enum { L_SOURCE = 0, L_DEPOSITED, L_ESCAPED, L_DISCARDED, L_DMAX, L_SIGSUM, L_SI
 __host__ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1) {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-#ifdef __CUDA_ARCH__
-        const uint32_t hi0 = __umulhi(0xD2511F53u, c.x), lo0 = 0xD2511F53u * c.x;
-        const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z), lo1 = 0xCD9E8D57u * c.z;
-#else
         const uint64_t p0 = uint64_t(0xD2511F53u) * c.x, p1 = uint64_t(0xCD9E8D57u) * c.z;
-        const uint32_t hi0 = uint32_t(p0 >> 32), lo0 = uint32_t(p0);
-        const uint32_t hi1 = uint32_t(p1 >> 32), lo1 = uint32_t(p1);
-#endif
-        c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
+        c = make_uint4(uint32_t(p1 >> 32) ^ c.y ^ k0, uint32_t(p1), uint32_t(p0 >> 32) ^ c.w ^ k1, uint32_t(p0));
         k0 += 0x9E3779B9u;
         k1 += 0xBB67AE85u;
     }
     return c;
 }
 
-// 23-bit uniform in the open interval (0,1): (floor(x/2^9) + 1/2) / 2^23 is
-// exactly representable in FP32, so it never rounds to 0 or 1.
+// 23-bit uniform in the open interval (0,1): (floor(x/2^9) + 1/2) / 2^23,
+// exactly representable in FP32, so it never rounds to 0 or 1.  The top 23
+// bits become the mantissa of a float in [1, 2) (one funnel shift), and
+// subtracting 1 - 2^-24 is exact.
 __device__ __forceinline__ float u01(uint32_t x) {
-    return (float(x >> 9) + 0.5f) * 1.1920928955078125e-07f;
+    return __uint_as_float(__funnelshift_r(x, 0x7Fu, 9)) - 0.999999940395355224609375f;
 }
 
 // Id of the k-th banked secondary: the SplitMix64 output function
@@ -187,11 +182,15 @@ __device__ __forceinline__ void source_load(const Queue& q, uint32_t s, Part& p)
 // Rotate (u,v,w) by polar cosine `cost` and azimuth phi given as (cp, sp).
 // Azimuth reference: e1 = (u w, v w, -(1-w^2))/s, e2 = (-v, u, 0)/s with
 // s = sqrt(1-w^2); for s^2 < 1e-10 the x and y axes.  The result is
-// renormalised.
-__device__ __forceinline__ void rotate(float& u, float& v, float& w, float cost, float cp,
-                                       float sp) {
-    const float sint = sqrtf(fmaxf(0.f, 1.f - cost * cost));
-    const float s2 = 1.f - w * w;
+// renormalised.  Which products are fused is spelled out, here and wherever a
+// sum of two products decides a history: left to the compiler it changes
+// with the surrounding code, and a history's result with it.  TURNED: the
+// Moller primary, whose (cp, sp) are the delta ray's negated, fuses the
+// other product of each pair.
+template <bool TURNED = false>
+__device__ __forceinline__ void rotate(float& u, float& v, float& w, float cost, float cp, float sp) {
+    const float sint = sqrtf(fmaxf(0.f, fmaf(-cost, cost, 1.f)));
+    const float s2 = fmaf(-w, w, 1.f);
     float un, vn, wn;
     if (s2 < 1e-10f) {
         un = cost * u + sint * cp;
@@ -200,12 +199,16 @@ __device__ __forceinline__ void rotate(float& u, float& v, float& w, float cost,
     } else {
         const float s = sqrtf(s2);
         const float is = 1.f / s;
-        un = cost * u + sint * (cp * u * w - sp * v) * is;
-        vn = cost * v + sint * (cp * v * w + sp * u) * is;
-        wn = cost * w - sint * cp * s;
+        const float cu = __fmul_rn(cp, u), cv = __fmul_rn(cp, v);
+        // a = cp u w - sp v, b = cp v w + sp u
+        const float a = TURNED ? fmaf(cu, w, -__fmul_rn(sp, v)) : fmaf(-sp, v, __fmul_rn(cu, w));
+        const float b = TURNED ? fmaf(sp, u, __fmul_rn(cv, w)) : fmaf(cv, w, __fmul_rn(sp, u));
+        un = fmaf(cost, u, __fmul_rn(__fmul_rn(sint, a), is));
+        vn = fmaf(cost, v, __fmul_rn(__fmul_rn(sint, b), is));
+        wn = fmaf(cost, w, -__fmul_rn(__fmul_rn(sint, cp), s));
     }
-    const float n = rsqrtf(un * un + vn * vn + wn * wn);
-    u = un * n; v = vn * n; w = wn * n;
+    const float n = rsqrtf(fmaf(wn, wn, fmaf(un, un, __fmul_rn(vn, vn))));
+    u = __fmul_rn(un, n); v = __fmul_rn(vn, n); w = __fmul_rn(wn, n);
 }
 
 // cos and sin of 2*pi*r for r in (0,1): evaluated at the angle 2*pi*r - pi in

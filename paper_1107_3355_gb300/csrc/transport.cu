@@ -8,8 +8,10 @@
 // terminates, so warps stay full until the input is drained instead of
 // idling on their longest history.  A lane advances its particle by one
 // step per iteration:
-//   photon:   Woodcock flights against the majorant until a real collision
-//             (Sec. 2.1), then one Compton / photoelectric / pair event;
+//   photon:   one Woodcock flight against the majorant (Sec. 2.1); photons
+//             that collide wait in shared memory until the warp has 32 of
+//             them, and their Compton / photoelectric / pair events run
+//             together;
 //   electron: one condensed-history step (CSDA loss over the step, random
 //             hinge multiple scattering, voxel walk depositing along the
 //             path) and, at a hard-event candidate, Moller or
@@ -35,16 +37,22 @@ constexpr float kEs = 21.2f;            // Rossi-Greisen scattering energy, MeV
 constexpr uint32_t kFull = 0xffffffffu;
 
 // CTA shape each phase kernel is compiled for: threads per CTA and the
-// resident CTAs per SM that fix its register budget.  The photon kernel fits
-// 64 registers at 4 x 256 threads; so does the whole-step electron kernel,
-// with a few spilled words, and the extra warps hide more latency than the
-// spills cost (6 MV slab electron phase -4.6 %).  The resumable electron
+// resident CTAs per SM that fix its register budget.  The photon kernel's
+// stacks take 3.8 KB of shared memory a warp: one CTA of 768 threads stages
+// the tables once and leaves the L1 its half (1024 threads at 64 registers
+// spill and were 4 % slower, 640 threads 4-6 %).  The whole-step electron
+// kernel fits 64 registers at 4 x 256 threads with a few spilled words, and
+// the extra warps hide more latency than the spills cost (6 MV slab electron
+// phase -4.6 %).  The resumable electron
 // kernel keeps its step state across the loop top: at 2 x 448 threads (72
 // registers, 24 bytes spilled, 28 warps per SM) it beats 3 x 256 (80
 // registers, no spill, 24 warps) by 2.7 % on the CT plan; at 4 x 256 (64
 // registers) it spills that state, +12 %.
+#ifndef GDPM_THREADS_PHOTON
+#define GDPM_THREADS_PHOTON 768
+#endif
 #ifndef GDPM_MIN_CTAS_PHOTON
-#define GDPM_MIN_CTAS_PHOTON 4
+#define GDPM_MIN_CTAS_PHOTON 1
 #endif
 #ifndef GDPM_MIN_CTAS_ELECTRON_WHOLE
 #define GDPM_MIN_CTAS_ELECTRON_WHOLE 4
@@ -57,18 +65,11 @@ constexpr uint32_t kFull = 0xffffffffu;
 #endif
 template <int PT>
 struct PhaseShape {
-    static constexpr int threads = PT == 2 ? GDPM_THREADS_ELECTRON : 256;
+    static constexpr int threads = PT == 0 ? GDPM_THREADS_PHOTON : PT == 2 ? GDPM_THREADS_ELECTRON : 256;
     static constexpr int ctas = PT == 0 ? GDPM_MIN_CTAS_PHOTON
                                 : PT == 1 ? GDPM_MIN_CTAS_ELECTRON_WHOLE
                                           : GDPM_MIN_CTAS_ELECTRON;
 };
-
-// Threads per CTA of phase kernel PT: its own shape, or the context's
-// GDPM_PARAM_BLOCK_THREADS when set (at most 256, within every kernel's bound).
-int phase_threads(const gdpm_ctx* ctx, int pt) {
-    if (ctx->block_threads > 0) return ctx->block_threads;
-    return pt == 0 ? PhaseShape<0>::threads : pt == 1 ? PhaseShape<1>::threads : PhaseShape<2>::threads;
-}
 
 // ---------------------------------------------------------------- ledger/tally
 struct Acc {
@@ -97,7 +98,11 @@ struct Sec {
     float E1, E2, dx, dy, dz;
 };
 
-// Deposit e MeV in voxel vox of the tally of the batch in `flags`.
+// Deposit e MeV in voxel vox of the tally of the batch in `flags`.  GEN: the
+// general form, which looks at the tally mode and, below, at the per-history
+// records; the phase kernels also exist without it (FP64 tally, no records),
+// which saves its tests at every deposit and event.
+template <bool GEN>
 __device__ __forceinline__ void tally(const SimParams& P, uint32_t flags, uint32_t vox0, float e) {
     size_t vox = size_t(vox0) + size_t((flags & kBatchMask) >> kBatchShift) * P.batch_stride;
 #if GDPM_CHECKED
@@ -106,7 +111,7 @@ __device__ __forceinline__ void tally(const SimParams& P, uint32_t flags, uint32
         vox = P.tally_lo;
     }
 #endif
-    if (P.tally_mode == 0) {
+    if (!GEN || P.tally_mode == 0) {
         atomicAdd(&P.edep[vox], double(e));
     } else {
         // FP32 pair: hi accumulates, lo collects the exact rounding error of
@@ -123,11 +128,13 @@ __device__ __forceinline__ uint32_t vox_of(const SimParams& P, int ix, int iy, i
     return uint32_t(ix) + uint32_t(P.nx) * (uint32_t(iy) + uint32_t(P.ny) * uint32_t(iz));
 }
 
+template <bool GEN>
 __device__ __forceinline__ void hist_count(const SimParams& P, uint32_t hist, int k) {
-    if (P.hrec) atomicAdd(&P.hrec[size_t(GDPM_IDX(P.status, hist, P.n_records, ST_B_RECORD)) * 4 + k], 1);
+    if (GEN && P.hrec) atomicAdd(&P.hrec[size_t(GDPM_IDX(P.status, hist, P.n_records, ST_B_RECORD)) * 4 + k], 1);
 }
+template <bool GEN>
 __device__ __forceinline__ void hist_add(const SimParams& P, uint32_t hist, int k, double v) {
-    if (P.hrec) atomicAdd(&P.hrecd[size_t(GDPM_IDX(P.status, hist, P.n_records, ST_B_RECORD)) * 2 + k], v);
+    if (GEN && P.hrec) atomicAdd(&P.hrecd[size_t(GDPM_IDX(P.status, hist, P.n_records, ST_B_RECORD)) * 2 + k], v);
 }
 #if GDPM_CHECKED
 __device__ __forceinline__ uint32_t n_voxels(const SimParams& P) {
@@ -139,24 +146,25 @@ __device__ __forceinline__ uint32_t n_voxels(const SimParams& P) {
 // Klein-Nishina in eps = E'/E by the two-branch mixture method: with weight
 // ln(1/eps0) sample from 1/eps, with weight (1-eps0^2)/2 from eps, accept
 // with 1 - eps sin^2(theta)/(1+eps^2).  Draws: (branch, eps, accept, phi).
-__device__ __forceinline__ void sample_kn(Part& p, const SimParams& P, float E, float& eps,
-                                          float& cost, float& rphi) {
+__device__ __forceinline__ bool kn_trial(uint4 r, float E, float& eps, float& cost, float& rphi) {
     const float k = E * (1.f / kMC2f);
     const float e0 = 1.f / fmaf(2.f, k, 1.f);
     const float a1 = -__logf(e0), a2 = 0.5f * (1.f - e0 * e0);
-    float t = 0.f;
-    eps = 1.f;
-    rphi = 0.5f;
-    for (int it = 0; it < 4096; ++it) {
-        const float4 c = draw(p, P.key0, P.key1);
-        if (c.x * (a1 + a2) < a1) eps = __expf(-a1 * c.y);
-        else eps = sqrtf(fmaf(1.f - e0 * e0, c.y, e0 * e0));
-        t = (1.f - eps) / (k * eps);
-        const float g = 1.f - eps * t * (2.f - t) / fmaf(eps, eps, 1.f);
-        rphi = c.w;
-        if (c.z <= g) break;
-    }
+    const float4 c = make_float4(u01(r.x), u01(r.y), u01(r.z), u01(r.w));
+    if (c.x * (a1 + a2) < a1) eps = __expf(-a1 * c.y);
+    else eps = sqrtf(fmaf(1.f - e0 * e0, c.y, e0 * e0));
+    const float t = (1.f - eps) / (k * eps);
+    const float g = 1.f - eps * t * (2.f - t) / fmaf(eps, eps, 1.f);
+    rphi = c.w;
     cost = 1.f - t;
+    return c.z <= g;
+}
+// A whole Klein-Nishina event (checks of the sampler).
+__device__ __forceinline__ void sample_kn(Part& p, const SimParams& P, float E, float& eps,
+                                          float& cost, float& rphi) {
+    for (int it = 0; it < 4096; ++it)
+        if (kn_trial(philox_block(p.hist, p.pidlo, p.pidhi, p.ctr++, P.key0, P.key1), E, eps, cost, rphi))
+            break;
 }
 
 // Moller: eps = W/T on [W_cc/T, 1/2] from the 1/eps^2 proposal, accepted with
@@ -370,7 +378,7 @@ __device__ bool make_primary(const SimParams& P, const PhaseArgs& A, uint32_t id
     acc.src += p.E;
     if (!enter_box(P, p)) {
         acc.esc += p.E;
-        hist_add(P, p.hist, 0, p.E);
+        hist_add<true>(P, p.hist, 0, p.E);
         return false;
     }
     voxel_of(P, p);
@@ -378,121 +386,125 @@ __device__ bool make_primary(const SimParams& P, const PhaseArgs& A, uint32_t id
 }
 
 // ---------------------------------------------------------------- photon step
-// Woodcock flights a photon takes per iteration of the phase loop.  A photon
-// crossing air or lung makes many virtual flights against a majorant set by
-// bone; past this many it continues in the next iteration, so it does not
-// hold the warp while the other lanes interact and are refilled.  Between
-// flights a photon carries nothing but its position and draw counter, so
-// the cap changes no draw and no result.  3 was measured best against 2, 4,
-// 5, 6, 8 and no cap (CT plan: photon phase -17 %).
-constexpr int kFlightsPerTrip = 3;
-
 struct PhSmem {
     const float* maj;
     const float* tot;
     const float2* cum;
 };
 
-__device__ void photon_step(const SimParams& P, const PhSmem& S, Part& p, bool& active, Acc& acc,
-                            Ev& ev, Sec& sec) {
+// Outcome of a flight: the photon makes a virtual (delta) collision and flies
+// on, leaves the phantom, or waits for its event.
+enum class Flight { fly, gone, wait };
+
+// What a waiting photon waits for is kept in its state: a photoelectric event
+// sets kAbsorbed in its flags (no photon uses the positron bit), a pair has
+// the sign of its energy set, a Compton event neither.
+constexpr uint32_t kAbsorbed = 0x80000000u;
+
+// One Woodcock flight against the majorant (Sec. 2.1) with the draw x.
+template <bool GEN>
+__device__ __forceinline__ Flight photon_flight(const SimParams& P, const PhSmem& S, Part& p, uint4 x,
+                                                Acc& acc, Ev& ev) {
     const DevTables& T = P.T;
-    if (p.E < T.eabs_ph) {   // only a source photon below the cutoff reaches here
-        tally(P, p.flags, vox_of(P, p.ix, p.iy, p.iz), p.E);
-        ev.b += EV_TERM;
-        active = false;
-        return;
-    }
-    // Woodcock flights at fixed energy until a real collision (or escape), so
-    // that the interaction below runs with the warp's lanes together; at most
-    // kFlightsPerTrip of them per iteration.
     int i;
     float f;
     grid_pos(T, p.E, i, f);
     const float mm = lerpf(S.maj[i], S.maj[i + 1], f);
     const float inv_mm = 1.f / mm;
-    float4 r;
-    uint32_t vox;
-    float mt;
-    int mi;
-    for (int flight = 0;; ++flight) {
-        // a photon still in virtual flights after kFlightsPerTrip of them
-        // goes on in the next iteration (the same draws: one block a flight)
-        if (flight == kFlightsPerTrip) return;
-        r = draw(p, P.key0, P.key1);
-        const float s = -__logf(r.x) * inv_mm;
-        p.x = fmaf(s, p.u, p.x);
-        p.y = fmaf(s, p.v, p.y);
-        p.z = fmaf(s, p.w, p.z);
-        if (!inside(P, p.x, p.y, p.z)) {
-            acc.esc += p.E;
-            hist_add(P, p.hist, 0, p.E);
-            ev.b += EV_TERM;
-            active = false;
-            return;
-        }
-        ++ev.n;
-        voxel_of(P, p);
-        vox = GDPM_IDX(P.status, vox_of(P, p.ix, p.iy, p.iz), n_voxels(P), ST_B_VOXEL);
-        const int m = GDPM_IDX(P.status, int(__ldg(&P.mat[vox])), T.n_mat, ST_B_TABLE);
-        const float rho = __ldg(&P.rho[vox]);
-        mi = m * T.n_e + i;
-        mt = lerpf(S.tot[mi], S.tot[mi + 1], f);
-        if (r.y * mm < mt * rho) break;             // real; otherwise a virtual (delta) collision
+    const float s = -__logf(u01(x.x)) * inv_mm;
+    p.x = fmaf(s, p.u, p.x);
+    p.y = fmaf(s, p.v, p.y);
+    p.z = fmaf(s, p.w, p.z);
+    if (!inside(P, p.x, p.y, p.z)) {
+        acc.esc += p.E;
+        hist_add<GEN>(P, p.hist, 0, p.E);
+        ev.b += EV_TERM;
+        return Flight::gone;
     }
+    ++ev.n;
+    voxel_of(P, p);
+    const uint32_t vox = GDPM_IDX(P.status, vox_of(P, p.ix, p.iy, p.iz), n_voxels(P), ST_B_VOXEL);
+    const int m = GDPM_IDX(P.status, int(__ldg(&P.mat[vox])), T.n_mat, ST_B_TABLE);
+    const float rho = __ldg(&P.rho[vox]);
+    const int mi = m * T.n_e + i;
+    const float mt = lerpf(S.tot[mi], S.tot[mi + 1], f);
+    if (!(u01(x.y) * mm < mt * rho)) return Flight::fly;
     ev.a += EV_REAL;
-    hist_count(P, p.hist, 0);
+    hist_count<GEN>(P, p.hist, 0);
     const float2 c0 = S.cum[mi], c1 = S.cum[mi + 1];
-    const float rr = r.z * mt;
-    sec.n = 1;
-    sec.photon = false;
-    sec.dx = p.u; sec.dy = p.v; sec.dz = p.w;
-    if (rr < lerpf(c0.x, c1.x, f)) {
-        // Compton (Klein-Nishina); recoil electron along E u - E' u'
-        ev.a += EV_COMPTON;
-        const float E = p.E;
-        float eps, cost, rphi;
-        sample_kn(p, P, E, eps, cost, rphi);
-        float cp, sp;
-        cossin_2pi(rphi, cp, sp);
-        rotate(p.u, p.v, p.w, cost, cp, sp);
-        const float Ep = eps * E;
-        sec.E1 = E - Ep;
-        float dx = E * sec.dx - Ep * p.u, dy = E * sec.dy - Ep * p.v, dz = E * sec.dz - Ep * p.w;
-        const float en = rsqrtf(dx * dx + dy * dy + dz * dz);
-        sec.dx = dx * en; sec.dy = dy * en; sec.dz = dz * en;
-        sec.pos2 = false;
-        if (Ep < T.eabs_ph) {
-            tally(P, p.flags, vox, Ep);
-            ev.b += EV_LOCAL + EV_TERM;
-            active = false;
+    const float rr = u01(x.z) * mt;
+    if (!(rr < lerpf(c0.x, c1.x, f))) {
+        if (rr < lerpf(c0.y, c1.y, f)) {
+            p.flags |= kAbsorbed;
         } else {
-            p.E = Ep;
+            p.E = -p.E;
+            --p.ctr;        // the event shares the energy with this draw's last uniform
         }
-    } else if (rr < lerpf(c0.y, c1.y, f)) {
-        // photoelectric: photon absorbed, photoelectron along the photon (or
-        // at Sauter's angle to it, physics variant)
-        ev.a += EV_PHOTO;
-        ev.b += EV_TERM;
-        sec.E1 = p.E;
-        sec.pos2 = false;
-        active = false;
-        if (T.flags & GDPM_FLAG_SAUTER) {
-            float mu, rphi, cp, sp;
-            sample_sauter(p, P, p.E, mu, rphi);
-            cossin_2pi(rphi, cp, sp);
-            rotate(sec.dx, sec.dy, sec.dz, mu, cp, sp);
-        }
-    } else {
-        // pair: electron takes r.w of the kinetic energy, positron the rest
-        ev.a += EV_PAIR;
-        ev.b += EV_TERM;
-        const float tav = p.E - 2.f * kMC2f;
-        sec.E1 = r.w * tav;
-        sec.E2 = tav - sec.E1;
-        sec.n = 2;
-        sec.pos2 = true;
-        active = false;
     }
+    return Flight::wait;
+}
+
+// The event a photon waits for, with the draw x at its counter: pair
+// production (the electron takes the flight's last uniform of the kinetic
+// energy, the positron the rest), photoelectric absorption (photoelectron
+// along the photon, or at Sauter's angle to it, physics variant), or one
+// trial of a Compton event (`force` accepts any).  False when the trial was
+// rejected.  After a Compton event the photon has turned and lost energy,
+// with a recoil electron along E u - E' u', and `goes_on` says whether it
+// stays above its absorption energy (below it, it is deposited here).
+template <bool GEN>
+__device__ __forceinline__ bool photon_event(const SimParams& P, Part& p, uint4 x, bool force, bool& goes_on,
+                                             Ev& ev, Sec& sec) {
+    const float E = p.E;
+    sec.n = 1;
+    sec.dx = p.u; sec.dy = p.v; sec.dz = p.w;
+    sec.pos2 = false;
+    if (E < 0.f || (p.flags & kAbsorbed)) {
+        ev.b += EV_TERM;
+        if (E < 0.f) {
+            ev.a += EV_PAIR;
+            const float tav = -E - 2.f * kMC2f;
+            sec.E1 = u01(x.w) * tav;
+            sec.E2 = tav - sec.E1;
+            sec.n = 2;
+            sec.pos2 = true;
+        } else {
+            ev.a += EV_PHOTO;
+            p.flags &= ~kAbsorbed;
+            sec.E1 = E;
+            if (P.T.flags & GDPM_FLAG_SAUTER) {
+                float mu, rphi, cp, sp;
+                sample_sauter(p, P, E, mu, rphi);
+                cossin_2pi(rphi, cp, sp);
+                rotate(sec.dx, sec.dy, sec.dz, mu, cp, sp);
+            }
+        }
+        return true;
+    }
+    ++p.ctr;
+    float eps, cost, rphi;
+    if (!kn_trial(x, E, eps, cost, rphi) && !force) {
+        sec.n = 0;
+        return false;
+    }
+    ev.a += EV_COMPTON;
+    float cp, sp;
+    cossin_2pi(rphi, cp, sp);
+    rotate(p.u, p.v, p.w, cost, cp, sp);
+    const float Ep = __fmul_rn(eps, E);
+    sec.E1 = __fsub_rn(E, Ep);
+    const float dx = fmaf(E, sec.dx, -__fmul_rn(Ep, p.u)), dy = fmaf(E, sec.dy, -__fmul_rn(Ep, p.v)),
+                dz = fmaf(E, sec.dz, -__fmul_rn(Ep, p.w));
+    const float en = rsqrtf(fmaf(dz, dz, fmaf(dx, dx, __fmul_rn(dy, dy))));
+    sec.dx = dx * en; sec.dy = dy * en; sec.dz = dz * en;
+    goes_on = !(Ep < P.T.eabs_ph);
+    if (goes_on) {
+        p.E = Ep;
+    } else {
+        tally<GEN>(P, p.flags, vox_of(P, p.ix, p.iy, p.iz), Ep);
+        ev.b += EV_LOCAL + EV_TERM;
+    }
+    return true;
 }
 
 // ---------------------------------------------------------------- electron step
@@ -540,6 +552,7 @@ struct ElStep {
 // One DDA trip: the particle either ends its leg inside the current voxel
 // (1) or moves to the voxel's exit face, tallies, and crosses (0, or 2 when
 // it leaves the phantom).
+template <bool GEN>
 __device__ __forceinline__ int walk_trip(const SimParams& P, Part& p, ElStep& s, float iu, float iv,
                                          float iw, int sx, int sy, int sz, uint32_t& vox,
                                          uint32_t& crossings, float& pend) {
@@ -566,7 +579,7 @@ __device__ __forceinline__ int walk_trip(const SimParams& P, Part& p, ElStep& s,
     p.z = fmaf(tb, p.w, p.z);
     const float piece = rho * tb;
     const float e = s.dpm * piece;
-    if (e + pend > 0.f) tally(P, p.flags, vox, e + pend);
+    if (e + pend > 0.f) tally<GEN>(P, p.flags, vox, e + pend);
     s.dep += e;
     pend = 0.f;
     s.left -= piece;
@@ -613,6 +626,7 @@ __device__ __forceinline__ void hinge(Part& p, ElStep& s, float& pend) {
 // direction (a NaN position falls to the z branch), and the walk leaves the
 // grid within nx + ny + nz trips.  (A counted guard here cost 8-14 % of the
 // electron phase in code generation, for no case it could catch.)
+template <bool GEN>
 __device__ int walk_whole(const SimParams& P, Part& p, ElStep& s, uint32_t& crossings, float& pend) {
 #pragma unroll 1
     for (;;) {
@@ -624,7 +638,7 @@ __device__ int walk_whole(const SimParams& P, Part& p, ElStep& s, uint32_t& cros
         int res;
 #pragma unroll 1
         do {
-            res = walk_trip(P, p, s, iu, iv, iw, sx, sy, sz, vox, crossings, pend);
+            res = walk_trip<GEN>(P, p, s, iu, iv, iw, sx, sy, sz, vox, crossings, pend);
         } while (res == 0);
         if (res == 2 || s.leg == 2) return res;
         hinge<false>(p, s, pend);
@@ -633,6 +647,7 @@ __device__ int walk_whole(const SimParams& P, Part& p, ElStep& s, uint32_t& cros
 
 // Resumable form: at most kWalkTrips trips, turning at the hinge within the
 // budget.
+template <bool GEN>
 __device__ int walk_resumable(const SimParams& P, Part& p, ElStep& s, uint32_t& crossings,
                               float& pend) {
     float iu = p.u != 0.f ? 1.f / p.u : 0.f;
@@ -642,7 +657,7 @@ __device__ int walk_resumable(const SimParams& P, Part& p, ElStep& s, uint32_t& 
     uint32_t vox = vox_of(P, p.ix, p.iy, p.iz);
 #pragma unroll 1
     for (int trip = 0; trip < kWalkTrips; ++trip) {
-        const int res = walk_trip(P, p, s, iu, iv, iw, sx, sy, sz, vox, crossings, pend);
+        const int res = walk_trip<GEN>(P, p, s, iu, iv, iw, sx, sy, sz, vox, crossings, pend);
         if (res == 2 || (res == 1 && s.leg == 2)) return res;
         if (res == 1) {
             hinge<true>(p, s, pend);
@@ -655,6 +670,7 @@ __device__ int walk_resumable(const SimParams& P, Part& p, ElStep& s, uint32_t& 
     return 0;
 }
 
+template <bool GEN>
 __device__ void electron_escape(const SimParams& P, Part& p, float energy, Acc& acc) {
     double e = energy;
     if (p.flags & kPositron) {
@@ -662,7 +678,7 @@ __device__ void electron_escape(const SimParams& P, Part& p, float energy, Acc& 
         else acc.disc += 2.0 * kMC2;
     }
     acc.esc += e;
-    hist_add(P, p.hist, 0, e);
+    hist_add<GEN>(P, p.hist, 0, e);
 }
 
 // One condensed-history step of an electron or positron (Sec. 2.1), or its
@@ -671,7 +687,7 @@ __device__ void electron_escape(const SimParams& P, Part& p, float energy, Acc& 
 // voxel walk may take several calls (several iterations of the phase loop),
 // and the step's end (escape, absorption, hard-event candidate) runs in the
 // call whose walk reaches it.
-template <bool RESUME>
+template <bool RESUME, bool GEN>
 __device__ __forceinline__ void electron_step(const SimParams& P, const ElSmem& S, Part& p, bool& active,
                                               Acc& acc, Ev& ev, Sec& sec, float& pend, ElStep& carried) {
     const DevTables& T = P.T;
@@ -685,7 +701,7 @@ __device__ __forceinline__ void electron_step(const SimParams& P, const ElSmem& 
         if (!absorb) {
             const float4 r = draw(p, P.key0, P.key1);
             ev.b += EV_STEP;
-            hist_count(P, p.hist, 1);
+            hist_count<GEN>(P, p.hist, 1);
             // material and density of the start voxel, loaded together
             const uint32_t vox0 = GDPM_IDX(P.status, vox_of(P, p.ix, p.iy, p.iz), n_voxels(P), ST_B_VOXEL);
             const int m = GDPM_IDX(P.status, int(__ldg(&P.mat[vox0])), T.n_mat, ST_B_TABLE);
@@ -719,7 +735,7 @@ __device__ __forceinline__ void electron_step(const SimParams& P, const ElSmem& 
             }
             const float Tk = p.E;
             const float dT = Tk - Tend;
-            if (P.hrec) hist_add(P, p.hist, 1, double(xs));
+            hist_add<GEN>(P, p.hist, 1, double(xs));
             // multiple scattering at the mid-step energy
             const float Tm = 0.5f * (Tk + Tend);
             const float pbc = Tm * (Tm + 2.f * kMC2f) / (Tm + kMC2f);
@@ -754,12 +770,12 @@ __device__ __forceinline__ void electron_step(const SimParams& P, const ElSmem& 
         }
     }
     if (!absorb) {
-        const int res = RESUME ? walk_resumable(P, p, st, ev.n, pend) : walk_whole(P, p, st, ev.n, pend);
+        const int res = RESUME ? walk_resumable<GEN>(P, p, st, ev.n, pend) : walk_whole<GEN>(P, p, st, ev.n, pend);
         if (res == 0) return;            // the walk goes on in the next iteration
         st.leg = 0;
         const float Tk = p.E;
         if (res == 2) {
-            electron_escape(P, p, Tk - st.dep, acc);
+            electron_escape<GEN>(P, p, Tk - st.dep, acc);
             ev.b += EV_TERM;
             active = false;
             return;
@@ -786,7 +802,7 @@ __device__ __forceinline__ void electron_step(const SimParams& P, const ElSmem& 
             }
             const float sh = sm + sb;
             if (v.x * T.sigmax[m] < sh) {
-                hist_count(P, p.hist, 2);
+                hist_count<GEN>(P, p.hist, 2);
                 sec.n = 1;
                 sec.pos2 = false;
                 if (v.y * sh < sm) {
@@ -802,7 +818,7 @@ __device__ __forceinline__ void electron_step(const SimParams& P, const ElSmem& 
                     rotate(sec.dx, sec.dy, sec.dz, cd, c, sn);
                     sec.photon = false;
                     sec.E1 = W;
-                    rotate(p.u, p.v, p.w, cpr, -c, -sn);
+                    rotate<true>(p.u, p.v, p.w, cpr, -c, -sn);
                     p.E = Tp;
                 } else {
                     ev.c += EV_BREMS;
@@ -819,7 +835,7 @@ __device__ __forceinline__ void electron_step(const SimParams& P, const ElSmem& 
         // end of track: residual energy deposited here; a positron then
         // annihilates into two back-to-back 0.511 MeV photons (isotropic),
         // or its rest energy is discarded (Sec. 2.1, Sec. 4)
-        tally(P, p.flags, vox_of(P, p.ix, p.iy, p.iz), p.E + pend);
+        tally<GEN>(P, p.flags, vox_of(P, p.ix, p.iy, p.iz), p.E + pend);
         pend = 0.f;
         ev.b += EV_TERM;
         active = false;
@@ -925,21 +941,23 @@ __device__ __forceinline__ uint32_t reserve(Slots& sl, uint32_t c, uint32_t* cou
 // Bank the secondaries the lanes' last steps created (call with the whole
 // warp): below-cutoff electrons and photons deposit on the spot, the rest
 // get slots in the warp's reservations and counter-derived ids.
+template <int PT, bool GEN>
 __device__ __forceinline__ void bank_pending(const SimParams& P, const PhaseArgs& A, Part& p,
                                              const Sec& sec, Slots (&sl)[2], WarpCnt& wc) {
+    const bool photon = PT != 0 && sec.photon;      // photons create electrons only
     const uint32_t lane = lane_id();
     for (int k = 0; k < 2; ++k) {
         const bool want = k < sec.n;
         if (!__any_sync(kFull, want)) return;
         const bool pos = k == 1 && sec.pos2;
         const float E = k ? sec.E2 : sec.E1;
-        const float sg = (k == 1 && sec.photon) ? -1.f : 1.f;
-        const bool push = want && (pos || E >= (sec.photon ? P.T.eabs_ph : P.T.eabs_el));
-        if (want && !push) tally(P, p.flags, vox_of(P, p.ix, p.iy, p.iz), E);
+        const float sg = (k == 1 && photon) ? -1.f : 1.f;
+        const bool push = want && (pos || E >= (photon ? P.T.eabs_ph : P.T.eabs_el));
+        if (want && !push) tally<GEN>(P, p.flags, vox_of(P, p.ix, p.iy, p.iz), E);
         wc.w0 += __popc(__ballot_sync(kFull, want && !push));
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {           // q = 0 electron queue, 1 photon queue
-            const bool mine = push && (sec.photon == (q == 1));
+        for (int q = 0; q < (PT == 0 ? 1 : 2); ++q) {   // q = 0 electron queue, 1 photon queue
+            const bool mine = push && (photon == (q == 1));
             const uint32_t m = __ballot_sync(kFull, mine);
             if (!m) continue;
             const uint32_t c = __popc(m);
@@ -967,7 +985,7 @@ __device__ __forceinline__ void bank_pending(const SimParams& P, const PhaseArgs
                 const Queue& Q = q ? A.out_ph : A.out_el;
                 if (slot < Q.capacity) queue_store(Q, slot, ch);
                 else atomicOr(P.status, ST_QUEUE_OVERFLOW);
-                hist_count(P, p.hist, 3);
+                hist_count<GEN>(P, p.hist, 3);
             }
             if (q) wc.w1 += c; else wc.w0 += c << 16;
         }
@@ -995,13 +1013,93 @@ __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(
 // and 256); near the end of a phase the grabs turn exact.
 constexpr uint32_t kGrab = 128u;
 
-// One transport phase (Sec. 2.2.1 Step 3): a persistent loop per warp.
-// Loop top (whole warp): fold event counters now and then, bank the
-// secondaries of the last step, refill lanes whose particle ended.  Then
-// each lane takes one step of its own particle.  PT: 0 photons, 1 electrons
-// a whole step per iteration, 2 electrons with resumable steps.
+// What a warp leaves behind at the end of its phase: event counts, empty
+// marks on the queue slots it reserved but never wrote, its share of the
+// ledger; then the CTA's counters.
 template <int PT>
-__device__ __forceinline__ void phase_run(const SimParams& P, const PhaseArgs& A) {
+__device__ __forceinline__ void phase_end(const SimParams& P, const PhaseArgs& A, Acc& acc, Ev& ev,
+                                          WarpCnt& wc, const Slots (&sl)[2], uint32_t* s_cnt) {
+    const uint32_t lane = lane_id();
+    flush_events<PT>(ev, s_cnt);
+    flush_warp_counts<PT>(wc, s_cnt);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const Queue& Q = q ? A.out_ph : A.out_el;
+        const uint32_t slot = sl[q].base + lane;
+        if (lane < sl[q].left && slot < Q.capacity) queue_mark_empty(Q, slot);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        acc.src += __shfl_down_sync(kFull, acc.src, o);
+        acc.esc += __shfl_down_sync(kFull, acc.esc, o);
+        acc.disc += __shfl_down_sync(kFull, acc.disc, o);
+    }
+    if (lane == 0) {
+        if (acc.src != 0.0) atomicAdd(&P.ledger[L_SOURCE], acc.src);
+        if (acc.esc != 0.0) atomicAdd(&P.ledger[L_ESCAPED], acc.esc);
+        if (acc.disc != 0.0) atomicAdd(&P.ledger[L_DISCARDED], acc.disc);
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < C_NCOUNT; k += blockDim.x)
+        if (s_cnt[k]) atomicAdd(&P.counters[k], (unsigned long long)s_cnt[k]);
+}
+
+// Particle idx of the phase's input (its primaries first, then the queue)
+// into p; false for an empty slot (a primary that missed the phantom, which
+// k_sources accounts, or a reserved slot that was never written).
+__device__ __forceinline__ bool load_input(const SimParams& P, const PhaseArgs& A, uint32_t idx, Part& p,
+                                           bool& from_queue) {
+    if (idx < A.n_src) {
+        source_load(A.src, GDPM_IDX(P.status, idx, A.src.capacity, ST_B_QUEUE), p);
+        p.hist = A.src_first + idx;
+        return p.E >= 0.f;
+    }
+    queue_load(A.in, GDPM_IDX(P.status, idx - A.n_src, A.in.capacity, ST_B_QUEUE), p);
+    from_queue = p.E >= 0.f;
+    return from_queue;
+}
+
+// ---------------------------------------------------------------- photon phase
+// A warp's photons that are not in a lane: a stack in shared memory that
+// holds the ones ready to fly (from the bottom) and the ones waiting for a
+// Compton event (from the top).
+struct PhRec {
+    uint4 a, b, c;      // x y z E | u v w flags | history, particle id lo, hi, draw counter
+};
+constexpr uint32_t kPhReady = 16, kPhStack = kPhReady + 64;
+
+__device__ __forceinline__ void rec_store(PhRec& r, const Part& p) {
+    r.a = pack4(p.x, p.y, p.z, __float_as_uint(p.E));
+    r.b = pack4(p.u, p.v, p.w, p.flags);
+    r.c = make_uint4(p.hist, p.pidlo, p.pidhi, p.ctr);
+}
+__device__ __forceinline__ void rec_load(const PhRec& r, Part& p) {
+    const uint4 a = r.a, b = r.b, c = r.c;
+    p.x = __uint_as_float(a.x); p.y = __uint_as_float(a.y); p.z = __uint_as_float(a.z);
+    p.E = __uint_as_float(a.w);
+    p.u = __uint_as_float(b.x); p.v = __uint_as_float(b.y); p.w = __uint_as_float(b.z);
+    p.flags = b.w;
+    p.hist = c.x; p.pidlo = c.y; p.pidhi = c.z; p.ctr = c.w;
+}
+
+// The photon phase.  Every lane of a warp takes one Woodcock flight per round.
+// A photon that collides is set aside in shared memory and its lane takes
+// another photon; once 32 wait, a round runs one Klein-Nishina trial (or the
+// photoelectric absorption) of each, all lanes at work, and the accepted ones
+// go back to fly.  Flights, rejection trials and recoil banking in one lane's
+// own loop, as each lane reached them, kept 14 of 32 lanes active; now 27 are.
+// Measured (1e8 histories of the CT plan / 2.5e8 of the paper's lung slab):
+// 22.5 -> 20.6 ms / 36.0 -> 28.1 ms; 160 instead of 225 warp instructions a
+// history.  What is left is the latency of the voxel loads (24 warps) and
+// the round's own control.  New
+// photons come kPhReady at a time into the stack, not one by one as lanes
+// fall free.  Both kinds of round start with one draw, at one place in the
+// code: a single inlined copy of the generator, which leaves the loop without
+// calls and its constants in uniform registers.
+// Stack bounds: photons enter the warp (and free lanes take one) only while
+// at most 31 wait, and only up to kPhReady ready; 32 more are in the lanes.
+template <bool GEN>
+__device__ __forceinline__ void photon_run(const SimParams& P, const PhaseArgs& A) {
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t n_in = A.in_count ? min(*A.in_count, A.in.capacity) : 0u;
     const uint32_t total = A.n_src + n_in;
@@ -1009,31 +1107,154 @@ __device__ __forceinline__ void phase_run(const SimParams& P, const PhaseArgs& A
 
     const DevTables& T = P.T;
     const size_t ne = size_t(T.n_mat) * T.n_e;
-    PhSmem ps{};
-    ElSmem es{};
-    uint32_t* s_cnt;
-    if (PT == 0) {
-        float2* cum = reinterpret_cast<float2*>(smem);
-        float* tot = reinterpret_cast<float*>(smem + align16(ne * 8));
-        float* maj = reinterpret_cast<float*>(smem + align16(ne * 8) + align16(ne * 4));
-        s_cnt = reinterpret_cast<uint32_t*>(smem + align16(ne * 8) + align16(ne * 4) +
-                                            align16(size_t(T.n_e) * 4));
-        copy_to_smem(cum, T.ph_cum, ne * 8);
-        copy_to_smem(tot, T.ph_tot, ne * 4);
-        copy_to_smem(maj, P.maj, size_t(T.n_e) * 4);
-        ps.maj = maj; ps.tot = tot; ps.cum = cum;
-    } else {
-        float4* el = reinterpret_cast<float4*>(smem);
-        float* rinv = reinterpret_cast<float*>(smem + ne * 16);
-        const size_t nr = size_t(T.n_mat) * T.n_r;
-        float* atab = reinterpret_cast<float*>(smem + ne * 16 + align16(nr * 4));
-        s_cnt = reinterpret_cast<uint32_t*>(smem + ne * 16 + align16(nr * 4) +
-                                            align16(size_t(T.n_a) * 4));
-        copy_to_smem(el, T.el, ne * 16);
-        copy_to_smem(rinv, T.rinv, nr * 4);
-        copy_to_smem(atab, T.atab, size_t(T.n_a) * 4);
-        es.el = el; es.rinv = rinv; es.atab = atab;
+    float2* cum = reinterpret_cast<float2*>(smem);
+    float* tot = reinterpret_cast<float*>(smem + align16(ne * 8));
+    float* maj = reinterpret_cast<float*>(smem + align16(ne * 8) + align16(ne * 4));
+    unsigned char* after = smem + align16(ne * 8) + align16(ne * 4) + align16(size_t(T.n_e) * 4);
+    uint32_t* s_cnt = reinterpret_cast<uint32_t*>(after);
+    PhRec* stack = reinterpret_cast<PhRec*>(after + align16(C_NCOUNT * 4)) + (threadIdx.x >> 5) * kPhStack;
+    copy_to_smem(cum, T.ph_cum, ne * 8);
+    copy_to_smem(tot, T.ph_tot, ne * 4);
+    copy_to_smem(maj, P.maj, size_t(T.n_e) * 4);
+    const PhSmem ps{maj, tot, cum};
+    for (int k = threadIdx.x; k < C_NCOUNT; k += blockDim.x) s_cnt[k] = 0u;
+    __syncthreads();
+
+    Acc acc{0.0, 0.0, 0.0};
+    Part p{};
+    Ev ev{0u, 0u, 0u, 0u};
+    WarpCnt wc{0u, 0u, 0u};
+    Slots sl[2] = {{0u, 0u}, {0u, 0u}};
+    const uint32_t lane = lane_id(), lt = lanemask_lt();
+    bool active = false;
+    uint32_t alive = 0u;                         // ballot of `active`
+    uint32_t n_ready = 0u, n_wait = 0u;          // the stack: [0, n_ready) and [kPhStack - n_wait, kPhStack)
+    uint32_t st_base = 0u, st_left = 0u;         // the warp's block of work indices
+    bool st_exact = false, drained = false;      // drained: no input left
+    for (uint32_t it = 0, trials = 0;; ++it) {
+        if ((it % kFlushEvery) == kFlushEvery - 1u) {
+            flush_events<0>(ev, s_cnt);
+            flush_warp_counts<0>(wc, s_cnt);
+        }
+        while (n_wait < 32u && alive != kFull) {
+            const uint32_t nm = ~alive, need = __popc(nm);
+            // ---- input into the stack, up to kPhReady ready
+            if (n_ready < min(need, kPhReady) && !drained) {
+                if (st_left == 0u) {
+                    const uint32_t block = st_exact ? need : kGrab;
+                    uint32_t nb = 0u;
+                    if (lane == 0) nb = atomicAdd(A.head, block);
+                    nb = __shfl_sync(kFull, nb, 0);
+                    st_base = nb;
+                    st_left = nb < total ? min(block, total - nb) : 0u;
+                    if (nb >= total || total - nb < 2u * gridDim.x * blockDim.x) st_exact = true;
+                    drained = st_left == 0u;
+                }
+                const uint32_t k = min(kPhReady - n_ready, st_left);
+                Part q;
+                bool from_queue = false, have = false;
+                if (lane < k) have = load_input(P, A, st_base + lane, q, from_queue);
+                st_base += k;
+                st_left -= k;
+                wc.w2 += __popc(__ballot_sync(kFull, from_queue));
+                if (have && q.E < T.eabs_ph) {   // only a source photon below the cutoff
+                    voxel_of(P, q);
+                    tally<GEN>(P, q.flags, vox_of(P, q.ix, q.iy, q.iz), q.E);
+                    ev.b += EV_TERM;
+                    have = false;
+                }
+                const uint32_t m = __ballot_sync(kFull, have);
+                if (have) rec_store(stack[n_ready + __popc(m & lt)], q);
+                n_ready += __popc(m);
+                __syncwarp();
+            }
+            // ---- free lanes take ready photons
+            const uint32_t r = __popc(nm & lt);
+            if (!active && r < n_ready) {
+                rec_load(stack[n_ready - 1u - r], p);
+                active = true;
+            }
+            n_ready -= min(need, n_ready);
+            __syncwarp();
+            alive = __ballot_sync(kFull, active);
+            if (drained) break;
+        }
+        // ---- which round: events once 32 photons wait, or, when the input is
+        // drained, once no fewer wait than fly
+        const uint32_t fly = __popc(alive) + n_ready;
+        const bool events = n_wait >= 32u || (drained && n_wait >= fly);
+        if (fly + n_wait == 0u) break;
+        if (it >= P.max_iters) {
+            if (lane == 0) atomicOr(P.status, ST_ITER_CAP);
+            break;
+        }
+        const uint32_t k = min(n_wait, 32u);
+        const PhRec* const rec = stack + (kPhStack - n_wait) + (lane < k ? lane : 0u);   // the k last set aside
+        uint4 c = make_uint4(p.hist, p.pidlo, p.pidhi, p.ctr);
+        if (events) c = rec->c;
+        const uint4 x = philox4x32_10(c, P.key0, P.key1);
+        if (!events) {
+            trials = 0u;
+            Flight what = Flight::fly;
+            if (active) {
+                ++p.ctr;
+                what = photon_flight<GEN>(P, ps, p, x, acc, ev);
+                active = what == Flight::fly;
+            }
+            alive = __ballot_sync(kFull, active);
+            const uint32_t m = __ballot_sync(kFull, what == Flight::wait);
+            if (what == Flight::wait) rec_store(stack[kPhStack - 1u - n_wait - __popc(m & lt)], p);
+            n_wait += __popc(m);
+            __syncwarp();
+        } else {
+            ++trials;
+            Part q{};
+            Sec sec{};
+            bool goes_on = false, done = true;
+            if (lane < k) {
+                rec_load(*rec, q);
+                voxel_of(P, q);
+                done = photon_event<GEN>(P, q, x, trials > 4096u, goes_on, ev, sec);
+            }
+            n_wait -= k;
+            bank_pending<0, GEN>(P, A, q, sec, sl, wc);
+            __syncwarp();
+            const uint32_t gm = __ballot_sync(kFull, goes_on), wm = __ballot_sync(kFull, !done);
+            if (goes_on || !done)
+                rec_store(stack[goes_on ? n_ready + __popc(gm & lt) : kPhStack - 1u - n_wait - __popc(wm & lt)], q);
+            n_ready += __popc(gm);
+            n_wait += __popc(wm);
+            __syncwarp();
+        }
     }
+    phase_end<0>(P, A, acc, ev, wc, sl, s_cnt);
+}
+
+// ---------------------------------------------------------------- electron phase
+// The electron phase: loop top (whole warp): fold event counters now and
+// then, bank the secondaries of the last step, refill lanes whose particle
+// ended.  Then each lane takes one step of its own particle.  PT: 1 a whole
+// step per iteration, 2 resumable steps.
+template <int PT, bool GEN>
+__device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs& A) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const uint32_t n_in = A.in_count ? min(*A.in_count, A.in.capacity) : 0u;
+    const uint32_t total = A.n_src + n_in;
+    if (total == 0u || blockIdx.x * blockDim.x >= total) return;
+
+    const DevTables& T = P.T;
+    const size_t ne = size_t(T.n_mat) * T.n_e;
+    ElSmem es{};
+    float4* el = reinterpret_cast<float4*>(smem);
+    float* rinv = reinterpret_cast<float*>(smem + ne * 16);
+    const size_t nr = size_t(T.n_mat) * T.n_r;
+    float* atab = reinterpret_cast<float*>(smem + ne * 16 + align16(nr * 4));
+    uint32_t* s_cnt = reinterpret_cast<uint32_t*>(smem + ne * 16 + align16(nr * 4) +
+                                        align16(size_t(T.n_a) * 4));
+    copy_to_smem(el, T.el, ne * 16);
+    copy_to_smem(rinv, T.rinv, nr * 4);
+    copy_to_smem(atab, T.atab, size_t(T.n_a) * 4);
+    es.el = el; es.rinv = rinv; es.atab = atab;
     for (int k = threadIdx.x; k < C_NCOUNT; k += blockDim.x) s_cnt[k] = 0u;
     __syncthreads();
 
@@ -1058,7 +1279,7 @@ __device__ __forceinline__ void phase_run(const SimParams& P, const PhaseArgs& A
             flush_events<PT>(ev, s_cnt);
             flush_warp_counts<PT>(wc, s_cnt);
         }
-        bank_pending(P, A, p, sec, sl, wc);
+        bank_pending<PT, GEN>(P, A, p, sec, sl, wc);
         sec.n = 0;
         const bool need = !active && !exhausted;
         const uint32_t nm = __ballot_sync(kFull, need);
@@ -1081,20 +1302,9 @@ __device__ __forceinline__ void phase_run(const SimParams& P, const PhaseArgs& A
             if (need) {
                 const uint32_t r = __popc(nm & lanemask_lt());
                 const uint32_t idx = r < left0 ? base0 + r : nb + (r - left0);
-                if (idx < A.n_src) {
-                    // made by k_sources; a primary that missed the phantom
-                    // left its slot empty (E < 0) and is accounted there
-                    source_load(A.src, GDPM_IDX(P.status, idx, A.src.capacity, ST_B_QUEUE), p);
-                    active = p.E >= 0.f;
-                    if (active) {
-                        p.hist = A.src_first + idx;
-                        voxel_of(P, p);
-                    }
-                } else if (idx < total) {
-                    queue_load(A.in, GDPM_IDX(P.status, idx - A.n_src, A.in.capacity, ST_B_QUEUE), p);
-                    // a slot reserved but never written holds E < 0
-                    from_queue = p.E >= 0.f;
-                    active = from_queue;
+                if (idx < total) {
+                    active = load_input(P, A, idx, p, from_queue);
+                    if (active && idx < A.n_src) voxel_of(P, p);
                 } else {
                     exhausted = true;
                 }
@@ -1108,41 +1318,27 @@ __device__ __forceinline__ void phase_run(const SimParams& P, const PhaseArgs& A
         }
         // ---- each lane on its own: one step
         if (active) {
-            if (PT == 0) photon_step(P, ps, p, active, acc, ev, sec);
-            else electron_step<PT == 2>(P, es, p, active, acc, ev, sec, pend, est);
+            electron_step<PT == 2, GEN>(P, es, p, active, acc, ev, sec, pend, est);
         }
     }
     // only a phase stopped by its iteration cap leaves a track unfinished
-    if (PT != 0 && pend != 0.f) tally(P, p.flags, vox_of(P, p.ix, p.iy, p.iz), pend);
-    flush_events<PT>(ev, s_cnt);
-    flush_warp_counts<PT>(wc, s_cnt);
-    // reserved queue slots never written: mark them empty for the consumer
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const Queue& Q = q ? A.out_ph : A.out_el;
-        const uint32_t slot = sl[q].base + lane;
-        if (lane < sl[q].left && slot < Q.capacity) queue_mark_empty(Q, slot);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        acc.src += __shfl_down_sync(kFull, acc.src, o);
-        acc.esc += __shfl_down_sync(kFull, acc.esc, o);
-        acc.disc += __shfl_down_sync(kFull, acc.disc, o);
-    }
-    if (lane == 0) {
-        if (acc.src != 0.0) atomicAdd(&P.ledger[L_SOURCE], acc.src);
-        if (acc.esc != 0.0) atomicAdd(&P.ledger[L_ESCAPED], acc.esc);
-        if (acc.disc != 0.0) atomicAdd(&P.ledger[L_DISCARDED], acc.disc);
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < C_NCOUNT; k += blockDim.x)
-        if (s_cnt[k]) atomicAdd(&P.counters[k], (unsigned long long)s_cnt[k]);
+    if (pend != 0.f) tally<GEN>(P, p.flags, vox_of(P, p.ix, p.iy, p.iz), pend);
+    phase_end<PT>(P, A, acc, ev, wc, sl, s_cnt);
 }
 
-template <int PT>
+// One transport phase (Sec. 2.2.1 Step 3), a persistent loop per warp.  PT: 0
+// photons, 1 electrons a whole step per iteration, 2 electrons with resumable
+// steps.
+template <int PT, bool GEN>
+__device__ __forceinline__ void phase_run(const SimParams& P, const PhaseArgs& A) {
+    if constexpr (PT == 0) photon_run<GEN>(P, A);
+    else electron_run<PT, GEN>(P, A);
+}
+
+template <int PT, bool GEN>
 __global__ void __launch_bounds__(PhaseShape<PT>::threads, PhaseShape<PT>::ctas)
 k_phase(const SimParams P, const PhaseArgs A) {
-    phase_run<PT>(P, A);
+    phase_run<PT, GEN>(P, A);
 }
 
 
@@ -1280,7 +1476,7 @@ k_phase_loop(const SimParams P, const LoopArgs L) {
     __shared__ PhaseArgs sA;
     if (threadIdx.x == 0) sA = phase_args(L, *L.k + (PT == 0 ? 0u : 1u));
     __syncthreads();
-    phase_run<PT>(P, sA);
+    phase_run<PT, true>(P, sA);
 }
 
 // Primaries of this pass's source phase (before it runs).
@@ -1452,6 +1648,7 @@ __global__ void k_debug_sources(const SimParams P, const PhaseArgs A, uint64_t n
 
 }  // namespace
 
+// Shared memory of a phase's tables and counters.
 static size_t smem_of(const DevTables& T, int particle) {
     const size_t ne = size_t(T.n_mat) * T.n_e;
     const size_t cnt = align16(C_NCOUNT * 4);
@@ -1462,18 +1659,41 @@ static size_t smem_of(const DevTables& T, int particle) {
 
 int transport_smem(const gdpm_tables* t, int particle) { return int(smem_of(t->dev, particle)); }
 
+// A phase kernel's launch shape: its own CTA, or the context's
+// GDPM_PARAM_BLOCK_THREADS when set (at most 256, within every kernel's
+// bound); the tables and counters of a CTA and the warps' stacks in shared
+// memory.  Beside large tables a CTA has fewer warps.
+struct Launch {
+    int threads;
+    size_t smem;
+};
+static Launch phase_shape(const gdpm_ctx* ctx, const DevTables& T, int pt) {
+    constexpr size_t kMaxSmem = size_t(227) << 10;
+    const size_t tables = smem_of(T, pt == 0 ? GDPM_PHOTON : GDPM_ELECTRON);
+    const size_t stack = pt == 0 ? kPhStack * sizeof(PhRec) : 0;
+    int thr = ctx->block_threads > 0 ? ctx->block_threads
+              : pt == 0              ? PhaseShape<0>::threads
+              : pt == 1              ? PhaseShape<1>::threads
+                                     : PhaseShape<2>::threads;
+    if (stack) thr = std::min(thr, 32 * int((kMaxSmem - tables) / stack));
+    return Launch{thr, tables + stack * size_t(thr / 32)};
+}
+
 // Persistent grid: SM count x resident CTAs per SM for this shared-memory size.
 // share_eighths < 8 gives the grid that many eighths of the GPU: a large
 // request that runs while small ones are active leaves SMs free for them,
 // since persistent CTAs do not yield until their phase's input is drained.
 int launch_phase(gdpm_ctx* ctx, cudaStream_t st, int particle, const SimParams& P,
                  const PhaseArgs& A, uint32_t n_items_hint, uint32_t share_eighths) {
-    const size_t smem = smem_of(P.T, particle);
     const bool resumable = particle != GDPM_PHOTON && P.walk_resumable;
-    const int thr = phase_threads(ctx, particle == GDPM_PHOTON ? 0 : resumable ? 2 : 1);
-    const void* fn = particle == GDPM_PHOTON ? (const void*)k_phase<0>
-                     : resumable              ? (const void*)k_phase<2>
-                                              : (const void*)k_phase<1>;
+    const Launch shape = phase_shape(ctx, P.T, particle == GDPM_PHOTON ? 0 : resumable ? 2 : 1);
+    const int thr = shape.threads;
+    const size_t smem = shape.smem;
+    using Kernel = void (*)(const SimParams, const PhaseArgs);
+    const bool gen = P.tally_mode != 0 || P.hrec;
+    const Kernel fn = particle == GDPM_PHOTON ? (gen ? k_phase<0, true> : k_phase<0, false>)
+                      : resumable             ? (gen ? k_phase<2, true> : k_phase<2, false>)
+                                              : (gen ? k_phase<1, true> : k_phase<1, false>);
     GDPM_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
     int bps = ctx->blocks_per_sm;
     if (bps <= 0) {
@@ -1494,12 +1714,7 @@ int launch_phase(gdpm_ctx* ctx, cudaStream_t st, int particle, const SimParams& 
     const uint64_t cap = std::min(A.out_el.capacity, A.out_ph.capacity);
     const uint64_t bb = std::min<uint64_t>(32u, cap / (8u * warps));
     B.bank_block = bb >= 8u ? uint32_t(bb) : 0u;
-    if (particle == GDPM_PHOTON)
-        k_phase<0><<<grid, thr, smem, st>>>(P, B);
-    else if (resumable)
-        k_phase<2><<<grid, thr, smem, st>>>(P, B);
-    else
-        k_phase<1><<<grid, thr, smem, st>>>(P, B);
+    fn<<<grid, thr, smem, st>>>(P, B);
     GDPM_CUDA_TRY(cudaGetLastError());
     return GDPM_OK;
 }
@@ -1543,10 +1758,12 @@ int build_loop_graph(gdpm_ctx* ctx, const SimParams& P, LoopArgs& L, bool metrop
     const void* fn[2] = {(const void*)k_phase_loop<0>,
                          P.walk_resumable ? (const void*)k_phase_loop<2>
                                           : (const void*)k_phase_loop<1>};
-    const int thr[2] = {phase_threads(ctx, 0), phase_threads(ctx, P.walk_resumable ? 2 : 1)};
+    int thr[2];
     uint64_t warps = 0;
     for (int t = 0; t < 2; ++t) {
-        smem[t] = smem_of(P.T, t == 0 ? GDPM_PHOTON : GDPM_ELECTRON);
+        const Launch shape = phase_shape(ctx, P.T, t == 0 ? 0 : P.walk_resumable ? 2 : 1);
+        thr[t] = shape.threads;
+        smem[t] = shape.smem;
         GDPM_CUDA_TRY(cudaFuncSetAttribute(fn[t], cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem[t])));
         int bps = ctx->blocks_per_sm;
         if (bps <= 0) {
