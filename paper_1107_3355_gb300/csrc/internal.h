@@ -87,7 +87,11 @@ struct PhaseArgs {
     Queue out_ph, out_el;      // where secondaries are banked
     uint32_t* out_ph_count;
     uint32_t* out_el_count;
-    uint32_t bank_block;       // queue slots a warp reserves at a time (0: exactly what it pushes)
+    // queue slots a warp reserves at a time (0: exactly what it pushes), and at
+    // most half its even share of the phase's input: a small phase would leave
+    // the next one mostly reserved slots that were never written
+    uint32_t bank_block;
+    uint32_t share_shift;      // items >> share_shift: at most half a warp's even share of them
     // dose matrix: n_sub sub-problems (one per fluence-map row), sub-problem
     // k owning histories [sub_first[k], sub_first[k+1]) in nb_small batches
     // each; 0 for a single problem
@@ -110,6 +114,7 @@ struct LoopArgs {
     uint32_t* pick;
     uint32_t n_src, first, chunk;
     uint32_t nb_small, nb_rem, n_sub, sub_batches, bank_block;
+    uint32_t share_shift[2];   // of the photon and the electron phases
     int src_particle, max_phases;
 };
 

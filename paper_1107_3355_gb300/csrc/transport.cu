@@ -917,19 +917,19 @@ struct Slots {
 };
 
 // `c` consecutive slots for the warp's pushes to one queue: from the
-// reservation first, then a new reservation of max(missing, block) slots
-// (one atomic).  Returns the first slot of the new reservation (or of the
+// reservation first, then a new reservation of PhaseArgs::bank_block slots
+// (one atomic; fewer in a phase of few particles).  Returns the first slot of the new reservation (or of the
 // old one when it sufficed); a lane of rank r < old left writes slot
 // old.base + r, the others new + (r - old left).
-__device__ __forceinline__ uint32_t reserve(Slots& sl, uint32_t c, uint32_t* count, uint32_t block,
-                                            int leader) {
+__device__ __forceinline__ uint32_t reserve(Slots& sl, uint32_t c, uint32_t* count, const PhaseArgs& A,
+                                            uint32_t total, int leader) {
     if (c <= sl.left) {
         const uint32_t b = sl.base;
         sl.base += c;
         sl.left -= c;
         return b;
     }
-    const uint32_t miss = c - sl.left, want = max(miss, block);
+    const uint32_t miss = c - sl.left, want = max(miss, min(A.bank_block, total >> A.share_shift));
     uint32_t nb = 0;
     if (int(lane_id()) == leader) nb = atomicAdd(count, want);
     nb = __shfl_sync(kFull, nb, leader);
@@ -942,7 +942,7 @@ __device__ __forceinline__ uint32_t reserve(Slots& sl, uint32_t c, uint32_t* cou
 // warp): below-cutoff electrons and photons deposit on the spot, the rest
 // get slots in the warp's reservations and counter-derived ids.
 template <int PT, bool GEN>
-__device__ __forceinline__ void bank_pending(const SimParams& P, const PhaseArgs& A, Part& p,
+__device__ __forceinline__ void bank_pending(const SimParams& P, const PhaseArgs& A, uint32_t total, Part& p,
                                              const Sec& sec, Slots (&sl)[2], WarpCnt& wc) {
     const bool photon = PT != 0 && sec.photon;      // photons create electrons only
     const uint32_t lane = lane_id();
@@ -962,8 +962,7 @@ __device__ __forceinline__ void bank_pending(const SimParams& P, const PhaseArgs
             if (!m) continue;
             const uint32_t c = __popc(m);
             const uint32_t left0 = sl[q].left, base0 = sl[q].base;
-            const uint32_t nb = reserve(sl[q], c, q ? A.out_ph_count : A.out_el_count, A.bank_block,
-                                        __ffs(m) - 1);
+            const uint32_t nb = reserve(sl[q], c, q ? A.out_ph_count : A.out_el_count, A, total, __ffs(m) - 1);
             if (mine) {
                 Part ch;
                 ch.x = p.x; ch.y = p.y; ch.z = p.z;
@@ -1010,8 +1009,20 @@ __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(
 // then queued particles): one atomic per block instead of one per refill.
 // Every block boundary costs the warp a round trip to the shared counter,
 // so blocks are several refills deep (128: measured best against 32, 64
-// and 256); near the end of a phase the grabs turn exact.
+// and 256).  A block is at most half the warp's even share of the work left
+// (PhaseArgs::share_shift), so blocks shrink towards the end of a phase, down
+// to exactly what the warp needs, and no warp sits on spare work.
 constexpr uint32_t kGrab = 128u;
+
+// Lanes of a warp that take particles.  A phase with less than one particle
+// per lane (a small calculation, the last phases of any) is bound by the
+// latency of a warp's loop, which grows with the lanes that diverge in it:
+// its particles are spread over all resident warps.  Measured: 1e4 histories of
+// a pencil in water 0.29 -> 0.20 ms a call, one CT beamlet of 1e5 1.09 -> 0.94,
+// 1e6 20 MeV electrons on the 128^3 slab 6.0 -> 5.5 ms.
+__device__ __forceinline__ uint32_t phase_lanes(uint32_t total) {
+    return min((total - 1u) / (gridDim.x * (blockDim.x >> 5)) + 1u, 32u);
+}
 
 // What a warp leaves behind at the end of its phase: event counts, empty
 // marks on the queue slots it reserved but never wrote, its share of the
@@ -1066,7 +1077,7 @@ __device__ __forceinline__ bool load_input(const SimParams& P, const PhaseArgs& 
 struct PhRec {
     uint4 a, b, c;      // x y z E | u v w flags | history, particle id lo, hi, draw counter
 };
-constexpr uint32_t kPhReady = 16, kPhStack = kPhReady + 64;
+constexpr uint32_t kPhReady = 32, kPhStack = kPhReady + 64;
 
 __device__ __forceinline__ void rec_store(PhRec& r, const Part& p) {
     r.a = pack4(p.x, p.y, p.z, __float_as_uint(p.E));
@@ -1103,7 +1114,8 @@ __device__ __forceinline__ void photon_run(const SimParams& P, const PhaseArgs& 
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t n_in = A.in_count ? min(*A.in_count, A.in.capacity) : 0u;
     const uint32_t total = A.n_src + n_in;
-    if (total == 0u || blockIdx.x * blockDim.x >= total) return;
+    if (blockIdx.x >= total) return;
+    const uint32_t lanes = phase_lanes(total), full = kFull >> (32u - lanes);
 
     const DevTables& T = P.T;
     const size_t ne = size_t(T.n_mat) * T.n_e;
@@ -1130,24 +1142,23 @@ __device__ __forceinline__ void photon_run(const SimParams& P, const PhaseArgs& 
     uint32_t alive = 0u;                         // ballot of `active`
     uint32_t n_ready = 0u, n_wait = 0u;          // the stack: [0, n_ready) and [kPhStack - n_wait, kPhStack)
     uint32_t st_base = 0u, st_left = 0u;         // the warp's block of work indices
-    bool st_exact = false, drained = false;      // drained: no input left
+    bool drained = false;                        // no input left
     for (uint32_t it = 0, trials = 0;; ++it) {
         if ((it % kFlushEvery) == kFlushEvery - 1u) {
             flush_events<0>(ev, s_cnt);
             flush_warp_counts<0>(wc, s_cnt);
         }
-        while (n_wait < 32u && alive != kFull) {
-            const uint32_t nm = ~alive, need = __popc(nm);
+        while (n_wait < 32u && alive != full) {
+            const uint32_t nm = full & ~alive, need = __popc(nm);
             // ---- input into the stack, up to kPhReady ready
             if (n_ready < min(need, kPhReady) && !drained) {
                 if (st_left == 0u) {
-                    const uint32_t block = st_exact ? need : kGrab;
+                    const uint32_t block = max(need, min((total - min(total, st_base)) >> A.share_shift, kGrab));
                     uint32_t nb = 0u;
                     if (lane == 0) nb = atomicAdd(A.head, block);
                     nb = __shfl_sync(kFull, nb, 0);
                     st_base = nb;
                     st_left = nb < total ? min(block, total - nb) : 0u;
-                    if (nb >= total || total - nb < 2u * gridDim.x * blockDim.x) st_exact = true;
                     drained = st_left == 0u;
                 }
                 const uint32_t k = min(kPhReady - n_ready, st_left);
@@ -1170,7 +1181,7 @@ __device__ __forceinline__ void photon_run(const SimParams& P, const PhaseArgs& 
             }
             // ---- free lanes take ready photons
             const uint32_t r = __popc(nm & lt);
-            if (!active && r < n_ready) {
+            if (!active && r < n_ready && lane < lanes) {
                 rec_load(stack[n_ready - 1u - r], p);
                 active = true;
             }
@@ -1217,7 +1228,7 @@ __device__ __forceinline__ void photon_run(const SimParams& P, const PhaseArgs& 
                 done = photon_event<GEN>(P, q, x, trials > 4096u, goes_on, ev, sec);
             }
             n_wait -= k;
-            bank_pending<0, GEN>(P, A, q, sec, sl, wc);
+            bank_pending<0, GEN>(P, A, total, q, sec, sl, wc);
             __syncwarp();
             const uint32_t gm = __ballot_sync(kFull, goes_on), wm = __ballot_sync(kFull, !done);
             if (goes_on || !done)
@@ -1240,7 +1251,7 @@ __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t n_in = A.in_count ? min(*A.in_count, A.in.capacity) : 0u;
     const uint32_t total = A.n_src + n_in;
-    if (total == 0u || blockIdx.x * blockDim.x >= total) return;
+    if (blockIdx.x >= total) return;
 
     const DevTables& T = P.T;
     const size_t ne = size_t(T.n_mat) * T.n_e;
@@ -1264,22 +1275,19 @@ __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs
     Ev ev{0u, 0u, 0u, 0u};
     WarpCnt wc{0u, 0u, 0u};
     Slots sl[2] = {{0u, 0u}, {0u, 0u}};
-    bool active = false, exhausted = false;
+    const uint32_t lane = lane_id();
+    bool active = false, exhausted = lane >= phase_lanes(total);
     float pend = 0.f;   // electron energy owed to its current voxel (see walk)
     ElStep est{};       // electron step in progress (leg 0: none)
-    // the warp's block of work indices [st_base, st_base + st_left); near
-    // the end of the phase (less than two per lane of the grid left) the
-    // warp takes exactly what it needs, so no warp sits on spare work
+    // the warp's block of work indices [st_base, st_base + st_left)
     uint32_t st_base = 0u, st_left = 0u;
-    bool st_exact = false;
-    const uint32_t lane = lane_id();
     for (uint32_t it = 0;; ++it) {
         // ---- whole warp: account and bank the last step, then refill
         if ((it % kFlushEvery) == kFlushEvery - 1u) {
             flush_events<PT>(ev, s_cnt);
             flush_warp_counts<PT>(wc, s_cnt);
         }
-        bank_pending<PT, GEN>(P, A, p, sec, sl, wc);
+        bank_pending<PT, GEN>(P, A, total, p, sec, sl, wc);
         sec.n = 0;
         const bool need = !active && !exhausted;
         const uint32_t nm = __ballot_sync(kFull, need);
@@ -1288,12 +1296,12 @@ __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs
             const uint32_t left0 = st_left, base0 = st_base;
             uint32_t nb = 0u;
             if (k > st_left) {
-                const uint32_t miss = k - st_left, want = st_exact ? miss : max(miss, kGrab);
+                const uint32_t miss = k - st_left;
+                const uint32_t want = max(miss, min((total - min(total, st_base)) >> A.share_shift, kGrab));
                 if (lane == 0) nb = atomicAdd(A.head, want);
                 nb = __shfl_sync(kFull, nb, 0);
                 st_base = nb + miss;
                 st_left = want - miss;
-                if (nb >= total || total - nb < 2u * gridDim.x * blockDim.x) st_exact = true;
             } else {
                 st_base += k;
                 st_left -= k;
@@ -1433,6 +1441,7 @@ __device__ __forceinline__ PhaseArgs phase_args(const LoopArgs& L, uint32_t k) {
     A.bank_block = L.bank_block;
     A.src = L.qsrc;
     const bool ph = (k % 2u) == 0u;
+    A.share_shift = L.share_shift[ph ? 0 : 1];
     const bool src_phase = ph == (L.src_particle == GDPM_PHOTON);
     if (src_phase) {
         const uint32_t j = L.src_particle == GDPM_PHOTON ? k / 2u : (k - 1u) / 2u;
@@ -1657,6 +1666,14 @@ static size_t smem_of(const DevTables& T, int particle) {
     return ne * 16 + align16(size_t(T.n_mat) * T.n_r * 4) + align16(size_t(T.n_a) * 4) + cnt;
 }
 
+// log2 of at least twice the warps of a phase: items >> shift is at most half
+// a warp's even share of them.
+static uint32_t share_shift(uint32_t warps) {
+    uint32_t s = 1u;
+    while ((1ull << s) < 2ull * warps) ++s;
+    return s;
+}
+
 int transport_smem(const gdpm_tables* t, int particle) { return int(smem_of(t->dev, particle)); }
 
 // A phase kernel's launch shape: its own CTA, or the context's
@@ -1703,8 +1720,7 @@ int launch_phase(gdpm_ctx* ctx, cudaStream_t st, int particle, const SimParams& 
     uint32_t grid = uint32_t(ctx->sm_count) * uint32_t(bps);
     if (share_eighths < 8) grid = std::max<uint32_t>(uint32_t(ctx->sm_count), grid * share_eighths / 8);
     if (n_items_hint > 0) {
-        const uint32_t need = (n_items_hint + thr - 1) / thr;
-        grid = need < grid ? need : grid;
+        grid = std::min(grid, n_items_hint);   // a CTA has at least one particle
     }
     if (grid == 0) grid = 1;
     // queue slots a warp reserves at a time: up to 32, while all warps'
@@ -1714,6 +1730,7 @@ int launch_phase(gdpm_ctx* ctx, cudaStream_t st, int particle, const SimParams& 
     const uint64_t cap = std::min(A.out_el.capacity, A.out_ph.capacity);
     const uint64_t bb = std::min<uint64_t>(32u, cap / (8u * warps));
     B.bank_block = bb >= 8u ? uint32_t(bb) : 0u;
+    B.share_shift = share_shift(uint32_t(warps));
     fn<<<grid, thr, smem, st>>>(P, B);
     GDPM_CUDA_TRY(cudaGetLastError());
     return GDPM_OK;
@@ -1772,6 +1789,7 @@ int build_loop_graph(gdpm_ctx* ctx, const SimParams& P, LoopArgs& L, bool metrop
         }
         grid[t] = uint32_t(ctx->sm_count) * uint32_t(bps);
         warps = std::max<uint64_t>(warps, uint64_t(grid[t]) * uint64_t(thr[t] / 32));
+        L.share_shift[t] = share_shift(grid[t] * uint32_t(thr[t] / 32));
     }
     const uint64_t cap = std::min(L.qph.capacity, L.qe0.capacity);
     const uint64_t bb = std::min<uint64_t>(32u, cap / (8u * warps));

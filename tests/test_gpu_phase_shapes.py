@@ -1,0 +1,53 @@
+"""A history's result depends on its id alone: not on how many warps run a
+phase, how many particles a warp holds, or which particles share its stack in
+shared memory.  The same histories under several launch shapes."""
+import numpy as np
+import pytest
+
+from paper_1107_3355_gb300 import gdpm as G
+from paper_1107_3355_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+KEYS = ["n_primary", "ph_created", "ph_terminated", "ph_flights", "ph_real", "compton", "photoelectric",
+        "pair", "el_created", "el_terminated", "el_steps", "moller", "brems", "annihilations",
+        "local_deposits", "crossings"]
+
+
+def problem(kind, n):
+    if kind == "compton":                       # 1 MeV photons in water
+        return W.tiny_problem(n, n_batches=2)
+    ph = W.slab_phantom((17, 23, 40), (0.5, 0.5, 0.5))
+    if kind == "photoelectric":                 # 60 keV photons, Sauter angles, electrons followed to 20 keV
+        return W.Problem(ph, W.pencil_source(ph, 0.06), n, 2, eabs_photon=0.01, eabs_electron=0.02,
+                         e_min=0.005, e_max=0.1, flags=W.FLAG_SAUTER)
+    if kind == "pair":                          # 15 MeV photons: pairs, positrons, annihilation photons
+        return W.Problem(ph, W.pencil_source(ph, 15.0), n, 2, eabs_photon=0.05, eabs_electron=0.2,
+                         e_min=0.005, e_max=16.0)
+    return W.Problem(ph, W.pencil_source(ph, 12.0, W.ELECTRON), n, 2, eabs_photon=0.05, eabs_electron=0.2,
+                     e_min=0.005, e_max=16.0)
+
+
+# fewer particles than warps, about a warp's worth, more than one per lane of
+# the narrow shapes; shapes down to two warps on the whole GPU
+@pytest.mark.parametrize("kind", ["compton", "photoelectric", "pair", "electron"])
+@pytest.mark.parametrize("n", [2, 33, 4097, 60_000])
+def test_results_do_not_depend_on_launch_shape(kind, n):
+    prob = problem(kind, n)
+    ref = None
+    for params in ({}, {G.GDPM_PARAM_BLOCK_THREADS: 64, G.GDPM_PARAM_BLOCKS_PER_SM: 1},
+                   {G.GDPM_PARAM_BLOCK_THREADS: 256}, {G.GDPM_PARAM_SOURCE_CHUNK: max(1, n // 3)},
+                   {G.GDPM_PARAM_ELECTRON_WALK: 1}, {G.GDPM_PARAM_GRAPH: 1}):
+        eng = G.Engine(prob, params=params)
+        try:
+            d, _, st = eng.run()
+            d = d.cpu().numpy()
+        finally:
+            eng.close()
+        events = [st[k] for k in KEYS]
+        assert st["ph_created"] == st["ph_terminated"] and st["el_created"] == st["el_terminated"]
+        if ref is None:
+            ref = d, events
+        assert events == ref[1], params
+        # the same FP64 deposits in another order
+        assert np.all(np.abs(d - ref[0]) <= 1e-11 * ref[0]), params
