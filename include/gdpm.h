@@ -194,13 +194,12 @@ enum {
                                         that reaches it abandons its particles and the call
                                         returns GDPM_E_TIMEOUT; the next call starts clean. */
     GDPM_PARAM_ELECTRON_WALK = 20,   /* electron phase form, same results either way: 1
-                                        resumable steps, whose voxel walk takes at most 3 trips
-                                        per loop iteration and resumes in the next, so a track
-                                        with many voxel crossings does not hold its warp; 0 a
-                                        whole condensed-history step per iteration; 2 (default)
-                                        resumable where the phantom holds voxels below 0.05
-                                        g/cm3 (air: electrons there take steps hundreds of
-                                        voxels long), whole steps otherwise */
+                                        resumable steps, whose voxel walk takes at most 2
+                                        crossings per round of the phase loop and resumes in
+                                        the next, so a track with many voxel crossings does
+                                        not hold its warp; 0 a whole condensed-history step
+                                        per round; 2 (default) the engine's choice (resumable
+                                        steps) */
     GDPM_PARAM_SERVE_BIG_SLOTS = 21, /* serving slots for large requests, in arrival order
                                         (1..15, fewer than GDPM_PARAM_SERVE_SLOTS; default 1);
                                         the other slots serve small requests.  Set before the

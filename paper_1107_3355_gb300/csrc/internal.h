@@ -129,11 +129,11 @@ struct SimParams {
     DevSource S;
     uint32_t key0, key1;
     double* edep;              // FP64 batch tally (MeV)
-    uint64_t batch_stride;     // voxels between batch grids (0: one grid for the current batch)
+    uint32_t batch_stride;     // voxels between batch grids (0: one grid for the current batch)
     float* edep_hi;            // FP32 compensated tally
     float* edep_lo;
     int tally_mode;
-    int walk_resumable;        // electron phase form of this run: 1 resumable steps, 0 whole steps
+    int walk_trips;            // stretches of an electron's voxel walk per round of the phase loop
     unsigned long long* counters;
     double* ledger;
     uint32_t* status;
@@ -172,7 +172,6 @@ struct gdpm_phantom {
     float dx = 0, dy = 0, dz = 0;
     gdpm::Buffer mat, rho, rhomax;   // rhomax: 256 floats, max density per material index
     float rhomax_host[256] = {};
-    float rhomin_host = 0.f;                   // smallest voxel density
     std::map<uint64_t, gdpm::Buffer> maj;    // Woodcock majorant per table set id
 };
 
@@ -273,11 +272,8 @@ struct Runner {
     std::vector<unsigned char> loop_key;
 };
 int runner_init(Runner& r, cudaStream_t stream, bool own_stream);
-// Density below which a voxel counts as air (g/cm3): the electron phase form
-// and the Sec. 3.1 metric's default tissue threshold use it.
-constexpr float kAirDensity = 0.05f;
-// Electron phase form of a run on this phantom: 1 resumable steps, 0 whole steps.
-int walk_form(const gdpm_ctx* ctx, const gdpm_phantom* ph);
+// Electron phase form of a run: 1 resumable steps, 0 whole steps.
+int walk_form(const gdpm_ctx* ctx);
 
 // Host helpers shared by gdpm_simulate's runner and the allocation-free
 // entry point (api.cu).
@@ -332,9 +328,7 @@ struct gdpm_ctx {
     int profile = 0;
     int overlap_fold = 1;
     int use_graph = 0;                         // device-driven phase loop (CUDA graph)
-    int electron_walk = 2;                     // 1: resumable electron steps (k_phase<2>); 0: whole
-                                               // steps (k_phase<1>); 2: resumable where the phantom
-                                               // holds air-like voxels (< 0.05 g/cm3)
+    int electron_walk = 2;                     // GDPM_PARAM_ELECTRON_WALK
     float metric_min_rho = 0.05f;              // sigma/Dmax over voxels at least this dense
     int batch_mode = 0;                        // 0 auto, 1 sequential, 2 side by side
     uint64_t concurrent_max_hist = 4000000000ull;   // auto: histories per batch for side by side

@@ -2,25 +2,21 @@
 //
 // Photon and electron transport run in separate phases (Sec. 2.2.1: only
 // one particle type is in flight at a time; secondaries go to per-type
-// stacks).  Each phase is one persistent launch: every warp keeps its 32
-// lanes busy by refilling a lane from the phase's input (a queue of banked
-// particles, plus freshly generated primaries) whenever the lane's particle
-// terminates, so warps stay full until the input is drained instead of
-// idling on their longest history.  A lane advances its particle by one
-// step per iteration:
-//   photon:   one Woodcock flight against the majorant (Sec. 2.1); photons
-//             that collide wait in shared memory until the warp has 32 of
-//             them, and their Compton / photoelectric / pair events run
-//             together;
-//   electron: one condensed-history step (CSDA loss over the step, random
-//             hinge multiple scattering, voxel walk depositing along the
-//             path) and, at a hard-event candidate, Moller or
-//             bremsstrahlung (Sec. 2.1).
-// A step runs with whatever lanes it diverges into and uses no warp-wide
-// operation.  It leaves its event counts and the secondaries it created in
-// registers; at the top of the next iteration, where all 32 lanes are
-// present, the warp banks those secondaries into the queues and adds the
-// counts with full-warp ballots and reductions.
+// stacks).  Each phase is one persistent launch.  A warp works in rounds:
+//   flight / step round: every lane advances its own particle, a photon by
+//             one Woodcock flight against the majorant, an electron by a
+//             condensed-history step (CSDA loss over the step, random hinge
+//             multiple scattering, voxel walk depositing along the path) or a
+//             part of its walk (Sec. 2.1);
+//   event round: what the particles of a step round ran into (Compton,
+//             photoelectric and pair events; hard-event candidates, Moller
+//             trials, bremsstrahlung, annihilation) happens to few of a
+//             warp's lanes at a time, so those particles wait in the warp's
+//             stack in shared memory and are taken 32 at a time, one draw
+//             each; their secondaries are banked with full-warp ballots.
+// A lane whose particle waits or has ended takes another from the stack, which
+// is refilled from the phase's input (freshly generated primaries, then the
+// queue of banked particles), so warps stay full until the input is drained.
 // Tables live in shared memory (Sec. 2.2.2 reads them by linear
 // interpolation); random numbers come from Philox4x32-10 keyed per history
 // and particle, so results do not depend on scheduling.
@@ -37,57 +33,34 @@ constexpr float kEs = 21.2f;            // Rossi-Greisen scattering energy, MeV
 constexpr uint32_t kFull = 0xffffffffu;
 
 // CTA shape each phase kernel is compiled for: threads per CTA and the
-// resident CTAs per SM that fix its register budget.  The photon kernel's
-// stacks take 3.8 KB of shared memory a warp: one CTA of 768 threads stages
-// the tables once and leaves the L1 its half (1024 threads at 64 registers
-// spill and were 4 % slower, 640 threads 4-6 %).  The whole-step electron
-// kernel fits 64 registers at 4 x 256 threads with a few spilled words, and
-// the extra warps hide more latency than the spills cost (6 MV slab electron
-// phase -4.6 %).  The resumable electron
-// kernel keeps its step state across the loop top: at 2 x 448 threads (72
-// registers, 24 bytes spilled, 28 warps per SM) it beats 3 x 256 (80
-// registers, no spill, 24 warps) by 2.7 % on the CT plan; at 4 x 256 (64
-// registers) it spills that state, +12 %.
+// resident CTAs per SM that fix its register budget.  A warp's stack takes
+// 4.6 KB (photons) or 6.0 KB (electrons) of shared memory, so one CTA stages
+// the tables once and leaves the L1 what it can.  768 threads and 80
+// registers measured best over the workloads: photons at 1024 (64 registers)
+// gain 7 % on the paper's slabs and lose 3 % on the CT phantom, whose voxels
+// miss the smaller L1; electrons at 896 (72 registers) lose 5-8 %, at 640 4 %.
 #ifndef GDPM_THREADS_PHOTON
 #define GDPM_THREADS_PHOTON 768
 #endif
 #ifndef GDPM_MIN_CTAS_PHOTON
 #define GDPM_MIN_CTAS_PHOTON 1
 #endif
-#ifndef GDPM_MIN_CTAS_ELECTRON_WHOLE
-#define GDPM_MIN_CTAS_ELECTRON_WHOLE 4
-#endif
 #ifndef GDPM_THREADS_ELECTRON
-#define GDPM_THREADS_ELECTRON 448
+#define GDPM_THREADS_ELECTRON 768
 #endif
 #ifndef GDPM_MIN_CTAS_ELECTRON
-#define GDPM_MIN_CTAS_ELECTRON 2
+#define GDPM_MIN_CTAS_ELECTRON 1
 #endif
 template <int PT>
 struct PhaseShape {
-    static constexpr int threads = PT == 0 ? GDPM_THREADS_PHOTON : PT == 2 ? GDPM_THREADS_ELECTRON : 256;
-    static constexpr int ctas = PT == 0 ? GDPM_MIN_CTAS_PHOTON
-                                : PT == 1 ? GDPM_MIN_CTAS_ELECTRON_WHOLE
-                                          : GDPM_MIN_CTAS_ELECTRON;
+    static constexpr int threads = PT == 0 ? GDPM_THREADS_PHOTON : GDPM_THREADS_ELECTRON;
+    static constexpr int ctas = PT == 0 ? GDPM_MIN_CTAS_PHOTON : GDPM_MIN_CTAS_ELECTRON;
 };
 
 // ---------------------------------------------------------------- ledger/tally
 struct Acc {
-    double src, esc, disc;
+    double src, esc;
 };
-
-// Per-lane event counters: one byte per kind of event, four kinds to a
-// word, plus the flight (photon) or voxel-crossing (electron) count.  Each
-// kind happens at most once per lane and iteration, so folding the bytes
-// into the block's counters every kFlushEvery (< 256) iterations keeps them
-// from overflowing.
-struct Ev {
-    uint32_t a, b, c, n;
-};
-constexpr uint32_t EV_REAL = 1u, EV_COMPTON = 1u << 8, EV_PHOTO = 1u << 16, EV_PAIR = 1u << 24;  // a
-constexpr uint32_t EV_TERM = 1u, EV_LOCAL = 1u << 8, EV_STEP = 1u << 16, EV_MOLLER = 1u << 24;   // b
-constexpr uint32_t EV_BREMS = 1u, EV_ANNIHIL = 1u << 8;                                          // c
-constexpr uint32_t kFlushEvery = 128u;
 
 // Secondaries created by one step: n of them (0..2) at the particle's
 // current position; the second is a positron (pair) or, for photons, the
@@ -104,7 +77,7 @@ struct Sec {
 // which saves its tests at every deposit and event.
 template <bool GEN>
 __device__ __forceinline__ void tally(const SimParams& P, uint32_t flags, uint32_t vox0, float e) {
-    size_t vox = size_t(vox0) + size_t((flags & kBatchMask) >> kBatchShift) * P.batch_stride;
+    size_t vox = uint64_t((flags & kBatchMask) >> kBatchShift) * P.batch_stride + vox0;
 #if GDPM_CHECKED
     if (vox < P.tally_lo || vox >= P.tally_hi) {
         bounds_fail(P.status, ST_B_TALLY);
@@ -169,23 +142,25 @@ __device__ __forceinline__ void sample_kn(Part& p, const SimParams& P, float E, 
 
 // Moller: eps = W/T on [W_cc/T, 1/2] from the 1/eps^2 proposal, accepted with
 // eps^2 f(eps) / (2 + c1/4).  Draws: (eps, accept, phi, -).
-__device__ __forceinline__ void sample_moller(Part& p, const SimParams& P, float T, float wcc,
-                                              float& eps, float& rphi) {
+__device__ __forceinline__ bool moller_trial(uint4 x, float T, float wcc, float& eps, float& rphi) {
     const float tau = T * (1.f / kMC2f);
     const float g = tau / (tau + 1.f);
     const float c1 = g * g, c2 = (2.f * tau + 1.f) / ((tau + 1.f) * (tau + 1.f));
     const float ec = wcc / T;
     const float bound = 2.f + 0.25f * c1;
-    eps = ec;
-    rphi = 0.5f;
-    for (int it = 0; it < 4096; ++it) {
-        const float4 w = draw(p, P.key0, P.key1);
-        eps = ec / (1.f - w.x * (1.f - 2.f * ec));
-        const float x = eps / (1.f - eps);
-        const float gg = 1.f + x * x + c1 * eps * eps - c2 * x;
-        rphi = w.z;
-        if (w.y * bound <= gg) break;
-    }
+    const float4 w = make_float4(u01(x.x), u01(x.y), u01(x.z), u01(x.w));
+    eps = ec / (1.f - w.x * (1.f - 2.f * ec));
+    const float y = eps / (1.f - eps);
+    const float gg = 1.f + y * y + c1 * eps * eps - c2 * y;
+    rphi = w.z;
+    return w.y * bound <= gg;
+}
+// A whole Moller event (checks of the sampler).
+__device__ __forceinline__ void sample_moller(Part& p, const SimParams& P, float T, float wcc, float& eps,
+                                              float& rphi) {
+    for (int it = 0; it < 4096; ++it)
+        if (moller_trial(philox_block(p.hist, p.pidlo, p.pidhi, p.ctr++, P.key0, P.key1), T, wcc, eps, rphi))
+            break;
 }
 
 // Sauter's K-shell photoelectron distribution (physics variant) in
@@ -404,7 +379,7 @@ constexpr uint32_t kAbsorbed = 0x80000000u;
 // One Woodcock flight against the majorant (Sec. 2.1) with the draw x.
 template <bool GEN>
 __device__ __forceinline__ Flight photon_flight(const SimParams& P, const PhSmem& S, Part& p, uint4 x,
-                                                Acc& acc, Ev& ev) {
+                                                double& esc) {
     const DevTables& T = P.T;
     int i;
     float f;
@@ -416,12 +391,10 @@ __device__ __forceinline__ Flight photon_flight(const SimParams& P, const PhSmem
     p.y = fmaf(s, p.v, p.y);
     p.z = fmaf(s, p.w, p.z);
     if (!inside(P, p.x, p.y, p.z)) {
-        acc.esc += p.E;
+        esc += p.E;
         hist_add<GEN>(P, p.hist, 0, p.E);
-        ev.b += EV_TERM;
         return Flight::gone;
     }
-    ++ev.n;
     voxel_of(P, p);
     const uint32_t vox = GDPM_IDX(P.status, vox_of(P, p.ix, p.iy, p.iz), n_voxels(P), ST_B_VOXEL);
     const int m = GDPM_IDX(P.status, int(__ldg(&P.mat[vox])), T.n_mat, ST_B_TABLE);
@@ -429,7 +402,6 @@ __device__ __forceinline__ Flight photon_flight(const SimParams& P, const PhSmem
     const int mi = m * T.n_e + i;
     const float mt = lerpf(S.tot[mi], S.tot[mi + 1], f);
     if (!(u01(x.y) * mm < mt * rho)) return Flight::fly;
-    ev.a += EV_REAL;
     hist_count<GEN>(P, p.hist, 0);
     const float2 c0 = S.cum[mi], c1 = S.cum[mi + 1];
     const float rr = u01(x.z) * mt;
@@ -448,46 +420,41 @@ __device__ __forceinline__ Flight photon_flight(const SimParams& P, const PhSmem
 // production (the electron takes the flight's last uniform of the kinetic
 // energy, the positron the rest), photoelectric absorption (photoelectron
 // along the photon, or at Sauter's angle to it, physics variant), or one
-// trial of a Compton event (`force` accepts any).  False when the trial was
-// rejected.  After a Compton event the photon has turned and lost energy,
-// with a recoil electron along E u - E' u', and `goes_on` says whether it
-// stays above its absorption energy (below it, it is deposited here).
+// trial of a Compton event (`force` accepts any).  After a Compton event the
+// photon has turned and lost energy, with a recoil electron along
+// E u - E' u', and `goes_on` says whether it stays above its absorption
+// energy (below it, it is deposited here).
+enum class PhEvent { none, compton, photo, pair };
 template <bool GEN>
-__device__ __forceinline__ bool photon_event(const SimParams& P, Part& p, uint4 x, bool force, bool& goes_on,
-                                             Ev& ev, Sec& sec) {
+__device__ __forceinline__ PhEvent photon_event(const SimParams& P, Part& p, uint4 x, bool force, bool& goes_on,
+                                                Sec& sec) {
     const float E = p.E;
-    sec.n = 1;
     sec.dx = p.u; sec.dy = p.v; sec.dz = p.w;
-    sec.pos2 = false;
-    if (E < 0.f || (p.flags & kAbsorbed)) {
-        ev.b += EV_TERM;
-        if (E < 0.f) {
-            ev.a += EV_PAIR;
-            const float tav = -E - 2.f * kMC2f;
-            sec.E1 = u01(x.w) * tav;
-            sec.E2 = tav - sec.E1;
-            sec.n = 2;
-            sec.pos2 = true;
-        } else {
-            ev.a += EV_PHOTO;
-            p.flags &= ~kAbsorbed;
-            sec.E1 = E;
-            if (P.T.flags & GDPM_FLAG_SAUTER) {
-                float mu, rphi, cp, sp;
-                sample_sauter(p, P, E, mu, rphi);
-                cossin_2pi(rphi, cp, sp);
-                rotate(sec.dx, sec.dy, sec.dz, mu, cp, sp);
-            }
+    sec.photon = sec.pos2 = false;
+    if (E < 0.f) {
+        const float tav = -E - 2.f * kMC2f;
+        sec.E1 = u01(x.w) * tav;
+        sec.E2 = tav - sec.E1;
+        sec.n = 2;
+        sec.pos2 = true;
+        return PhEvent::pair;
+    }
+    if (p.flags & kAbsorbed) {
+        p.flags &= ~kAbsorbed;
+        sec.n = 1;
+        sec.E1 = E;
+        if (P.T.flags & GDPM_FLAG_SAUTER) {
+            float mu, rphi, cp, sp;
+            sample_sauter(p, P, E, mu, rphi);
+            cossin_2pi(rphi, cp, sp);
+            rotate(sec.dx, sec.dy, sec.dz, mu, cp, sp);
         }
-        return true;
+        return PhEvent::photo;
     }
     ++p.ctr;
     float eps, cost, rphi;
-    if (!kn_trial(x, E, eps, cost, rphi) && !force) {
-        sec.n = 0;
-        return false;
-    }
-    ev.a += EV_COMPTON;
+    if (!kn_trial(x, E, eps, cost, rphi) && !force) return PhEvent::none;
+    sec.n = 1;
     float cp, sp;
     cossin_2pi(rphi, cp, sp);
     rotate(p.u, p.v, p.w, cost, cp, sp);
@@ -498,13 +465,9 @@ __device__ __forceinline__ bool photon_event(const SimParams& P, Part& p, uint4 
     const float en = rsqrtf(fmaf(dz, dz, fmaf(dx, dx, __fmul_rn(dy, dy))));
     sec.dx = dx * en; sec.dy = dy * en; sec.dz = dz * en;
     goes_on = !(Ep < P.T.eabs_ph);
-    if (goes_on) {
-        p.E = Ep;
-    } else {
-        tally<GEN>(P, p.flags, vox_of(P, p.ix, p.iy, p.iz), Ep);
-        ev.b += EV_LOCAL + EV_TERM;
-    }
-    return true;
+    if (goes_on) p.E = Ep;
+    else tally<GEN>(P, p.flags, vox_of(P, p.ix, p.iy, p.iz), Ep);
+    return PhEvent::compton;
 }
 
 // ---------------------------------------------------------------- electron step
@@ -514,401 +477,320 @@ struct ElSmem {
     const float* atab;
 };
 
-// The electron phase runs in one of two forms with identical arithmetic
-// (GDPM_PARAM_ELECTRON_WALK): a lane takes a whole condensed-history step
-// per iteration of the phase loop (kernel k_phase<1>), or a resumable step
-// whose voxel walk takes at most kWalkTrips trips of the DDA loop per
-// iteration and resumes in the next (k_phase<2>).  The resumable form keeps
-// a lane with many voxel crossings from holding its warp while the other
-// lanes' steps end and they are refilled; it pays for that with step state
-// that lives across the loop top.
-constexpr int kWalkTrips = 3;
+// An electron or positron in a lane: its voxel is packed (10 bits an axis),
+// pend is energy it owes to that voxel and has not tallied yet.
+struct Electron {
+    float x, y, z, u, v, w, E, pend;
+    uint32_t vox, hist, pidlo, pidhi, ctr, flags;
+};
 
-// An electron step in progress: the CH step of Sec. 2.1 is set up once
-// (limits, end energy, hinge deflection), then its straight legs are walked
-// through the voxels over one or more loop iterations.
+// The condensed-history step in progress (Sec. 2.1): set up once (limits, end
+// energy, hinge deflection), then its straight legs are walked through the
+// voxels over one or more rounds of the phase loop.
 struct ElStep {
     float left;        // mass thickness left in the current leg (g/cm2)
     float m1;          // mass thickness of the second leg
     float dpm;         // energy loss per unit mass thickness along the step
-    float u1, v1, w1;  // resumable form: the direction after the hinge; whole-step
-                       // form: the deflection cos(theta), cos(phi), sin(phi)
+    float u1, v1, w1;  // the direction after the hinge
     float Tend;        // energy at the end of the step
     float dep;         // energy of the step tallied or owed to a voxel so far
     float rho;         // density of the particle's current voxel
-    int leg;           // 0: no step in progress; 1 or 2: walking that leg
-    int lim_m;         // what ends the step (bits 0-1), start material (bits 2+)
+    uint32_t what;     // bits 0-1: 0 no step in progress, 1 or 2 walking that leg; bits 2-3: what
+                       // ends the step (0 reach E_abs, 1 hard candidate, 2 MS step); bits 4+: start material
 };
 
-// Voxel walk (3-D DDA) of the step in progress, depositing dpm MeV per
-// g/cm2 in each voxel: along leg 1 (zeta x_s), turn to the deflected
-// direction at the hinge, along leg 2 ((1 - zeta) x_s).  pend is energy
-// already owed to the current voxel but not yet tallied: it goes out with
-// the first piece tallied on leaving the voxel, so a track issues one atomic
-// per voxel it visits rather than one per piece; the last piece of leg 2 is
-// left to the caller.  Returns 0 when the trip budget ran out (resumable
-// form), 1 at the end of leg 2, 2 when the particle left the phantom.
-//
-// One DDA trip: the particle either ends its leg inside the current voxel
-// (1) or moves to the voxel's exit face, tallies, and crosses (0, or 2 when
-// it leaves the phantom).
+// Outcome of a lane's round: the particle stays in its lane, its track has
+// ended, or it waits for an event.
+enum class Round { go, ended, wait };
+// Events a waiting particle waits for.
+constexpr uint32_t kCandidate = 0u, kMoller = 1u, kAnnihilation = 2u;
+
+__device__ __forceinline__ uint32_t vox_packed(int ix, int iy, int iz) {
+    return uint32_t(ix) | (uint32_t(iy) << 10) | (uint32_t(iz) << 20);
+}
+__device__ __forceinline__ uint32_t vox_linear(const SimParams& P, uint32_t v) {
+    return (v & 1023u) + uint32_t(P.nx) * (((v >> 10) & 1023u) + uint32_t(P.ny) * (v >> 20));
+}
+
+// End of track: residual energy deposited in the voxel; a positron then waits
+// to annihilate, or its rest energy is discarded (Sec. 2.1, Sec. 4).
 template <bool GEN>
-__device__ __forceinline__ int walk_trip(const SimParams& P, Part& p, ElStep& s, float iu, float iv,
-                                         float iw, int sx, int sy, int sz, uint32_t& vox,
-                                         uint32_t& crossings, float& pend) {
-    const float tx = p.u != 0.f ? (float(p.ix + (sx > 0)) * P.dx - p.x) * iu : kInf;
-    const float ty = p.v != 0.f ? (float(p.iy + (sy > 0)) * P.dy - p.y) * iv : kInf;
-    const float tz = p.w != 0.f ? (float(p.iz + (sz > 0)) * P.dz - p.z) * iw : kInf;
-    float tb;
-    int ab;
-    if (tx <= ty && tx <= tz) { tb = tx; ab = 0; }
-    else if (ty <= tz) { tb = ty; ab = 1; }
-    else { tb = tz; ab = 2; }
-    tb = fmaxf(tb, 0.f);
-    const float rho = s.rho;
-    if (rho * tb >= s.left) {
-        // the leg ends in this voxel
-        const float t = s.left / rho;
-        p.x = fmaf(t, p.u, p.x);
-        p.y = fmaf(t, p.v, p.y);
-        p.z = fmaf(t, p.w, p.z);
-        return 1;
+__device__ __forceinline__ Round absorb(const SimParams& P, Electron& p, uint32_t& kind) {
+    tally<GEN>(P, p.flags, vox_linear(P, p.vox), p.E + p.pend);
+    p.pend = 0.f;
+    if (!(p.flags & kPositron)) return Round::ended;
+    if (!P.S.annihilation) {
+        atomicAdd(&P.ledger[L_DISCARDED], 2.0 * kMC2);
+        return Round::ended;
     }
-    p.x = fmaf(tb, p.u, p.x);
-    p.y = fmaf(tb, p.v, p.y);
-    p.z = fmaf(tb, p.w, p.z);
-    const float piece = rho * tb;
-    const float e = s.dpm * piece;
-    if (e + pend > 0.f) tally<GEN>(P, p.flags, vox, e + pend);
-    s.dep += e;
-    pend = 0.f;
-    s.left -= piece;
-    ++crossings;
-    if (ab == 0) {
-        p.ix += sx;
-        if (p.ix < 0 || p.ix >= P.nx) return 2;
-        vox += sx;
-    } else if (ab == 1) {
-        p.iy += sy;
-        if (p.iy < 0 || p.iy >= P.ny) return 2;
-        vox = sy > 0 ? vox + P.nx : vox - P.nx;
-    } else {
-        p.iz += sz;
-        if (p.iz < 0 || p.iz >= P.nz) return 2;
-        const uint32_t plane = uint32_t(P.nx) * uint32_t(P.ny);
-        vox = sz > 0 ? vox + plane : vox - plane;
-    }
-    vox = GDPM_IDX(P.status, uint32_t(vox), n_voxels(P), ST_B_VOXEL);
-    s.rho = __ldg(&P.rho[vox]);
-    return 0;
+    kind = kAnnihilation;
+    return Round::wait;
 }
 
-// The hinge: the rest of leg 1 stays owed to the current voxel, then the
-// particle turns to the deflected direction (precomputed by the resumable
-// form, rotated here by the whole-step form) and starts leg 2.
-template <bool RESUME>
-__device__ __forceinline__ void hinge(Part& p, ElStep& s, float& pend) {
-    pend += s.dpm * s.left;
-    s.dep += s.dpm * s.left;
-    if (RESUME) {
-        p.u = s.u1; p.v = s.v1; p.w = s.w1;
-    } else {
-        rotate(p.u, p.v, p.w, s.u1, s.v1, s.w1);
-    }
-    s.leg = 2;
-    s.left = s.m1;
-}
-
-// Whole-step form: the legs one after another, with the warp's lanes
-// finishing leg 1 together before any turns.  The trip loop ends by
-// construction: within a leg the signs sx, sy, sz are fixed, so every trip
-// either ends the leg or moves one voxel index one step in its fixed
-// direction (a NaN position falls to the z branch), and the walk leaves the
-// grid within nx + ny + nz trips.  (A counted guard here cost 8-14 % of the
-// electron phase in code generation, for no case it could catch.)
+// Set up a step with the draw x: step limits as mass thickness in the start
+// voxel's material, energy at its end, deflection at the random hinge.
 template <bool GEN>
-__device__ int walk_whole(const SimParams& P, Part& p, ElStep& s, uint32_t& crossings, float& pend) {
-#pragma unroll 1
-    for (;;) {
-        const float iu = p.u != 0.f ? 1.f / p.u : 0.f;
-        const float iv = p.v != 0.f ? 1.f / p.v : 0.f;
-        const float iw = p.w != 0.f ? 1.f / p.w : 0.f;
-        const int sx = p.u > 0.f ? 1 : -1, sy = p.v > 0.f ? 1 : -1, sz = p.w > 0.f ? 1 : -1;
-        uint32_t vox = vox_of(P, p.ix, p.iy, p.iz);
-        int res;
-#pragma unroll 1
-        do {
-            res = walk_trip<GEN>(P, p, s, iu, iv, iw, sx, sy, sz, vox, crossings, pend);
-        } while (res == 0);
-        if (res == 2 || s.leg == 2) return res;
-        hinge<false>(p, s, pend);
-    }
-}
-
-// Resumable form: at most kWalkTrips trips, turning at the hinge within the
-// budget.
-template <bool GEN>
-__device__ int walk_resumable(const SimParams& P, Part& p, ElStep& s, uint32_t& crossings,
-                              float& pend) {
-    float iu = p.u != 0.f ? 1.f / p.u : 0.f;
-    float iv = p.v != 0.f ? 1.f / p.v : 0.f;
-    float iw = p.w != 0.f ? 1.f / p.w : 0.f;
-    int sx = p.u > 0.f ? 1 : -1, sy = p.v > 0.f ? 1 : -1, sz = p.w > 0.f ? 1 : -1;
-    uint32_t vox = vox_of(P, p.ix, p.iy, p.iz);
-#pragma unroll 1
-    for (int trip = 0; trip < kWalkTrips; ++trip) {
-        const int res = walk_trip<GEN>(P, p, s, iu, iv, iw, sx, sy, sz, vox, crossings, pend);
-        if (res == 2 || (res == 1 && s.leg == 2)) return res;
-        if (res == 1) {
-            hinge<true>(p, s, pend);
-            iu = p.u != 0.f ? 1.f / p.u : 0.f;
-            iv = p.v != 0.f ? 1.f / p.v : 0.f;
-            iw = p.w != 0.f ? 1.f / p.w : 0.f;
-            sx = p.u > 0.f ? 1 : -1; sy = p.v > 0.f ? 1 : -1; sz = p.w > 0.f ? 1 : -1;
-        }
-    }
-    return 0;
-}
-
-template <bool GEN>
-__device__ void electron_escape(const SimParams& P, Part& p, float energy, Acc& acc) {
-    double e = energy;
-    if (p.flags & kPositron) {
-        if (P.S.annihilation) e += 2.0 * kMC2;
-        else acc.disc += 2.0 * kMC2;
-    }
-    acc.esc += e;
-    hist_add<GEN>(P, p.hist, 0, e);
-}
-
-// One condensed-history step of an electron or positron (Sec. 2.1), or its
-// absorption.  Whole-step form (RESUME false): set up, walk and end in one
-// call.  Resumable form: the step is set up when none is in progress, its
-// voxel walk may take several calls (several iterations of the phase loop),
-// and the step's end (escape, absorption, hard-event candidate) runs in the
-// call whose walk reaches it.
-template <bool RESUME, bool GEN>
-__device__ __forceinline__ void electron_step(const SimParams& P, const ElSmem& S, Part& p, bool& active,
-                                              Acc& acc, Ev& ev, Sec& sec, float& pend, ElStep& carried) {
+__device__ __forceinline__ void electron_setup(const SimParams& P, const ElSmem& S, const Electron& p, uint4 x,
+                                               ElStep& st) {
     const DevTables& T = P.T;
-    // the whole-step form keeps its step state local to this call
-    ElStep local;
-    ElStep& st = RESUME ? carried : local;
-    if (!RESUME) st.leg = 0;
-    bool absorb = false;
-    if (st.leg == 0) {
-        absorb = p.E < T.eabs_el;
-        if (!absorb) {
-            const float4 r = draw(p, P.key0, P.key1);
-            ev.b += EV_STEP;
-            hist_count<GEN>(P, p.hist, 1);
-            // material and density of the start voxel, loaded together
-            const uint32_t vox0 = GDPM_IDX(P.status, vox_of(P, p.ix, p.iy, p.iz), n_voxels(P), ST_B_VOXEL);
-            const int m = GDPM_IDX(P.status, int(__ldg(&P.mat[vox0])), T.n_mat, ST_B_TABLE);
-            st.rho = __ldg(&P.rho[vox0]);
+    const float4 r = make_float4(u01(x.x), u01(x.y), u01(x.z), u01(x.w));
+    hist_count<GEN>(P, p.hist, 1);
+    // material and density of the start voxel, loaded together
+    const uint32_t vox0 = GDPM_IDX(P.status, vox_linear(P, p.vox), n_voxels(P), ST_B_VOXEL);
+    const int m = GDPM_IDX(P.status, int(__ldg(&P.mat[vox0])), T.n_mat, ST_B_TABLE);
+    st.rho = __ldg(&P.rho[vox0]);
+    int i;
+    float f;
+    grid_pos(T, p.E, i, f);
+    const int mi = m * T.n_e + i;
+    const float4 a0 = S.el[mi], a1 = S.el[mi + 1];
+    const float R0 = lerpf(a0.x, a1.x, f);
+    const float xms = lerpf(a0.y, a1.y, f);
+    const float xcut = R0 - T.r_eabs[m];
+    const float xhard = (T.flags & GDPM_FLAG_NO_HARD) ? kInf : -__logf(r.x) * T.inv_sigmax[m];
+    uint32_t lim;
+    float xs;
+    if (xcut <= xms && xcut <= xhard) { lim = 0u; xs = xcut; }
+    else if (xhard <= xms) { lim = 1u; xs = xhard; }
+    else { lim = 2u; xs = xms; }
+    xs = fmaxf(xs, 0.f);
+    float Tend;
+    if (lim == 0u) {
+        Tend = T.eabs_el;
+    } else {
+        const float rr = (R0 - xs - T.rinv_lo[m]) * T.rinv_idr[m];
+        const int j = min(max(int(floorf(rr)), 0), T.n_r - 2);
+        const float g = fminf(fmaxf(rr - float(j), 0.f), 1.f);
+        const float* ri = S.rinv + m * T.n_r;
+        Tend = fminf(lerpf(ri[j], ri[j + 1], g), p.E);
+    }
+    const float Tk = p.E;
+    const float dT = Tk - Tend;
+    hist_add<GEN>(P, p.hist, 1, double(xs));
+    // multiple scattering at the mid-step energy
+    const float Tm = 0.5f * (Tk + Tend);
+    const float pbc = Tm * (Tm + 2.f * kMC2f) / (Tm + kMC2f);
+    const float q = kEs / pbc;
+    const float G1 = xs * q * q * 0.5f * T.inv_x0[m];
+    float mu;
+    if (G1 >= 1.f) {
+        mu = 2.f * r.z - 1.f;
+    } else {
+        const float Asc = screening_A(T, S.atab, G1);
+        mu = 1.f - 2.f * Asc * r.z / (1.f - r.z + Asc);
+    }
+    float cp, sp;
+    cossin_2pi(r.w, cp, sp);
+    // leg 1 keeps the step's start direction, so the deflection is applied to
+    // it here, with all lanes that start a step together
+    st.u1 = p.u; st.v1 = p.v; st.w1 = p.w;
+    rotate(st.u1, st.v1, st.w1, mu, cp, sp);
+    st.dpm = xs > 0.f ? dT / xs : 0.f;
+    st.dep = 0.f;
+    st.Tend = Tend;
+    // random hinge: zeta x_s straight, deflect, (1 - zeta) x_s straight
+    st.left = r.y * xs;
+    st.m1 = (1.f - r.y) * xs;
+    st.what = 1u | (lim << 2) | (uint32_t(m) << 4);
+}
+
+// Voxel walk (3-D DDA) of the step in progress, depositing dpm MeV per g/cm2
+// in each voxel: along leg 1 (zeta x_s), turn to the deflected direction at
+// the hinge, along leg 2 ((1 - zeta) x_s).  A track tallies once per voxel it
+// visits, on leaving it (pend); the last piece of leg 2 is left to the
+// caller.
+struct Walk {
+    float iu, iv, iw;      // 1 / direction (0 for a zero component)
+    float ou, ov, ow;      // added to the distance: kInf for a zero component
+    float fx, fy, fz;      // voxel indices
+    uint32_t lin;          // linear voxel index
+    float tb;              // distance to the exit face
+    int axis;              // of the exit face
+};
+__device__ __forceinline__ void walk_aim(const Electron& p, Walk& k) {
+    k.iu = p.u != 0.f ? 1.f / p.u : 0.f; k.ou = p.u != 0.f ? 0.f : kInf;
+    k.iv = p.v != 0.f ? 1.f / p.v : 0.f; k.ov = p.v != 0.f ? 0.f : kInf;
+    k.iw = p.w != 0.f ? 1.f / p.w : 0.f; k.ow = p.w != 0.f ? 0.f : kInf;
+}
+// Move to the end of the leg (true) or to the exit face of the voxel.
+__device__ __forceinline__ bool walk_move(const SimParams& P, Electron& p, const ElStep& s, Walk& k) {
+    const float tx = fmaf(fmaf(k.fx + (p.u > 0.f ? 1.f : 0.f), P.dx, -p.x), k.iu, k.ou);
+    const float ty = fmaf(fmaf(k.fy + (p.v > 0.f ? 1.f : 0.f), P.dy, -p.y), k.iv, k.ov);
+    const float tz = fmaf(fmaf(k.fz + (p.w > 0.f ? 1.f : 0.f), P.dz, -p.z), k.iw, k.ow);
+    const bool cx = tx <= ty && tx <= tz, cy = ty <= tz;
+    k.axis = cx ? 0 : cy ? 1 : 2;
+    k.tb = fmaxf(cx ? tx : cy ? ty : tz, 0.f);
+    const bool ends = __fmul_rn(s.rho, k.tb) >= s.left;
+    const float t = ends ? s.left / s.rho : k.tb;
+    p.x = fmaf(t, p.u, p.x);
+    p.y = fmaf(t, p.v, p.y);
+    p.z = fmaf(t, p.w, p.z);
+    return ends;
+}
+// Cross the exit face; false when the particle leaves the phantom.
+template <bool GEN>
+__device__ __forceinline__ bool walk_cross(const SimParams& P, Electron& p, ElStep& s, Walk& k,
+                                           uint32_t& crossings) {
+    const float piece = __fmul_rn(s.rho, k.tb);
+    const float owed = fmaf(s.dpm, piece, p.pend);
+    if (owed > 0.f) tally<GEN>(P, p.flags, k.lin, owed);
+    s.dep = fmaf(s.dpm, piece, s.dep);
+    p.pend = 0.f;
+    s.left = __fsub_rn(s.left, piece);
+    ++crossings;
+    const bool up = (k.axis == 0 ? p.u : k.axis == 1 ? p.v : p.w) > 0.f;
+    const uint32_t n = k.axis == 0 ? P.nx : k.axis == 1 ? P.ny : P.nz;
+    const uint32_t d = k.axis == 0 ? 1u : k.axis == 1 ? uint32_t(P.nx) : uint32_t(P.nx) * uint32_t(P.ny);
+    const uint32_t shift = 10u * uint32_t(k.axis);
+    const uint32_t at = ((p.vox >> shift) & 1023u) + (up ? 1u : ~0u);       // wraps below zero
+    if (at >= n) return false;
+    p.vox = up ? p.vox + (1u << shift) : p.vox - (1u << shift);
+    const float f = float(at);
+    if (k.axis == 0) k.fx = f;
+    else if (k.axis == 1) k.fy = f;
+    else k.fz = f;
+    k.lin = up ? k.lin + d : k.lin - d;
+    k.lin = GDPM_IDX(P.status, k.lin, n_voxels(P), ST_B_VOXEL);
+    s.rho = __ldg(&P.rho[k.lin]);
+    return true;
+}
+// One stretch of the walk: to the end of leg 1, the turn at the hinge and the
+// end of leg 2, or to the next crossing on the way, so that the lanes that
+// end a leg do it together and those that cross a face do that together.
+// Returns 0 when the step goes on, 1 at the end of leg 2, 2 when the particle
+// left the phantom.
+template <bool GEN>
+__device__ __forceinline__ int walk_stretch(const SimParams& P, Electron& p, ElStep& s, Walk& k,
+                                            uint32_t& crossings) {
+    bool ends = walk_move(P, p, s, k);
+    if (ends && (s.what & 3u) == 1u) {
+        // the hinge: the rest of leg 1 stays owed to the current voxel
+        p.pend = fmaf(s.dpm, s.left, p.pend);
+        s.dep = fmaf(s.dpm, s.left, s.dep);
+        p.u = s.u1; p.v = s.v1; p.w = s.w1;
+        s.what ^= 3u;                         // leg 1 -> leg 2
+        s.left = s.m1;
+        walk_aim(p, k);
+        ends = walk_move(P, p, s, k);
+    }
+    if (ends) return 1;
+    return walk_cross<GEN>(P, p, s, k, crossings) ? 0 : 2;
+}
+
+// A lane's round: set up a step when none is in progress (`starts`, with the
+// draw x), walk, and at the step's end escape, be absorbed, or wait for the
+// hard-event candidate.
+template <bool GEN>
+__device__ __forceinline__ Round electron_round(const SimParams& P, const ElSmem& S, Electron& p, ElStep& st,
+                                                uint4 x, double& esc, uint32_t& crossings, uint32_t& kind) {
+    if ((st.what & 3u) == 0u) {
+        ++p.ctr;
+        electron_setup<GEN>(P, S, p, x, st);
+    }
+    Walk k;
+    k.lin = vox_linear(P, p.vox);
+    k.fx = float(p.vox & 1023u); k.fy = float((p.vox >> 10) & 1023u); k.fz = float(p.vox >> 20);
+    walk_aim(p, k);
+    int res = walk_stretch<GEN>(P, p, st, k, crossings);
+#pragma unroll 1
+    for (int n = 1; res == 0 && n < P.walk_trips; ++n) res = walk_stretch<GEN>(P, p, st, k, crossings);
+    if (res == 0) return Round::go;
+    st.what &= ~3u;
+    if (res == 2) {
+        double e = p.E - st.dep;
+        if (p.flags & kPositron) {
+            if (P.S.annihilation) e += 2.0 * kMC2;
+            else atomicAdd(&P.ledger[L_DISCARDED], 2.0 * kMC2);
+        }
+        esc += e;
+        hist_add<GEN>(P, p.hist, 0, e);
+        return Round::ended;
+    }
+    // the step's remainder stays owed to the voxel the step ends in
+    p.pend += (p.E - st.Tend) - st.dep;
+    p.E = st.Tend;
+    const uint32_t lim = (st.what >> 2) & 3u;
+    if (lim == 1u) {
+        kind = kCandidate | ((st.what >> 4) << 2);
+        return Round::wait;
+    }
+    if (lim == 0u || p.E < P.T.eabs_el) return absorb<GEN>(P, p, kind);
+    return Round::go;
+}
+
+// One draw of the event a particle waits for.  A hard-event candidate is
+// accepted with Sigma_h(T)/Sigma_max of the step's start material, as
+// bremsstrahlung (done with this draw) or as a Moller event, which then takes
+// one rejection trial per draw (`force` accepts any); a positron at rest
+// annihilates.  Returns go when the particle takes its next step, wait when
+// it needs another draw, ended at the end of its track.
+template <bool GEN>
+__device__ __forceinline__ Round electron_event(const SimParams& P, const ElSmem& S, Electron& p, uint32_t& kind,
+                                                uint4 x, bool force, Sec& sec) {
+    const DevTables& T = P.T;
+    ++p.ctr;
+    sec.dx = p.u; sec.dy = p.v; sec.dz = p.w;
+    sec.photon = sec.pos2 = false;
+    const uint32_t what = kind & 3u;
+    if (what == kCandidate) {
+        const int m = int(kind >> 2);
+        const float Tn = p.E, wcc = T.eabs_el, wcb = T.eabs_ph;
+        float sm = 0.f, sb = 0.f;
+        if (Tn > wcb || Tn > 2.f * wcc) {
             int i;
             float f;
-            grid_pos(T, p.E, i, f);
-            const int mi = m * T.n_e + i;
-            const float4 a0 = S.el[mi], a1 = S.el[mi + 1];
-            // step limits as mass thickness in the start material: reach E_abs,
-            // hard-event candidate, or the multiple-scattering step
-            const float R0 = lerpf(a0.x, a1.x, f);
-            const float xms = lerpf(a0.y, a1.y, f);
-            const float xcut = R0 - T.r_eabs[m];
-            const float xhard = (T.flags & GDPM_FLAG_NO_HARD) ? kInf : -__logf(r.x) * T.inv_sigmax[m];
-            int lim;   // what ends the step: 0 reach E_abs, 1 hard candidate, 2 MS step
-            float xs;
-            if (xcut <= xms && xcut <= xhard) { lim = 0; xs = xcut; }
-            else if (xhard <= xms) { lim = 1; xs = xhard; }
-            else { lim = 2; xs = xms; }
-            xs = fmaxf(xs, 0.f);
-            float Tend;
-            if (lim == 0) {
-                Tend = T.eabs_el;
-            } else {
-                const float rr = (R0 - xs - T.rinv_lo[m]) * T.rinv_idr[m];
-                const int j = min(max(int(floorf(rr)), 0), T.n_r - 2);
-                const float g = fminf(fmaxf(rr - float(j), 0.f), 1.f);
-                const float* ri = S.rinv + m * T.n_r;
-                Tend = fminf(lerpf(ri[j], ri[j + 1], g), p.E);
-            }
-            const float Tk = p.E;
-            const float dT = Tk - Tend;
-            hist_add<GEN>(P, p.hist, 1, double(xs));
-            // multiple scattering at the mid-step energy
-            const float Tm = 0.5f * (Tk + Tend);
-            const float pbc = Tm * (Tm + 2.f * kMC2f) / (Tm + kMC2f);
-            const float q = kEs / pbc;
-            const float G1 = xs * q * q * 0.5f * T.inv_x0[m];
-            float mu;
-            if (G1 >= 1.f) {
-                mu = 2.f * r.z - 1.f;
-            } else {
-                const float Asc = screening_A(T, S.atab, G1);
-                mu = 1.f - 2.f * Asc * r.z / (1.f - r.z + Asc);
-            }
-            float cp, sp;
-            cossin_2pi(r.w, cp, sp);
-            if (RESUME) {
-                // the direction after the hinge: leg 1 keeps the step's start
-                // direction, so the deflection is applied to it here, with all
-                // lanes that start a step together
-                st.u1 = p.u; st.v1 = p.v; st.w1 = p.w;
-                rotate(st.u1, st.v1, st.w1, mu, cp, sp);
-            } else {
-                st.u1 = mu; st.v1 = cp; st.w1 = sp;
-            }
-            st.dpm = xs > 0.f ? dT / xs : 0.f;
-            st.dep = 0.f;
-            st.Tend = Tend;
-            // random hinge: zeta x_s straight, deflect, (1 - zeta) x_s straight
-            st.left = r.y * xs;
-            st.m1 = (1.f - r.y) * xs;
-            st.leg = 1;
-            st.lim_m = lim | (m << 2);
+            grid_pos(T, Tn, i, f);
+            const int mj = m * T.n_e + i;
+            const float4 a0 = S.el[mj], a1 = S.el[mj + 1];
+            if (Tn > 2.f * wcc) sm = lerpf(a0.z, a1.z, f);
+            if (Tn > wcb) sb = lerpf(a0.w, a1.w, f);
         }
+        const float sh = sm + sb;
+        if (u01(x.x) * T.sigmax[m] < sh) {
+            hist_count<GEN>(P, p.hist, 2);
+            if (u01(x.y) * sh < sm) {
+                kind = kMoller;
+                return Round::wait;
+            }
+            const float k = wcb * exp2f(u01(x.z) * __log2f(Tn / wcb));
+            sec.n = 1;
+            sec.photon = true;
+            sec.E1 = k;
+            p.E = Tn - k;
+        }
+    } else if (what == kMoller) {
+        const float Tn = p.E;
+        float eps, rphi;
+        if (!moller_trial(x, Tn, T.eabs_el, eps, rphi) && !force) return Round::wait;
+        float c, sn;
+        cossin_2pi(rphi, c, sn);
+        const float W = eps * Tn, Tp = Tn - W;
+        const float cd = sqrtf(W * (Tn + 2.f * kMC2f) / (Tn * (W + 2.f * kMC2f)));
+        const float cpr = sqrtf(Tp * (Tn + 2.f * kMC2f) / (Tn * (Tp + 2.f * kMC2f)));
+        rotate(sec.dx, sec.dy, sec.dz, cd, c, sn);
+        sec.n = 1;
+        sec.E1 = W;
+        rotate<true>(p.u, p.v, p.w, cpr, -c, -sn);
+        p.E = Tp;
+    } else {
+        // two back-to-back 0.511 MeV photons (isotropic)
+        const float cost = 2.f * u01(x.x) - 1.f;
+        const float sint = sqrtf(fmaxf(0.f, 1.f - cost * cost));
+        float cp, sp;
+        cossin_2pi(u01(x.y), cp, sp);
+        sec.n = 2;
+        sec.photon = true;
+        sec.E1 = sec.E2 = kMC2f;
+        sec.dx = sint * cp; sec.dy = sint * sp; sec.dz = cost;
+        return Round::ended;
     }
-    if (!absorb) {
-        const int res = RESUME ? walk_resumable<GEN>(P, p, st, ev.n, pend) : walk_whole<GEN>(P, p, st, ev.n, pend);
-        if (res == 0) return;            // the walk goes on in the next iteration
-        st.leg = 0;
-        const float Tk = p.E;
-        if (res == 2) {
-            electron_escape<GEN>(P, p, Tk - st.dep, acc);
-            ev.b += EV_TERM;
-            active = false;
-            return;
-        }
-        // the step's remainder stays owed to the voxel the step ends in
-        pend += (Tk - st.Tend) - st.dep;
-        p.E = st.Tend;
-        const int lim = st.lim_m & 3, m = st.lim_m >> 2;
-        if (lim == 0) {
-            absorb = true;
-        } else if (lim == 1) {
-            // hard-event candidate: accept with Sigma_h(T)/Sigma_max (start material)
-            const float4 v = draw(p, P.key0, P.key1);
-            const float Tn = p.E, wcc = T.eabs_el, wcb = T.eabs_ph;
-            float sm = 0.f, sb = 0.f;
-            if (Tn > wcb || Tn > 2.f * wcc) {
-                int i;
-                float f;
-                grid_pos(T, Tn, i, f);
-                const int mj = m * T.n_e + i;
-                const float4 a0 = S.el[mj], a1 = S.el[mj + 1];
-                if (Tn > 2.f * wcc) sm = lerpf(a0.z, a1.z, f);
-                if (Tn > wcb) sb = lerpf(a0.w, a1.w, f);
-            }
-            const float sh = sm + sb;
-            if (v.x * T.sigmax[m] < sh) {
-                hist_count<GEN>(P, p.hist, 2);
-                sec.n = 1;
-                sec.pos2 = false;
-                if (v.y * sh < sm) {
-                    ev.b += EV_MOLLER;
-                    float eps, rphi;
-                    sample_moller(p, P, Tn, wcc, eps, rphi);
-                    float c, sn;
-                    cossin_2pi(rphi, c, sn);
-                    const float W = eps * Tn, Tp = Tn - W;
-                    const float cd = sqrtf(W * (Tn + 2.f * kMC2f) / (Tn * (W + 2.f * kMC2f)));
-                    const float cpr = sqrtf(Tp * (Tn + 2.f * kMC2f) / (Tn * (Tp + 2.f * kMC2f)));
-                    sec.dx = p.u; sec.dy = p.v; sec.dz = p.w;
-                    rotate(sec.dx, sec.dy, sec.dz, cd, c, sn);
-                    sec.photon = false;
-                    sec.E1 = W;
-                    rotate<true>(p.u, p.v, p.w, cpr, -c, -sn);
-                    p.E = Tp;
-                } else {
-                    ev.c += EV_BREMS;
-                    const float k = wcb * exp2f(v.z * __log2f(Tn / wcb));
-                    sec.photon = true;
-                    sec.E1 = k;
-                    sec.dx = p.u; sec.dy = p.v; sec.dz = p.w;
-                    p.E = Tn - k;
-                }
-            }
-        }
-    }
-    if (absorb) {
-        // end of track: residual energy deposited here; a positron then
-        // annihilates into two back-to-back 0.511 MeV photons (isotropic),
-        // or its rest energy is discarded (Sec. 2.1, Sec. 4)
-        tally<GEN>(P, p.flags, vox_of(P, p.ix, p.iy, p.iz), p.E + pend);
-        pend = 0.f;
-        ev.b += EV_TERM;
-        active = false;
-        if (p.flags & kPositron) {
-            if (!P.S.annihilation) {
-                acc.disc += 2.0 * kMC2;
-            } else {
-                const float4 a = draw(p, P.key0, P.key1);
-                const float cost = 2.f * a.x - 1.f;
-                const float sint = sqrtf(fmaxf(0.f, 1.f - cost * cost));
-                float cp, sp;
-                cossin_2pi(a.y, cp, sp);
-                ev.c += EV_ANNIHIL;
-                sec.n = 2;
-                sec.photon = true;
-                sec.pos2 = false;
-                sec.E1 = sec.E2 = kMC2f;
-                sec.dx = sint * cp; sec.dy = sint * sp; sec.dz = cost;
-            }
-        }
-    }
+    return p.E < T.eabs_el ? absorb<GEN>(P, p, kind) : Round::go;
 }
 
 // ---------------------------------------------------------------- warp-uniform parts
-// Fold the lanes' event counters into the block's (call with the whole warp).
-template <int PT>
-__device__ __forceinline__ void flush_events(Ev& ev, uint32_t* s_cnt) {
-    const bool lead = lane_id() == 0;
-    const uint32_t n = __reduce_add_sync(kFull, ev.n);
-    if (lead && n) atomicAdd(&s_cnt[PT == 0 ? C_PH_FLIGHTS : C_CROSS], n);
-    const uint32_t w[3] = {ev.a, ev.b, ev.c};
-    const int slots[10] = {C_PH_REAL, C_COMPTON, C_PHOTO, C_PAIR,
-                           PT == 0 ? C_PH_TERMINATED : C_EL_TERMINATED, C_LOCAL_DEP,
-                           C_EL_STEPS, C_MOLLER, C_BREMS, C_ANNIHIL};
-#pragma unroll
-    for (int k = 0; k < 10; ++k) {
-        const uint32_t c = __reduce_add_sync(kFull, (w[k >> 2] >> (8 * (k & 3))) & 0xFFu);
-        if (lead && c) atomicAdd(&s_cnt[slots[k]], c);
-    }
-    ev = Ev{0u, 0u, 0u, 0u};
-}
-
-// Warp-uniform tallies of the loop top (identical in every lane), two
-// 16-bit counts to a word: (local deposits, electron pushes), (photon
-// pushes, primaries), (pops, primaries that miss the phantom).  At most 32
-// per count and iteration, folded with the event counters.
-struct WarpCnt {
-    uint32_t w0, w1, w2;
-};
-
-template <int PT>
-__device__ __forceinline__ void flush_warp_counts(WarpCnt& wc, uint32_t* s_cnt) {
-    if (lane_id() == 0) {
-        const uint32_t local = wc.w0 & 0xFFFFu, push_el = wc.w0 >> 16;
-        const uint32_t push_ph = wc.w1 & 0xFFFFu, primary = wc.w1 >> 16;
-        const uint32_t pop = wc.w2 & 0xFFFFu, missed = wc.w2 >> 16;
-        if (local) atomicAdd(&s_cnt[C_LOCAL_DEP], local);
-        if (push_el) {
-            atomicAdd(&s_cnt[C_PUSH_EL], push_el);
-            atomicAdd(&s_cnt[C_EL_CREATED], push_el);
-        }
-        if (push_ph) {
-            atomicAdd(&s_cnt[C_PUSH_PH], push_ph);
-            atomicAdd(&s_cnt[C_PH_CREATED], push_ph);
-        }
-        if (primary) {
-            atomicAdd(&s_cnt[C_PRIMARY], primary);
-            atomicAdd(&s_cnt[PT == 0 ? C_PH_CREATED : C_EL_CREATED], primary);
-        }
-        if (pop) atomicAdd(&s_cnt[PT == 0 ? C_POP_PH : C_POP_EL], pop);
-        if (missed) atomicAdd(&s_cnt[PT == 0 ? C_PH_TERMINATED : C_EL_TERMINATED], missed);
-    }
-    wc = WarpCnt{0u, 0u, 0u};
+// Add n to counter k of the CTA (call with the whole warp).
+__device__ __forceinline__ void count(uint32_t* s_cnt, int k, uint32_t n) {
+    if (lane_id() == 0) atomicAdd(&s_cnt[k], n);
 }
 
 // Queue slots a warp holds: [base, base + left) reserved but not yet written.
@@ -918,34 +800,35 @@ struct Slots {
 
 // `c` consecutive slots for the warp's pushes to one queue: from the
 // reservation first, then a new reservation of PhaseArgs::bank_block slots
-// (one atomic; fewer in a phase of few particles).  Returns the first slot of the new reservation (or of the
-// old one when it sufficed); a lane of rank r < old left writes slot
-// old.base + r, the others new + (r - old left).
-__device__ __forceinline__ uint32_t reserve(Slots& sl, uint32_t c, uint32_t* count, const PhaseArgs& A,
-                                            uint32_t total, int leader) {
-    if (c <= sl.left) {
-        const uint32_t b = sl.base;
+// (one atomic; fewer in a phase of few particles).  Returns the slot of the
+// push of rank r.
+__device__ __forceinline__ uint32_t reserve(Slots& sl, uint32_t c, uint32_t r, uint32_t* counter,
+                                            const PhaseArgs& A, uint32_t total) {
+    const uint32_t base = sl.base, left = sl.left;
+    if (c <= left) {
         sl.base += c;
         sl.left -= c;
-        return b;
+        return base + r;
     }
-    const uint32_t miss = c - sl.left, want = max(miss, min(A.bank_block, total >> A.share_shift));
+    const uint32_t miss = c - left, want = max(miss, min(A.bank_block, total >> A.share_shift));
     uint32_t nb = 0;
-    if (int(lane_id()) == leader) nb = atomicAdd(count, want);
-    nb = __shfl_sync(kFull, nb, leader);
+    if (lane_id() == 0) nb = atomicAdd(counter, want);
+    nb = __shfl_sync(kFull, nb, 0);
     sl.base = nb + miss;
     sl.left = want - miss;
-    return nb;
+    return r < left ? base + r : nb + (r - left);
 }
 
-// Bank the secondaries the lanes' last steps created (call with the whole
-// warp): below-cutoff electrons and photons deposit on the spot, the rest
-// get slots in the warp's reservations and counter-derived ids.
-template <int PT, bool GEN>
-__device__ __forceinline__ void bank_pending(const SimParams& P, const PhaseArgs& A, uint32_t total, Part& p,
-                                             const Sec& sec, Slots (&sl)[2], WarpCnt& wc) {
-    const bool photon = PT != 0 && sec.photon;      // photons create electrons only
-    const uint32_t lane = lane_id();
+// Bank the secondaries of a round of events (call with the whole warp):
+// below-cutoff electrons and photons deposit on the spot, the rest get slots
+// in the warp's reservations and counter-derived ids.  vox: the parents'
+// packed voxels; pushes: the warp's pushes to the electron queue (0) and the
+// photon queue (1).  PT 0: photons create electrons only.
+template <int PT, bool GEN, class Parent>
+__device__ __forceinline__ void bank(const SimParams& P, const PhaseArgs& A, uint32_t total, Parent& p,
+                                     uint32_t vox, const Sec& sec, Slots (&sl)[PT + 1],
+                                     uint32_t (&pushes)[PT + 1]) {
+    const bool photon = PT != 0 && sec.photon;
     for (int k = 0; k < 2; ++k) {
         const bool want = k < sec.n;
         if (!__any_sync(kFull, want)) return;
@@ -953,40 +836,33 @@ __device__ __forceinline__ void bank_pending(const SimParams& P, const PhaseArgs
         const float E = k ? sec.E2 : sec.E1;
         const float sg = (k == 1 && photon) ? -1.f : 1.f;
         const bool push = want && (pos || E >= (photon ? P.T.eabs_ph : P.T.eabs_el));
-        if (want && !push) tally<GEN>(P, p.flags, vox_of(P, p.ix, p.iy, p.iz), E);
-        wc.w0 += __popc(__ballot_sync(kFull, want && !push));
+        if (want && !push) tally<GEN>(P, p.flags, vox_linear(P, vox), E);
 #pragma unroll
         for (int q = 0; q < (PT == 0 ? 1 : 2); ++q) {   // q = 0 electron queue, 1 photon queue
             const bool mine = push && (photon == (q == 1));
             const uint32_t m = __ballot_sync(kFull, mine);
             if (!m) continue;
-            const uint32_t c = __popc(m);
-            const uint32_t left0 = sl[q].left, base0 = sl[q].base;
-            const uint32_t nb = reserve(sl[q], c, q ? A.out_ph_count : A.out_el_count, A, total, __ffs(m) - 1);
+            const uint32_t c = __popc(m), r = __popc(m & lanemask_lt());
+            const uint32_t slot = reserve(sl[q], c, r, q ? A.out_ph_count : A.out_el_count, A, total);
             if (mine) {
-                Part ch;
-                ch.x = p.x; ch.y = p.y; ch.z = p.z;
-                ch.u = sg * sec.dx; ch.v = sg * sec.dy; ch.w = sg * sec.dz;
-                ch.E = E;
-                ch.ix = p.ix; ch.iy = p.iy; ch.iz = p.iz;
-                ch.hist = p.hist;
                 const uint64_t id = child_id(uint64_t(p.pidlo) | (uint64_t(p.pidhi) << 32), p.flags & kChildMask);
                 // the child index cannot wrap into the slot bits (no particle
                 // comes near 65535 secondaries; flag it if one ever did)
                 if ((p.flags & kChildMask) == kChildMask) atomicOr(P.status, ST_QUEUE_OVERFLOW);
-                ch.pidlo = uint32_t(id);
-                ch.pidhi = uint32_t(id >> 32);
-                ch.ctr = 0;
-                ch.flags = (p.flags & kBatchMask) | (pos ? kPositron : 0u);
+                const uint32_t flags = (p.flags & kBatchMask) | (pos ? kPositron : 0u);
                 ++p.flags;
-                const uint32_t r = __popc(m & lanemask_lt());
-                const uint32_t slot = c <= left0 ? base0 + r : (r < left0 ? base0 + r : nb + (r - left0));
                 const Queue& Q = q ? A.out_ph : A.out_el;
-                if (slot < Q.capacity) queue_store(Q, slot, ch);
-                else atomicOr(P.status, ST_QUEUE_OVERFLOW);
+                if (slot < Q.capacity) {
+                    uint4* rec = Q.rec + size_t(slot) * (kQueueWords / 4);
+                    rec[0] = pack4(p.x, p.y, p.z, __float_as_uint(E));
+                    rec[1] = pack4(sg * sec.dx, sg * sec.dy, sg * sec.dz, vox);
+                    rec[2] = make_uint4(p.hist, uint32_t(id), uint32_t(id >> 32), flags);
+                } else {
+                    atomicOr(P.status, ST_QUEUE_OVERFLOW);
+                }
                 hist_count<GEN>(P, p.hist, 3);
             }
-            if (q) wc.w1 += c; else wc.w0 += c << 16;
+            pushes[q] += c;
         }
     }
 }
@@ -1024,35 +900,33 @@ __device__ __forceinline__ uint32_t phase_lanes(uint32_t total) {
     return min((total - 1u) / (gridDim.x * (blockDim.x >> 5)) + 1u, 32u);
 }
 
-// What a warp leaves behind at the end of its phase: event counts, empty
-// marks on the queue slots it reserved but never wrote, its share of the
-// ledger; then the CTA's counters.
+// What a warp leaves behind at the end of its phase: empty marks on the queue
+// slots it reserved but never wrote, its share of the ledger; then the CTA's
+// counters (Compton events are the other real collisions; a photoelectric
+// event ends its photon without a deposit; a push creates a particle).
 template <int PT>
-__device__ __forceinline__ void phase_end(const SimParams& P, const PhaseArgs& A, Acc& acc, Ev& ev,
-                                          WarpCnt& wc, const Slots (&sl)[2], uint32_t* s_cnt) {
+__device__ __forceinline__ void phase_end(const SimParams& P, const PhaseArgs& A, double esc,
+                                          const Slots (&sl)[PT + 1], uint32_t* s_cnt) {
     const uint32_t lane = lane_id();
-    flush_events<PT>(ev, s_cnt);
-    flush_warp_counts<PT>(wc, s_cnt);
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < PT + 1; ++q) {
         const Queue& Q = q ? A.out_ph : A.out_el;
-        const uint32_t slot = sl[q].base + lane;
-        if (lane < sl[q].left && slot < Q.capacity) queue_mark_empty(Q, slot);
+        const Slots h = sl[q];
+        const uint32_t slot = h.base + lane;
+        if (lane < h.left && slot < Q.capacity) queue_mark_empty(Q, slot);
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        acc.src += __shfl_down_sync(kFull, acc.src, o);
-        acc.esc += __shfl_down_sync(kFull, acc.esc, o);
-        acc.disc += __shfl_down_sync(kFull, acc.disc, o);
-    }
-    if (lane == 0) {
-        if (acc.src != 0.0) atomicAdd(&P.ledger[L_SOURCE], acc.src);
-        if (acc.esc != 0.0) atomicAdd(&P.ledger[L_ESCAPED], acc.esc);
-        if (acc.disc != 0.0) atomicAdd(&P.ledger[L_DISCARDED], acc.disc);
-    }
+    for (int o = 16; o > 0; o >>= 1) esc += __shfl_down_sync(kFull, esc, o);
+    if (lane == 0 && esc != 0.0) atomicAdd(&P.ledger[L_ESCAPED], esc);
     __syncthreads();
-    for (int k = threadIdx.x; k < C_NCOUNT; k += blockDim.x)
-        if (s_cnt[k]) atomicAdd(&P.counters[k], (unsigned long long)s_cnt[k]);
+    for (int k = threadIdx.x; k < C_NCOUNT; k += blockDim.x) {
+        const uint32_t n = k == C_COMPTON      ? s_cnt[C_PH_REAL] - s_cnt[C_PHOTO] - s_cnt[C_PAIR]
+                           : k == C_LOCAL_DEP  ? s_cnt[C_LOCAL_DEP] - s_cnt[C_PHOTO]
+                           : k == C_EL_CREATED ? s_cnt[C_PUSH_EL]
+                           : k == C_PH_CREATED ? s_cnt[C_PUSH_PH]
+                                               : s_cnt[k];
+        if (n) atomicAdd(&P.counters[k], (unsigned long long)n);
+    }
 }
 
 // Particle idx of the phase's input (its primaries first, then the queue)
@@ -1132,22 +1006,19 @@ __device__ __forceinline__ void photon_run(const SimParams& P, const PhaseArgs& 
     for (int k = threadIdx.x; k < C_NCOUNT; k += blockDim.x) s_cnt[k] = 0u;
     __syncthreads();
 
-    Acc acc{0.0, 0.0, 0.0};
+    double esc = 0.0;
     Part p{};
-    Ev ev{0u, 0u, 0u, 0u};
-    WarpCnt wc{0u, 0u, 0u};
-    Slots sl[2] = {{0u, 0u}, {0u, 0u}};
     const uint32_t lane = lane_id(), lt = lanemask_lt();
     bool active = false;
     uint32_t alive = 0u;                         // ballot of `active`
+    uint32_t n_flights = 0u;                     // the lane's, inside the phantom
+    uint32_t n_in_warp = 0u, n_done = 0u, n_on = 0u;   // the warp's: photons taken in, events, photons that went on
+    Slots sl[1] = {{0u, 0u}};
+    uint32_t pushes[1] = {0u};
     uint32_t n_ready = 0u, n_wait = 0u;          // the stack: [0, n_ready) and [kPhStack - n_wait, kPhStack)
     uint32_t st_base = 0u, st_left = 0u;         // the warp's block of work indices
     bool drained = false;                        // no input left
     for (uint32_t it = 0, trials = 0;; ++it) {
-        if ((it % kFlushEvery) == kFlushEvery - 1u) {
-            flush_events<0>(ev, s_cnt);
-            flush_warp_counts<0>(wc, s_cnt);
-        }
         while (n_wait < 32u && alive != full) {
             const uint32_t nm = full & ~alive, need = __popc(nm);
             // ---- input into the stack, up to kPhReady ready
@@ -1167,16 +1038,20 @@ __device__ __forceinline__ void photon_run(const SimParams& P, const PhaseArgs& 
                 if (lane < k) have = load_input(P, A, st_base + lane, q, from_queue);
                 st_base += k;
                 st_left -= k;
-                wc.w2 += __popc(__ballot_sync(kFull, from_queue));
-                if (have && q.E < T.eabs_ph) {   // only a source photon below the cutoff
-                    voxel_of(P, q);
-                    tally<GEN>(P, q.flags, vox_of(P, q.ix, q.iy, q.iz), q.E);
-                    ev.b += EV_TERM;
-                    have = false;
+                count(s_cnt, C_POP_PH, __popc(__ballot_sync(kFull, from_queue)));
+                const bool low = have && q.E < T.eabs_ph;   // only a source photon
+                if (__any_sync(kFull, low)) {
+                    if (low) {
+                        voxel_of(P, q);
+                        tally<GEN>(P, q.flags, vox_of(P, q.ix, q.iy, q.iz), q.E);
+                        have = false;
+                    }
+                    count(s_cnt, C_PH_TERMINATED, __popc(__ballot_sync(kFull, low)));
                 }
                 const uint32_t m = __ballot_sync(kFull, have);
                 if (have) rec_store(stack[n_ready + __popc(m & lt)], q);
                 n_ready += __popc(m);
+                n_in_warp += __popc(m);
                 __syncwarp();
             }
             // ---- free lanes take ready photons
@@ -1209,11 +1084,12 @@ __device__ __forceinline__ void photon_run(const SimParams& P, const PhaseArgs& 
             Flight what = Flight::fly;
             if (active) {
                 ++p.ctr;
-                what = photon_flight<GEN>(P, ps, p, x, acc, ev);
+                what = photon_flight<GEN>(P, ps, p, x, esc);
                 active = what == Flight::fly;
+                n_flights += what != Flight::gone;
             }
-            alive = __ballot_sync(kFull, active);
             const uint32_t m = __ballot_sync(kFull, what == Flight::wait);
+            alive = __ballot_sync(kFull, active);
             if (what == Flight::wait) rec_store(stack[kPhStack - 1u - n_wait - __popc(m & lt)], p);
             n_wait += __popc(m);
             __syncwarp();
@@ -1221,126 +1097,260 @@ __device__ __forceinline__ void photon_run(const SimParams& P, const PhaseArgs& 
             ++trials;
             Part q{};
             Sec sec{};
-            bool goes_on = false, done = true;
+            bool goes_on = false;
+            PhEvent what = PhEvent::none;
             if (lane < k) {
                 rec_load(*rec, q);
                 voxel_of(P, q);
-                done = photon_event<GEN>(P, q, x, trials > 4096u, goes_on, ev, sec);
+                what = photon_event<GEN>(P, q, x, trials > 4096u, goes_on, sec);
             }
             n_wait -= k;
-            bank_pending<0, GEN>(P, A, total, q, sec, sl, wc);
+            bank<0, GEN>(P, A, total, q, vox_packed(q.ix, q.iy, q.iz), sec, sl, pushes);
             __syncwarp();
-            const uint32_t gm = __ballot_sync(kFull, goes_on), wm = __ballot_sync(kFull, !done);
-            if (goes_on || !done)
+            const uint32_t gm = __ballot_sync(kFull, goes_on);
+            const uint32_t wm = __ballot_sync(kFull, lane < k && what == PhEvent::none);
+            if (lane < k && (goes_on || what == PhEvent::none))
                 rec_store(stack[goes_on ? n_ready + __popc(gm & lt) : kPhStack - 1u - n_wait - __popc(wm & lt)], q);
+            if (__any_sync(kFull, what > PhEvent::compton)) {
+                count(s_cnt, C_PHOTO, __popc(__ballot_sync(kFull, what == PhEvent::photo)));
+                count(s_cnt, C_PAIR, __popc(__ballot_sync(kFull, what == PhEvent::pair)));
+            }
+            n_done += k - __popc(wm);
+            n_on += __popc(gm);
             n_ready += __popc(gm);
             n_wait += __popc(wm);
             __syncwarp();
         }
     }
-    phase_end<0>(P, A, acc, ev, wc, sl, s_cnt);
+    // every photon taken in escaped or ended in an event; a Compton event that
+    // ends its photon deposits it (a photoelectric one does not, see
+    // phase_end), and every event has one secondary (a pair two), banked or
+    // deposited
+    n_flights = __reduce_add_sync(kFull, n_flights);
+    count(s_cnt, C_PH_FLIGHTS, n_flights);
+    count(s_cnt, C_PH_TERMINATED, n_in_warp);
+    count(s_cnt, C_PH_REAL, n_done);
+    count(s_cnt, C_LOCAL_DEP, 2u * n_done - n_on - pushes[0]);
+    count(s_cnt, C_PUSH_EL, pushes[0]);
+    phase_end<0>(P, A, esc, sl, s_cnt);
 }
 
 // ---------------------------------------------------------------- electron phase
-// The electron phase: loop top (whole warp): fold event counters now and
-// then, bank the secondaries of the last step, refill lanes whose particle
-// ended.  Then each lane takes one step of its own particle.  PT: 1 a whole
-// step per iteration, 2 resumable steps.
-template <int PT, bool GEN>
+// A warp's electrons that are not in a lane: a stack in shared memory like
+// the photons', in planes of 16 bytes (a 64-byte record would put every
+// second lane on the same banks).
+constexpr uint32_t kElReady = 32, kElWait = 32, kElStack = kElReady + kElWait + 32;
+struct ElStack {
+    uint4 a[kElStack], b[kElStack], c[kElStack], d[kElStack];
+    Slots held[2];      // the warp's queue reservations, used only by event rounds
+};
+
+__device__ __forceinline__ void el_store(ElStack& s, uint32_t i, const Electron& p, uint32_t kind) {
+    s.a[i] = pack4(p.x, p.y, p.z, __float_as_uint(p.E));
+    s.b[i] = pack4(p.u, p.v, p.w, p.vox);
+    s.c[i] = make_uint4(p.hist, p.pidlo, p.pidhi, p.ctr);
+    s.d[i] = make_uint4(__float_as_uint(p.pend), p.flags, kind, 0u);
+}
+__device__ __forceinline__ uint32_t el_load(const ElStack& s, uint32_t i, Electron& p) {
+    const uint4 a = s.a[i], b = s.b[i], c = s.c[i], d = s.d[i];
+    p.x = __uint_as_float(a.x); p.y = __uint_as_float(a.y); p.z = __uint_as_float(a.z);
+    p.E = __uint_as_float(a.w);
+    p.u = __uint_as_float(b.x); p.v = __uint_as_float(b.y); p.w = __uint_as_float(b.z);
+    p.vox = b.w;
+    p.hist = c.x; p.pidlo = c.y; p.pidhi = c.z; p.ctr = c.w;
+    p.pend = __uint_as_float(d.x);
+    p.flags = d.y;
+    return d.z;
+}
+
+// The electron phase, in rounds like the photon phase.  In a step round every
+// lane sets up a step (unless one is in progress) and walks it.  A step that
+// ends in a hard-event candidate, and a positron at rest, waits in shared
+// memory; once kElWait wait, an event round gives each of 32 its next draw.
+// In one lane's own loop, as each lane reached them, the draw, walk, candidate
+// and Moller code ran with 14.8 of 32 lanes active and 271 warp instructions
+// a history; now 20 and 205.  Measured against that (1e8 histories of the CT
+// plan; 2.5e8 of the paper's lung slab; 2.5e6 20 MeV electrons on its bone
+// slab): electron phase 29.6 -> 25.7, 54.8 -> 50.0, 7.0 -> 5.6 ms.
+template <bool GEN>
 __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs& A) {
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t n_in = A.in_count ? min(*A.in_count, A.in.capacity) : 0u;
     const uint32_t total = A.n_src + n_in;
     if (blockIdx.x >= total) return;
+    const uint32_t lanes = phase_lanes(total), full = kFull >> (32u - lanes);
 
     const DevTables& T = P.T;
     const size_t ne = size_t(T.n_mat) * T.n_e;
-    ElSmem es{};
     float4* el = reinterpret_cast<float4*>(smem);
     float* rinv = reinterpret_cast<float*>(smem + ne * 16);
     const size_t nr = size_t(T.n_mat) * T.n_r;
     float* atab = reinterpret_cast<float*>(smem + ne * 16 + align16(nr * 4));
-    uint32_t* s_cnt = reinterpret_cast<uint32_t*>(smem + ne * 16 + align16(nr * 4) +
-                                        align16(size_t(T.n_a) * 4));
+    unsigned char* after = smem + ne * 16 + align16(nr * 4) + align16(size_t(T.n_a) * 4);
+    uint32_t* s_cnt = reinterpret_cast<uint32_t*>(after);
+    ElStack& stack = reinterpret_cast<ElStack*>(after + align16(C_NCOUNT * 4))[threadIdx.x >> 5];
+    if (lane_id() < 4u) (&stack.held[0].base)[lane_id()] = 0u;
     copy_to_smem(el, T.el, ne * 16);
     copy_to_smem(rinv, T.rinv, nr * 4);
     copy_to_smem(atab, T.atab, size_t(T.n_a) * 4);
-    es.el = el; es.rinv = rinv; es.atab = atab;
+    const ElSmem es{el, rinv, atab};
     for (int k = threadIdx.x; k < C_NCOUNT; k += blockDim.x) s_cnt[k] = 0u;
     __syncthreads();
 
-    Acc acc{0.0, 0.0, 0.0};
-    Part p{};
-    Sec sec{};
-    Ev ev{0u, 0u, 0u, 0u};
-    WarpCnt wc{0u, 0u, 0u};
-    Slots sl[2] = {{0u, 0u}, {0u, 0u}};
-    const uint32_t lane = lane_id();
-    bool active = false, exhausted = lane >= phase_lanes(total);
-    float pend = 0.f;   // electron energy owed to its current voxel (see walk)
-    ElStep est{};       // electron step in progress (leg 0: none)
-    // the warp's block of work indices [st_base, st_base + st_left)
-    uint32_t st_base = 0u, st_left = 0u;
-    for (uint32_t it = 0;; ++it) {
-        // ---- whole warp: account and bank the last step, then refill
-        if ((it % kFlushEvery) == kFlushEvery - 1u) {
-            flush_events<PT>(ev, s_cnt);
-            flush_warp_counts<PT>(wc, s_cnt);
-        }
-        bank_pending<PT, GEN>(P, A, total, p, sec, sl, wc);
-        sec.n = 0;
-        const bool need = !active && !exhausted;
-        const uint32_t nm = __ballot_sync(kFull, need);
-        if (nm) {
-            const uint32_t k = __popc(nm);
-            const uint32_t left0 = st_left, base0 = st_base;
-            uint32_t nb = 0u;
-            if (k > st_left) {
-                const uint32_t miss = k - st_left;
-                const uint32_t want = max(miss, min((total - min(total, st_base)) >> A.share_shift, kGrab));
-                if (lane == 0) nb = atomicAdd(A.head, want);
-                nb = __shfl_sync(kFull, nb, 0);
-                st_base = nb + miss;
-                st_left = want - miss;
-            } else {
+    double esc = 0.0;
+    Electron p{};
+    ElStep st{};
+    const uint32_t lane = lane_id(), lt = lanemask_lt();
+    bool active = false;
+    uint32_t alive = 0u;                         // ballot of `active`
+    uint32_t n_steps = 0u, n_ended = 0u;         // the warp's
+    uint32_t crossings = 0u;                     // the lane's
+    uint32_t n_ready = 0u, n_wait = 0u;          // the stack: [0, n_ready) and [kElStack - n_wait, kElStack)
+    uint32_t st_base = 0u, st_left = 0u;         // the warp's block of work indices
+    bool drained = false;                        // no input left
+    for (uint32_t it = 0, draws = 0;; ++it) {
+        while (n_wait < kElWait && alive != full) {
+            const uint32_t nm = full & ~alive, need = __popc(nm);
+            // ---- input into the stack, up to kElReady ready
+            if (n_ready < min(need, kElReady) && !drained) {
+                if (st_left == 0u) {
+                    const uint32_t block = max(need, min((total - min(total, st_base)) >> A.share_shift, kGrab));
+                    uint32_t nb = 0u;
+                    if (lane == 0) nb = atomicAdd(A.head, block);
+                    nb = __shfl_sync(kFull, nb, 0);
+                    st_base = nb;
+                    st_left = nb < total ? min(block, total - nb) : 0u;
+                    drained = st_left == 0u;
+                }
+                const uint32_t k = min(kElReady - n_ready, st_left);
+                Part q;
+                Electron e{};
+                bool from_queue = false, have = false;
+                if (lane < k) {
+                    have = load_input(P, A, st_base + lane, q, from_queue);
+                    if (have && !from_queue) voxel_of(P, q);
+                    e = Electron{q.x, q.y, q.z, q.u, q.v, q.w, q.E, 0.f, vox_packed(q.ix, q.iy, q.iz),
+                                 q.hist, q.pidlo, q.pidhi, q.ctr, q.flags};
+                }
                 st_base += k;
                 st_left -= k;
-            }
-            bool from_queue = false;
-            if (need) {
-                const uint32_t r = __popc(nm & lanemask_lt());
-                const uint32_t idx = r < left0 ? base0 + r : nb + (r - left0);
-                if (idx < total) {
-                    active = load_input(P, A, idx, p, from_queue);
-                    if (active && idx < A.n_src) voxel_of(P, p);
-                } else {
-                    exhausted = true;
+                count(s_cnt, C_POP_EL, __popc(__ballot_sync(kFull, from_queue)));
+                // below the cutoff: a source electron, or a positron, which
+                // annihilates
+                const bool low = have && e.E < T.eabs_el;
+                if (__any_sync(kFull, low)) {
+                    uint32_t kind = 0u;
+                    const bool wait = low && absorb<GEN>(P, e, kind) == Round::wait;
+                    const uint32_t wm = __ballot_sync(kFull, wait);
+                    if (wait) el_store(stack, kElStack - 1u - n_wait - __popc(wm & lt), e, kind);
+                    n_wait += __popc(wm);
+                    n_ended += __popc(__ballot_sync(kFull, low)) - __popc(wm);
+                    have = have && !low;
                 }
+                const uint32_t m = __ballot_sync(kFull, have);
+                if (have) el_store(stack, n_ready + __popc(m & lt), e, 0u);
+                n_ready += __popc(m);
+                __syncwarp();
             }
-            wc.w2 += __popc(__ballot_sync(kFull, from_queue));
+            // ---- free lanes take ready electrons
+            const uint32_t r = __popc(nm & lt);
+            if (!active && r < n_ready && lane < lanes) {
+                el_load(stack, n_ready - 1u - r, p);
+                active = true;
+                st.what = 0u;
+            }
+            n_ready -= min(need, n_ready);
+            __syncwarp();
+            alive = __ballot_sync(kFull, active);
+            if (drained) break;
         }
-        if (__all_sync(kFull, exhausted)) break;
+        // ---- which round: events once kElWait electrons wait, or, when the
+        // input is drained, once no fewer wait than walk
+        const uint32_t walking = __popc(alive) + n_ready;
+        const bool events = n_wait >= kElWait || (drained && n_wait >= walking);
+        if (walking + n_wait == 0u) break;
         if (it >= P.max_iters) {
             if (lane == 0) atomicOr(P.status, ST_ITER_CAP);
             break;
         }
-        // ---- each lane on its own: one step
-        if (active) {
-            electron_step<PT == 2, GEN>(P, es, p, active, acc, ev, sec, pend, est);
+        const uint32_t k = min(n_wait, 32u);
+        const uint32_t top = kElStack - n_wait + (lane < k ? lane : 0u);     // the k last set aside
+        uint4 c = make_uint4(p.hist, p.pidlo, p.pidhi, p.ctr);
+        if (events) c = stack.c[top];
+        const uint4 x = philox4x32_10(c, P.key0, P.key1);
+        if (!events) {
+            draws = 0u;
+            uint32_t kind = 0u;
+            Round what = Round::go;
+            n_steps += __popc(__ballot_sync(kFull, active && (st.what & 3u) == 0u));
+            if (active) {
+                what = electron_round<GEN>(P, es, p, st, x, esc, crossings, kind);
+                active = what == Round::go;
+            }
+            const uint32_t m = __ballot_sync(kFull, what == Round::wait);
+            n_ended += __popc(alive);
+            alive = __ballot_sync(kFull, active);
+            n_ended -= __popc(m) + __popc(alive);
+            if (what == Round::wait) el_store(stack, kElStack - 1u - n_wait - __popc(m & lt), p, kind);
+            n_wait += __popc(m);
+            __syncwarp();
+        } else {
+            ++draws;
+            Electron q{};
+            Sec sec{};
+            uint32_t kind = 0u, was = 0u;
+            Round what = Round::ended;
+            if (lane < k) {
+                was = kind = el_load(stack, top, q);
+                what = electron_event<GEN>(P, es, q, kind, x, draws > 4096u, sec);
+            }
+            n_wait -= k;
+            if (__any_sync(kFull, sec.n > 0)) {
+                Slots sl[2] = {stack.held[0], stack.held[1]};
+                uint32_t pushes[2] = {0u, 0u};
+                bank<1, GEN>(P, A, total, q, q.vox, sec, sl, pushes);
+                const uint32_t mol = __popc(__ballot_sync(kFull, sec.n > 0 && (was & 3u) == kMoller));
+                const uint32_t brems = __popc(__ballot_sync(kFull, sec.n > 0 && (was & 3u) == kCandidate));
+                const uint32_t annihil = __popc(__ballot_sync(kFull, sec.n > 1));
+                if (lane == 0) {
+                    stack.held[0] = sl[0];
+                    stack.held[1] = sl[1];
+                }
+                // one shared-memory atomic for the six counters
+                const uint32_t n = lane == 0 ? mol : lane == 1 ? brems : lane == 2 ? annihil
+                                   : lane == 3 ? pushes[0] : lane == 4 ? pushes[1]
+                                               : mol + brems + 2u * annihil - pushes[0] - pushes[1];
+                const int slot = lane == 0 ? C_MOLLER : lane == 1 ? C_BREMS : lane == 2 ? C_ANNIHIL
+                                 : lane == 3 ? C_PUSH_EL : lane == 4 ? C_PUSH_PH : C_LOCAL_DEP;
+                if (lane < 6u) atomicAdd(&s_cnt[slot], n);
+            }
+            __syncwarp();
+            const uint32_t gm = __ballot_sync(kFull, lane < k && what == Round::go);
+            const uint32_t wm = __ballot_sync(kFull, lane < k && what == Round::wait);
+            if (lane < k && what != Round::ended)
+                el_store(stack, what == Round::go ? n_ready + __popc(gm & lt)
+                                                  : kElStack - 1u - n_wait - __popc(wm & lt), q, kind);
+            n_ended += k - __popc(gm) - __popc(wm);
+            n_ready += __popc(gm);
+            n_wait += __popc(wm);
+            __syncwarp();
         }
     }
     // only a phase stopped by its iteration cap leaves a track unfinished
-    if (pend != 0.f) tally<GEN>(P, p.flags, vox_of(P, p.ix, p.iy, p.iz), pend);
-    phase_end<PT>(P, A, acc, ev, wc, sl, s_cnt);
+    if (active && p.pend != 0.f) tally<GEN>(P, p.flags, vox_linear(P, p.vox), p.pend);
+    count(s_cnt, C_EL_STEPS, n_steps);
+    count(s_cnt, C_EL_TERMINATED, n_ended);
+    count(s_cnt, C_CROSS, __reduce_add_sync(kFull, crossings));
+    const Slots sl[2] = {stack.held[0], stack.held[1]};
+    phase_end<1>(P, A, esc, sl, s_cnt);
 }
 
 // One transport phase (Sec. 2.2.1 Step 3), a persistent loop per warp.  PT: 0
-// photons, 1 electrons a whole step per iteration, 2 electrons with resumable
-// steps.
+// photons, 1 electrons.
 template <int PT, bool GEN>
 __device__ __forceinline__ void phase_run(const SimParams& P, const PhaseArgs& A) {
     if constexpr (PT == 0) photon_run<GEN>(P, A);
-    else electron_run<PT, GEN>(P, A);
+    else electron_run<GEN>(P, A);
 }
 
 template <int PT, bool GEN>
@@ -1369,7 +1379,7 @@ __device__ __forceinline__ void make_sources(const SimParams& P, const PhaseArgs
     __syncthreads();
     const uint32_t* ptab = n_prefix ? s_prefix : nullptr;
     const float* ctab = n_cdf ? s_cdf : nullptr;
-    Acc acc{0.0, 0.0, 0.0};
+    Acc acc{0.0, 0.0};
     uint32_t made = 0u, missed = 0u;
     for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < A.n_src;
          idx += gridDim.x * blockDim.x) {
@@ -1474,8 +1484,7 @@ __device__ __forceinline__ PhaseArgs phase_args(const LoopArgs& L, uint32_t k) {
 
 // One pass of the device-driven loop runs photon phase k and electron
 // phase k+1, k = *L.k (even); PT selects which of the two this launch is
-// (0 the photon phase; 1 or 2 the electron phase in its whole-step or
-// resumable form).
+// (0 the photon phase, 1 the electron phase).
 // The phase's arguments are derived in shared memory from k.  (A kernel of
 // its own: the host loop's k_phase takes them as kernel parameters, which
 // keeps more registers for the transport loop.)
@@ -1647,7 +1656,7 @@ __global__ void k_debug_sources(const SimParams P, const PhaseArgs A, uint64_t n
     for (uint64_t s = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; s < n;
          s += uint64_t(gridDim.x) * blockDim.x) {
         Part p{};
-        Acc acc{0, 0, 0};
+        Acc acc{0, 0};
         const bool in = make_primary(P, A, uint32_t(s), p, acc);
         double* o = out + 8 * s;
         o[0] = p.x; o[1] = p.y; o[2] = p.z; o[3] = p.u; o[4] = p.v; o[5] = p.w; o[6] = p.E;
@@ -1687,12 +1696,11 @@ struct Launch {
 static Launch phase_shape(const gdpm_ctx* ctx, const DevTables& T, int pt) {
     constexpr size_t kMaxSmem = size_t(227) << 10;
     const size_t tables = smem_of(T, pt == 0 ? GDPM_PHOTON : GDPM_ELECTRON);
-    const size_t stack = pt == 0 ? kPhStack * sizeof(PhRec) : 0;
+    const size_t stack = pt == 0 ? kPhStack * sizeof(PhRec) : sizeof(ElStack);
     int thr = ctx->block_threads > 0 ? ctx->block_threads
               : pt == 0              ? PhaseShape<0>::threads
-              : pt == 1              ? PhaseShape<1>::threads
-                                     : PhaseShape<2>::threads;
-    if (stack) thr = std::min(thr, 32 * int((kMaxSmem - tables) / stack));
+                                     : PhaseShape<1>::threads;
+    thr = std::min(thr, 32 * int((kMaxSmem - tables) / stack));
     return Launch{thr, tables + stack * size_t(thr / 32)};
 }
 
@@ -1702,14 +1710,12 @@ static Launch phase_shape(const gdpm_ctx* ctx, const DevTables& T, int pt) {
 // since persistent CTAs do not yield until their phase's input is drained.
 int launch_phase(gdpm_ctx* ctx, cudaStream_t st, int particle, const SimParams& P,
                  const PhaseArgs& A, uint32_t n_items_hint, uint32_t share_eighths) {
-    const bool resumable = particle != GDPM_PHOTON && P.walk_resumable;
-    const Launch shape = phase_shape(ctx, P.T, particle == GDPM_PHOTON ? 0 : resumable ? 2 : 1);
+    const Launch shape = phase_shape(ctx, P.T, particle == GDPM_PHOTON ? 0 : 1);
     const int thr = shape.threads;
     const size_t smem = shape.smem;
     using Kernel = void (*)(const SimParams, const PhaseArgs);
     const bool gen = P.tally_mode != 0 || P.hrec;
     const Kernel fn = particle == GDPM_PHOTON ? (gen ? k_phase<0, true> : k_phase<0, false>)
-                      : resumable             ? (gen ? k_phase<2, true> : k_phase<2, false>)
                                               : (gen ? k_phase<1, true> : k_phase<1, false>);
     GDPM_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
     int bps = ctx->blocks_per_sm;
@@ -1772,13 +1778,11 @@ int build_loop_graph(gdpm_ctx* ctx, const SimParams& P, LoopArgs& L, bool metrop
     *exec = nullptr;
     uint32_t grid[2];
     size_t smem[2];
-    const void* fn[2] = {(const void*)k_phase_loop<0>,
-                         P.walk_resumable ? (const void*)k_phase_loop<2>
-                                          : (const void*)k_phase_loop<1>};
+    const void* fn[2] = {(const void*)k_phase_loop<0>, (const void*)k_phase_loop<1>};
     int thr[2];
     uint64_t warps = 0;
     for (int t = 0; t < 2; ++t) {
-        const Launch shape = phase_shape(ctx, P.T, t == 0 ? 0 : P.walk_resumable ? 2 : 1);
+        const Launch shape = phase_shape(ctx, P.T, t);
         thr[t] = shape.threads;
         smem[t] = shape.smem;
         GDPM_CUDA_TRY(cudaFuncSetAttribute(fn[t], cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem[t])));
