@@ -383,6 +383,7 @@ SimParams base_params(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb, uint32_t
     P.T = tb->dev;
     P.key0 = uint32_t(ctx->seed);
     P.key1 = uint32_t(ctx->seed >> 32) ^ request_id;
+    P.keys = round_keys(P.key0, P.key1);
     P.tally_mode = ctx->tally_mode;
     P.walk_trips = walk_form(ctx) ? 2 : 1 << 30;
     P.max_iters = ctx->max_iters;   // loop trips per warp and phase (GDPM_PARAM_MAX_ITERS)

@@ -69,6 +69,30 @@ __host__ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, ui
     return c;
 }
 
+// The ten round keys of a key (k0, k1), and a block with round keys made
+// before (they are the same for every block of a run).
+struct RoundKeys {
+    uint2 k[10];
+};
+__host__ __device__ __forceinline__ RoundKeys round_keys(uint32_t k0, uint32_t k1) {
+    RoundKeys r;
+    for (int i = 0; i < 10; ++i) {
+        r.k[i] = make_uint2(k0, k1);
+        k0 += 0x9E3779B9u;
+        k1 += 0xBB67AE85u;
+    }
+    return r;
+}
+__device__ __forceinline__ uint4 philox4x32_10(uint4 c, const RoundKeys& K) {
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        const uint64_t p0 = uint64_t(0xD2511F53u) * c.x, p1 = uint64_t(0xCD9E8D57u) * c.z;
+        c = make_uint4(uint32_t(p1 >> 32) ^ c.y ^ K.k[r].x, uint32_t(p1), uint32_t(p0 >> 32) ^ c.w ^ K.k[r].y,
+                       uint32_t(p0));
+    }
+    return c;
+}
+
 // 23-bit uniform in the open interval (0,1): (floor(x/2^9) + 1/2) / 2^23,
 // exactly representable in FP32, so it never rounds to 0 or 1.  The top 23
 // bits become the mantissa of a float in [1, 2) (one funnel shift), and

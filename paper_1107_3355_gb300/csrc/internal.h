@@ -128,6 +128,7 @@ struct SimParams {
     DevTables T;
     DevSource S;
     uint32_t key0, key1;
+    RoundKeys keys;            // of (key0, key1)
     double* edep;              // FP64 batch tally (MeV)
     uint32_t batch_stride;     // voxels between batch grids (0: one grid for the current batch)
     float* edep_hi;            // FP32 compensated tally

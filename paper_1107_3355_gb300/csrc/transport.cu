@@ -471,10 +471,14 @@ __device__ __forceinline__ PhEvent photon_event(const SimParams& P, Part& p, uin
 }
 
 // ---------------------------------------------------------------- electron step
+struct __align__(16) ElMat {      // a material's constants of a step (shared memory)
+    float r_eabs, inv_sigmax, rinv_lo, rinv_idr, inv_x0, sigmax, pad[2];
+};
 struct ElSmem {
     const float4* el;
     const float* rinv;
     const float* atab;
+    const ElMat* mat;
 };
 
 // An electron or positron in a lane: its voxel is packed (10 bits an axis),
@@ -528,17 +532,14 @@ __device__ __forceinline__ Round absorb(const SimParams& P, Electron& p, uint32_
 }
 
 // Set up a step with the draw x: step limits as mass thickness in the start
-// voxel's material, energy at its end, deflection at the random hinge.
+// voxel's material (`mat`), energy at its end, deflection at the random hinge.
 template <bool GEN>
 __device__ __forceinline__ void electron_setup(const SimParams& P, const ElSmem& S, const Electron& p, uint4 x,
-                                               ElStep& st) {
+                                               int mat, ElStep& st) {
     const DevTables& T = P.T;
     const float4 r = make_float4(u01(x.x), u01(x.y), u01(x.z), u01(x.w));
     hist_count<GEN>(P, p.hist, 1);
-    // material and density of the start voxel, loaded together
-    const uint32_t vox0 = GDPM_IDX(P.status, vox_linear(P, p.vox), n_voxels(P), ST_B_VOXEL);
-    const int m = GDPM_IDX(P.status, int(__ldg(&P.mat[vox0])), T.n_mat, ST_B_TABLE);
-    st.rho = __ldg(&P.rho[vox0]);
+    const int m = GDPM_IDX(P.status, mat, T.n_mat, ST_B_TABLE);
     int i;
     float f;
     grid_pos(T, p.E, i, f);
@@ -546,8 +547,9 @@ __device__ __forceinline__ void electron_setup(const SimParams& P, const ElSmem&
     const float4 a0 = S.el[mi], a1 = S.el[mi + 1];
     const float R0 = lerpf(a0.x, a1.x, f);
     const float xms = lerpf(a0.y, a1.y, f);
-    const float xcut = R0 - T.r_eabs[m];
-    const float xhard = (T.flags & GDPM_FLAG_NO_HARD) ? kInf : -__logf(r.x) * T.inv_sigmax[m];
+    const ElMat M = S.mat[m];
+    const float xcut = R0 - M.r_eabs;
+    const float xhard = (T.flags & GDPM_FLAG_NO_HARD) ? kInf : -__logf(r.x) * M.inv_sigmax;
     uint32_t lim;
     float xs;
     if (xcut <= xms && xcut <= xhard) { lim = 0u; xs = xcut; }
@@ -558,7 +560,7 @@ __device__ __forceinline__ void electron_setup(const SimParams& P, const ElSmem&
     if (lim == 0u) {
         Tend = T.eabs_el;
     } else {
-        const float rr = (R0 - xs - T.rinv_lo[m]) * T.rinv_idr[m];
+        const float rr = (R0 - xs - M.rinv_lo) * M.rinv_idr;
         const int j = min(max(int(floorf(rr)), 0), T.n_r - 2);
         const float g = fminf(fmaxf(rr - float(j), 0.f), 1.f);
         const float* ri = S.rinv + m * T.n_r;
@@ -571,7 +573,7 @@ __device__ __forceinline__ void electron_setup(const SimParams& P, const ElSmem&
     const float Tm = 0.5f * (Tk + Tend);
     const float pbc = Tm * (Tm + 2.f * kMC2f) / (Tm + kMC2f);
     const float q = kEs / pbc;
-    const float G1 = xs * q * q * 0.5f * T.inv_x0[m];
+    const float G1 = xs * q * q * 0.5f * M.inv_x0;
     float mu;
     if (G1 >= 1.f) {
         mu = 2.f * r.z - 1.f;
@@ -682,10 +684,11 @@ __device__ __forceinline__ int walk_stretch(const SimParams& P, Electron& p, ElS
 // hard-event candidate.
 template <bool GEN>
 __device__ __forceinline__ Round electron_round(const SimParams& P, const ElSmem& S, Electron& p, ElStep& st,
-                                                uint4 x, double& esc, uint32_t& crossings, uint32_t& kind) {
+                                                uint4 x, int mat, double& esc, uint32_t& crossings,
+                                                uint32_t& kind) {
     if ((st.what & 3u) == 0u) {
         ++p.ctr;
-        electron_setup<GEN>(P, S, p, x, st);
+        electron_setup<GEN>(P, S, p, x, mat, st);
     }
     Walk k;
     k.lin = vox_linear(P, p.vox);
@@ -746,7 +749,7 @@ __device__ __forceinline__ Round electron_event(const SimParams& P, const ElSmem
             if (Tn > wcb) sb = lerpf(a0.w, a1.w, f);
         }
         const float sh = sm + sb;
-        if (u01(x.x) * T.sigmax[m] < sh) {
+        if (u01(x.x) * S.mat[m].sigmax < sh) {
             hist_count<GEN>(P, p.hist, 2);
             if (u01(x.y) * sh < sm) {
                 kind = kMoller;
@@ -1078,7 +1081,7 @@ __device__ __forceinline__ void photon_run(const SimParams& P, const PhaseArgs& 
         const PhRec* const rec = stack + (kPhStack - n_wait) + (lane < k ? lane : 0u);   // the k last set aside
         uint4 c = make_uint4(p.hist, p.pidlo, p.pidhi, p.ctr);
         if (events) c = rec->c;
-        const uint4 x = philox4x32_10(c, P.key0, P.key1);
+        const uint4 x = philox4x32_10(c, P.keys);
         if (!events) {
             trials = 0u;
             Flight what = Flight::fly;
@@ -1188,12 +1191,17 @@ __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs
     float* atab = reinterpret_cast<float*>(smem + ne * 16 + align16(nr * 4));
     unsigned char* after = smem + ne * 16 + align16(nr * 4) + align16(size_t(T.n_a) * 4);
     uint32_t* s_cnt = reinterpret_cast<uint32_t*>(after);
-    ElStack& stack = reinterpret_cast<ElStack*>(after + align16(C_NCOUNT * 4))[threadIdx.x >> 5];
+    ElMat* mats = reinterpret_cast<ElMat*>(after + align16(C_NCOUNT * 4));
+    ElStack& stack = reinterpret_cast<ElStack*>(mats + kMaxMat)[threadIdx.x >> 5];
+    if (threadIdx.x < uint32_t(T.n_mat)) {
+        const int m = int(threadIdx.x);
+        mats[m] = ElMat{T.r_eabs[m], T.inv_sigmax[m], T.rinv_lo[m], T.rinv_idr[m], T.inv_x0[m], T.sigmax[m]};
+    }
     if (lane_id() < 4u) (&stack.held[0].base)[lane_id()] = 0u;
     copy_to_smem(el, T.el, ne * 16);
     copy_to_smem(rinv, T.rinv, nr * 4);
     copy_to_smem(atab, T.atab, size_t(T.n_a) * 4);
-    const ElSmem es{el, rinv, atab};
+    const ElSmem es{el, rinv, atab, mats};
     for (int k = threadIdx.x; k < C_NCOUNT; k += blockDim.x) s_cnt[k] = 0u;
     __syncthreads();
 
@@ -1276,15 +1284,24 @@ __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs
         const uint32_t k = min(n_wait, 32u);
         const uint32_t top = kElStack - n_wait + (lane < k ? lane : 0u);     // the k last set aside
         uint4 c = make_uint4(p.hist, p.pidlo, p.pidhi, p.ctr);
-        if (events) c = stack.c[top];
-        const uint4 x = philox4x32_10(c, P.key0, P.key1);
+        // material and density of the voxel a step starts in: the loads run
+        // while the draw is made
+        int mat = 0;
+        if (events) {
+            c = stack.c[top];
+        } else if (active && (st.what & 3u) == 0u) {
+            const uint32_t vox0 = GDPM_IDX(P.status, vox_linear(P, p.vox), n_voxels(P), ST_B_VOXEL);
+            mat = int(__ldg(&P.mat[vox0]));
+            st.rho = __ldg(&P.rho[vox0]);
+        }
+        const uint4 x = philox4x32_10(c, P.keys);
         if (!events) {
             draws = 0u;
             uint32_t kind = 0u;
             Round what = Round::go;
             n_steps += __popc(__ballot_sync(kFull, active && (st.what & 3u) == 0u));
             if (active) {
-                what = electron_round<GEN>(P, es, p, st, x, esc, crossings, kind);
+                what = electron_round<GEN>(P, es, p, st, x, mat, esc, crossings, kind);
                 active = what == Round::go;
             }
             const uint32_t m = __ballot_sync(kFull, what == Round::wait);
@@ -1672,7 +1689,8 @@ static size_t smem_of(const DevTables& T, int particle) {
     const size_t cnt = align16(C_NCOUNT * 4);
     if (particle == GDPM_PHOTON)
         return align16(ne * 8) + align16(ne * 4) + align16(size_t(T.n_e) * 4) + cnt;
-    return ne * 16 + align16(size_t(T.n_mat) * T.n_r * 4) + align16(size_t(T.n_a) * 4) + cnt;
+    return ne * 16 + align16(size_t(T.n_mat) * T.n_r * 4) + align16(size_t(T.n_a) * 4) + cnt +
+           kMaxMat * sizeof(ElMat);
 }
 
 // log2 of at least twice the warps of a phase: items >> shift is at most half
