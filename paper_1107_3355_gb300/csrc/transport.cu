@@ -679,13 +679,18 @@ __device__ __forceinline__ int walk_stretch(const SimParams& P, Electron& p, ElS
     return walk_cross<GEN>(P, p, s, k, crossings) ? 0 : 2;
 }
 
+// Stretches per round once the phase's input is drained: a lane whose step
+// ends has nothing to take over, so the lanes with many crossings (air) need
+// not give up the warp.
+constexpr int kDrainedStretches = 16;
+
 // A lane's round: set up a step when none is in progress (`starts`, with the
 // draw x), walk, and at the step's end escape, be absorbed, or wait for the
 // hard-event candidate.
 template <bool GEN>
 __device__ __forceinline__ Round electron_round(const SimParams& P, const ElSmem& S, Electron& p, ElStep& st,
-                                                uint4 x, int mat, double& esc, uint32_t& crossings,
-                                                uint32_t& kind) {
+                                                uint4 x, int mat, int stretches, double& esc,
+                                                uint32_t& crossings, uint32_t& kind) {
     if ((st.what & 3u) == 0u) {
         ++p.ctr;
         electron_setup<GEN>(P, S, p, x, mat, st);
@@ -696,7 +701,7 @@ __device__ __forceinline__ Round electron_round(const SimParams& P, const ElSmem
     walk_aim(p, k);
     int res = walk_stretch<GEN>(P, p, st, k, crossings);
 #pragma unroll 1
-    for (int n = 1; res == 0 && n < P.walk_trips; ++n) res = walk_stretch<GEN>(P, p, st, k, crossings);
+    for (int n = 1; res == 0 && n < stretches; ++n) res = walk_stretch<GEN>(P, p, st, k, crossings);
     if (res == 0) return Round::go;
     st.what &= ~3u;
     if (res == 2) {
@@ -1301,7 +1306,8 @@ __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs
             Round what = Round::go;
             n_steps += __popc(__ballot_sync(kFull, active && (st.what & 3u) == 0u));
             if (active) {
-                what = electron_round<GEN>(P, es, p, st, x, mat, esc, crossings, kind);
+                what = electron_round<GEN>(P, es, p, st, x, mat, drained ? max(P.walk_trips, kDrainedStretches) : P.walk_trips, esc,
+                                           crossings, kind);
                 active = what == Round::go;
             }
             const uint32_t m = __ballot_sync(kFull, what == Round::wait);
