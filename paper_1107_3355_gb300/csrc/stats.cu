@@ -159,14 +159,16 @@ __device__ __forceinline__ double root(double var) {
 // would change no bit of a sum); a warp spends FP64 operations for the lane
 // with the most.  Those tallies are then zeroed, after all of the chunk's
 // loads, which leaves the grids ready for the next calculation.
-// Measured with the finalize work in the same kernel (below): CT phantom, 10
-// grids of one beamlet's 1e5 histories 0.98 -> 0.24 ms; 128^3 slab, 100 grids
-// of 1e4 histories each 0.93 -> 0.45 ms; CT plan, 100 grids of 1e6 histories
-// each 3.7 -> 2.7 ms (6.7 GB read).  16 batches at a time and 64 registers
-// were best: 8 (40 registers) +14 %, 32 (128 registers) +25-33 %.
+// Measured with the finalize work in the same kernel (below) and the metric:
+// CT phantom, 10 grids of one beamlet's 1e5 histories 0.98 -> 0.19 ms; 128^3
+// slab, 100 grids of 1e4 histories each 0.93 -> 0.38 ms; CT plan, 100 grids of
+// 1e6 histories each 3.7 -> 2.6 ms (6.7 GB read).  10 batches at a time (whole
+// chunks of the usual 10, 20 and 100) at five CTAs per SM were best: 16 at
+// four +9 to +20 %, 20 to 32 at two or three +15 to +60 %.
 template <int VPT, int UB>
 __device__ __forceinline__ void batch_sums(const SimParams& P, size_t V, size_t first, size_t v,
-                                           int b0, int b1, double (&se)[VPT], double (&sq)[VPT]) {
+                                           int b0, int b1, double (&se)[VPT], double (&sq)[VPT],
+                                           uint32_t (&have)[VPT]) {
     const bool pair = P.tally_mode != 0;
     for (int b = b0; b < b1; b += UB) {
         uint32_t mask[VPT] = {};
@@ -199,6 +201,7 @@ __device__ __forceinline__ void batch_sums(const SimParams& P, size_t V, size_t 
 #pragma unroll
         for (int i = 0; i < VPT; ++i) {
             const size_t ki = k0 + i * blockDim.x;
+            have[i] |= mask[i];
             for (uint32_t m = mask[i]; m; m &= m - 1u) {
                 const size_t k = ki + size_t(__ffs(m) - 1) * V;
                 const double e = pair ? double(P.edep_hi[k]) + double(P.edep_lo[k]) : P.edep[k];
@@ -218,11 +221,48 @@ __device__ __forceinline__ void batch_sums(const SimParams& P, size_t V, size_t 
     }
 }
 
+// The tallies themselves instead of their sums, for at most 4 batches: the
+// sums are then made with the rest of a voxel's FP64 work, by full warps.
+template <int VPT, int NB>
+__device__ __forceinline__ void batch_tallies(const SimParams& P, size_t V, size_t first, size_t v, int nbatch,
+                                              double (&e)[VPT][NB], uint32_t (&have)[VPT]) {
+    const bool pair = P.tally_mode != 0;
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int i = 0; i < VPT; ++i) {
+            const size_t vi = v + size_t(i) * blockDim.x, k = (first + size_t(b)) * V + vi;
+            const bool in = b < nbatch && vi < V;
+            if (!pair) {
+                e[i][b] = in ? P.edep[k] : 0.0;
+                have[i] |= uint32_t(__double2hiint(e[i][b]) | __double2loint(e[i][b]));
+            } else {
+                const float hi = in ? P.edep_hi[k] : 0.f, lo = in ? P.edep_lo[k] : 0.f;
+                e[i][b] = double(hi) + double(lo);
+                have[i] |= __float_as_uint(hi) | __float_as_uint(lo);
+            }
+        }
+#pragma unroll
+    for (int i = 0; i < VPT; ++i)
+        if (have[i])
+#pragma unroll
+            for (int b = 0; b < NB; ++b)
+                if (b < nbatch) {
+                    const size_t k = (first + size_t(b)) * V + v + size_t(i) * blockDim.x;
+                    if (!pair) {
+                        P.edep[k] = 0.0;
+                    } else {
+                        P.edep_hi[k] = 0.f;
+                        P.edep_lo[k] = 0.f;
+                    }
+                }
+}
+
 // Voxels with dose, gathered by the threads of a CTA so that the FP64 work
 // per voxel (weights, mean, 1/mass, square root: about 30 operations) runs
 // with full warps however few of a warp's voxels hold dose.
 struct FoldItem {
-    double eb, qb, es, qs;      // sums over the long batches and over the short ones
+    double v[4];      // sums over the long batches (e, e^2) and over the short ones, or the tallies
 };
 constexpr int kFoldThreads = 256;
 struct FoldList {
@@ -231,47 +271,77 @@ struct FoldList {
     uint32_t n;
 };
 
-// Loop of a fold over the CTA's voxels: sum each voxel's tallies, hand a
+// Loop of a fold over the CTA's voxels: read each voxel's tallies, hand a
 // voxel without dose to `empty(voxel)` and the others, in full CTA-loads, to
-// `full(voxel, item)`.
+// `full(voxel, eb, qb, es, qs)`.  UB: batches read at a time (batch_sums), or
+// 0 for at most 4 batches (batch_tallies).
 template <int VPT, int UB, class Full, class Empty>
 __device__ __forceinline__ void fold_voxels(const SimParams& P, size_t V, size_t first, int nbig, int nbatch,
                                             FoldList& L, Full full, Empty empty) {
+    auto item = [&](uint32_t j) {
+        const FoldItem t = L.item[j];
+        if constexpr (UB > 0) {
+            full(size_t(L.vox[j]), t.v[0], t.v[1], t.v[2], t.v[3]);
+        } else {
+            double s[2] = {0.0, 0.0}, q[2] = {0.0, 0.0};
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+                if (b < nbatch) {
+                    if (b < nbig) {
+                        s[0] += t.v[b];
+                        q[0] = fma(t.v[b], t.v[b], q[0]);
+                    } else {
+                        s[1] += t.v[b];
+                        q[1] = fma(t.v[b], t.v[b], q[1]);
+                    }
+                }
+            full(size_t(L.vox[j]), s[0], q[0], s[1], q[1]);
+        }
+    };
     if (threadIdx.x == 0) L.n = 0u;
     __syncthreads();
     for (size_t base = size_t(blockIdx.x) * kFoldThreads * VPT; base < V;
          base += size_t(gridDim.x) * kFoldThreads * VPT) {
         const size_t v = base + threadIdx.x;
-        double eb[VPT] = {}, qb[VPT] = {}, es[VPT] = {}, qs[VPT] = {};
-        if (nbig > 0) batch_sums<VPT, UB>(P, V, first, v, 0, nbig, eb, qb);
-        batch_sums<VPT, UB>(P, V, first, v, nbig, nbatch, es, qs);
+        FoldItem it[VPT];
+        uint32_t some[VPT] = {};
+        if constexpr (UB > 0) {
+            double eb[VPT] = {}, qb[VPT] = {}, es[VPT] = {}, qs[VPT] = {};
+            if (nbig > 0) batch_sums<VPT, UB>(P, V, first, v, 0, nbig, eb, qb, some);
+            batch_sums<VPT, UB>(P, V, first, v, nbig, nbatch, es, qs, some);
+#pragma unroll
+            for (int i = 0; i < VPT; ++i) it[i] = FoldItem{{eb[i], qb[i], es[i], qs[i]}};
+        } else {
+            double e[VPT][4];
+            batch_tallies<VPT, 4>(P, V, first, v, nbatch, e, some);
+#pragma unroll
+            for (int i = 0; i < VPT; ++i) it[i] = FoldItem{{e[i][0], e[i][1], e[i][2], e[i][3]}};
+        }
 #pragma unroll
         for (int i = 0; i < VPT; ++i) {
             const size_t vi = v + size_t(i) * kFoldThreads;
-            // the sum of squares is zero only when every tally is
-            const bool have = vi < V && (qb[i] != 0.0 || qs[i] != 0.0);
+            const bool have = some[i] != 0u;
             if (vi < V && !have) empty(vi);
             const uint32_t m = __ballot_sync(0xffffffffu, have);
             uint32_t at = 0u;
             if (m && (threadIdx.x & 31u) == 0u) at = atomicAdd(&L.n, uint32_t(__popc(m)));
             at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & lanemask_lt());
             if (have) {
-                L.item[at] = FoldItem{eb[i], qb[i], es[i], qs[i]};
+                L.item[at] = it[i];
                 L.vox[at] = uint32_t(vi);
             }
             __syncthreads();
             // at most 255 left over plus 256 new ones: one full load at a time
             const uint32_t n = L.n;
             if (n >= uint32_t(kFoldThreads)) {
-                const uint32_t j = n - kFoldThreads + threadIdx.x;
-                full(size_t(L.vox[j]), L.item[j]);
+                item(n - kFoldThreads + threadIdx.x);
                 __syncthreads();
                 if (threadIdx.x == 0) L.n = n - kFoldThreads;
             }
             __syncthreads();
         }
     }
-    if (threadIdx.x < L.n) full(size_t(L.vox[threadIdx.x]), L.item[threadIdx.x]);
+    if (threadIdx.x < L.n) item(threadIdx.x);
 }
 
 // All batches at once (batches run side by side, one tally grid each): per
@@ -281,23 +351,22 @@ __device__ __forceinline__ void fold_voxels(const SimParams& P, size_t V, size_t
 // Dmax), with no sums written and read back.  Otherwise the sums of a run in
 // parts accumulate in out1, out2.  The grids are left zeroed.
 template <bool FINAL, int VPT, int UB>
-__global__ void __launch_bounds__(kFoldThreads, 4) k_fold_batches(SimParams P, size_t V, int nbatch,
+__global__ void __launch_bounds__(kFoldThreads, 5) k_fold_batches(SimParams P, size_t V, int nbatch,
                                                                double inv_big, double inv_small, int n_big,
                                                                double* __restrict__ out1,
-                                                               double* __restrict__ out2, double dvol,
+                                                               double* __restrict__ out2, double inv_n,
+                                                               double inv_nn1, double dvol,
                                                                unsigned long long* dmax_bits,
                                                                float metric_min_rho) {
     __shared__ double s_red[32];
     __shared__ FoldList L;
     double dep = 0.0, mx = 0.0;
-    const double inv_n = 1.0 / nbatch;
-    const double inv_nn1 = FINAL ? 1.0 / (double(nbatch) * (nbatch - 1)) : 0.0;
     fold_voxels<VPT, UB>(
         P, V, 0, min(n_big, nbatch), nbatch, L,
-        [&](size_t v, const FoldItem& t) {
-            dep += t.eb + t.es;
-            const double a1 = fma(t.eb, inv_big, t.es * inv_small);
-            const double a2 = fma(t.qb, inv_big * inv_big, t.qs * (inv_small * inv_small));
+        [&](size_t v, double eb, double qb, double es, double qs) {
+            dep += eb + es;
+            const double a1 = fma(eb, inv_big, es * inv_small);
+            const double a2 = fma(qb, inv_big * inv_big, qs * (inv_small * inv_small));
             if (FINAL) {
                 const double mean = a1 * inv_n;
                 const double var = fmax(0.0, (a2 - nbatch * mean * mean) * inv_nn1);
@@ -336,11 +405,12 @@ __global__ void __launch_bounds__(kFoldThreads, 4) k_fold_batches(SimParams P, s
 // sub-problem k, whose first nbig[k] batches are the long ones.  The grids
 // are left zeroed.  With two batches a thread has only two tallies a voxel to
 // load, so it takes four voxels.  64 beamlets x 2 batches on the 128^3 slab
-// (134M voxels of output): memset and fold 17 -> 3.7 ms.
+// (134M voxels of output, 12 % of them with dose): memset and fold 17 -> 1.9 ms.
 template <int VPT, int UB>
 __global__ void __launch_bounds__(kFoldThreads) k_fold_sub(SimParams P, size_t V, uint32_t k0, int nb,
                                                            const double* __restrict__ inv_n,
                                                            const uint32_t* __restrict__ nbig, double dvol,
+                                                           double inv_nb, double inv_nn1,
                                                            double* __restrict__ dose,
                                                            double* __restrict__ sigma) {
     __shared__ double s_red[32];
@@ -353,15 +423,14 @@ __global__ void __launch_bounds__(kFoldThreads) k_fold_sub(SimParams P, size_t V
     double dep = 0.0;
     fold_voxels<VPT, UB>(
         P, V, size_t(k) * nb, int(min(nbig[k], uint32_t(nb))), nb, L,
-        [&](size_t v, const FoldItem& t) {
-            dep += t.eb + t.es;
-            const double a1 = fma(t.eb, ib, t.es * is);
-            const double a2 = fma(t.qb, ib * ib, t.qs * (is * is));
+        [&](size_t v, double eb, double qb, double es, double qs) {
+            dep += eb + es;
+            const double a1 = fma(eb, ib, es * is);
+            const double a2 = fma(qb, ib * ib, qs * (is * is));
             const double im = inverse_mass(P.rho[v], dvol);
-            const double mean = a1 / nb;
+            const double mean = a1 * inv_nb;
             dk[v] = mean * im;
-            if (with_sigma)
-                sk[v] = root(fmax(0.0, (a2 - nb * mean * mean) / (double(nb) * (nb - 1)))) * im;
+            if (with_sigma) sk[v] = root(fmax(0.0, (a2 - nb * mean * mean) * inv_nn1)) * im;
         },
         [&](size_t v) {
             dk[v] = 0.0;
@@ -491,9 +560,9 @@ static unsigned fold_grid(gdpm_ctx* ctx, size_t V, int vpt, int ctas_per_sm) {
 
 int launch_fold_batches(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t V, int n_batches,
                         uint32_t nb_small, uint32_t nb_rem, double* s1, double* s2) {
-    k_fold_batches<false, 1, 16><<<fold_grid(ctx, V, 1, 8), kFoldThreads, 0, st>>>(
+    k_fold_batches<false, 1, 10><<<fold_grid(ctx, V, 1, 5), kFoldThreads, 0, st>>>(
         P, V, n_batches, 1.0 / double(nb_small + 1), 1.0 / double(nb_small), int(nb_rem), s1, s2, 0.0,
-        nullptr, 0.f);
+        0.0, 0.0, nullptr, 0.f);
     GDPM_CUDA_TRY(cudaGetLastError());
     return GDPM_OK;
 }
@@ -512,9 +581,9 @@ int launch_fold_final(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t
                       uint32_t nb_small, uint32_t nb_rem, double* dose, double* sigma) {
     const double dvol = double(P.dx) * P.dy * P.dz;
     unsigned long long* dmax_bits = reinterpret_cast<unsigned long long*>(&P.ledger[L_DMAX]);
-    k_fold_batches<true, 1, 16><<<fold_grid(ctx, V, 1, 8), kFoldThreads, 0, st>>>(
+    k_fold_batches<true, 1, 10><<<fold_grid(ctx, V, 1, 5), kFoldThreads, 0, st>>>(
         P, V, n_batches, 1.0 / double(nb_small + 1), 1.0 / double(nb_small), int(nb_rem), dose, sigma,
-        dvol, dmax_bits, ctx->metric_min_rho);
+        1.0 / n_batches, 1.0 / (double(n_batches) * (n_batches - 1)), dvol, dmax_bits, ctx->metric_min_rho);
     GDPM_CUDA_TRY(cudaGetLastError());
     return launch_metric(ctx, st, P, V, dose, sigma);
 }
@@ -523,8 +592,11 @@ int launch_fold_sub(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t V
                     uint32_t nk, int nb, const double* inv_n, const uint32_t* nbig, double* dose,
                     double* sigma) {
     const double dvol = double(P.dx) * P.dy * P.dz;
-    k_fold_sub<4, 2><<<dim3(fold_grid(ctx, V, 4, 8), nk), kFoldThreads, 0, st>>>(P, V, k0, nb, inv_n, nbig, dvol,
-                                                                        dose, sigma);
+    const double inv_nb = 1.0 / nb, inv_nn1 = nb > 1 ? 1.0 / (double(nb) * (nb - 1)) : 0.0;
+    const dim3 grid(fold_grid(ctx, V, 4, 2), nk);   // two CTAs per SM and beamlet: 8 were 6 % slower
+    if (nb <= 4) k_fold_sub<4, 0><<<grid, kFoldThreads, 0, st>>>(P, V, k0, nb, inv_n, nbig, dvol, inv_nb, inv_nn1, dose,
+                                                                 sigma);
+    else k_fold_sub<4, 4><<<grid, kFoldThreads, 0, st>>>(P, V, k0, nb, inv_n, nbig, dvol, inv_nb, inv_nn1, dose, sigma);
     GDPM_CUDA_TRY(cudaGetLastError());
     return GDPM_OK;
 }

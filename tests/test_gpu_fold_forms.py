@@ -37,3 +37,27 @@ def test_side_by_side_fold_equals_sequential(shape, batches, tally):
     assert (d1 > 0).any()
     assert abs(a["deposited"] - b["deposited"]) <= 1e-12 * a["deposited"]
     assert abs(a["sigma_over_dmax"] - b["sigma_over_dmax"]) <= 1e-6 * a["sigma_over_dmax"] + 1e-9
+
+
+# a dose matrix of one beamlet holds the histories of that beamlet's own
+# calculation; up to 4 batches keep their tallies apart until the last kernel
+# step, more are summed first
+@pytest.mark.parametrize("batches", [2, 3, 4, 5, 11])
+@pytest.mark.parametrize("tally", [0, 1])
+def test_matrix_fold_equals_calculation(batches, tally):
+    ph = W.homogeneous_phantom((19, 23, 29), (0.5, 0.5, 0.5), W.WATER, 1.0)
+    n = 10_000 + batches // 2
+    src = W.single_beamlet(ph, 0.0, -0.5, -0.5, 1.0)
+    prob = W.Problem(ph, src, n, batches, eabs_photon=0.05, eabs_electron=0.2, e_min=0.005, e_max=6.5,
+                     sub_histories=(n,))
+    eng = G.Engine(prob, params={G.GDPM_PARAM_TALLY_MODE: tally})
+    try:
+        d1, s1, _ = eng.run()
+        for _ in range(2):
+            d2, s2, _ = eng.run_beamlets()
+        d1, s1, d2, s2 = (t.cpu().numpy().ravel() for t in (d1, s1, d2, s2))
+    finally:
+        eng.close()
+    assert (d1 > 0).any()
+    assert np.all(np.abs(d1 - d2) <= 1e-12 * d1)
+    assert np.all(np.abs(s1 ** 2 - s2 ** 2) <= 1e-12 * d1 ** 2 + 1e-12 * s1 ** 2)
