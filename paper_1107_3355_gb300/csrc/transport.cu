@@ -71,12 +71,22 @@ struct Sec {
     float E1, E2, dx, dy, dz;
 };
 
-// Deposit e MeV in voxel vox of the tally of the batch in `flags`.  GEN: the
-// general form, which looks at the tally mode and, below, at the per-history
-// records; the phase kernels also exist without it (FP64 tally, no records),
-// which saves its tests at every deposit and event.
-template <bool GEN>
-__device__ __forceinline__ void tally(const SimParams& P, uint32_t flags, uint32_t vox0, float e) {
+// Forms of the phase kernels: FP64 tally or FP32 pair tally, without
+// per-history records, and the general form, which looks at both at every
+// deposit and event.
+constexpr int kPlain = 0, kPair = 1, kGeneral = 2;
+
+// Deposit e MeV in voxel vox of the tally of the batch in `flags`.
+// FP32 pair: hi accumulates, lo collects the exact rounding error of each
+// addition (TwoSum on the value the atomic returned); the second half
+// (tally_end) can come after other work, which then hides the atomic's return
+// trip.
+struct Deposit {
+    size_t vox;
+    float e, old;
+};
+template <int GEN>
+__device__ __forceinline__ Deposit tally_begin(const SimParams& P, uint32_t flags, uint32_t vox0, float e) {
     size_t vox = uint64_t((flags & kBatchMask) >> kBatchShift) * P.batch_stride + vox0;
 #if GDPM_CHECKED
     if (vox < P.tally_lo || vox >= P.tally_hi) {
@@ -84,30 +94,35 @@ __device__ __forceinline__ void tally(const SimParams& P, uint32_t flags, uint32
         vox = P.tally_lo;
     }
 #endif
-    if (!GEN || P.tally_mode == 0) {
-        atomicAdd(&P.edep[vox], double(e));
-    } else {
-        // FP32 pair: hi accumulates, lo collects the exact rounding error of
-        // each addition (TwoSum on the value the atomic returned).
-        const float old = atomicAdd(&P.edep_hi[vox], e);
-        const float s = old + e;
-        const float bb = s - old;
-        const float err = (old - (s - bb)) + (e - bb);
-        if (err != 0.f) atomicAdd(&P.edep_lo[vox], err);
-    }
+    Deposit d{vox, e, 0.f};
+    if (GEN == kPlain || (GEN == kGeneral && P.tally_mode == 0)) atomicAdd(&P.edep[vox], double(e));
+    else d.old = atomicAdd(&P.edep_hi[vox], e);
+    return d;
+}
+template <int GEN>
+__device__ __forceinline__ void tally_end(const SimParams& P, const Deposit& d) {
+    if (GEN == kPlain || (GEN == kGeneral && P.tally_mode == 0)) return;
+    const float s = d.old + d.e;
+    const float bb = s - d.old;
+    const float err = (d.old - (s - bb)) + (d.e - bb);
+    if (err != 0.f) atomicAdd(&P.edep_lo[d.vox], err);
+}
+template <int GEN>
+__device__ __forceinline__ void tally(const SimParams& P, uint32_t flags, uint32_t vox0, float e) {
+    tally_end<GEN>(P, tally_begin<GEN>(P, flags, vox0, e));
 }
 
 __device__ __forceinline__ uint32_t vox_of(const SimParams& P, int ix, int iy, int iz) {
     return uint32_t(ix) + uint32_t(P.nx) * (uint32_t(iy) + uint32_t(P.ny) * uint32_t(iz));
 }
 
-template <bool GEN>
+template <int GEN>
 __device__ __forceinline__ void hist_count(const SimParams& P, uint32_t hist, int k) {
-    if (GEN && P.hrec) atomicAdd(&P.hrec[size_t(GDPM_IDX(P.status, hist, P.n_records, ST_B_RECORD)) * 4 + k], 1);
+    if (GEN == kGeneral && P.hrec) atomicAdd(&P.hrec[size_t(GDPM_IDX(P.status, hist, P.n_records, ST_B_RECORD)) * 4 + k], 1);
 }
-template <bool GEN>
+template <int GEN>
 __device__ __forceinline__ void hist_add(const SimParams& P, uint32_t hist, int k, double v) {
-    if (GEN && P.hrec) atomicAdd(&P.hrecd[size_t(GDPM_IDX(P.status, hist, P.n_records, ST_B_RECORD)) * 2 + k], v);
+    if (GEN == kGeneral && P.hrec) atomicAdd(&P.hrecd[size_t(GDPM_IDX(P.status, hist, P.n_records, ST_B_RECORD)) * 2 + k], v);
 }
 #if GDPM_CHECKED
 __device__ __forceinline__ uint32_t n_voxels(const SimParams& P) {
@@ -353,7 +368,7 @@ __device__ bool make_primary(const SimParams& P, const PhaseArgs& A, uint32_t id
     acc.src += p.E;
     if (!enter_box(P, p)) {
         acc.esc += p.E;
-        hist_add<true>(P, p.hist, 0, p.E);
+        hist_add<kGeneral>(P, p.hist, 0, p.E);
         return false;
     }
     voxel_of(P, p);
@@ -377,7 +392,7 @@ enum class Flight { fly, gone, wait };
 constexpr uint32_t kAbsorbed = 0x80000000u;
 
 // One Woodcock flight against the majorant (Sec. 2.1) with the draw x.
-template <bool GEN>
+template <int GEN>
 __device__ __forceinline__ Flight photon_flight(const SimParams& P, const PhSmem& S, Part& p, uint4 x,
                                                 double& esc) {
     const DevTables& T = P.T;
@@ -425,7 +440,7 @@ __device__ __forceinline__ Flight photon_flight(const SimParams& P, const PhSmem
 // E u - E' u', and `goes_on` says whether it stays above its absorption
 // energy (below it, it is deposited here).
 enum class PhEvent { none, compton, photo, pair };
-template <bool GEN>
+template <int GEN>
 __device__ __forceinline__ PhEvent photon_event(const SimParams& P, Part& p, uint4 x, bool force, bool& goes_on,
                                                 Sec& sec) {
     const float E = p.E;
@@ -518,7 +533,7 @@ __device__ __forceinline__ uint32_t vox_linear(const SimParams& P, uint32_t v) {
 
 // End of track: residual energy deposited in the voxel; a positron then waits
 // to annihilate, or its rest energy is discarded (Sec. 2.1, Sec. 4).
-template <bool GEN>
+template <int GEN>
 __device__ __forceinline__ Round absorb(const SimParams& P, Electron& p, uint32_t& kind) {
     tally<GEN>(P, p.flags, vox_linear(P, p.vox), p.E + p.pend);
     p.pend = 0.f;
@@ -533,7 +548,7 @@ __device__ __forceinline__ Round absorb(const SimParams& P, Electron& p, uint32_
 
 // Set up a step with the draw x: step limits as mass thickness in the start
 // voxel's material (`mat`), energy at its end, deflection at the random hinge.
-template <bool GEN>
+template <int GEN>
 __device__ __forceinline__ void electron_setup(const SimParams& P, const ElSmem& S, const Electron& p, uint4 x,
                                                int mat, ElStep& st) {
     const DevTables& T = P.T;
@@ -630,12 +645,13 @@ __device__ __forceinline__ bool walk_move(const SimParams& P, Electron& p, const
     return ends;
 }
 // Cross the exit face; false when the particle leaves the phantom.
-template <bool GEN>
+template <int GEN>
 __device__ __forceinline__ bool walk_cross(const SimParams& P, Electron& p, ElStep& s, Walk& k,
                                            uint32_t& crossings) {
     const float piece = __fmul_rn(s.rho, k.tb);
     const float owed = fmaf(s.dpm, piece, p.pend);
-    if (owed > 0.f) tally<GEN>(P, p.flags, k.lin, owed);
+    Deposit dep{0, 0.f, 0.f};
+    if (owed > 0.f) dep = tally_begin<GEN>(P, p.flags, k.lin, owed);
     s.dep = fmaf(s.dpm, piece, s.dep);
     p.pend = 0.f;
     s.left = __fsub_rn(s.left, piece);
@@ -645,7 +661,10 @@ __device__ __forceinline__ bool walk_cross(const SimParams& P, Electron& p, ElSt
     const uint32_t d = k.axis == 0 ? 1u : k.axis == 1 ? uint32_t(P.nx) : uint32_t(P.nx) * uint32_t(P.ny);
     const uint32_t shift = 10u * uint32_t(k.axis);
     const uint32_t at = ((p.vox >> shift) & 1023u) + (up ? 1u : ~0u);       // wraps below zero
-    if (at >= n) return false;
+    if (at >= n) {
+        tally_end<GEN>(P, dep);
+        return false;
+    }
     p.vox = up ? p.vox + (1u << shift) : p.vox - (1u << shift);
     const float f = float(at);
     if (k.axis == 0) k.fx = f;
@@ -654,6 +673,7 @@ __device__ __forceinline__ bool walk_cross(const SimParams& P, Electron& p, ElSt
     k.lin = up ? k.lin + d : k.lin - d;
     k.lin = GDPM_IDX(P.status, k.lin, n_voxels(P), ST_B_VOXEL);
     s.rho = __ldg(&P.rho[k.lin]);
+    tally_end<GEN>(P, dep);
     return true;
 }
 // One stretch of the walk: to the end of leg 1, the turn at the hinge and the
@@ -661,7 +681,7 @@ __device__ __forceinline__ bool walk_cross(const SimParams& P, Electron& p, ElSt
 // end a leg do it together and those that cross a face do that together.
 // Returns 0 when the step goes on, 1 at the end of leg 2, 2 when the particle
 // left the phantom.
-template <bool GEN>
+template <int GEN>
 __device__ __forceinline__ int walk_stretch(const SimParams& P, Electron& p, ElStep& s, Walk& k,
                                             uint32_t& crossings) {
     bool ends = walk_move(P, p, s, k);
@@ -687,7 +707,7 @@ constexpr int kDrainedStretches = 16;
 // A lane's round: set up a step when none is in progress (`starts`, with the
 // draw x), walk, and at the step's end escape, be absorbed, or wait for the
 // hard-event candidate.
-template <bool GEN>
+template <int GEN>
 __device__ __forceinline__ Round electron_round(const SimParams& P, const ElSmem& S, Electron& p, ElStep& st,
                                                 uint4 x, int mat, int stretches, double& esc,
                                                 uint32_t& crossings, uint32_t& kind) {
@@ -732,7 +752,7 @@ __device__ __forceinline__ Round electron_round(const SimParams& P, const ElSmem
 // one rejection trial per draw (`force` accepts any); a positron at rest
 // annihilates.  Returns go when the particle takes its next step, wait when
 // it needs another draw, ended at the end of its track.
-template <bool GEN>
+template <int GEN>
 __device__ __forceinline__ Round electron_event(const SimParams& P, const ElSmem& S, Electron& p, uint32_t& kind,
                                                 uint4 x, bool force, Sec& sec) {
     const DevTables& T = P.T;
@@ -832,7 +852,7 @@ __device__ __forceinline__ uint32_t reserve(Slots& sl, uint32_t c, uint32_t r, u
 // in the warp's reservations and counter-derived ids.  vox: the parents'
 // packed voxels; pushes: the warp's pushes to the electron queue (0) and the
 // photon queue (1).  PT 0: photons create electrons only.
-template <int PT, bool GEN, class Parent>
+template <int PT, int GEN, class Parent>
 __device__ __forceinline__ void bank(const SimParams& P, const PhaseArgs& A, uint32_t total, Parent& p,
                                      uint32_t vox, const Sec& sec, Slots (&sl)[PT + 1],
                                      uint32_t (&pushes)[PT + 1]) {
@@ -991,7 +1011,7 @@ __device__ __forceinline__ void rec_load(const PhRec& r, Part& p) {
 // calls and its constants in uniform registers.
 // Stack bounds: photons enter the warp (and free lanes take one) only while
 // at most 31 wait, and only up to kPhReady ready; 32 more are in the lanes.
-template <bool GEN>
+template <int GEN>
 __device__ __forceinline__ void photon_run(const SimParams& P, const PhaseArgs& A) {
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t n_in = A.in_count ? min(*A.in_count, A.in.capacity) : 0u;
@@ -1180,7 +1200,7 @@ __device__ __forceinline__ uint32_t el_load(const ElStack& s, uint32_t i, Electr
 // a history; now 20 and 205.  Measured against that (1e8 histories of the CT
 // plan; 2.5e8 of the paper's lung slab; 2.5e6 20 MeV electrons on its bone
 // slab): electron phase 29.6 -> 25.7, 54.8 -> 50.0, 7.0 -> 5.6 ms.
-template <bool GEN>
+template <int GEN>
 __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs& A) {
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t n_in = A.in_count ? min(*A.in_count, A.in.capacity) : 0u;
@@ -1370,13 +1390,13 @@ __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs
 
 // One transport phase (Sec. 2.2.1 Step 3), a persistent loop per warp.  PT: 0
 // photons, 1 electrons.
-template <int PT, bool GEN>
+template <int PT, int GEN>
 __device__ __forceinline__ void phase_run(const SimParams& P, const PhaseArgs& A) {
     if constexpr (PT == 0) photon_run<GEN>(P, A);
     else electron_run<GEN>(P, A);
 }
 
-template <int PT, bool GEN>
+template <int PT, int GEN>
 __global__ void __launch_bounds__(PhaseShape<PT>::threads, PhaseShape<PT>::ctas)
 k_phase(const SimParams P, const PhaseArgs A) {
     phase_run<PT, GEN>(P, A);
@@ -1597,7 +1617,7 @@ k_phase_loop(const SimParams P, const LoopArgs L) {
     __shared__ PhaseArgs sA;
     if (threadIdx.x == 0) sA = phase_args(L, *L.k + (PT == 0 ? 0u : 1u));
     __syncthreads();
-    phase_run<PT, true>(P, sA);
+    phase_run<PT, kGeneral>(P, sA);
 }
 
 // Primaries of this pass's source phase (before it runs).
@@ -1776,9 +1796,9 @@ int launch_phase(gdpm_ctx* ctx, cudaStream_t st, int particle, const SimParams& 
     const int thr = shape.threads;
     const size_t smem = shape.smem;
     using Kernel = void (*)(const SimParams, const PhaseArgs);
-    const bool gen = P.tally_mode != 0 || P.hrec;
-    const Kernel fn = particle == GDPM_PHOTON ? (gen ? k_phase<0, true> : k_phase<0, false>)
-                                              : (gen ? k_phase<1, true> : k_phase<1, false>);
+    static const Kernel kernels[2][3] = {{k_phase<0, kPlain>, k_phase<0, kPair>, k_phase<0, kGeneral>},
+                                         {k_phase<1, kPlain>, k_phase<1, kPair>, k_phase<1, kGeneral>}};
+    const Kernel fn = kernels[particle == GDPM_PHOTON ? 0 : 1][P.hrec ? kGeneral : P.tally_mode ? kPair : kPlain];
     GDPM_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
     int bps = ctx->blocks_per_sm;
     if (bps <= 0) {
