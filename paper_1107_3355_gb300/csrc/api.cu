@@ -98,9 +98,7 @@ void runner_free(Runner& r) {
     if (r.side) cudaStreamSynchronize(r.side);
     Workspace& w = r.ws;
     Buffer* bs[] = {&w.edep, &w.edep2, &w.hi2, &w.lo2, &w.s1, &w.s2, &w.hi, &w.lo, &w.qph,
-                    &w.qel0, &w.qel1, &w.qsrc, &w.ctl, &w.prefix, &w.counters, &w.ledger, &w.status,
-                    &w.edges, &w.beamlets, &w.bl_cdf, &w.bl_row, &w.bl_f, &w.al_cut,
-                    &w.al_alias, &w.chains, &w.pick, &w.sub_first, &w.sub_inv, &w.sub_nbig,
+                    &w.qel0, &w.qel1, &w.qsrc, &w.ctl, &w.inputs, &w.run, &w.chains, &w.pick, &w.sub_first, &w.sub_inv, &w.sub_nbig,
                     &w.loop_k, &w.stage};
     for (Buffer* b : bs) release(*b);
     if (r.loop_exec) cudaGraphExecDestroy(r.loop_exec);
@@ -109,7 +107,8 @@ void runner_free(Runner& r) {
     r.loop_graph = nullptr;
     r.loop_key.clear();
     if (w.pinned_host.p) cudaFreeHost(w.pinned_host.p);
-    w.pinned_host.p = nullptr;
+    if (w.pinned_stage.p) cudaFreeHost(w.pinned_stage.p);
+    w.pinned_host.p = w.pinned_stage.p = nullptr;
     for (cudaEvent_t e : r.prof_events) cudaEventDestroy(e);
     r.prof_events.clear();
     cudaEvent_t evs[] = {r.ev0, r.ev1, r.batch_done[0], r.batch_done[1], r.fold_done[0], r.fold_done[1]};
@@ -224,6 +223,10 @@ static int source_copy(const gdpm_source_desc* s, gdpm_source_state& st) {
 void beamlet_tables_host(const std::vector<double>& rows17, BeamletHost& out, bool all_rows) {
     const int nb = int(rows17.size() / 17);
     out = BeamletHost{};
+    out.rows.reserve(size_t(nb) * 16);
+    out.row.reserve(nb);
+    out.f.reserve(nb);
+    out.cdf.reserve(nb);
     double tot = 0;
     for (int b = 0; b < nb; ++b) tot += rows17[size_t(b) * 17 + 16];
     double acc = 0;
@@ -311,40 +314,91 @@ void source_fields(const gdpm_source_state& s, DevSource& d) {
     d.al_alias = nullptr;
 }
 
-static int source_upload(Runner& r, const gdpm_source_state& s, DevSource& d, bool all_rows = false) {
+// The small inputs of a calculation -- the spectrum allotment `prefix` (may be
+// null), the spectrum's edges and the fluence map with its samplers' tables --
+// to the device in one copy, from the runner's pinned staging block: the copy
+// is asynchronous and the block lives as long as the runner, whose every call
+// ends with its stream synchronized.  What exceeds the block (a plan of more
+// than about 2700 beamlets) goes from pageable memory and is waited for.
+constexpr size_t kStageBytes = size_t(256) << 10;
+static int source_upload(Runner& r, const gdpm_source_state& s, DevSource& d, bool all_rows = false,
+                         const std::vector<uint32_t>* prefix = nullptr) {
     const gdpm_source_desc& g = s.desc;
+    Workspace& w = r.ws;
     source_fields(s, d);
     std::vector<float> e(s.edges.begin(), s.edges.end());
-    int rc = ensure(r.ws.edges, e.size() * 4);
-    if (rc) return rc;
-    GDPM_CUDA_TRY(cudaMemcpyAsync(r.ws.edges.p, e.data(), e.size() * 4, cudaMemcpyHostToDevice, r.stream));
-    d.edges = static_cast<const float*>(r.ws.edges.p);
     BeamletHost bh;
     if (g.geometry == GDPM_GEO_BEAMLETS) beamlet_tables_host(s.beamlets, bh, all_rows);
-    if (!bh.f.empty()) {
-        const size_t nbl = bh.f.size();
-        Workspace& w = r.ws;
-        if ((rc = ensure(w.beamlets, nbl * 64)) || (rc = ensure(w.bl_cdf, nbl * 4)) ||
-            (rc = ensure(w.bl_row, nbl * 4)) || (rc = ensure(w.bl_f, nbl * 8)) ||
-            (rc = ensure(w.al_cut, nbl * 8)) || (rc = ensure(w.al_alias, nbl * 4)))
-            return rc;
-        GDPM_CUDA_TRY(cudaMemcpyAsync(w.beamlets.p, bh.rows.data(), nbl * 64, cudaMemcpyHostToDevice, r.stream));
-        GDPM_CUDA_TRY(cudaMemcpyAsync(w.bl_cdf.p, bh.cdf_up.data(), nbl * 4, cudaMemcpyHostToDevice, r.stream));
-        GDPM_CUDA_TRY(cudaMemcpyAsync(w.bl_row.p, bh.row.data(), nbl * 4, cudaMemcpyHostToDevice, r.stream));
-        GDPM_CUDA_TRY(cudaMemcpyAsync(w.bl_f.p, bh.f.data(), nbl * 8, cudaMemcpyHostToDevice, r.stream));
-        GDPM_CUDA_TRY(cudaMemcpyAsync(w.al_cut.p, bh.cut_t.data(), nbl * 8, cudaMemcpyHostToDevice, r.stream));
-        GDPM_CUDA_TRY(cudaMemcpyAsync(w.al_alias.p, bh.alias.data(), nbl * 4, cudaMemcpyHostToDevice, r.stream));
-        d.n_beamlets = int(nbl);
-        d.beamlets = static_cast<const float*>(w.beamlets.p);
-        d.bl_cdf = static_cast<const float*>(w.bl_cdf.p);
-        d.bl_row = static_cast<const int*>(w.bl_row.p);
-        d.bl_f = static_cast<const double*>(w.bl_f.p);
-        d.al_cut = static_cast<const uint64_t*>(w.al_cut.p);
-        d.al_alias = static_cast<const int*>(w.al_alias.p);
+    const size_t nbl = bh.f.size();
+    struct Piece {
+        const void* host;
+        size_t bytes, at;
+    };
+    Piece pc[8] = {{prefix ? prefix->data() : nullptr, prefix ? prefix->size() * 4 : 0, 0},
+                   {e.data(), e.size() * 4, 0},
+                   {bh.rows.data(), nbl * 64, 0},
+                   {bh.cdf_up.data(), nbl * 4, 0},
+                   {bh.row.data(), nbl * 4, 0},
+                   {bh.f.data(), nbl * 8, 0},
+                   {bh.cut_t.data(), nbl * 8, 0},
+                   {bh.alias.data(), nbl * 4, 0}};
+    size_t total = 0;
+    for (Piece& q : pc) {
+        q.at = total;
+        total += (q.bytes + 255) & ~size_t(255);
     }
-    // the host vectors above are staged by the copies; make the copies
-    // complete before they go out of scope
-    GDPM_CUDA_TRY(cudaStreamSynchronize(r.stream));
+    int rc = ensure(w.inputs, total);
+    if (rc) return rc;
+    if (!w.pinned_stage.p) {
+        void* h = nullptr;
+        GDPM_CUDA_TRY(cudaMallocHost(&h, kStageBytes));
+        w.pinned_stage.p = h;
+        w.pinned_stage.bytes = kStageBytes;
+    }
+    std::vector<unsigned char> big;
+    const bool staged = total <= kStageBytes;
+    if (!staged) big.resize(total);
+    unsigned char* host = staged ? static_cast<unsigned char*>(w.pinned_stage.p) : big.data();
+    for (const Piece& q : pc)
+        if (q.bytes) std::memcpy(host + q.at, q.host, q.bytes);
+    GDPM_CUDA_TRY(cudaMemcpyAsync(w.inputs.p, host, total, cudaMemcpyHostToDevice, r.stream));
+    if (!staged) GDPM_CUDA_TRY(cudaStreamSynchronize(r.stream));   // before `big` goes out of scope
+    unsigned char* dev = static_cast<unsigned char*>(w.inputs.p);
+    w.prefix = prefix ? reinterpret_cast<const uint32_t*>(dev + pc[0].at) : nullptr;
+    w.prefix_n = prefix ? uint32_t(prefix->size()) : 0u;
+    d.edges = reinterpret_cast<const float*>(dev + pc[1].at);
+    if (nbl) {
+        d.n_beamlets = int(nbl);
+        d.beamlets = reinterpret_cast<const float*>(dev + pc[2].at);
+        d.bl_cdf = reinterpret_cast<const float*>(dev + pc[3].at);
+        d.bl_row = reinterpret_cast<const int*>(dev + pc[4].at);
+        d.bl_f = reinterpret_cast<const double*>(dev + pc[5].at);
+        d.al_cut = reinterpret_cast<const uint64_t*>(dev + pc[6].at);
+        d.al_alias = reinterpret_cast<const int*>(dev + pc[7].at);
+    }
+    return GDPM_OK;
+}
+
+// A run's counters, ledger and status words, one after another in one device
+// block: cleared by one memset and read back by one copy.
+constexpr size_t kRunLedger = C_NCOUNT * 8, kRunStatus = kRunLedger + L_NLEDGER * 8, kRunBytes = kRunStatus + 16;
+static void point_run_block(const Workspace& w, SimParams& P) {
+    unsigned char* b = static_cast<unsigned char*>(w.run.p);
+    P.counters = reinterpret_cast<unsigned long long*>(b);
+    P.ledger = reinterpret_cast<double*>(b + kRunLedger);
+    P.status = reinterpret_cast<uint32_t*>(b + kRunStatus);
+}
+struct RunBlock {      // its copy in the runner's pinned block (valid once the stream is synchronized)
+    const unsigned long long* counters;
+    const double* ledger;
+    const uint32_t* status;
+};
+static int read_run_block(const Workspace& w, cudaStream_t s, RunBlock& b) {
+    unsigned char* h = static_cast<unsigned char*>(w.pinned_host.p) + 64;
+    GDPM_CUDA_TRY(cudaMemcpyAsync(h, w.run.p, kRunBytes, cudaMemcpyDeviceToHost, s));
+    b.counters = reinterpret_cast<const unsigned long long*>(h);
+    b.ledger = reinterpret_cast<const double*>(h + kRunLedger);
+    b.status = reinterpret_cast<const uint32_t*>(h + kRunStatus);
     return GDPM_OK;
 }
 
@@ -469,9 +523,7 @@ static int prepare_workspace(gdpm_ctx* ctx, Runner& r, size_t V, uint32_t cap, u
     if ((rc = ensure(ws.qsrc, size_t(chunk) * kSourceWords * 4))) return rc;
     ws.cap_src = chunk;
     if ((rc = ensure(ws.ctl, size_t(ctx->max_phases + 4) * 16)) ||
-        (rc = ensure(ws.prefix, size_t(n_batches) * (n_bins + 1) * 4)) ||
-        (rc = ensure(ws.counters, C_NCOUNT * 8)) || (rc = ensure(ws.ledger, L_NLEDGER * 8)) ||
-        (rc = ensure(ws.status, 16)))
+        (rc = ensure(ws.run, kRunBytes)))
         return rc;
     if (!ws.pinned_host.p) {
         void* h = nullptr;
@@ -520,7 +572,7 @@ static LoopArgs loop_args(gdpm_ctx* ctx, Runner& r, const SimParams& P, const gd
     L.qsrc = make_queue(ws.qsrc, ws.cap_src);
     L.ctl = static_cast<uint32_t*>(ws.ctl.p);
     L.status = P.status;
-    L.bin_prefix = static_cast<const uint32_t*>(ws.prefix.p);
+    L.bin_prefix = ws.prefix;
     L.prefix_n = ws.prefix_n;
     L.sub_first = sub_first;
     const bool metro = P.S.sampler == GDPM_SAMPLE_METROPOLIS && P.S.n_beamlets > 0 && n_sub == 0;
@@ -563,7 +615,7 @@ static int run_phases(gdpm_ctx* ctx, Runner& r, const SimParams& P, const gdpm_s
         A.n_sub = n_sub;
         A.sub_batches = sub_batches;
         A.sub_first = sub_first;
-        A.bin_prefix = static_cast<const uint32_t*>(ws.prefix.p);
+        A.bin_prefix = ws.prefix;
         A.prefix_n = ws.prefix_n;
         if (ph == photon_src && left > 0) {
             A.n_src = uint32_t(std::min<uint64_t>(left, chunk));
@@ -606,7 +658,7 @@ static int run_phases(gdpm_ctx* ctx, Runner& r, const SimParams& P, const gdpm_s
         const size_t pi = prof_begin(ctx, r, s, ph ? 0 : 1);
         const uint32_t share = (r.serving && !r.small && ctx->small_running.load() > 0)
                                    ? uint32_t(ctx->serve_share8) : 8u;
-        int rc = launch_phase(ctx, s, ph ? GDPM_PHOTON : GDPM_ELECTRON, P, A, hint, share);
+        int rc = launch_phase(ctx, r, s, ph ? GDPM_PHOTON : GDPM_ELECTRON, P, A, hint, share);
         prof_end(ctx, r, s, pi);
         if (rc) return rc;
         ++phases;
@@ -614,10 +666,10 @@ static int run_phases(gdpm_ctx* ctx, Runner& r, const SimParams& P, const gdpm_s
         ++since;
         if (!ph && left == 0 && since >= 2 * ctx->speculative) {
             // pending after electron phase k-1: photons P[k], electrons E[k+1]
-            GDPM_CUDA_TRY(cudaMemcpyAsync(host, ctl + size_t(k) * 4 + 1, 4, cudaMemcpyDeviceToHost, s));
-            GDPM_CUDA_TRY(cudaMemcpyAsync(host + 1, ctl + size_t(k + 1) * 4 + 2, 4, cudaMemcpyDeviceToHost, s));
+            // (rows k and k+1 are neighbours: one copy holds both counts)
+            GDPM_CUDA_TRY(cudaMemcpyAsync(host, ctl + size_t(k) * 4 + 1, 24, cudaMemcpyDeviceToHost, s));
             GDPM_CUDA_TRY(cudaStreamSynchronize(s));
-            if (host[0] == 0 && host[1] == 0) break;
+            if (host[0] == 0 && host[5] == 0) break;
             since = 0;
         }
     }
@@ -727,9 +779,7 @@ int simulate_impl(gdpm_ctx* ctx, Runner& r, gdpm_phantom* ph, gdpm_tables* tb,
         const uint64_t nb = n_hist / n_batches + (uint64_t(b) < n_hist % n_batches ? 1 : 0);
         allot_prefix(src.weights, nb, &prefix[size_t(b) * (n_bins + 1)]);
     }
-    GDPM_CUDA_TRY(cudaMemcpyAsync(ws.prefix.p, prefix.data(), prefix.size() * 4, cudaMemcpyHostToDevice, s));
-    ws.prefix_n = uint32_t(prefix.size());
-    if ((rc = source_upload(r, src, P.S))) return rc;
+    if ((rc = source_upload(r, src, P.S, false, &prefix))) return rc;
     int64_t aux = 0;          // launches besides the transport phases
     if (P.S.sampler == GDPM_SAMPLE_METROPOLIS && P.S.n_beamlets > 0) {
         if ((rc = ensure(ws.chains, size_t(P.S.n_chains) * 4)) || (rc = ensure(ws.pick, size_t(chunk) * 4)))
@@ -737,9 +787,7 @@ int simulate_impl(gdpm_ctx* ctx, Runner& r, gdpm_phantom* ph, gdpm_tables* tb,
         if ((rc = launch_metropolis_init(s, P, static_cast<uint32_t*>(ws.chains.p)))) return rc;
         ++aux;
     }
-    P.counters = static_cast<unsigned long long*>(ws.counters.p);
-    P.ledger = static_cast<double*>(ws.ledger.p);
-    P.status = static_cast<uint32_t*>(ws.status.p);
+    point_run_block(ws, P);
     P.hrec = hrec;
     P.hrecd = hrecd;
     P.n_records = hrec ? ctx->hrec_n : 0;
@@ -768,9 +816,7 @@ int simulate_impl(gdpm_ctx* ctx, Runner& r, gdpm_phantom* ph, gdpm_tables* tb,
         GDPM_CUDA_TRY(cudaMemsetAsync(ws.hi2.p, 0, V * 4, s));
         GDPM_CUDA_TRY(cudaMemsetAsync(ws.lo2.p, 0, V * 4, s));
     }
-    GDPM_CUDA_TRY(cudaMemsetAsync(ws.counters.p, 0, C_NCOUNT * 8, s));
-    GDPM_CUDA_TRY(cudaMemsetAsync(ws.ledger.p, 0, L_NLEDGER * 8, s));
-    GDPM_CUDA_TRY(cudaMemsetAsync(ws.status.p, 0, 16, s));
+    GDPM_CUDA_TRY(cudaMemsetAsync(ws.run.p, 0, kRunBytes, s));
     if (hrec) {
         GDPM_CUDA_TRY(cudaMemsetAsync(hrec, 0, n_hist * 16, s));
         GDPM_CUDA_TRY(cudaMemsetAsync(hrecd, 0, n_hist * 16, s));
@@ -847,18 +893,13 @@ int simulate_impl(gdpm_ctx* ctx, Runner& r, gdpm_phantom* ph, gdpm_tables* tb,
         if (dose_out) GDPM_CUDA_TRY(cudaMemcpyAsync(dose_out, dd, V * 8, cudaMemcpyDefault, s));
         if (sigma_out) GDPM_CUDA_TRY(cudaMemcpyAsync(sigma_out, ds, V * 8, cudaMemcpyDefault, s));
     }
-    unsigned char* h = static_cast<unsigned char*>(ws.pinned_host.p);
-    unsigned long long* hc = reinterpret_cast<unsigned long long*>(h + 64);
-    double* hl = reinterpret_cast<double*>(h + 64 + C_NCOUNT * 8);
-    uint32_t* hs = reinterpret_cast<uint32_t*>(h + 64 + C_NCOUNT * 8 + L_NLEDGER * 8);
-    GDPM_CUDA_TRY(cudaMemcpyAsync(hc, ws.counters.p, C_NCOUNT * 8, cudaMemcpyDeviceToHost, s));
-    GDPM_CUDA_TRY(cudaMemcpyAsync(hl, ws.ledger.p, L_NLEDGER * 8, cudaMemcpyDeviceToHost, s));
-    GDPM_CUDA_TRY(cudaMemcpyAsync(hs, ws.status.p, 4, cudaMemcpyDeviceToHost, s));
+    RunBlock rb;
+    if ((rc = read_run_block(ws, s, rb))) return rc;
     GDPM_CUDA_TRY(cudaStreamSynchronize(s));
     if (conc) ws.edep_clean = grids;        // the fold has cleared every grid of this calculation
     if (st) {
         std::memset(st, 0, sizeof(*st));
-        fill_stats(hc, hl, st);
+        fill_stats(rb.counters, rb.ledger, st);
         if (graph_k) phases = int64_t(*graph_k);
         st->phases = phases;
         st->launches = phases + aux + (conc ? 1 : 2);   // + the metric (and the finalize)
@@ -867,9 +908,9 @@ int simulate_impl(gdpm_ctx* ctx, Runner& r, gdpm_phantom* ph, gdpm_tables* tb,
         st->transport_ms = ms;
     }
     prof_collect(r, st);
-    if (*hs & ST_BOUNDS) return GDPM_E_BOUNDS;
-    if (*hs & ST_QUEUE_OVERFLOW) return GDPM_E_QUEUE_OVERFLOW;
-    if (*hs & (ST_ITER_CAP | ST_PHASE_CAP)) return GDPM_E_TIMEOUT;
+    if (*rb.status & ST_BOUNDS) return GDPM_E_BOUNDS;
+    if (*rb.status & ST_QUEUE_OVERFLOW) return GDPM_E_QUEUE_OVERFLOW;
+    if (*rb.status & (ST_ITER_CAP | ST_PHASE_CAP)) return GDPM_E_TIMEOUT;
     return GDPM_OK;
 }
 
@@ -1356,10 +1397,7 @@ int gdpm_simulate_part(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb, uint64_
     std::vector<uint32_t> prefix(size_t(n_batches) * (n_bins + 1));
     for (int b = 0; b < n_batches; ++b)
         allot_prefix(src.weights, hb(b + 1) - hb(b), &prefix[size_t(b) * (n_bins + 1)]);
-    if ((rc = ensure(ws.prefix, prefix.size() * 4))) return rc;
-    GDPM_CUDA_TRY(cudaMemcpyAsync(ws.prefix.p, prefix.data(), prefix.size() * 4, cudaMemcpyHostToDevice, s));
-    ws.prefix_n = uint32_t(prefix.size());
-    if ((rc = source_upload(r, src, P.S))) return rc;
+    if ((rc = source_upload(r, src, P.S, false, &prefix))) return rc;
     int64_t aux = 0;
     if (P.S.sampler == GDPM_SAMPLE_METROPOLIS && P.S.n_beamlets > 0) {
         // the chains run from their start through the histories before h0
@@ -1372,9 +1410,7 @@ int gdpm_simulate_part(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb, uint64_
             return rc;
         aux += 2;
     }
-    P.counters = static_cast<unsigned long long*>(ws.counters.p);
-    P.ledger = static_cast<double*>(ws.ledger.p);
-    P.status = static_cast<uint32_t*>(ws.status.p);
+    point_run_block(ws, P);
     // the part's grids hold batches first_batch.. as slots 0..n_part-1
     const uintptr_t shift = uintptr_t(first_batch) * V;
     P.batch_stride = uint32_t(V);
@@ -1384,9 +1420,7 @@ int gdpm_simulate_part(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb, uint64_
     P.edep_hi = reinterpret_cast<float*>(reinterpret_cast<uintptr_t>(ws.edep.p) - shift * 4);
     P.edep_lo = reinterpret_cast<float*>(reinterpret_cast<uintptr_t>(ws.edep.p) + (V * size_t(n_part) - shift) * 4);
     GDPM_CUDA_TRY(cudaMemsetAsync(ws.edep.p, 0, V * size_t(n_part) * 8, s));
-    GDPM_CUDA_TRY(cudaMemsetAsync(ws.counters.p, 0, C_NCOUNT * 8, s));
-    GDPM_CUDA_TRY(cudaMemsetAsync(ws.ledger.p, 0, L_NLEDGER * 8, s));
-    GDPM_CUDA_TRY(cudaMemsetAsync(ws.status.p, 0, 16, s));
+    GDPM_CUDA_TRY(cudaMemsetAsync(ws.run.p, 0, kRunBytes, s));
     // the caller's sums, on the device for the fold
     const bool dev = is_device_ptr(sum1) && is_device_ptr(sum2);
     double *d1 = sum1, *d2 = sum2;
@@ -1420,17 +1454,12 @@ int gdpm_simulate_part(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb, uint64_
         GDPM_CUDA_TRY(cudaMemcpyAsync(sum1, d1, V * 8, cudaMemcpyDefault, s));
         GDPM_CUDA_TRY(cudaMemcpyAsync(sum2, d2, V * 8, cudaMemcpyDefault, s));
     }
-    unsigned char* hp = static_cast<unsigned char*>(ws.pinned_host.p);
-    unsigned long long* hc = reinterpret_cast<unsigned long long*>(hp + 64);
-    double* hl = reinterpret_cast<double*>(hp + 64 + C_NCOUNT * 8);
-    uint32_t* hs = reinterpret_cast<uint32_t*>(hp + 64 + C_NCOUNT * 8 + L_NLEDGER * 8);
-    GDPM_CUDA_TRY(cudaMemcpyAsync(hc, ws.counters.p, C_NCOUNT * 8, cudaMemcpyDeviceToHost, s));
-    GDPM_CUDA_TRY(cudaMemcpyAsync(hl, ws.ledger.p, L_NLEDGER * 8, cudaMemcpyDeviceToHost, s));
-    GDPM_CUDA_TRY(cudaMemcpyAsync(hs, ws.status.p, 4, cudaMemcpyDeviceToHost, s));
+    RunBlock rb;
+    if ((rc = read_run_block(ws, s, rb))) return rc;
     GDPM_CUDA_TRY(cudaStreamSynchronize(s));
     if (st) {
         std::memset(st, 0, sizeof(*st));
-        fill_stats(hc, hl, st);
+        fill_stats(rb.counters, rb.ledger, st);
         st->phases = phases;
         st->launches = phases + aux;
         float ms = 0;
@@ -1438,9 +1467,9 @@ int gdpm_simulate_part(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb, uint64_
         st->transport_ms = ms;
     }
     prof_collect(r, st);
-    if (*hs & ST_BOUNDS) return GDPM_E_BOUNDS;
-    if (*hs & ST_QUEUE_OVERFLOW) return GDPM_E_QUEUE_OVERFLOW;
-    if (*hs & (ST_ITER_CAP | ST_PHASE_CAP)) return GDPM_E_TIMEOUT;
+    if (*rb.status & ST_BOUNDS) return GDPM_E_BOUNDS;
+    if (*rb.status & ST_QUEUE_OVERFLOW) return GDPM_E_QUEUE_OVERFLOW;
+    if (*rb.status & (ST_ITER_CAP | ST_PHASE_CAP)) return GDPM_E_TIMEOUT;
     return GDPM_OK;
 }
 
@@ -1454,7 +1483,7 @@ int gdpm_finalize(gdpm_ctx* ctx, gdpm_phantom* ph, int n_batches, const double* 
     Workspace& ws = r.ws;
     int rc;
     if ((rc = ensure(ws.s1, V * 8)) || (rc = ensure(ws.s2, V * 8)) || (rc = ensure(ws.stage, V * 16)) ||
-        (rc = ensure(ws.ledger, L_NLEDGER * 8)))
+        (rc = ensure(ws.run, kRunBytes)))
         return rc;
     if (!ws.pinned_host.p) {
         void* h = nullptr;
@@ -1464,11 +1493,11 @@ int gdpm_finalize(gdpm_ctx* ctx, gdpm_phantom* ph, int n_batches, const double* 
     }
     GDPM_CUDA_TRY(cudaMemcpyAsync(ws.s1.p, sum1, V * 8, cudaMemcpyDefault, s));
     GDPM_CUDA_TRY(cudaMemcpyAsync(ws.s2.p, sum2, V * 8, cudaMemcpyDefault, s));
-    GDPM_CUDA_TRY(cudaMemsetAsync(ws.ledger.p, 0, L_NLEDGER * 8, s));
+    GDPM_CUDA_TRY(cudaMemsetAsync(ws.run.p, 0, kRunBytes, s));
     SimParams P{};
     P.dx = ph->dx; P.dy = ph->dy; P.dz = ph->dz;
     P.rho = static_cast<const float*>(ph->rho.p);
-    P.ledger = static_cast<double*>(ws.ledger.p);
+    point_run_block(ws, P);
     double* dd = static_cast<double*>(ws.stage.p);
     double* ds = dd + V;
     if ((rc = launch_finalize_into(ctx, s, P, V, n_batches, static_cast<const double*>(ws.s1.p),
@@ -1476,8 +1505,9 @@ int gdpm_finalize(gdpm_ctx* ctx, gdpm_phantom* ph, int n_batches, const double* 
         return rc;
     if (dose_out) GDPM_CUDA_TRY(cudaMemcpyAsync(dose_out, dd, V * 8, cudaMemcpyDefault, s));
     if (sigma_out) GDPM_CUDA_TRY(cudaMemcpyAsync(sigma_out, ds, V * 8, cudaMemcpyDefault, s));
-    double* hl = reinterpret_cast<double*>(static_cast<unsigned char*>(ws.pinned_host.p) + 64 + C_NCOUNT * 8);
-    GDPM_CUDA_TRY(cudaMemcpyAsync(hl, ws.ledger.p, L_NLEDGER * 8, cudaMemcpyDeviceToHost, s));
+    RunBlock rb;
+    if ((rc = read_run_block(ws, s, rb))) return rc;
+    const double* hl = rb.ledger;
     GDPM_CUDA_TRY(cudaStreamSynchronize(s));
     if (st) {
         std::memset(st, 0, sizeof(*st));
@@ -1666,15 +1696,12 @@ int gdpm_simulate_beamlets(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb,
     if ((rc = ensure(ws.sub_first, first.size() * 4)) || (rc = ensure(ws.sub_inv, inv.size() * 8)) ||
         (rc = ensure(ws.sub_nbig, nbig.size() * 4)))
         return rc;
-    GDPM_CUDA_TRY(cudaMemcpyAsync(ws.prefix.p, prefix.data(), prefix.size() * 4, cudaMemcpyHostToDevice, s));
-    ws.prefix_n = uint32_t(prefix.size());
     GDPM_CUDA_TRY(cudaMemcpyAsync(ws.sub_first.p, first.data(), first.size() * 4, cudaMemcpyHostToDevice, s));
     GDPM_CUDA_TRY(cudaMemcpyAsync(ws.sub_inv.p, inv.data(), inv.size() * 8, cudaMemcpyHostToDevice, s));
     GDPM_CUDA_TRY(cudaMemcpyAsync(ws.sub_nbig.p, nbig.data(), nbig.size() * 4, cudaMemcpyHostToDevice, s));
-    if ((rc = source_upload(r, src, P.S, true))) return rc;    // syncs: host vectors may go
-    P.counters = static_cast<unsigned long long*>(ws.counters.p);
-    P.ledger = static_cast<double*>(ws.ledger.p);
-    P.status = static_cast<uint32_t*>(ws.status.p);
+    if ((rc = source_upload(r, src, P.S, true, &prefix))) return rc;
+    GDPM_CUDA_TRY(cudaStreamSynchronize(s));   // the host vectors may go out of scope
+    point_run_block(ws, P);
     P.batch_stride = uint32_t(V);
     P.tally_hi = V * uint64_t(slots);
     P.edep = static_cast<double*>(ws.edep.p);
@@ -1691,9 +1718,7 @@ int gdpm_simulate_beamlets(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb,
     // the previous calculation's fold cleared the grids it read
     const size_t grids = V * size_t(slots) * 8;
     if (ws.edep_zero < grids) GDPM_CUDA_TRY(cudaMemsetAsync(ws.edep.p, 0, grids, s));
-    GDPM_CUDA_TRY(cudaMemsetAsync(ws.counters.p, 0, C_NCOUNT * 8, s));
-    GDPM_CUDA_TRY(cudaMemsetAsync(ws.ledger.p, 0, L_NLEDGER * 8, s));
-    GDPM_CUDA_TRY(cudaMemsetAsync(ws.status.p, 0, 16, s));
+    GDPM_CUDA_TRY(cudaMemsetAsync(ws.run.p, 0, kRunBytes, s));
     r.prof_kind.clear();
     GDPM_CUDA_TRY(cudaEventRecord(r.ev0, s));
     int64_t phases = 0, aux = 0;
@@ -1743,18 +1768,13 @@ int gdpm_simulate_beamlets(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb,
                 GDPM_CUDA_TRY(cudaMemcpyAsync(sigma_out + size_t(k0) * V, ss, size_t(nk) * V * 8, cudaMemcpyDefault, s));
         }
     }
-    unsigned char* h = static_cast<unsigned char*>(ws.pinned_host.p);
-    unsigned long long* hc = reinterpret_cast<unsigned long long*>(h + 64);
-    double* hl = reinterpret_cast<double*>(h + 64 + C_NCOUNT * 8);
-    uint32_t* hs = reinterpret_cast<uint32_t*>(h + 64 + C_NCOUNT * 8 + L_NLEDGER * 8);
-    GDPM_CUDA_TRY(cudaMemcpyAsync(hc, ws.counters.p, C_NCOUNT * 8, cudaMemcpyDeviceToHost, s));
-    GDPM_CUDA_TRY(cudaMemcpyAsync(hl, ws.ledger.p, L_NLEDGER * 8, cudaMemcpyDeviceToHost, s));
-    GDPM_CUDA_TRY(cudaMemcpyAsync(hs, ws.status.p, 4, cudaMemcpyDeviceToHost, s));
+    RunBlock rb;
+    if ((rc = read_run_block(ws, s, rb))) return rc;
     GDPM_CUDA_TRY(cudaStreamSynchronize(s));
     ws.edep_clean = grids;                  // k_fold_sub has cleared every slot's grid
     if (st) {
         std::memset(st, 0, sizeof(*st));
-        fill_stats(hc, hl, st);
+        fill_stats(rb.counters, rb.ledger, st);
         if (graph_k) phases = int64_t(*graph_k);
         st->phases = phases;
         st->launches = phases + aux;
@@ -1763,9 +1783,9 @@ int gdpm_simulate_beamlets(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb,
         st->transport_ms = ms;
     }
     prof_collect(r, st);
-    if (*hs & ST_BOUNDS) return GDPM_E_BOUNDS;
-    if (*hs & ST_QUEUE_OVERFLOW) return GDPM_E_QUEUE_OVERFLOW;
-    if (*hs & (ST_ITER_CAP | ST_PHASE_CAP)) return GDPM_E_TIMEOUT;
+    if (*rb.status & ST_BOUNDS) return GDPM_E_BOUNDS;
+    if (*rb.status & ST_QUEUE_OVERFLOW) return GDPM_E_QUEUE_OVERFLOW;
+    if (*rb.status & (ST_ITER_CAP | ST_PHASE_CAP)) return GDPM_E_TIMEOUT;
     return GDPM_OK;
 }
 
@@ -1874,16 +1894,14 @@ int gdpm_debug_sources(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb, uint64_
     const int n_bins = int(ctx->src.weights.size());
     std::vector<uint32_t> prefix(n_bins + 1);
     allot_prefix(ctx->src.weights, nb0, prefix.data());
-    if ((rc = ensure(r.ws.prefix, prefix.size() * 4))) return rc;
-    GDPM_CUDA_TRY(cudaMemcpyAsync(r.ws.prefix.p, prefix.data(), prefix.size() * 4, cudaMemcpyHostToDevice, r.stream));
     SimParams P = base_params(ctx, ph, tb, ctx->request_id);
     if ((rc = get_majorant(ctx, r.stream, ph, tb, &P.maj))) return rc;
-    if ((rc = source_upload(r, ctx->src, P.S))) return rc;
+    if ((rc = source_upload(r, ctx->src, P.S, false, &prefix))) return rc;
     PhaseArgs A{};
     A.src_first = uint32_t(first);
     A.nb_small = uint32_t(n_histories / n_batches);
     A.nb_rem = uint32_t(n_histories % n_batches);
-    A.bin_prefix = static_cast<const uint32_t*>(r.ws.prefix.p);
+    A.bin_prefix = r.ws.prefix;
     if ((rc = run_chains(r, P, first + n))) return rc;
     if (P.S.sampler == GDPM_SAMPLE_METROPOLIS && P.S.n_beamlets > 0)
         A.bl_pick = static_cast<const uint32_t*>(r.ws.pick.p) + first;

@@ -202,23 +202,24 @@ struct Workspace {
     Buffer qsrc;                           // primaries of one source phase
     uint32_t cap_src = 0;
     Buffer ctl;                            // per-phase counters (uint32)
-    Buffer prefix;                         // per-batch spectrum prefix counts
-    uint32_t prefix_n = 0;                 // entries in use
-    Buffer counters, ledger, status;       // run statistics
-    Buffer edges, beamlets, bl_cdf;        // source arrays
-    Buffer bl_row, bl_f, al_cut, al_alias; // beamlet samplers
+    Buffer inputs;                         // a calculation's small inputs (source_upload):
+    const uint32_t* prefix = nullptr;      //   per-batch spectrum prefix counts,
+    uint32_t prefix_n = 0;                 //   how many; edges, fluence map, samplers
+    Buffer run;                            // run statistics: counters, ledger, status
     Buffer chains, pick;                   // Metropolis chain states; picks of one phase
     Buffer sub_first, sub_inv, sub_nbig;   // dose matrix: sub-problem history ranges, batch sizes
     Buffer loop_k;                         // device-driven phase loop: the phase index
     Buffer stage;                          // device staging for host outputs
     Buffer pinned_host;                    // pinned host block for small readbacks
+    Buffer pinned_stage;                   // pinned staging block of the inputs
 };
 
 // Launch wrappers (defined next to their kernels); all work goes to `st`.
 int build_tables_device(gdpm_ctx* ctx, gdpm_tables* t, const gdpm_material_desc* mats);
 int phantom_density_max(gdpm_ctx* ctx, gdpm_phantom* ph);
 int launch_majorant_into(cudaStream_t st, gdpm_phantom* ph, gdpm_tables* t, float* maj);
-int launch_phase(gdpm_ctx* ctx, cudaStream_t st, int particle, const SimParams& P,
+struct Runner;
+int launch_phase(gdpm_ctx* ctx, Runner& r, cudaStream_t st, int particle, const SimParams& P,
                  const PhaseArgs& A, uint32_t n_items_hint, uint32_t share_eighths = 8);
 int launch_fold_into(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t V, uint32_t nb,
                      double* s1, double* s2);
@@ -271,6 +272,13 @@ struct Runner {
     cudaGraph_t loop_graph = nullptr;
     cudaGraphExec_t loop_exec = nullptr;
     std::vector<unsigned char> loop_key;
+    // resident CTAs per SM of the phase kernels this runner launched (asking
+    // the runtime costs as much as a launch)
+    struct Resident {
+        const void* fn = nullptr;
+        int threads = 0, ctas = 0;
+        size_t smem = 0;
+    } resident[6];
 };
 int runner_init(Runner& r, cudaStream_t stream, bool own_stream);
 // Electron phase form of a run: 1 resumable steps, 0 whole steps.

@@ -254,7 +254,7 @@ extern "C" int gdpm_simulate_noalloc(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_table
                 A.out_el = qe[((k + 2) / 2) % 2];
                 A.out_el_count = ctl + size_t(k + 2) * 4 + 2;
             }
-            if ((run_rc = launch_phase(ctx, s, ph_phase ? GDPM_PHOTON : GDPM_ELECTRON, P, A,
+            if ((run_rc = launch_phase(ctx, ctx->run, s, ph_phase ? GDPM_PHOTON : GDPM_ELECTRON, P, A,
                                        A.in_count ? 0u : A.n_src)))
                 break;
             ++phases;

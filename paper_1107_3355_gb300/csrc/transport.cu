@@ -1771,12 +1771,12 @@ int transport_smem(const gdpm_tables* t, int particle) { return int(smem_of(t->d
 // GDPM_PARAM_BLOCK_THREADS when set (at most 256, within every kernel's
 // bound); the tables and counters of a CTA and the warps' stacks in shared
 // memory.  Beside large tables a CTA has fewer warps.
+constexpr size_t kMaxSmem = size_t(227) << 10;
 struct Launch {
     int threads;
     size_t smem;
 };
 static Launch phase_shape(const gdpm_ctx* ctx, const DevTables& T, int pt) {
-    constexpr size_t kMaxSmem = size_t(227) << 10;
     const size_t tables = smem_of(T, pt == 0 ? GDPM_PHOTON : GDPM_ELECTRON);
     const size_t stack = pt == 0 ? kPhStack * sizeof(PhRec) : sizeof(ElStack);
     int thr = ctx->block_threads > 0 ? ctx->block_threads
@@ -1790,7 +1790,7 @@ static Launch phase_shape(const gdpm_ctx* ctx, const DevTables& T, int pt) {
 // share_eighths < 8 gives the grid that many eighths of the GPU: a large
 // request that runs while small ones are active leaves SMs free for them,
 // since persistent CTAs do not yield until their phase's input is drained.
-int launch_phase(gdpm_ctx* ctx, cudaStream_t st, int particle, const SimParams& P,
+int launch_phase(gdpm_ctx* ctx, Runner& r, cudaStream_t st, int particle, const SimParams& P,
                  const PhaseArgs& A, uint32_t n_items_hint, uint32_t share_eighths) {
     const Launch shape = phase_shape(ctx, P.T, particle == GDPM_PHOTON ? 0 : 1);
     const int thr = shape.threads;
@@ -1799,12 +1799,21 @@ int launch_phase(gdpm_ctx* ctx, cudaStream_t st, int particle, const SimParams& 
     static const Kernel kernels[2][3] = {{k_phase<0, kPlain>, k_phase<0, kPair>, k_phase<0, kGeneral>},
                                          {k_phase<1, kPlain>, k_phase<1, kPair>, k_phase<1, kGeneral>}};
     const Kernel fn = kernels[particle == GDPM_PHOTON ? 0 : 1][P.hrec ? kGeneral : P.tally_mode ? kPair : kPlain];
-    GDPM_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-    int bps = ctx->blocks_per_sm;
-    if (bps <= 0) {
-        GDPM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, thr, smem));
-        if (bps < 1) return GDPM_E_ARG;
+    Runner::Resident* known = nullptr;
+    for (Runner::Resident& q : r.resident) {
+        if (q.fn == (const void*)fn && q.threads == thr && q.smem == smem) known = &q;
+        if (known) break;
     }
+    if (!known) {
+        int ctas = 0;
+        GDPM_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kMaxSmem)));
+        GDPM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, fn, thr, smem));
+        for (int k = 5; k > 0; --k) r.resident[k] = r.resident[k - 1];
+        r.resident[0] = Runner::Resident{(const void*)fn, thr, ctas, smem};
+        known = &r.resident[0];
+    }
+    const int bps = ctx->blocks_per_sm > 0 ? ctx->blocks_per_sm : known->ctas;
+    if (bps < 1) return GDPM_E_ARG;
     uint32_t grid = uint32_t(ctx->sm_count) * uint32_t(bps);
     if (share_eighths < 8) grid = std::max<uint32_t>(uint32_t(ctx->sm_count), grid * share_eighths / 8);
     if (n_items_hint > 0) {
