@@ -152,7 +152,9 @@ __device__ __forceinline__ float4 draw(Part& p, uint32_t k0, uint32_t k1) {
 // A banked particle has made no draw yet (draw counter 0).  A primary's
 // history is its phase's first plus its slot, its particle id 1, its draw
 // counter 1 and its voxel follows from its position.  E < 0 marks an empty
-// slot.  One address and three loads per refill, where 13 arrays of one word
+// slot.  A record is written once and read once, with streaming accesses: the
+// L2 is for the phantom and the tallies (CT plan photon phase -3 %).
+// One address and three loads per refill, where 13 arrays of one word
 // took 13 of each: CT plan, photon phase 23.9 -> 22.5 ms, electron phase
 // 31.7 -> 30.1 ms (1e8 histories).
 struct Queue {
@@ -176,7 +178,7 @@ __device__ __forceinline__ void queue_mark_empty(const Queue& q, uint32_t s) {
 }
 __device__ __forceinline__ void queue_load(const Queue& q, uint32_t s, Part& p) {
     const uint4* r = q.rec + size_t(s) * (kQueueWords / 4);
-    const uint4 a = r[0], b = r[1], c = r[2];
+    const uint4 a = __ldcs(r), b = __ldcs(r + 1), c = __ldcs(r + 2);
     p.x = __uint_as_float(a.x); p.y = __uint_as_float(a.y); p.z = __uint_as_float(a.z);
     p.E = __uint_as_float(a.w);
     p.u = __uint_as_float(b.x); p.v = __uint_as_float(b.y); p.w = __uint_as_float(b.z);
@@ -186,15 +188,15 @@ __device__ __forceinline__ void queue_load(const Queue& q, uint32_t s, Part& p) 
 }
 __device__ __forceinline__ void source_store(const Queue& q, uint32_t s, const Part& p) {
     uint4* r = q.rec + size_t(s) * (kSourceWords / 4);
-    r[0] = pack4(p.x, p.y, p.z, __float_as_uint(p.E));
-    r[1] = pack4(p.u, p.v, p.w, p.flags);
+    __stcs(&r[0], pack4(p.x, p.y, p.z, __float_as_uint(p.E)));
+    __stcs(&r[1], pack4(p.u, p.v, p.w, p.flags));
 }
 __device__ __forceinline__ void source_mark_empty(const Queue& q, uint32_t s) {
     q.rec[size_t(s) * (kSourceWords / 4)].w = __float_as_uint(-1.f);
 }
 __device__ __forceinline__ void source_load(const Queue& q, uint32_t s, Part& p) {
     const uint4* r = q.rec + size_t(s) * (kSourceWords / 4);
-    const uint4 a = r[0], b = r[1];
+    const uint4 a = __ldcs(r), b = __ldcs(r + 1);
     p.x = __uint_as_float(a.x); p.y = __uint_as_float(a.y); p.z = __uint_as_float(a.z);
     p.E = __uint_as_float(a.w);
     p.u = __uint_as_float(b.x); p.v = __uint_as_float(b.y); p.w = __uint_as_float(b.z);

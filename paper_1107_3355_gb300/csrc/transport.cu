@@ -882,9 +882,9 @@ __device__ __forceinline__ void bank(const SimParams& P, const PhaseArgs& A, uin
                 const Queue& Q = q ? A.out_ph : A.out_el;
                 if (slot < Q.capacity) {
                     uint4* rec = Q.rec + size_t(slot) * (kQueueWords / 4);
-                    rec[0] = pack4(p.x, p.y, p.z, __float_as_uint(E));
-                    rec[1] = pack4(sg * sec.dx, sg * sec.dy, sg * sec.dz, vox);
-                    rec[2] = make_uint4(p.hist, uint32_t(id), uint32_t(id >> 32), flags);
+                    __stcs(&rec[0], pack4(p.x, p.y, p.z, __float_as_uint(E)));
+                    __stcs(&rec[1], pack4(sg * sec.dx, sg * sec.dy, sg * sec.dz, vox));
+                    __stcs(&rec[2], make_uint4(p.hist, uint32_t(id), uint32_t(id >> 32), flags));
                 } else {
                     atomicOr(P.status, ST_QUEUE_OVERFLOW);
                 }
