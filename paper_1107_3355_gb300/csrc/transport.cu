@@ -838,7 +838,11 @@ __device__ __forceinline__ uint32_t reserve(Slots& sl, uint32_t c, uint32_t r, u
         sl.left -= c;
         return base + r;
     }
-    const uint32_t miss = c - left, want = max(miss, min(A.bank_block, total >> A.share_shift));
+    // beyond 32 slots at most an eighth of the warp's even share of the phase's
+    // items, so that a small phase leaves its queue dense
+    const uint32_t share = total >> A.share_shift;
+    const uint32_t miss = c - left;
+    const uint32_t want = max(miss, min(A.bank_block, max(min(share, 32u), share >> 2)));
     uint32_t nb = 0;
     if (lane_id() == 0) nb = atomicAdd(counter, want);
     nb = __shfl_sync(kFull, nb, 0);
@@ -940,8 +944,8 @@ __device__ __forceinline__ void phase_end(const SimParams& P, const PhaseArgs& A
     for (int q = 0; q < PT + 1; ++q) {
         const Queue& Q = q ? A.out_ph : A.out_el;
         const Slots h = sl[q];
-        const uint32_t slot = h.base + lane;
-        if (lane < h.left && slot < Q.capacity) queue_mark_empty(Q, slot);
+        for (uint32_t i = lane; i < h.left; i += 32u)
+            if (h.base + i < Q.capacity) queue_mark_empty(Q, h.base + i);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) esc += __shfl_down_sync(kFull, esc, o);
@@ -1765,6 +1769,19 @@ static uint32_t share_shift(uint32_t warps) {
     return s;
 }
 
+// Queue slots a warp reserves at a time: up to 32, while all warps' spare
+// slots stay below an eighth of the queue, and up to kBankBlock where they
+// stay below 1/256 of it; exact below 8.  A reservation is an atomic whose
+// answer the warp waits for, a third of a photon phase's banking at 32 slots
+// each: at 128 the photon phases of 1e8 CT histories take 17.9 ms instead of
+// 19.1 (64: 18.0, 256: 18.0).
+constexpr uint64_t kBankBlock = 128u;
+static uint32_t bank_block(uint64_t capacity, uint64_t warps) {
+    const uint64_t b = std::max(std::min<uint64_t>(32u, capacity / (8u * warps)),
+                                std::min(kBankBlock, capacity / (256u * warps)));
+    return b >= 8u ? uint32_t(b) : 0u;
+}
+
 int transport_smem(const gdpm_tables* t, int particle) { return int(smem_of(t->dev, particle)); }
 
 // A phase kernel's launch shape: its own CTA, or the context's
@@ -1820,13 +1837,9 @@ int launch_phase(gdpm_ctx* ctx, Runner& r, cudaStream_t st, int particle, const 
         grid = std::min(grid, n_items_hint);   // a CTA has at least one particle
     }
     if (grid == 0) grid = 1;
-    // queue slots a warp reserves at a time: up to 32, while all warps'
-    // spare slots stay below an eighth of the queue; exact below 8
     PhaseArgs B = A;
     const uint64_t warps = uint64_t(grid) * uint64_t(thr / 32);
-    const uint64_t cap = std::min(A.out_el.capacity, A.out_ph.capacity);
-    const uint64_t bb = std::min<uint64_t>(32u, cap / (8u * warps));
-    B.bank_block = bb >= 8u ? uint32_t(bb) : 0u;
+    B.bank_block = bank_block(std::min(A.out_el.capacity, A.out_ph.capacity), warps);
     B.share_shift = share_shift(uint32_t(warps));
     fn<<<grid, thr, smem, st>>>(P, B);
     GDPM_CUDA_TRY(cudaGetLastError());
@@ -1886,9 +1899,7 @@ int build_loop_graph(gdpm_ctx* ctx, const SimParams& P, LoopArgs& L, bool metrop
         warps = std::max<uint64_t>(warps, uint64_t(grid[t]) * uint64_t(thr[t] / 32));
         L.share_shift[t] = share_shift(grid[t] * uint32_t(thr[t] / 32));
     }
-    const uint64_t cap = std::min(L.qph.capacity, L.qe0.capacity);
-    const uint64_t bb = std::min<uint64_t>(32u, cap / (8u * warps));
-    L.bank_block = bb >= 8u ? uint32_t(bb) : 0u;
+    L.bank_block = bank_block(std::min(L.qph.capacity, L.qe0.capacity), warps);
 
     cudaGraph_t g = nullptr;
     GDPM_CUDA_TRY(cudaGraphCreate(&g, 0));
