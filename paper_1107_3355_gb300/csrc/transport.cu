@@ -1751,14 +1751,17 @@ __global__ void k_debug_sources(const SimParams P, const PhaseArgs A, uint64_t n
 
 }  // namespace
 
-// Shared memory of a phase's tables and counters.
-static size_t smem_of(const DevTables& T, int particle) {
+// Shared memory of the staged tables and the CTA's counters, which bounds the
+// tables a context accepts, and with the electrons' per-material constants.
+static size_t tables_smem(const DevTables& T, int particle) {
     const size_t ne = size_t(T.n_mat) * T.n_e;
     const size_t cnt = align16(C_NCOUNT * 4);
     if (particle == GDPM_PHOTON)
         return align16(ne * 8) + align16(ne * 4) + align16(size_t(T.n_e) * 4) + cnt;
-    return ne * 16 + align16(size_t(T.n_mat) * T.n_r * 4) + align16(size_t(T.n_a) * 4) + cnt +
-           kMaxMat * sizeof(ElMat);
+    return ne * 16 + align16(size_t(T.n_mat) * T.n_r * 4) + align16(size_t(T.n_a) * 4) + cnt;
+}
+static size_t smem_of(const DevTables& T, int particle) {
+    return tables_smem(T, particle) + (particle == GDPM_PHOTON ? 0 : kMaxMat * sizeof(ElMat));
 }
 
 // log2 of at least twice the warps of a phase: items >> shift is at most half
@@ -1782,7 +1785,7 @@ static uint32_t bank_block(uint64_t capacity, uint64_t warps) {
     return b >= 8u ? uint32_t(b) : 0u;
 }
 
-int transport_smem(const gdpm_tables* t, int particle) { return int(smem_of(t->dev, particle)); }
+int transport_smem(const gdpm_tables* t, int particle) { return int(tables_smem(t->dev, particle)); }
 
 // A phase kernel's launch shape: its own CTA, or the context's
 // GDPM_PARAM_BLOCK_THREADS when set (at most 256, within every kernel's
@@ -1832,7 +1835,7 @@ int launch_phase(gdpm_ctx* ctx, Runner& r, cudaStream_t st, int particle, const 
     const int bps = ctx->blocks_per_sm > 0 ? ctx->blocks_per_sm : known->ctas;
     if (bps < 1) return GDPM_E_ARG;
     uint32_t grid = uint32_t(ctx->sm_count) * uint32_t(bps);
-    if (share_eighths < 8) grid = std::max<uint32_t>(uint32_t(ctx->sm_count), grid * share_eighths / 8);
+    if (share_eighths < 8) grid = std::max(1u, grid * share_eighths / 8);
     if (n_items_hint > 0) {
         grid = std::min(grid, n_items_hint);   // a CTA has at least one particle
     }
