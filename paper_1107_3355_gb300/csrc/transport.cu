@@ -35,12 +35,13 @@ constexpr uint32_t kFull = 0xffffffffu;
 // CTA shape each phase kernel is compiled for: threads per CTA and the
 // resident CTAs per SM that fix its register budget.  A warp's stack takes
 // 4.6 KB (photons) or 6.0 KB (electrons) of shared memory, so one CTA stages
-// the tables once and leaves the L1 what it can.  768 threads and 80
-// registers measured best over the workloads: photons at 1024 (64 registers)
-// gain 7 % on the paper's slabs and lose 3 % on the CT phantom, whose voxels
-// miss the smaller L1; electrons at 896 (72 registers) lose 5-8 %, at 640 4 %.
+// the tables once and leaves the L1 what it can.  Photons: 896 threads and 72
+// registers, which wide phases fill (narrow_threads for the others); 1e8 CT
+// histories take 16.8 ms of photon phases instead of 17.9 at 768 and 17.1 at
+// 1024 (64 registers), the lung slab's 2.5e8 25.2 instead of 27.0 and 24.8.
+// Electrons at 896 lose 5-8 %, at 640 4 %.
 #ifndef GDPM_THREADS_PHOTON
-#define GDPM_THREADS_PHOTON 768
+#define GDPM_THREADS_PHOTON 896
 #endif
 #ifndef GDPM_MIN_CTAS_PHOTON
 #define GDPM_MIN_CTAS_PHOTON 1
@@ -1792,15 +1793,23 @@ int transport_smem(const gdpm_tables* t, int particle) { return int(tables_smem(
 // bound); the tables and counters of a CTA and the warps' stacks in shared
 // memory.  Beside large tables a CTA has fewer warps.
 constexpr size_t kMaxSmem = size_t(227) << 10;
+// A photon phase that starts fewer than kWideItems histories per thread (the
+// later generations among them) runs narrow: its last rounds, which few lanes
+// fill, cost more than more warps hide.  1e6
+// photons on 128^3 (7 a thread) take 0.50 ms of photon phases at 768 threads
+// and 0.55 at 896, a 1e5 beamlet 0.26 and 0.27; 1e7 CT photons (73 a thread)
+// 2.11 and 2.03, 3.3e7 lung photons 7 % less at 896.
+constexpr int kNarrowThreads = std::min(768, PhaseShape<0>::threads);
+constexpr uint64_t kWideItems = 64u;
 struct Launch {
     int threads;
     size_t smem;
 };
-static Launch phase_shape(const gdpm_ctx* ctx, const DevTables& T, int pt) {
+static Launch phase_shape(const gdpm_ctx* ctx, const DevTables& T, int pt, bool narrow) {
     const size_t tables = smem_of(T, pt == 0 ? GDPM_PHOTON : GDPM_ELECTRON);
     const size_t stack = pt == 0 ? kPhStack * sizeof(PhRec) : sizeof(ElStack);
     int thr = ctx->block_threads > 0 ? ctx->block_threads
-              : pt == 0              ? PhaseShape<0>::threads
+              : pt == 0              ? (narrow ? kNarrowThreads : PhaseShape<0>::threads)
                                      : PhaseShape<1>::threads;
     thr = std::min(thr, 32 * int((kMaxSmem - tables) / stack));
     return Launch{thr, tables + stack * size_t(thr / 32)};
@@ -1812,7 +1821,8 @@ static Launch phase_shape(const gdpm_ctx* ctx, const DevTables& T, int pt) {
 // since persistent CTAs do not yield until their phase's input is drained.
 int launch_phase(gdpm_ctx* ctx, Runner& r, cudaStream_t st, int particle, const SimParams& P,
                  const PhaseArgs& A, uint32_t n_items_hint, uint32_t share_eighths) {
-    const Launch shape = phase_shape(ctx, P.T, particle == GDPM_PHOTON ? 0 : 1);
+    const uint64_t wide = kWideItems * uint64_t(ctx->sm_count) * uint64_t(PhaseShape<0>::threads);
+    const Launch shape = phase_shape(ctx, P.T, particle == GDPM_PHOTON ? 0 : 1, A.n_src < wide);
     const int thr = shape.threads;
     const size_t smem = shape.smem;
     using Kernel = void (*)(const SimParams, const PhaseArgs);
@@ -1889,7 +1899,7 @@ int build_loop_graph(gdpm_ctx* ctx, const SimParams& P, LoopArgs& L, bool metrop
     int thr[2];
     uint64_t warps = 0;
     for (int t = 0; t < 2; ++t) {
-        const Launch shape = phase_shape(ctx, P.T, t);
+        const Launch shape = phase_shape(ctx, P.T, t, false);
         thr[t] = shape.threads;
         smem[t] = shape.smem;
         GDPM_CUDA_TRY(cudaFuncSetAttribute(fn[t], cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem[t])));

@@ -51,3 +51,22 @@ def test_results_do_not_depend_on_launch_shape(kind, n):
         assert events == ref[1], params
         # the same FP64 deposits in another order
         assert np.all(np.abs(d - ref[0]) <= 1e-11 * ref[0]), params
+
+
+# A source phase of 9e6 photons fills the wide photon shape; in chunks of half
+# of them, every phase runs the narrow one.  A voxel's dose is a sum of up to
+# 9e6 positive FP64 deposits, whose order moves it by about sqrt(9e6) half-ulps.
+@pytest.mark.parametrize("kind", ["compton", "pair"])
+def test_wide_and_narrow_photon_phases(kind):
+    n = 9_000_000
+    prob = problem(kind, n)
+    runs = []
+    for params in ({G.GDPM_PARAM_SOURCE_CHUNK: n}, {G.GDPM_PARAM_SOURCE_CHUNK: n // 2}):
+        eng = G.Engine(prob, params=params)
+        try:
+            d, _, st = eng.run()
+            runs.append((d.cpu().numpy(), [st[k] for k in KEYS]))
+        finally:
+            eng.close()
+    assert runs[0][1] == runs[1][1]
+    assert np.all(np.abs(runs[0][0] - runs[1][0]) <= 1e-11 * runs[0][0])
