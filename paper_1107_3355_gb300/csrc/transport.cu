@@ -506,12 +506,11 @@ struct Electron {
 
 // The condensed-history step in progress (Sec. 2.1): set up once (limits, end
 // energy, hinge deflection), then its straight legs are walked through the
-// voxels over one or more rounds of the phase loop.
+// voxels over one or more rounds of the phase loop.  What leg 2 needs is in
+// the lane's ElStack::hinge.
 struct ElStep {
     float left;        // mass thickness left in the current leg (g/cm2)
-    float m1;          // mass thickness of the second leg
     float dpm;         // energy loss per unit mass thickness along the step
-    float u1, v1, w1;  // the direction after the hinge
     float Tend;        // energy at the end of the step
     float dep;         // energy of the step tallied or owed to a voxel so far
     float rho;         // density of the particle's current voxel
@@ -551,7 +550,7 @@ __device__ __forceinline__ Round absorb(const SimParams& P, Electron& p, uint32_
 // voxel's material (`mat`), energy at its end, deflection at the random hinge.
 template <int GEN>
 __device__ __forceinline__ void electron_setup(const SimParams& P, const ElSmem& S, const Electron& p, uint4 x,
-                                               int mat, ElStep& st) {
+                                               int mat, ElStep& st, float4& hinge) {
     const DevTables& T = P.T;
     const float4 r = make_float4(u01(x.x), u01(x.y), u01(x.z), u01(x.w));
     hist_count<GEN>(P, p.hist, 1);
@@ -601,14 +600,14 @@ __device__ __forceinline__ void electron_setup(const SimParams& P, const ElSmem&
     cossin_2pi(r.w, cp, sp);
     // leg 1 keeps the step's start direction, so the deflection is applied to
     // it here, with all lanes that start a step together
-    st.u1 = p.u; st.v1 = p.v; st.w1 = p.w;
-    rotate(st.u1, st.v1, st.w1, mu, cp, sp);
+    float u1 = p.u, v1 = p.v, w1 = p.w;
+    rotate(u1, v1, w1, mu, cp, sp);
     st.dpm = xs > 0.f ? dT / xs : 0.f;
     st.dep = 0.f;
     st.Tend = Tend;
     // random hinge: zeta x_s straight, deflect, (1 - zeta) x_s straight
     st.left = r.y * xs;
-    st.m1 = (1.f - r.y) * xs;
+    hinge = make_float4(u1, v1, w1, (1.f - r.y) * xs);
     st.what = 1u | (lim << 2) | (uint32_t(m) << 4);
 }
 
@@ -684,15 +683,16 @@ __device__ __forceinline__ bool walk_cross(const SimParams& P, Electron& p, ElSt
 // left the phantom.
 template <int GEN>
 __device__ __forceinline__ int walk_stretch(const SimParams& P, Electron& p, ElStep& s, Walk& k,
-                                            uint32_t& crossings) {
+                                            const float4& hinge, uint32_t& crossings) {
     bool ends = walk_move(P, p, s, k);
     if (ends && (s.what & 3u) == 1u) {
         // the hinge: the rest of leg 1 stays owed to the current voxel
         p.pend = fmaf(s.dpm, s.left, p.pend);
         s.dep = fmaf(s.dpm, s.left, s.dep);
-        p.u = s.u1; p.v = s.v1; p.w = s.w1;
+        const float4 h = hinge;
+        p.u = h.x; p.v = h.y; p.w = h.z;
         s.what ^= 3u;                         // leg 1 -> leg 2
-        s.left = s.m1;
+        s.left = h.w;
         walk_aim(p, k);
         ends = walk_move(P, p, s, k);
     }
@@ -710,19 +710,18 @@ constexpr int kDrainedStretches = 16;
 // hard-event candidate.
 template <int GEN>
 __device__ __forceinline__ Round electron_round(const SimParams& P, const ElSmem& S, Electron& p, ElStep& st,
-                                                uint4 x, int mat, int stretches, double& esc,
+                                                uint4 x, int mat, float4& hinge, int stretches, double& esc,
                                                 uint32_t& crossings, uint32_t& kind) {
     if ((st.what & 3u) == 0u) {
-        ++p.ctr;
-        electron_setup<GEN>(P, S, p, x, mat, st);
+        electron_setup<GEN>(P, S, p, x, mat, st, hinge);
     }
     Walk k;
     k.lin = vox_linear(P, p.vox);
     k.fx = float(p.vox & 1023u); k.fy = float((p.vox >> 10) & 1023u); k.fz = float(p.vox >> 20);
     walk_aim(p, k);
-    int res = walk_stretch<GEN>(P, p, st, k, crossings);
+    int res = walk_stretch<GEN>(P, p, st, k, hinge, crossings);
 #pragma unroll 1
-    for (int n = 1; res == 0 && n < stretches; ++n) res = walk_stretch<GEN>(P, p, st, k, crossings);
+    for (int n = 1; res == 0 && n < stretches; ++n) res = walk_stretch<GEN>(P, p, st, k, hinge, crossings);
     if (res == 0) return Round::go;
     st.what &= ~3u;
     if (res == 2) {
@@ -1176,6 +1175,15 @@ constexpr uint32_t kElReady = 32, kElWait = 32, kElStack = kElReady + kElWait + 
 struct ElStack {
     uint4 a[kElStack], b[kElStack], c[kElStack], d[kElStack];
     Slots held[2];      // the warp's queue reservations, used only by event rounds
+    // What a lane needs once a round or a step, kept out of its registers (24
+    // instead of 72 bytes of spills): history, id and draw counter of its
+    // electron; direction after the hinge and mass thickness of leg 2.  1e8 CT
+    // histories: electron phases 24.0 -> 23.3 ms, lung slab 47.1 -> 46.2.  The
+    // KB a warp leaves room for 24 warps beside 58 KB of tables (4 materials
+    // of 512 energies take 53); beside 8 materials' 103 KB 17 run and 1e6
+    // 20 MeV electrons take 4.19 instead of 4.01 ms.
+    uint4 ids[32];
+    float4 hinge[32];
 };
 
 __device__ __forceinline__ void el_store(ElStack& s, uint32_t i, const Electron& p, uint32_t kind) {
@@ -1294,6 +1302,7 @@ __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs
             const uint32_t r = __popc(nm & lt);
             if (!active && r < n_ready && lane < lanes) {
                 el_load(stack, n_ready - 1u - r, p);
+                stack.ids[lane] = make_uint4(p.hist, p.pidlo, p.pidhi, p.ctr);
                 active = true;
                 st.what = 0u;
             }
@@ -1313,7 +1322,7 @@ __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs
         }
         const uint32_t k = min(n_wait, 32u);
         const uint32_t top = kElStack - n_wait + (lane < k ? lane : 0u);     // the k last set aside
-        uint4 c = make_uint4(p.hist, p.pidlo, p.pidhi, p.ctr);
+        uint4 c = stack.ids[lane];
         // material and density of the voxel a step starts in: the loads run
         // while the draw is made
         int mat = 0;
@@ -1331,7 +1340,10 @@ __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs
             Round what = Round::go;
             n_steps += __popc(__ballot_sync(kFull, active && (st.what & 3u) == 0u));
             if (active) {
-                what = electron_round<GEN>(P, es, p, st, x, mat, drained ? max(P.walk_trips, kDrainedStretches) : P.walk_trips, esc,
+                if ((st.what & 3u) == 0u) stack.ids[lane].w = c.w + 1u;
+                p.hist = c.x;
+                what = electron_round<GEN>(P, es, p, st, x, mat, stack.hinge[lane],
+                                           drained ? max(P.walk_trips, kDrainedStretches) : P.walk_trips, esc,
                                            crossings, kind);
                 active = what == Round::go;
             }
@@ -1339,7 +1351,11 @@ __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs
             n_ended += __popc(alive);
             alive = __ballot_sync(kFull, active);
             n_ended -= __popc(m) + __popc(alive);
-            if (what == Round::wait) el_store(stack, kElStack - 1u - n_wait - __popc(m & lt), p, kind);
+            if (what == Round::wait) {
+                const uint4 id = stack.ids[lane];
+                p.hist = id.x; p.pidlo = id.y; p.pidhi = id.z; p.ctr = id.w;
+                el_store(stack, kElStack - 1u - n_wait - __popc(m & lt), p, kind);
+            }
             n_wait += __popc(m);
             __syncwarp();
         } else {
