@@ -233,7 +233,7 @@ __device__ __forceinline__ void voxel_of(const SimParams& P, Part& p) {
 
 // Move a primary from outside onto the phantom surface (ray-box slabs); the
 // entry coordinate is set exactly on the face.  False if the ray misses.
-__device__ bool enter_box(const SimParams& P, Part& p) {
+__device__ __forceinline__ bool enter_box(const SimParams& P, Part& p) {
     if (inside(P, p.x, p.y, p.z)) return true;
     const float o[3] = {p.x, p.y, p.z}, d[3] = {p.u, p.v, p.w}, L[3] = {P.Lx, P.Ly, P.Lz};
     float tmin = -kInf, tmax = kInf;
@@ -252,8 +252,10 @@ __device__ bool enter_box(const SimParams& P, Part& p) {
     if (amin < 0 || tmax <= tmin || tmax <= 0.f) return false;
     float q[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) q[a] = fminf(fmaxf(fmaf(tmin, d[a], o[a]), 0.f), L[a]);
-    q[amin] = d[amin] > 0.f ? 0.f : L[amin];
+    for (int a = 0; a < 3; ++a) {
+        q[a] = fminf(fmaxf(fmaf(tmin, d[a], o[a]), 0.f), L[a]);
+        if (a == amin) q[a] = d[a] > 0.f ? 0.f : L[a];   // by value: an index would put the arrays in local memory
+    }
     p.x = q[0]; p.y = q[1]; p.z = q[2];
     return true;
 }
@@ -288,8 +290,8 @@ __device__ __forceinline__ int pick_beamlet(const DevSource& S, const PhaseArgs&
 // prefix_tab / cdf_tab: copies of A.bin_prefix and S.bl_cdf (e.g. in shared
 // memory), or null to read the originals.
 __device__ bool make_primary(const SimParams& P, const PhaseArgs& A, uint32_t idx, Part& p,
-                             Acc& acc, const uint32_t* prefix_tab = nullptr,
-                             const float* cdf_tab = nullptr) {
+                             Acc& acc, uint32_t inv_big, uint32_t inv_small,
+                             const uint32_t* prefix_tab = nullptr, const float* cdf_tab = nullptr) {
     const DevSource& S = P.S;
     const uint32_t h = A.src_first + idx;
     // a dose-matrix run: sub-problem k holds histories [sub_first[k],
@@ -311,20 +313,26 @@ __device__ bool make_primary(const SimParams& P, const PhaseArgs& A, uint32_t id
     // the first nb_rem hold nb_small + 1 histories)
     const uint32_t hl = h - h0;
     const uint32_t big = nb_small + 1u, split = nb_rem * big;
-    uint32_t b, local;
-    if (hl < split) {
-        b = hl / big;
-        local = hl - b * big;
-    } else {
-        b = nb_rem + (hl - split) / nb_small;
-        local = (hl - split) - (b - nb_rem) * nb_small;
+    // hl < split: histories of the long batches.  The quotient by the batch
+    // size from its reciprocal, floor((2^32 - 1) / size), is one too small at
+    // most
+    const bool first = hl < split;
+    const uint32_t size = first ? big : nb_small, at = first ? hl : hl - split;
+    const uint32_t inv = A.n_sub ? 0xffffffffu / size : first ? inv_big : inv_small;
+    uint32_t b = __umulhi(at, inv), local = at - b * size;
+    if (local >= size) {
+        ++b;
+        local -= size;
     }
+    if (!first) b += nb_rem;
     const uint32_t slot = A.n_sub ? k * A.sub_batches + b : b;
     const uint32_t* prefix = (prefix_tab ? prefix_tab : A.bin_prefix) + size_t(slot) * (S.n_bins + 1);
     p.hist = h;
     p.pidlo = 1u; p.pidhi = 0u; p.ctr = 0u;
     p.flags = (slot << kBatchShift) & kBatchMask;
-    const float4 r = draw(p, P.key0, P.key1);
+    const uint4 rx = philox4x32_10(make_uint4(h, 1u, 0u, 0u), P.keys);
+    ++p.ctr;
+    const float4 r = make_float4(u01(rx.x), u01(rx.y), u01(rx.z), u01(rx.w));
     int lo = 0, hi = S.n_bins;
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
@@ -358,13 +366,13 @@ __device__ bool make_primary(const SimParams& P, const PhaseArgs& A, uint32_t id
             a0 = q3.x; a1 = q3.y; b0 = q3.z; b1 = q3.w;
         }
         const float su = fmaf(a1 - a0, r.x, a0), sv = fmaf(b1 - b0, r.y, b0);
-        const float ax = cen[0] + su * au[0] + sv * av[0];
-        const float ay = cen[1] + su * au[1] + sv * av[1];
-        const float az = cen[2] + su * au[2] + sv * av[2];
+        const float ax = fmaf(sv, av[0], fmaf(su, au[0], cen[0]));
+        const float ay = fmaf(sv, av[1], fmaf(su, au[1], cen[1]));
+        const float az = fmaf(sv, av[2], fmaf(su, au[2], cen[2]));
         p.x = src[0]; p.y = src[1]; p.z = src[2];
         const float dx = ax - p.x, dy = ay - p.y, dz = az - p.z;
-        const float n = rsqrtf(dx * dx + dy * dy + dz * dz);
-        p.u = dx * n; p.v = dy * n; p.w = dz * n;
+        const float n = rsqrtf(fmaf(dz, dz, fmaf(dx, dx, __fmul_rn(dy, dy))));
+        p.u = __fmul_rn(dx, n); p.v = __fmul_rn(dy, n); p.w = __fmul_rn(dz, n);
     }
     acc.src += p.E;
     if (!enter_box(P, p)) {
@@ -1425,6 +1433,10 @@ k_phase(const SimParams P, const PhaseArgs A) {
 
 
 // ---------------------------------------------------------------- sources
+// Source CTAs: one of 1024 threads per SM for phases that fill them, which
+// stages its tables once and leaves the L1 to the beamlets' rows (eight of
+// 256, of which six are resident, take 7 % longer); CTAs of 256 below.
+constexpr int kSourceThreads = 1024;
 // The primaries of one source phase (Sec. 2.3), made with every lane busy
 // before the phase runs: primary idx goes to slot idx of A.src.  One that
 // misses the phantom leaves its slot empty (E < 0) and is accounted here:
@@ -1432,6 +1444,11 @@ k_phase(const SimParams P, const PhaseArgs A) {
 // The spectrum prefix counts of the batches and the cumulative beamlet
 // weights are searched for every primary: a CTA copies them to shared
 // memory when they fit (n_prefix, n_cdf of them; see sources_smem).
+// Bound by its instructions and the latency of its searches, not by the 32
+// bytes a primary it writes.  1e8 primaries of the CT plan 2.21 -> 1.79 ms,
+// 2.5e8 of the lung slab's field 3.32 -> 2.93 ms: the box entry without arrays
+// in local memory, the batch index without two divisions and the draw's round
+// keys took 0.30 and 0.19 of that, the CTA shape 0.13 and 0.20.
 template <int PT>
 __device__ __forceinline__ void make_sources(const SimParams& P, const PhaseArgs& A, uint32_t n_prefix,
                                              uint32_t n_cdf) {
@@ -1444,11 +1461,12 @@ __device__ __forceinline__ void make_sources(const SimParams& P, const PhaseArgs
     const uint32_t* ptab = n_prefix ? s_prefix : nullptr;
     const float* ctab = n_cdf ? s_cdf : nullptr;
     Acc acc{0.0, 0.0};
+    const uint32_t inv_big = 0xffffffffu / (A.nb_small + 1u), inv_small = 0xffffffffu / max(A.nb_small, 1u);
     uint32_t made = 0u, missed = 0u;
     for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < A.n_src;
          idx += gridDim.x * blockDim.x) {
         Part p{};
-        if (make_primary(P, A, idx, p, acc, ptab, ctab)) {
+        if (make_primary(P, A, idx, p, acc, inv_big, inv_small, ptab, ctab)) {
             source_store(A.src, GDPM_IDX(P.status, idx, A.src.capacity, ST_B_QUEUE), p);
         } else {
             source_mark_empty(A.src, GDPM_IDX(P.status, idx, A.src.capacity, ST_B_QUEUE));
@@ -1475,7 +1493,7 @@ __device__ __forceinline__ void make_sources(const SimParams& P, const PhaseArgs
 }
 
 template <int PT>
-__global__ void __launch_bounds__(256) k_sources(const SimParams P, const PhaseArgs A, uint32_t n_prefix,
+__global__ void __launch_bounds__(kSourceThreads) k_sources(const SimParams P, const PhaseArgs A, uint32_t n_prefix,
                                                  uint32_t n_cdf) {
     make_sources<PT>(P, A, n_prefix, n_cdf);
 }
@@ -1643,7 +1661,7 @@ k_phase_loop(const SimParams P, const LoopArgs L) {
 
 // Primaries of this pass's source phase (before it runs).
 template <int PT>
-__global__ void __launch_bounds__(256) k_sources_loop(const SimParams P, const LoopArgs L, uint32_t n_prefix,
+__global__ void __launch_bounds__(kSourceThreads) k_sources_loop(const SimParams P, const LoopArgs L, uint32_t n_prefix,
                                                       uint32_t n_cdf) {
     const PhaseArgs A = phase_args(L, *L.k + uint32_t(PT));
     if (A.n_src) make_sources<PT>(P, A, n_prefix, n_cdf);
@@ -1759,7 +1777,8 @@ __global__ void k_debug_sources(const SimParams P, const PhaseArgs A, uint64_t n
          s += uint64_t(gridDim.x) * blockDim.x) {
         Part p{};
         Acc acc{0, 0};
-        const bool in = make_primary(P, A, uint32_t(s), p, acc);
+        const bool in = make_primary(P, A, uint32_t(s), p, acc, 0xffffffffu / (A.nb_small + 1u),
+                                     0xffffffffu / max(A.nb_small, 1u));
         double* o = out + 8 * s;
         o[0] = p.x; o[1] = p.y; o[2] = p.z; o[3] = p.u; o[4] = p.v; o[5] = p.w; o[6] = p.E;
         o[7] = in ? 1.0 : 0.0;
@@ -1829,6 +1848,13 @@ static Launch phase_shape(const gdpm_ctx* ctx, const DevTables& T, int pt, bool 
                                      : PhaseShape<1>::threads;
     thr = std::min(thr, 32 * int((kMaxSmem - tables) / stack));
     return Launch{thr, tables + stack * size_t(thr / 32)};
+}
+
+// CTAs of n primaries: see kSourceThreads.
+static void source_shape(const gdpm_ctx* ctx, uint32_t n, uint32_t& grid, uint32_t& threads) {
+    const uint32_t sms = uint32_t(ctx->sm_count);
+    threads = n / uint32_t(kSourceThreads) >= sms ? uint32_t(kSourceThreads) : 256u;
+    grid = threads == 256u ? n / 256u + 1u : sms;
 }
 
 // Persistent grid: SM count x resident CTAs per SM for this shared-memory size.
@@ -1974,10 +2000,11 @@ int build_loop_graph(gdpm_ctx* ctx, const SimParams& P, LoopArgs& L, bool metrop
         add((const void*)k_metropolis_loop, dim3((P.S.n_chains + kMetroChains - 1) / kMetroChains),
             dim3(kMetroThreads), 0, metro_args_v);
     {
-        const uint32_t sg = std::max(1u, std::min((L.chunk + 255u) / 256u, uint32_t(ctx->sm_count) * 8u));
+        uint32_t sg, sthr;
+        source_shape(ctx, L.chunk, sg, sthr);
         const void* sf = L.src_particle == GDPM_PHOTON ? (const void*)k_sources_loop<0> : (const void*)k_sources_loop<1>;
         if (e == cudaSuccess) e = cudaFuncSetAttribute(sf, cudaFuncAttributeMaxDynamicSharedMemorySize, int(src_sm));
-        add(sf, dim3(sg), dim3(256), src_sm, src_args_v);
+        add(sf, dim3(sg), dim3(sthr), src_sm, src_args_v);
     }
     add(fn[0], dim3(grid[0]), dim3(thr[0]), smem[0], phase_args_v);
     add(fn[1], dim3(grid[1]), dim3(thr[1]), smem[1], phase_args_v);
@@ -1996,16 +2023,17 @@ int build_loop_graph(gdpm_ctx* ctx, const SimParams& P, LoopArgs& L, bool metrop
 }
 
 int launch_sources(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, const PhaseArgs& A) {
-    const uint32_t grid = std::max(1u, std::min((A.n_src + 255u) / 256u, uint32_t(ctx->sm_count) * 8u));
+    uint32_t grid, threads;
+    source_shape(ctx, A.n_src, grid, threads);
     uint32_t np, nc;
     sources_smem(A.prefix_n, cdf_entries(P, A), np, nc);
     const size_t sm = size_t(nc) * 4 + size_t(np) * 4;
     if (P.S.particle == GDPM_PHOTON) {
         GDPM_CUDA_TRY(cudaFuncSetAttribute(k_sources<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm)));
-        k_sources<0><<<grid, 256, sm, st>>>(P, A, np, nc);
+        k_sources<0><<<grid, threads, sm, st>>>(P, A, np, nc);
     } else {
         GDPM_CUDA_TRY(cudaFuncSetAttribute(k_sources<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm)));
-        k_sources<1><<<grid, 256, sm, st>>>(P, A, np, nc);
+        k_sources<1><<<grid, threads, sm, st>>>(P, A, np, nc);
     }
     GDPM_CUDA_TRY(cudaGetLastError());
     return GDPM_OK;

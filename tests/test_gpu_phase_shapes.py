@@ -70,3 +70,26 @@ def test_wide_and_narrow_photon_phases(kind):
             eng.close()
     assert runs[0][1] == runs[1][1]
     assert np.all(np.abs(runs[0][0] - runs[1][0]) <= 1e-11 * runs[0][0])
+
+
+# Sources in CTAs of 1024 threads, one per SM, from 1024 primaries per SM on;
+# in chunks of 50 000 always in CTAs of 256.  Seven batches leave long and
+# short ones, and chunks start inside them; half of the field misses the
+# phantom.  The same deposits in another order.
+@pytest.mark.parametrize("n", [1024 * 152 - 1, 1024 * 152, 200_003])
+def test_source_launch_shapes(n):
+    ph = W.slab_phantom((17, 23, 40), (0.5, 0.5, 0.5))
+    prob = W.Problem(ph, W.field_source(ph, W.kramers_spectrum(), ssd=30.0, field=(14.0, 14.0)), n, 7,
+                     eabs_photon=0.05, eabs_electron=0.2, e_min=0.005, e_max=7.0)
+    runs = []
+    for chunk in (n, 50_000):
+        eng = G.Engine(prob, params={G.GDPM_PARAM_SOURCE_CHUNK: chunk})
+        try:
+            d, s, st = eng.run()
+            runs.append((d.cpu().numpy(), s.cpu().numpy(), [st[k] for k in KEYS]))
+        finally:
+            eng.close()
+    assert runs[0][2] == runs[1][2]
+    for a, b in zip(runs[0][:2], runs[1][:2]):
+        # sigma takes a difference of sums: 1e-11 of its voxel's dose
+        assert np.all(np.abs(a - b) <= 1e-11 * runs[0][0])
