@@ -419,9 +419,11 @@ static int get_majorant(gdpm_ctx* ctx, cudaStream_t st, gdpm_phantom* ph, gdpm_t
 
 // The electron phase form of a run (GDPM_PARAM_ELECTRON_WALK): automatic (2)
 // takes resumable steps.  A walk's stretches per round, 2, were measured against
-// 1, 3, 4 and whole steps: CT plan electron phase 25.7 ms against 26.7, 27.0,
-// 28.2 and 32.6; the paper's 6 MV lung slab 50.0 against 50.0, 51.7, 52.4 and
-// 57.5; 20 MeV electrons on its bone slab 5.60 against 6.22, 5.62, 5.73, 6.49.
+// 1, 3, 4 and whole steps when the CT plan's electron phase took 25.7 ms:
+// 26.7, 27.0, 28.2 and 32.6; the paper's 6 MV lung slab's 50.0 against 50.0,
+// 51.7, 52.4 and 57.5; 20 MeV electrons on its bone slab 5.60 against 6.22,
+// 5.62, 5.73, 6.49.  One stretch against two now: 24.2 and 23.4, 46.8 and
+// 46.2, 5.8 and 5.2.
 int walk_form(const gdpm_ctx* ctx) { return ctx->electron_walk == 2 ? 1 : ctx->electron_walk; }
 
 SimParams base_params(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb, uint32_t request_id) {

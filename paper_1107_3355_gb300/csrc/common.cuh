@@ -131,10 +131,7 @@ constexpr int kMaxSlots = 32767;
 // One Philox block for the transport kernels.  Out of line (it has no
 // warp-synchronous operations), so its ten unrolled rounds exist once in
 // the kernel instead of at every draw site.
-#ifndef GDPM_PHILOX_ATTR
-#define GDPM_PHILOX_ATTR __noinline__
-#endif
-static __device__ GDPM_PHILOX_ATTR uint4 philox_block(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
+static __device__ __noinline__ uint4 philox_block(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
                                            uint32_t k0, uint32_t k1) {
     return philox4x32_10(make_uint4(c0, c1, c2, c3), k0, k1);
 }

@@ -88,8 +88,9 @@ struct PhaseArgs {
     uint32_t* out_ph_count;
     uint32_t* out_el_count;
     // queue slots a warp reserves at a time (0: exactly what it pushes), and at
-    // most half its even share of the phase's input: a small phase would leave
-    // the next one mostly reserved slots that were never written
+    // most half its even share of the phase's input (an eighth beyond 32
+    // slots): a small phase would leave the next one mostly reserved slots
+    // that were never written
     uint32_t bank_block;
     uint32_t share_shift;      // items >> share_shift: at most half a warp's even share of them
     // dose matrix: n_sub sub-problems (one per fluence-map row), sub-problem

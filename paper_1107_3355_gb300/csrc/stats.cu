@@ -132,20 +132,33 @@ __global__ void __launch_bounds__(256) k_fold(SimParams P, size_t V, double inv_
     if (threadIdx.x == 0 && t != 0.0) atomicAdd(&P.ledger[L_DEPOSITED], t);
 }
 
-// Mean dose of a voxel and its standard error, MeV/g per history, from the
-// sums a1, a2 over nb batches of x_b = E_b/n_b and x_b^2.  FP64 division and
-// square root are slow on this part, so 1/mass and sqrt(var) start from FP32
-// estimates and take one FP64 Newton step each (relative error ~1e-14).
-__device__ __forceinline__ double inverse_mass(float rho, double dvol) {
-    const double mass = double(rho) * dvol;
-    const double im = double(1.0f / float(mass));
-    return im * fma(-mass, im, 2.0);
+// Mean dose of a voxel and its standard error, MeV/g per history.  With n_b
+// batches, x_b = E_b/n_b and volume V, the weights of a voxel's sums make
+// x = sum x_b / (n_b V) and q = sum x_b^2 / (n_b (n_b - 1) V^2) at once, so
+// that dose = x / rho and sigma = sqrt(q - x^2 / (n_b - 1)) / rho: about 16
+// FP64 operations a voxel instead of 30, on a pipe that a fold of 10 grids
+// kept three quarters busy (CT phantom, 10 grids of 1e6 histories: 0.54 ->
+// 0.46 ms).  FP64 division and square root are slow on this part:
+// 1/rho and sqrt() start from FP32 estimates and take one FP64 Newton step
+// each (relative error ~1e-14).
+struct FoldWeights {
+    double xb, xs, qb, qs;     // of the sums over the long batches and over the short ones
+    double k;                  // 1 / (n_b - 1)
+};
+__host__ __device__ __forceinline__ FoldWeights fold_weights(double inv_big, double inv_small, double x_scale,
+                                                             double q_scale, double k) {
+    return FoldWeights{inv_big * x_scale, inv_small * x_scale, inv_big * inv_big * q_scale,
+                       inv_small * inv_small * q_scale, k};
+}
+__device__ __forceinline__ double inverse(float rho) {
+    const double y = double(1.0f / rho);
+    return y * fma(-double(rho), y, 2.0);
 }
 __device__ __forceinline__ double root(double var) {
     if (!(var > 0.0)) return 0.0;
-    double y = double(rsqrtf(float(var)));
-    y = y * fma(-0.5 * var * y, y, 1.5);
-    return var * y;
+    const float y = rsqrtf(float(var));
+    const double g = var * double(y);
+    return fma(g, fma(-g, double(0.5f * y), 0.5), g);
 }
 
 // Sums of a thread's batch tallies b in [b0, b1) at its VPT voxels v,
@@ -161,8 +174,8 @@ __device__ __forceinline__ double root(double var) {
 // loads, which leaves the grids ready for the next calculation.
 // Measured with the finalize work in the same kernel (below) and the metric:
 // CT phantom, 10 grids of one beamlet's 1e5 histories 0.98 -> 0.19 ms; 128^3
-// slab, 100 grids of 1e4 histories each 0.93 -> 0.38 ms; CT plan, 100 grids of
-// 1e6 histories each 3.7 -> 2.6 ms (6.7 GB read).  10 batches at a time (whole
+// slab, 100 grids of 1e4 histories each 0.93 -> 0.37 ms; CT plan, 100 grids of
+// 1e6 histories each 3.7 -> 2.45 ms (6.7 GB read).  10 batches at a time (whole
 // chunks of the usual 10, 20 and 100) at five CTAs per SM were best: 16 at
 // four +9 to +20 %, 20 to 32 at two or three +15 to +60 %.
 template <int VPT, int UB>
@@ -352,10 +365,9 @@ __device__ __forceinline__ void fold_voxels(const SimParams& P, size_t V, size_t
 // parts accumulate in out1, out2.  The grids are left zeroed.
 template <bool FINAL, int VPT, int UB>
 __global__ void __launch_bounds__(kFoldThreads, 5) k_fold_batches(SimParams P, size_t V, int nbatch,
-                                                               double inv_big, double inv_small, int n_big,
+                                                               FoldWeights W, int n_big,
                                                                double* __restrict__ out1,
-                                                               double* __restrict__ out2, double inv_n,
-                                                               double inv_nn1, double dvol,
+                                                               double* __restrict__ out2,
                                                                unsigned long long* dmax_bits,
                                                                float metric_min_rho) {
     __shared__ double s_red[32];
@@ -364,21 +376,22 @@ __global__ void __launch_bounds__(kFoldThreads, 5) k_fold_batches(SimParams P, s
     fold_voxels<VPT, UB>(
         P, V, 0, min(n_big, nbatch), nbatch, L,
         [&](size_t v, double eb, double qb, double es, double qs) {
-            dep += eb + es;
-            const double a1 = fma(eb, inv_big, es * inv_small);
-            const double a2 = fma(qb, inv_big * inv_big, qs * (inv_small * inv_small));
+            double x = es * W.xs, q = qs * W.qs;
+            dep += es;
+            if (n_big > 0) {
+                x = fma(eb, W.xb, x);
+                q = fma(qb, W.qb, q);
+                dep += eb;
+            }
             if (FINAL) {
-                const double mean = a1 * inv_n;
-                const double var = fmax(0.0, (a2 - nbatch * mean * mean) * inv_nn1);
                 const float r = P.rho[v];
-                const double im = inverse_mass(r, dvol);
-                const double d = mean * im;
+                const double ir = inverse(r), d = x * ir;
                 out1[v] = d;
-                out2[v] = root(var) * im;
+                out2[v] = root(fma(-W.k * x, x, q)) * ir;
                 if (r >= metric_min_rho) mx = fmax(mx, d);
             } else {
-                out1[v] += a1;
-                out2[v] += a2;
+                out1[v] += x;
+                out2[v] += q;
             }
         },
         [&](size_t v) {
@@ -405,32 +418,37 @@ __global__ void __launch_bounds__(kFoldThreads, 5) k_fold_batches(SimParams P, s
 // sub-problem k, whose first nbig[k] batches are the long ones.  The grids
 // are left zeroed.  With two batches a thread has only two tallies a voxel to
 // load, so it takes four voxels.  64 beamlets x 2 batches on the 128^3 slab
-// (134M voxels of output, 12 % of them with dose): memset and fold 17 -> 1.9 ms.
+// (134M voxels of output, 12 % of them with dose): memset and fold 17 -> 1.5 ms.
 template <int VPT, int UB>
 __global__ void __launch_bounds__(kFoldThreads) k_fold_sub(SimParams P, size_t V, uint32_t k0, int nb,
                                                            const double* __restrict__ inv_n,
-                                                           const uint32_t* __restrict__ nbig, double dvol,
-                                                           double inv_nb, double inv_nn1,
+                                                           const uint32_t* __restrict__ nbig, double x_scale,
+                                                           double q_scale, double k_sigma,
                                                            double* __restrict__ dose,
                                                            double* __restrict__ sigma) {
     __shared__ double s_red[32];
     __shared__ FoldList L;
     const uint32_t k = k0 + blockIdx.y;
-    const double ib = inv_n[2 * k], is = inv_n[2 * k + 1];
+    const int n_big = int(min(nbig[k], uint32_t(nb)));
+    __shared__ FoldWeights W;      // visible after fold_voxels' first barrier
+    if (threadIdx.x == 0) W = fold_weights(inv_n[2 * k], inv_n[2 * k + 1], x_scale, q_scale, k_sigma);
     const bool with_sigma = sigma && nb > 1;
     double* const dk = dose + size_t(blockIdx.y) * V;
     double* const sk = with_sigma ? sigma + size_t(blockIdx.y) * V : nullptr;
     double dep = 0.0;
     fold_voxels<VPT, UB>(
-        P, V, size_t(k) * nb, int(min(nbig[k], uint32_t(nb))), nb, L,
+        P, V, size_t(k) * nb, n_big, nb, L,
         [&](size_t v, double eb, double qb, double es, double qs) {
-            dep += eb + es;
-            const double a1 = fma(eb, ib, es * is);
-            const double a2 = fma(qb, ib * ib, qs * (is * is));
-            const double im = inverse_mass(P.rho[v], dvol);
-            const double mean = a1 * inv_nb;
-            dk[v] = mean * im;
-            if (with_sigma) sk[v] = root(fmax(0.0, (a2 - nb * mean * mean) * inv_nn1)) * im;
+            double x = es * W.xs, q = qs * W.qs;
+            dep += es;
+            if (n_big > 0) {
+                x = fma(eb, W.xb, x);
+                q = fma(qb, W.qb, q);
+                dep += eb;
+            }
+            const double ir = inverse(P.rho[v]);
+            dk[v] = x * ir;
+            if (with_sigma) sk[v] = root(fma(-W.k * x, x, q)) * ir;
         },
         [&](size_t v) {
             dk[v] = 0.0;
@@ -448,19 +466,17 @@ __global__ void k_finalize(const double* __restrict__ s1, const double* __restri
                            double* __restrict__ dose, double* __restrict__ sigma,
                            unsigned long long* dmax_bits, float metric_min_rho) {
     double mx = 0.0;
-    const double inv_n = 1.0 / nb;
-    const double inv_nn1 = 1.0 / (double(nb) * (nb - 1));
+    const double x_scale = 1.0 / (nb * dvol), q_scale = x_scale / ((nb - 1) * dvol), k = 1.0 / (nb - 1);
     for (size_t v = blockIdx.x * size_t(blockDim.x) + threadIdx.x; v < V;
          v += size_t(gridDim.x) * blockDim.x) {
         const double a1 = s1[v], a2 = s2[v];
         double d = 0.0, sd = 0.0;
         if (a1 != 0.0 || a2 != 0.0) {
-            const double mean = a1 * inv_n;
-            const double var = fmax(0.0, (a2 - nb * mean * mean) * inv_nn1);
+            const double x = a1 * x_scale;
             const float r = rho[v];
-            const double im = inverse_mass(r, dvol);
-            d = mean * im;
-            sd = root(var) * im;
+            const double ir = inverse(r);
+            d = x * ir;
+            sd = root(fma(-k * x, x, a2 * q_scale)) * ir;
             if (r >= metric_min_rho) mx = fmax(mx, d);
         }
         if (dose) dose[v] = d;
@@ -565,8 +581,8 @@ static unsigned fold_grid(gdpm_ctx* ctx, size_t V, int vpt, int ctas_per_sm) {
 int launch_fold_batches(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t V, int n_batches,
                         uint32_t nb_small, uint32_t nb_rem, double* s1, double* s2) {
     k_fold_batches<false, 1, 10><<<fold_grid(ctx, V, 1, 5), kFoldThreads, 0, st>>>(
-        P, V, n_batches, 1.0 / double(nb_small + 1), 1.0 / double(nb_small), int(nb_rem), s1, s2, 0.0,
-        0.0, 0.0, nullptr, 0.f);
+        P, V, n_batches, fold_weights(1.0 / double(nb_small + 1), 1.0 / double(nb_small), 1.0, 1.0, 0.0), int(nb_rem),
+        s1, s2, nullptr, 0.f);
     GDPM_CUDA_TRY(cudaGetLastError());
     return GDPM_OK;
 }
@@ -586,8 +602,10 @@ int launch_fold_final(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t
     const double dvol = double(P.dx) * P.dy * P.dz;
     unsigned long long* dmax_bits = reinterpret_cast<unsigned long long*>(&P.ledger[L_DMAX]);
     k_fold_batches<true, 1, 10><<<fold_grid(ctx, V, 1, 5), kFoldThreads, 0, st>>>(
-        P, V, n_batches, 1.0 / double(nb_small + 1), 1.0 / double(nb_small), int(nb_rem), dose, sigma,
-        1.0 / n_batches, 1.0 / (double(n_batches) * (n_batches - 1)), dvol, dmax_bits, ctx->metric_min_rho);
+        P, V, n_batches,
+        fold_weights(1.0 / double(nb_small + 1), 1.0 / double(nb_small), 1.0 / (n_batches * dvol),
+                     1.0 / (double(n_batches) * (n_batches - 1) * dvol * dvol), 1.0 / (n_batches - 1)),
+        int(nb_rem), dose, sigma, dmax_bits, ctx->metric_min_rho);
     GDPM_CUDA_TRY(cudaGetLastError());
     return launch_metric(ctx, st, P, V, dose, sigma);
 }
@@ -596,11 +614,10 @@ int launch_fold_sub(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t V
                     uint32_t nk, int nb, const double* inv_n, const uint32_t* nbig, double* dose,
                     double* sigma) {
     const double dvol = double(P.dx) * P.dy * P.dz;
-    const double inv_nb = 1.0 / nb, inv_nn1 = nb > 1 ? 1.0 / (double(nb) * (nb - 1)) : 0.0;
+    const double x = 1.0 / (nb * dvol), k = nb > 1 ? 1.0 / (nb - 1) : 0.0, q = x * k / dvol;
     const dim3 grid(fold_grid(ctx, V, 4, 2), nk);   // two CTAs per SM and beamlet: 8 were 6 % slower
-    if (nb <= 4) k_fold_sub<4, 0><<<grid, kFoldThreads, 0, st>>>(P, V, k0, nb, inv_n, nbig, dvol, inv_nb, inv_nn1, dose,
-                                                                 sigma);
-    else k_fold_sub<4, 4><<<grid, kFoldThreads, 0, st>>>(P, V, k0, nb, inv_n, nbig, dvol, inv_nb, inv_nn1, dose, sigma);
+    if (nb <= 4) k_fold_sub<4, 0><<<grid, kFoldThreads, 0, st>>>(P, V, k0, nb, inv_n, nbig, x, q, k, dose, sigma);
+    else k_fold_sub<4, 4><<<grid, kFoldThreads, 0, st>>>(P, V, k0, nb, inv_n, nbig, x, q, k, dose, sigma);
     GDPM_CUDA_TRY(cudaGetLastError());
     return GDPM_OK;
 }

@@ -1015,9 +1015,10 @@ __device__ __forceinline__ void rec_load(const PhRec& r, Part& p) {
 // own loop, as each lane reached them, kept 14 of 32 lanes active; now 27 are.
 // Measured (1e8 histories of the CT plan / 2.5e8 of the paper's lung slab):
 // 22.5 -> 20.6 ms / 36.0 -> 28.1 ms; 160 instead of 225 warp instructions a
-// history.  What is left is the latency of the voxel loads (24 warps) and
-// the round's own control.  New
-// photons come kPhReady at a time into the stack, not one by one as lanes
+// history; with sparser queue reservations, streamed queues and 28 warps (see
+// bank_block, PhaseShape) 142 and 16.8 / 25.2 ms.  Issue slots are then 72 %
+// taken; what a warp waits for is the latency of the voxel loads, two a flight
+// at random voxels, of which 5 % hit the L1 and 75 % the L2.  New photons come kPhReady at a time into the stack, not one by one as lanes
 // fall free.  Both kinds of round start with one draw, at one place in the
 // code: a single inlined copy of the generator, which leaves the loop without
 // calls and its constants in uniform registers.
@@ -1218,9 +1219,15 @@ __device__ __forceinline__ uint32_t el_load(const ElStack& s, uint32_t i, Electr
 // memory; once kElWait wait, an event round gives each of 32 its next draw.
 // In one lane's own loop, as each lane reached them, the draw, walk, candidate
 // and Moller code ran with 14.8 of 32 lanes active and 271 warp instructions
-// a history; now 20 and 205.  Measured against that (1e8 histories of the CT
+// a history; now 20 and 214.  Measured against that (1e8 histories of the CT
 // plan; 2.5e8 of the paper's lung slab; 2.5e6 20 MeV electrons on its bone
-// slab): electron phase 29.6 -> 25.7, 54.8 -> 50.0, 7.0 -> 5.6 ms.
+// slab): electron phase 29.6 -> 25.7, 54.8 -> 50.0, 7.0 -> 5.6 ms; with the
+// constants, ids and hinge directions in shared memory 23.3, 46.2, 5.2 ms.
+// Bound by its instructions (75 % of the issue slots taken).  On the CT plan 27
+// lanes set up a step in a round and 31 start its walk; the hinge runs twice
+// with 14, a crossing twice with 7 and the second stretch once with 10, and 6
+// lanes are refilled.  Running the second stretch only for 6 to 12 lanes or
+// more, or the refill for 2 to 12, was slower by 1 to 10 %.
 template <int GEN>
 __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs& A) {
     extern __shared__ __align__(16) unsigned char smem[];
