@@ -140,15 +140,17 @@ __global__ void __launch_bounds__(256) k_fold(SimParams P, size_t V, double inv_
 // kept three quarters busy (CT phantom, 10 grids of 1e6 histories: 0.54 ->
 // 0.46 ms).  FP64 division and square root are slow on this part:
 // 1/rho and sqrt() start from FP32 estimates and take one FP64 Newton step
-// each (relative error ~1e-14).
+// each (relative error ~1e-14).  The variance is a small difference where all
+// batches dose a voxel alike, so the weights of the squares are made from the
+// rounded weights of the sums.
 struct FoldWeights {
     double xb, xs, qb, qs;     // of the sums over the long batches and over the short ones
     double k;                  // 1 / (n_b - 1)
 };
 __host__ __device__ __forceinline__ FoldWeights fold_weights(double inv_big, double inv_small, double x_scale,
-                                                             double q_scale, double k) {
-    return FoldWeights{inv_big * x_scale, inv_small * x_scale, inv_big * inv_big * q_scale,
-                       inv_small * inv_small * q_scale, k};
+                                                             double nb_k, double k) {
+    const double xb = inv_big * x_scale, xs = inv_small * x_scale;
+    return FoldWeights{xb, xs, xb * xb * nb_k, xs * xs * nb_k, k};
 }
 __device__ __forceinline__ double inverse(float rho) {
     const double y = double(1.0f / rho);
@@ -423,15 +425,14 @@ template <int VPT, int UB>
 __global__ void __launch_bounds__(kFoldThreads) k_fold_sub(SimParams P, size_t V, uint32_t k0, int nb,
                                                            const double* __restrict__ inv_n,
                                                            const uint32_t* __restrict__ nbig, double x_scale,
-                                                           double q_scale, double k_sigma,
-                                                           double* __restrict__ dose,
+                                                           double k_sigma, double* __restrict__ dose,
                                                            double* __restrict__ sigma) {
     __shared__ double s_red[32];
     __shared__ FoldList L;
     const uint32_t k = k0 + blockIdx.y;
     const int n_big = int(min(nbig[k], uint32_t(nb)));
     __shared__ FoldWeights W;      // visible after fold_voxels' first barrier
-    if (threadIdx.x == 0) W = fold_weights(inv_n[2 * k], inv_n[2 * k + 1], x_scale, q_scale, k_sigma);
+    if (threadIdx.x == 0) W = fold_weights(inv_n[2 * k], inv_n[2 * k + 1], x_scale, nb * k_sigma, k_sigma);
     const bool with_sigma = sigma && nb > 1;
     double* const dk = dose + size_t(blockIdx.y) * V;
     double* const sk = with_sigma ? sigma + size_t(blockIdx.y) * V : nullptr;
@@ -466,7 +467,7 @@ __global__ void k_finalize(const double* __restrict__ s1, const double* __restri
                            double* __restrict__ dose, double* __restrict__ sigma,
                            unsigned long long* dmax_bits, float metric_min_rho) {
     double mx = 0.0;
-    const double x_scale = 1.0 / (nb * dvol), q_scale = x_scale / ((nb - 1) * dvol), k = 1.0 / (nb - 1);
+    const double x_scale = 1.0 / (nb * dvol), k = 1.0 / (nb - 1), q_scale = x_scale * x_scale * (nb * k);
     for (size_t v = blockIdx.x * size_t(blockDim.x) + threadIdx.x; v < V;
          v += size_t(gridDim.x) * blockDim.x) {
         const double a1 = s1[v], a2 = s2[v];
@@ -601,10 +602,10 @@ int launch_fold_final(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t
                       uint32_t nb_small, uint32_t nb_rem, double* dose, double* sigma) {
     const double dvol = double(P.dx) * P.dy * P.dz;
     unsigned long long* dmax_bits = reinterpret_cast<unsigned long long*>(&P.ledger[L_DMAX]);
+    const double k = 1.0 / (n_batches - 1);
     k_fold_batches<true, 1, 10><<<fold_grid(ctx, V, 1, 5), kFoldThreads, 0, st>>>(
         P, V, n_batches,
-        fold_weights(1.0 / double(nb_small + 1), 1.0 / double(nb_small), 1.0 / (n_batches * dvol),
-                     1.0 / (double(n_batches) * (n_batches - 1) * dvol * dvol), 1.0 / (n_batches - 1)),
+        fold_weights(1.0 / double(nb_small + 1), 1.0 / double(nb_small), 1.0 / (n_batches * dvol), n_batches * k, k),
         int(nb_rem), dose, sigma, dmax_bits, ctx->metric_min_rho);
     GDPM_CUDA_TRY(cudaGetLastError());
     return launch_metric(ctx, st, P, V, dose, sigma);
@@ -614,10 +615,10 @@ int launch_fold_sub(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t V
                     uint32_t nk, int nb, const double* inv_n, const uint32_t* nbig, double* dose,
                     double* sigma) {
     const double dvol = double(P.dx) * P.dy * P.dz;
-    const double x = 1.0 / (nb * dvol), k = nb > 1 ? 1.0 / (nb - 1) : 0.0, q = x * k / dvol;
+    const double x = 1.0 / (nb * dvol), k = nb > 1 ? 1.0 / (nb - 1) : 0.0;
     const dim3 grid(fold_grid(ctx, V, 4, 2), nk);   // two CTAs per SM and beamlet: 8 were 6 % slower
-    if (nb <= 4) k_fold_sub<4, 0><<<grid, kFoldThreads, 0, st>>>(P, V, k0, nb, inv_n, nbig, x, q, k, dose, sigma);
-    else k_fold_sub<4, 4><<<grid, kFoldThreads, 0, st>>>(P, V, k0, nb, inv_n, nbig, x, q, k, dose, sigma);
+    if (nb <= 4) k_fold_sub<4, 0><<<grid, kFoldThreads, 0, st>>>(P, V, k0, nb, inv_n, nbig, x, k, dose, sigma);
+    else k_fold_sub<4, 4><<<grid, kFoldThreads, 0, st>>>(P, V, k0, nb, inv_n, nbig, x, k, dose, sigma);
     GDPM_CUDA_TRY(cudaGetLastError());
     return GDPM_OK;
 }
