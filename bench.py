@@ -102,10 +102,10 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 # traffic is null.
 TRAFFIC_SOURCES = ("transport.cu", "common.cuh", "internal.h")
 TRAFFIC = {
-    # profiles/dram_k_phase_ct256_imrt7_2e6hist.md: 2e6 histories, 10 batches
-    # side by side, 4 launches of each phase kernel
-    "ct256_imrt7": {"tally": "fp64", "sha1": "31312f47325a5bfd8a40fe10bd545f4941ec33d6",
-                    "bytes_per_history": {"electron phase": 338.9, "photon phase": 337.5}},
+    # profiles/k_phase_ct256_imrt7_1e7hist.md: 1e7 histories, 10 batches side
+    # by side, 4 launches of each phase kernel
+    "ct256_imrt7": {"tally": "fp64", "sha1": "735ad6ac81a35a179ad30b6ef94a3a5d23da00e3",
+                    "bytes_per_history": {"electron phase": 177.2, "photon phase": 189.0}},
 }
 
 
@@ -145,7 +145,7 @@ def parse():
                     help="dose tally: FP64 atomics, or FP32 hi/lo compensated pairs")
     ap.add_argument("--electron-walk", type=int, default=None, choices=[0, 1],
                     help="electron phase form (GDPM_PARAM_ELECTRON_WALK): 1 resumable steps "
-                         "(the library's default), 0 a whole step per loop iteration")
+                         "(the library's default), 0 a whole step per round")
     ap.add_argument("--autotune-ms", type=float, default=0.0,
                     help="run gdpm_autotune on the step's calculation for this wall-clock "
                          "budget before the warm-up, and time the configuration it sets")

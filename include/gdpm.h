@@ -161,7 +161,7 @@ enum {
     GDPM_PARAM_QUEUE_CAPACITY = 1,   /* particles per queue buffer (0 = automatic), <= 2^31 */
     GDPM_PARAM_BLOCK_THREADS = 2,    /* threads per block of every transport phase kernel:
                                         64..256, multiple of 32; 0 (default): each kernel's
-                                        own shape (256; 448 for resumable electron steps) */
+                                        own shape (768; 896 for large photon phases) */
     GDPM_PARAM_BLOCKS_PER_SM = 3,    /* persistent CTAs per SM (0 = occupancy) */
     GDPM_PARAM_TALLY_MODE = 4,       /* 0: FP64 atomics; 1: FP32 compensated hi/lo pair */
     GDPM_PARAM_SOURCE_CHUNK = 5,     /* max primaries per transport phase (0 = auto), <= 2^28 */
