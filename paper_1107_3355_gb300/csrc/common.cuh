@@ -201,6 +201,16 @@ __device__ __forceinline__ void source_load(const Queue& q, uint32_t s, Part& p)
     p.pidlo = 1u; p.pidhi = 0u; p.ctr = 1u;
 }
 
+// ---------------------------------------------------------------- Metropolis chains
+// Most steps a chain takes when C chains share n consecutive histories, and
+// the tiles of `tile` steps they fill.  Quotients first: n may reach 2^32 - 1
+// and C 2^24, so rounding up by adding to n would wrap.
+__host__ __device__ __forceinline__ uint32_t chain_steps(uint32_t n, uint32_t C) { return n / C + (n % C != 0u); }
+__host__ __device__ __forceinline__ uint32_t chain_tiles(uint32_t n, uint32_t C, uint32_t tile) {
+    const uint32_t most = chain_steps(n, C);
+    return most / tile + (most % tile != 0u);
+}
+
 // ---------------------------------------------------------------- geometry
 // Rotate (u,v,w) by polar cosine `cost` and azimuth phi given as (cp, sp).
 // Azimuth reference: e1 = (u w, v w, -(1-w^2))/s, e2 = (-v, u, 0)/s with

@@ -1559,7 +1559,7 @@ __device__ __forceinline__ void metropolis_run(const SimParams& P, uint32_t firs
     // the chain's first history of the range, and how many it has there
     const uint64_t h0 = uint64_t(first) + (uint64_t(c) + C - first % C) % C;
     const uint32_t steps = c < C && h0 < end ? uint32_t((end - 1u - h0) / C) + 1u : 0u;
-    const uint32_t most = (n + C - 1u) / C, tiles = (most + kMetroTile - 1u) / kMetroTile;
+    const uint32_t tiles = chain_tiles(n, C, kMetroTile);
     auto propose = [&](uint32_t t) {
         for (uint32_t j = warp - 1u; j < uint32_t(kMetroTile); j += kMetroThreads / 32 - 1) {
             const uint32_t step = t * kMetroTile + j;
