@@ -1861,7 +1861,11 @@ static int run_chains(Runner& r, const SimParams& P, uint64_t n_hist) {
         return rc;
     uint32_t* chains = static_cast<uint32_t*>(r.ws.chains.p);
     if ((rc = launch_metropolis_init(r.stream, P, chains))) return rc;
-    return launch_metropolis(r.stream, P, 0, uint32_t(n_hist), chains, static_cast<uint32_t*>(r.ws.pick.p));
+    // in two launches: n_hist may be 2^32, one more than a launch's count holds
+    uint32_t* pick = static_cast<uint32_t*>(r.ws.pick.p);
+    const uint32_t half = uint32_t(n_hist / 2);
+    if (half && (rc = launch_metropolis(r.stream, P, 0, half, chains, pick))) return rc;
+    return launch_metropolis(r.stream, P, half, uint32_t(n_hist - half), chains, pick + half);
 }
 
 int gdpm_debug_beamlets(gdpm_ctx* ctx, uint64_t first, uint64_t n, int32_t* out) {
@@ -1880,7 +1884,7 @@ int gdpm_debug_beamlets(gdpm_ctx* ctx, uint64_t first, uint64_t n, int32_t* out)
     if ((rc = run_chains(r, P, first + n))) return rc;
     const uint32_t* pick = P.S.sampler == GDPM_SAMPLE_METROPOLIS ? static_cast<const uint32_t*>(r.ws.pick.p) + first
                                                                   : nullptr;
-    if ((rc = launch_debug_beamlets(r.stream, P, uint32_t(first), uint32_t(n), pick, out))) return rc;
+    if ((rc = launch_debug_beamlets(r.stream, P, uint32_t(first), n, pick, out))) return rc;
     GDPM_CUDA_TRY(cudaStreamSynchronize(r.stream));
     return GDPM_OK;
 }

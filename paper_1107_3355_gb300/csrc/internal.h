@@ -247,7 +247,7 @@ int build_loop_graph(gdpm_ctx* ctx, const SimParams& P, LoopArgs& L, bool metrop
                      cudaGraph_t* graph, cudaGraphExec_t* exec);
 int launch_metropolis(cudaStream_t st, const SimParams& P, uint32_t first, uint32_t n,
                       uint32_t* chains, uint32_t* pick);
-int launch_debug_beamlets(cudaStream_t st, const SimParams& P, uint32_t first, uint32_t n,
+int launch_debug_beamlets(cudaStream_t st, const SimParams& P, uint32_t first, uint64_t n,
                           const uint32_t* pick, int32_t* out);
 int launch_fold_sub(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, size_t V, uint32_t k0,
                     uint32_t nk, int nb, const double* inv_n, const uint32_t* nbig, double* dose,

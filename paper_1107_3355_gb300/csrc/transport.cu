@@ -1774,16 +1774,16 @@ __global__ void __launch_bounds__(kMetroThreads) k_metropolis(const SimParams P,
 }
 
 // Beamlet rows of histories [first, first+n) (checks of the samplers).
-__global__ void k_debug_beamlets(const SimParams P, uint32_t first, uint32_t n,
+__global__ void k_debug_beamlets(const SimParams P, uint32_t first, uint64_t n,
                                  const uint32_t* pick, int32_t* out) {
-    for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
+    for (uint64_t s = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; s < n; s += uint64_t(gridDim.x) * blockDim.x) {
         Part p{};
-        p.hist = first + s;
+        p.hist = first + uint32_t(s);
         p.pidlo = 1u;
         const float4 r = draw(p, P.key0, P.key1);
         PhaseArgs A{};
         A.bl_pick = pick;
-        out[s] = P.S.bl_row[pick_beamlet(P.S, A, s, first + s, r.w, P.key0, P.key1, P.S.bl_cdf)];
+        out[s] = P.S.bl_row[pick_beamlet(P.S, A, uint32_t(s), first + uint32_t(s), r.w, P.key0, P.key1, P.S.bl_cdf)];
     }
 }
 
@@ -2081,9 +2081,9 @@ int launch_metropolis(cudaStream_t st, const SimParams& P, uint32_t first, uint3
     return GDPM_OK;
 }
 
-int launch_debug_beamlets(cudaStream_t st, const SimParams& P, uint32_t first, uint32_t n,
+int launch_debug_beamlets(cudaStream_t st, const SimParams& P, uint32_t first, uint64_t n,
                           const uint32_t* pick, int32_t* out) {
-    const uint32_t grid = std::max(1u, std::min(1024u, (n + 255) / 256));
+    const uint32_t grid = uint32_t(std::min<uint64_t>(1024u, (n + 255) / 256));
     k_debug_beamlets<<<grid, 256, 0, st>>>(P, first, n, pick, out);
     GDPM_CUDA_TRY(cudaGetLastError());
     return GDPM_OK;

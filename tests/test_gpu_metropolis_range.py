@@ -37,3 +37,12 @@ def test_picks_at_the_end_of_the_range(chains, end):
     prob = problem(chains)
     n = 2000
     assert np.array_equal(picks(prob, end - n, n), O.beamlet_picks(prob, end - n, n))
+
+
+# the last history id there is, one more than a launch's 32-bit count reaches
+@pytest.mark.parametrize("sampler", ["metropolis", "alias"])
+def test_picks_up_to_the_last_history_id(sampler):
+    prob = problem(2 ** 20)
+    prob.source.sampler = sampler
+    n = 300
+    assert np.array_equal(picks(prob, 2 ** 32 - n, n), O.beamlet_picks(prob, 2 ** 32 - n, n))
