@@ -1377,7 +1377,8 @@ int gdpm_simulate_part(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb, uint64_
     const gdpm_source_state& src = ctx->src;
     int rc = validate_run(ctx, ph, tb, src, n_histories, n_batches);
     if (rc) return rc;
-    if (first_batch < 0 || n_part < 1 || first_batch + n_part > n_batches || n_part > kMaxConcurrentBatches)
+    if (first_batch < 0 || n_part < 1 || n_part > n_batches || first_batch > n_batches - n_part ||
+        n_part > kMaxConcurrentBatches)
         return GDPM_E_ARG;
     GDPM_CUDA_TRY(cudaSetDevice(ctx->device));
     Runner& r = ctx->run;
@@ -1872,7 +1873,7 @@ int gdpm_debug_beamlets(gdpm_ctx* ctx, uint64_t first, uint64_t n, int32_t* out)
     if (!ctx) return GDPM_E_ARG;
     if (!ctx->src.set) return GDPM_E_STATE;
     if (ctx->src.desc.geometry != GDPM_GEO_BEAMLETS || !out || !is_device_ptr(out) ||
-        first + n > (1ull << 32) || n == 0)
+        n > (1ull << 32) || first > (1ull << 32) - n || n == 0)
         return GDPM_E_ARG;
     GDPM_CUDA_TRY(cudaSetDevice(ctx->device));
     Runner& r = ctx->run;
@@ -1895,7 +1896,7 @@ int gdpm_debug_sources(gdpm_ctx* ctx, gdpm_phantom* ph, gdpm_tables* tb, uint64_
     int rc = validate_run(ctx, ph, tb, ctx->src, n_histories, n_batches);
     if (rc) return rc;
     const uint64_t nb0 = n_histories / n_batches + (n_histories % n_batches ? 1 : 0);
-    if (!out || !is_device_ptr(out) || first + n > nb0) return GDPM_E_ARG;
+    if (!out || !is_device_ptr(out) || n > nb0 || first > nb0 - n) return GDPM_E_ARG;
     Runner& r = ctx->run;
     const int n_bins = int(ctx->src.weights.size());
     std::vector<uint32_t> prefix(n_bins + 1);
