@@ -18,11 +18,14 @@ struct gdpm_source_state;   // a context's source (below)
 
 namespace gdpm {
 
+// The runtime's own record of the error is cleared: left there, it would fail
+// the next call of this thread at its first launch check.
 #define GDPM_CUDA_TRY(expr)                                   \
     do {                                                      \
         cudaError_t _e = (expr);                              \
         if (_e != cudaSuccess) {                              \
             last_cuda_error() = _e;                           \
+            cudaGetLastError();                               \
             return GDPM_E_CUDA;                               \
         }                                                     \
     } while (0)
