@@ -1841,7 +1841,8 @@ int transport_smem(const gdpm_tables* t, int particle) { return int(tables_smem(
 // A phase kernel's launch shape: its own CTA, or the context's
 // GDPM_PARAM_BLOCK_THREADS when set (at most 256, within every kernel's
 // bound); the tables and counters of a CTA and the warps' stacks in shared
-// memory.  Beside large tables a CTA has fewer warps.
+// memory.  Beside large tables a CTA has fewer warps.  fixed_smem: shared
+// memory the kernel declares itself, which counts towards the same limit.
 constexpr size_t kMaxSmem = size_t(227) << 10;
 // A photon phase that starts fewer than kWideItems histories per thread (the
 // later generations among them) runs narrow: its last rounds, which few lanes
@@ -1855,13 +1856,13 @@ struct Launch {
     int threads;
     size_t smem;
 };
-static Launch phase_shape(const gdpm_ctx* ctx, const DevTables& T, int pt, bool narrow) {
+static Launch phase_shape(const gdpm_ctx* ctx, const DevTables& T, int pt, bool narrow, size_t fixed_smem = 0) {
     const size_t tables = smem_of(T, pt == 0 ? GDPM_PHOTON : GDPM_ELECTRON);
     const size_t stack = pt == 0 ? kPhStack * sizeof(PhRec) : sizeof(ElStack);
     int thr = ctx->block_threads > 0 ? ctx->block_threads
               : pt == 0              ? (narrow ? kNarrowThreads : PhaseShape<0>::threads)
                                      : PhaseShape<1>::threads;
-    thr = std::min(thr, 32 * int((kMaxSmem - tables) / stack));
+    thr = std::min(thr, 32 * int((kMaxSmem - fixed_smem - tables) / stack));
     return Launch{thr, tables + stack * size_t(thr / 32)};
 }
 
@@ -1969,7 +1970,9 @@ int build_loop_graph(gdpm_ctx* ctx, const SimParams& P, LoopArgs& L, bool metrop
     int thr[2];
     uint64_t warps = 0;
     for (int t = 0; t < 2; ++t) {
-        const Launch shape = phase_shape(ctx, P.T, t, false);
+        cudaFuncAttributes attr{};             // the arguments k_phase_loop derives in shared memory
+        GDPM_CUDA_TRY(cudaFuncGetAttributes(&attr, fn[t]));
+        const Launch shape = phase_shape(ctx, P.T, t, false, attr.sharedSizeBytes);
         thr[t] = shape.threads;
         smem[t] = shape.smem;
         GDPM_CUDA_TRY(cudaFuncSetAttribute(fn[t], cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem[t])));
