@@ -1521,7 +1521,9 @@ inline uint32_t cdf_entries(const SimParams& P, const PhaseArgs& A) {
 }
 
 // Entries of the prefix and cumulative-weight tables a source CTA stages in
-// shared memory (0: read from global memory), within a 40 KB budget.
+// shared memory (0: read from global memory), within a 40 KB budget: below the
+// 48 KB any launch may ask for, so no launch sets a limit that another host
+// thread's launch of the same kernel would run into.
 __host__ __device__ inline void sources_smem(uint32_t prefix_entries, uint32_t cdf_entries,
                                              uint32_t& n_prefix, uint32_t& n_cdf) {
     const size_t budget = 40u << 10;
@@ -2034,7 +2036,6 @@ int build_loop_graph(gdpm_ctx* ctx, const SimParams& P, LoopArgs& L, bool metrop
         uint32_t sg, sthr;
         source_shape(ctx, L.chunk, sg, sthr);
         const void* sf = L.src_particle == GDPM_PHOTON ? (const void*)k_sources_loop<0> : (const void*)k_sources_loop<1>;
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(sf, cudaFuncAttributeMaxDynamicSharedMemorySize, int(src_sm));
         add(sf, dim3(sg), dim3(sthr), src_sm, src_args_v);
     }
     add(fn[0], dim3(grid[0]), dim3(thr[0]), smem[0], phase_args_v);
@@ -2060,10 +2061,8 @@ int launch_sources(gdpm_ctx* ctx, cudaStream_t st, const SimParams& P, const Pha
     sources_smem(A.prefix_n, cdf_entries(P, A), np, nc);
     const size_t sm = size_t(nc) * 4 + size_t(np) * 4;
     if (P.S.particle == GDPM_PHOTON) {
-        GDPM_CUDA_TRY(cudaFuncSetAttribute(k_sources<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm)));
         k_sources<0><<<grid, threads, sm, st>>>(P, A, np, nc);
     } else {
-        GDPM_CUDA_TRY(cudaFuncSetAttribute(k_sources<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm)));
         k_sources<1><<<grid, threads, sm, st>>>(P, A, np, nc);
     }
     GDPM_CUDA_TRY(cudaGetLastError());
