@@ -1977,7 +1977,9 @@ int build_loop_graph(gdpm_ctx* ctx, const SimParams& P, LoopArgs& L, bool metrop
         const Launch shape = phase_shape(ctx, P.T, t, false, attr.sharedSizeBytes);
         thr[t] = shape.threads;
         smem[t] = shape.smem;
-        GDPM_CUDA_TRY(cudaFuncSetAttribute(fn[t], cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem[t])));
+        // one limit for every context's graph, as in launch_phase
+        GDPM_CUDA_TRY(cudaFuncSetAttribute(fn[t], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           int(kMaxSmem - attr.sharedSizeBytes)));
         int bps = ctx->blocks_per_sm;
         if (bps <= 0) {
             GDPM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn[t], thr[t], smem[t]));

@@ -38,3 +38,31 @@ def test_threads_with_small_and_large_source_tables():
         t.join()
     assert not failed
     assert len(counts[0]) == 1 and len(counts[1]) == 1
+
+
+def test_threads_building_graphs_beside_small_and_large_tables():
+    """The graph loop's kernels, whose shared memory grows with the tables."""
+    base = W.slab_electron_problem(n_histories=500, n_batches=2, shape=(16, 16, 32))
+    failed, counts = [], {32: set(), 2048: set()}
+
+    def work(n_energy):
+        try:
+            # small blocks: the tables are most of a CTA's shared memory
+            eng = G.Engine(base.with_(n_energy=n_energy), params={G.GDPM_PARAM_GRAPH: 1, G.GDPM_PARAM_BLOCK_THREADS: 64})
+            try:
+                for k in range(150):
+                    # another walk form is another graph
+                    G.gdpm_set_param(eng.ctx, G.GDPM_PARAM_ELECTRON_WALK, k % 2)
+                    counts[n_energy].add(eng.run()[2]["el_steps"])
+            finally:
+                eng.close()
+        except Exception as e:
+            failed.append((n_energy, repr(e)))
+
+    threads = [threading.Thread(target=work, args=(n,)) for n in (32, 2048, 32)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed
+    assert all(len(c) == 1 for c in counts.values())
