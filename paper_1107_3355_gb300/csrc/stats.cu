@@ -156,11 +156,17 @@ __device__ __forceinline__ double inverse(float rho) {
     const double y = double(1.0f / rho);
     return y * fma(-double(rho), y, 2.0);
 }
+// The estimate is taken of the variance's mantissa times 1 or 2 and the result
+// given half the exponent, with integers: the variance itself, in MeV^2 per
+// cm^6, leaves FP32's range where voxels are large and deposits small.
 __device__ __forceinline__ double root(double var) {
-    if (!(var > 0.0)) return 0.0;
-    const float y = rsqrtf(float(var));
-    const double g = var * double(y);
-    return fma(g, fma(-g, double(0.5f * y), 0.5), g);
+    const int hi = __double2hiint(var);
+    if (hi < 0x00100000 || hi >= 0x7ff00000) return 0.0;   // negative, zero or subnormal, not finite
+    const int e = ((hi >> 20) - 1023) & ~1;
+    const double m = __hiloint2double(hi - e * (1 << 20), __double2loint(var));   // var = m 2^e, m in [1, 4)
+    const float y = rsqrtf(float(m));
+    const double g = m * double(y), r = fma(g, fma(-g, double(0.5f * y), 0.5), g);
+    return __hiloint2double(__double2hiint(r) + (e / 2) * (1 << 20), __double2loint(r));
 }
 
 // Sums of a thread's batch tallies b in [b0, b1) at its VPT voxels v,
