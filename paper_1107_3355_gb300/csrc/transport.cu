@@ -499,11 +499,16 @@ struct __align__(16) ElMat {      // a material's constants of a step (shared me
     float r_eabs, inv_sigmax, rinv_lo, rinv_idr, inv_x0, sigmax, pad[2];
 };
 struct ElSmem {
-    const float4* el;
+    const float4* el;       // in shared memory, or in global memory (FAR)
     const float* rinv;
     const float* atab;
     const ElMat* mat;
 };
+// Entry i of the step and event table.
+template <bool FAR>
+__device__ __forceinline__ float4 el_entry(const ElSmem& S, int i) {
+    return FAR ? __ldg(S.el + i) : S.el[i];
+}
 
 // An electron or positron in a lane: its voxel is packed (10 bits an axis),
 // pend is energy it owes to that voxel and has not tallied yet.
@@ -556,7 +561,7 @@ __device__ __forceinline__ Round absorb(const SimParams& P, Electron& p, uint32_
 
 // Set up a step with the draw x: step limits as mass thickness in the start
 // voxel's material (`mat`), energy at its end, deflection at the random hinge.
-template <int GEN>
+template <int GEN, bool FAR>
 __device__ __forceinline__ void electron_setup(const SimParams& P, const ElSmem& S, const Electron& p, uint4 x,
                                                int mat, ElStep& st, float4& hinge) {
     const DevTables& T = P.T;
@@ -567,7 +572,7 @@ __device__ __forceinline__ void electron_setup(const SimParams& P, const ElSmem&
     float f;
     grid_pos(T, p.E, i, f);
     const int mi = m * T.n_e + i;
-    const float4 a0 = S.el[mi], a1 = S.el[mi + 1];
+    const float4 a0 = el_entry<FAR>(S, mi), a1 = el_entry<FAR>(S, mi + 1);
     const float R0 = lerpf(a0.x, a1.x, f);
     const float xms = lerpf(a0.y, a1.y, f);
     const ElMat M = S.mat[m];
@@ -716,12 +721,12 @@ constexpr int kDrainedStretches = 16;
 // A lane's round: set up a step when none is in progress (`starts`, with the
 // draw x), walk, and at the step's end escape, be absorbed, or wait for the
 // hard-event candidate.
-template <int GEN>
+template <int GEN, bool FAR>
 __device__ __forceinline__ Round electron_round(const SimParams& P, const ElSmem& S, Electron& p, ElStep& st,
                                                 uint4 x, int mat, float4& hinge, int stretches, double& esc,
                                                 uint32_t& crossings, uint32_t& kind) {
     if ((st.what & 3u) == 0u) {
-        electron_setup<GEN>(P, S, p, x, mat, st, hinge);
+        electron_setup<GEN, FAR>(P, S, p, x, mat, st, hinge);
     }
     Walk k;
     k.lin = vox_linear(P, p.vox);
@@ -760,7 +765,7 @@ __device__ __forceinline__ Round electron_round(const SimParams& P, const ElSmem
 // one rejection trial per draw (`force` accepts any); a positron at rest
 // annihilates.  Returns go when the particle takes its next step, wait when
 // it needs another draw, ended at the end of its track.
-template <int GEN>
+template <int GEN, bool FAR>
 __device__ __forceinline__ Round electron_event(const SimParams& P, const ElSmem& S, Electron& p, uint32_t& kind,
                                                 uint4 x, bool force, Sec& sec) {
     const DevTables& T = P.T;
@@ -777,7 +782,7 @@ __device__ __forceinline__ Round electron_event(const SimParams& P, const ElSmem
             float f;
             grid_pos(T, Tn, i, f);
             const int mj = m * T.n_e + i;
-            const float4 a0 = S.el[mj], a1 = S.el[mj + 1];
+            const float4 a0 = el_entry<FAR>(S, mj), a1 = el_entry<FAR>(S, mj + 1);
             if (Tn > 2.f * wcc) sm = lerpf(a0.z, a1.z, f);
             if (Tn > wcb) sb = lerpf(a0.w, a1.w, f);
         }
@@ -1196,8 +1201,7 @@ struct ElStack {
     // electron; direction after the hinge and mass thickness of leg 2.  1e8 CT
     // histories: electron phases 24.0 -> 23.3 ms, lung slab 47.1 -> 46.2.  The
     // KB a warp leaves room for 24 warps beside 58 KB of tables (4 materials
-    // of 512 energies take 53); beside 8 materials' 103 KB 17 run and 1e6
-    // 20 MeV electrons take 4.19 instead of 4.01 ms.
+    // of 512 energies take 53); beside more see kFarWarps.
     uint4 ids[32];
     float4 hinge[32];
 };
@@ -1235,17 +1239,18 @@ __device__ __forceinline__ uint32_t el_load(const ElStack& s, uint32_t i, Electr
 // with 14, a crossing twice with 7 and the second stretch once with 10, and 6
 // lanes are refilled.  Running the second stretch only for 6 to 12 lanes or
 // more, or the refill for 2 to 12, was slower by 1 to 10 %.
-template <int GEN>
+template <int GEN, bool FAR>
 __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs& A) {
     extern __shared__ __align__(16) unsigned char smem[];
     next_may_start();
     const DevTables& T = P.T;
     const size_t ne = size_t(T.n_mat) * T.n_e;
     float4* el = reinterpret_cast<float4*>(smem);
-    float* rinv = reinterpret_cast<float*>(smem + ne * 16);
+    const size_t el_bytes = FAR ? 0 : ne * 16;
+    float* rinv = reinterpret_cast<float*>(smem + el_bytes);
     const size_t nr = size_t(T.n_mat) * T.n_r;
-    float* atab = reinterpret_cast<float*>(smem + ne * 16 + align16(nr * 4));
-    unsigned char* after = smem + ne * 16 + align16(nr * 4) + align16(size_t(T.n_a) * 4);
+    float* atab = reinterpret_cast<float*>(smem + el_bytes + align16(nr * 4));
+    unsigned char* after = smem + el_bytes + align16(nr * 4) + align16(size_t(T.n_a) * 4);
     uint32_t* s_cnt = reinterpret_cast<uint32_t*>(after);
     ElMat* mats = reinterpret_cast<ElMat*>(after + align16(C_NCOUNT * 4));
     ElStack& stack = reinterpret_cast<ElStack*>(mats + kMaxMat)[threadIdx.x >> 5];
@@ -1254,10 +1259,10 @@ __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs
         mats[m] = ElMat{T.r_eabs[m], T.inv_sigmax[m], T.rinv_lo[m], T.rinv_idr[m], T.inv_x0[m], T.sigmax[m]};
     }
     if (lane_id() < 4u) (&stack.held[0].base)[lane_id()] = 0u;
-    copy_to_smem(el, T.el, ne * 16);
+    if (!FAR) copy_to_smem(el, T.el, ne * 16);
     copy_to_smem(rinv, T.rinv, nr * 4);
     copy_to_smem(atab, T.atab, size_t(T.n_a) * 4);
-    const ElSmem es{el, rinv, atab, mats};
+    const ElSmem es{FAR ? T.el : el, rinv, atab, mats};
     for (int k = threadIdx.x; k < C_NCOUNT; k += blockDim.x) s_cnt[k] = 0u;
     wait_for_previous();
     __syncthreads();
@@ -1364,7 +1369,7 @@ __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs
             if (active) {
                 if ((st.what & 3u) == 0u) stack.ids[lane].w = c.w + 1u;
                 p.hist = c.x;
-                what = electron_round<GEN>(P, es, p, st, x, mat, stack.hinge[lane],
+                what = electron_round<GEN, FAR>(P, es, p, st, x, mat, stack.hinge[lane],
                                            drained ? max(P.walk_trips, kDrainedStretches) : P.walk_trips, esc,
                                            crossings, kind);
                 active = what == Round::go;
@@ -1388,7 +1393,7 @@ __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs
             Round what = Round::ended;
             if (lane < k) {
                 was = kind = el_load(stack, top, q);
-                what = electron_event<GEN>(P, es, q, kind, x, draws > 4096u, sec);
+                what = electron_event<GEN, FAR>(P, es, q, kind, x, draws > 4096u, sec);
             }
             n_wait -= k;
             if (__any_sync(kFull, sec.n > 0)) {
@@ -1432,11 +1437,11 @@ __device__ __forceinline__ void electron_run(const SimParams& P, const PhaseArgs
 }
 
 // One transport phase (Sec. 2.2.1 Step 3), a persistent loop per warp.  PT: 0
-// photons, 1 electrons.
+// photons, 1 electrons, 2 electrons beside large tables (kFarWarps).
 template <int PT, int GEN>
 __device__ __forceinline__ void phase_run(const SimParams& P, const PhaseArgs& A) {
     if constexpr (PT == 0) photon_run<GEN>(P, A);
-    else electron_run<GEN>(P, A);
+    else electron_run<GEN, PT == 2>(P, A);
 }
 
 template <int PT, int GEN>
@@ -1813,8 +1818,12 @@ static size_t tables_smem(const DevTables& T, int particle) {
         return align16(ne * 8) + align16(ne * 4) + align16(size_t(T.n_e) * 4) + cnt;
     return ne * 16 + align16(size_t(T.n_mat) * T.n_r * 4) + align16(size_t(T.n_a) * 4) + cnt;
 }
-static size_t smem_of(const DevTables& T, int particle) {
-    return tables_smem(T, particle) + (particle == GDPM_PHOTON ? 0 : kMaxMat * sizeof(ElMat));
+// pt: 0 photons, 1 electrons, 2 electrons with the step and event table left
+// in global memory.
+static size_t smem_of(const DevTables& T, int pt) {
+    if (pt == 0) return tables_smem(T, GDPM_PHOTON);
+    const size_t el = pt == 2 ? size_t(T.n_mat) * T.n_e * 16 : 0;
+    return tables_smem(T, GDPM_ELECTRON) + kMaxMat * sizeof(ElMat) - el;
 }
 
 // log2 of at least twice the warps of a phase: items >> shift is at most half
@@ -1854,18 +1863,32 @@ constexpr size_t kMaxSmem = size_t(227) << 10;
 // 2.11 and 2.03, 3.3e7 lung photons 7 % less at 896.
 constexpr int kNarrowThreads = std::min(768, PhaseShape<0>::threads);
 constexpr uint64_t kWideItems = 64u;
+// Beside large tables the electrons' step and event table, two thirds of
+// theirs, stays in global memory (PT 2) and is read through the L1, so that
+// the warps' stacks find room.  Staged, it leaves 24 warps a CTA beside 4
+// materials of 512 energies, 18 beside 8, 11 beside 4 of 1500 and 4 beside the
+// largest tables (8 of 1024); in global memory 24, 24, 24 and 22.  The line
+// is where the two cost the same (staged -> global; 5e6 histories of the CT
+// plan, 5e6 photons and 3e5 20 MeV electrons on 128^3): 24 warps 3.67 -> 3.70,
+// 2.66 -> 2.69, 1.90 -> 1.92 ms; 20 warps 3.76 -> 3.73, 2.75 -> 2.71, 1.89 ->
+// 1.95; 18 warps 3.85 -> 3.75, 2.82 -> 2.71, 1.93 -> 1.94; 17 warps 3.90 ->
+// 3.75, 2.86 -> 2.72, 1.96 -> 1.95; 11 warps 4.31 -> 3.68, 3.25 -> 2.65, 2.22 ->
+// 1.94; 4 warps 7.33 -> 3.93, 5.73 -> 2.71, 3.87 -> 1.95.
+constexpr int kFarWarps = 18;
 struct Launch {
+    int pt;            // of the kernel: 0 photons, 1 electrons, 2 electrons beside large tables
     int threads;
     size_t smem;
 };
 static Launch phase_shape(const gdpm_ctx* ctx, const DevTables& T, int pt, bool narrow, size_t fixed_smem = 0) {
-    const size_t tables = smem_of(T, pt == 0 ? GDPM_PHOTON : GDPM_ELECTRON);
     const size_t stack = pt == 0 ? kPhStack * sizeof(PhRec) : sizeof(ElStack);
-    int thr = ctx->block_threads > 0 ? ctx->block_threads
-              : pt == 0              ? (narrow ? kNarrowThreads : PhaseShape<0>::threads)
-                                     : PhaseShape<1>::threads;
-    thr = std::min(thr, 32 * int((kMaxSmem - fixed_smem - tables) / stack));
-    return Launch{thr, tables + stack * size_t(thr / 32)};
+    const int want = ctx->block_threads > 0 ? ctx->block_threads
+                     : pt == 0              ? (narrow ? kNarrowThreads : PhaseShape<0>::threads)
+                                            : PhaseShape<1>::threads;
+    auto fit = [&](int k) { return std::min(want, 32 * int((kMaxSmem - fixed_smem - smem_of(T, k)) / stack)); };
+    int thr = fit(pt);
+    if (pt == 1 && thr < std::min(want, 32 * kFarWarps)) thr = fit(pt = 2);
+    return Launch{pt, thr, smem_of(T, pt) + stack * size_t(thr / 32)};
 }
 
 // CTAs of n primaries: see kSourceThreads.
@@ -1886,9 +1909,10 @@ int launch_phase(gdpm_ctx* ctx, Runner& r, cudaStream_t st, int particle, const 
     const int thr = shape.threads;
     const size_t smem = shape.smem;
     using Kernel = void (*)(const SimParams, const PhaseArgs);
-    static const Kernel kernels[2][3] = {{k_phase<0, kPlain>, k_phase<0, kPair>, k_phase<0, kGeneral>},
-                                         {k_phase<1, kPlain>, k_phase<1, kPair>, k_phase<1, kGeneral>}};
-    const Kernel fn = kernels[particle == GDPM_PHOTON ? 0 : 1][P.hrec ? kGeneral : P.tally_mode ? kPair : kPlain];
+    static const Kernel kernels[3][3] = {{k_phase<0, kPlain>, k_phase<0, kPair>, k_phase<0, kGeneral>},
+                                         {k_phase<1, kPlain>, k_phase<1, kPair>, k_phase<1, kGeneral>},
+                                         {k_phase<2, kPlain>, k_phase<2, kPair>, k_phase<2, kGeneral>}};
+    const Kernel fn = kernels[shape.pt][P.hrec ? kGeneral : P.tally_mode ? kPair : kPlain];
     Runner::Resident* known = nullptr;
     for (Runner::Resident& q : r.resident) {
         if (q.fn == (const void*)fn && q.threads == thr && q.smem == smem) known = &q;
@@ -1968,13 +1992,16 @@ int build_loop_graph(gdpm_ctx* ctx, const SimParams& P, LoopArgs& L, bool metrop
     *exec = nullptr;
     uint32_t grid[2];
     size_t smem[2];
-    const void* fn[2] = {(const void*)k_phase_loop<0>, (const void*)k_phase_loop<1>};
+    const void* const loops[3] = {(const void*)k_phase_loop<0>, (const void*)k_phase_loop<1>,
+                                  (const void*)k_phase_loop<2>};
+    const void* fn[2];
     int thr[2];
     uint64_t warps = 0;
     for (int t = 0; t < 2; ++t) {
         cudaFuncAttributes attr{};             // the arguments k_phase_loop derives in shared memory
-        GDPM_CUDA_TRY(cudaFuncGetAttributes(&attr, fn[t]));
+        GDPM_CUDA_TRY(cudaFuncGetAttributes(&attr, loops[t]));
         const Launch shape = phase_shape(ctx, P.T, t, false, attr.sharedSizeBytes);
+        fn[t] = loops[shape.pt];
         thr[t] = shape.threads;
         smem[t] = shape.smem;
         // one limit for every context's graph, as in launch_phase
