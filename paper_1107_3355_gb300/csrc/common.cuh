@@ -149,7 +149,7 @@ __device__ __forceinline__ float4 draw(Part& p, uint32_t k0, uint32_t k1) {
 // A banked particle has made no draw yet (draw counter 0).  A primary's
 // history is its phase's first plus its slot, its particle id 1, its draw
 // counter 1 and its voxel follows from its position.  E < 0 marks an empty
-// slot.  A record is written once and read once, with streaming accesses: the
+// slot.  bank() writes the banked ones.  A record is written once and read once, with streaming accesses: the
 // L2 is for the phantom and the tallies (CT plan photon phase -3 %).
 // One address and three loads per refill, where 13 arrays of one word
 // took 13 of each: CT plan, photon phase 23.9 -> 22.5 ms, electron phase
@@ -163,12 +163,6 @@ constexpr int kSourceWords = 8;
 
 __device__ __forceinline__ uint4 pack4(float a, float b, float c, uint32_t d) {
     return make_uint4(__float_as_uint(a), __float_as_uint(b), __float_as_uint(c), d);
-}
-__device__ __forceinline__ void queue_store(const Queue& q, uint32_t s, const Part& p) {
-    uint4* r = q.rec + size_t(s) * (kQueueWords / 4);
-    r[0] = pack4(p.x, p.y, p.z, __float_as_uint(p.E));
-    r[1] = pack4(p.u, p.v, p.w, uint32_t(p.ix) | (uint32_t(p.iy) << 10) | (uint32_t(p.iz) << 20));
-    r[2] = make_uint4(p.hist, p.pidlo, p.pidhi, p.flags);
 }
 __device__ __forceinline__ void queue_mark_empty(const Queue& q, uint32_t s) {
     q.rec[size_t(s) * (kQueueWords / 4)].w = __float_as_uint(-1.f);

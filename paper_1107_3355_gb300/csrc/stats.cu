@@ -1,7 +1,8 @@
 // Batch statistics (Sec. 2.2.1: mean dose and uncertainty from N_b batches;
 // Sec. 3.1: sigma/Dmax over the D > 0.5 Dmax region) and the per-phantom
-// Woodcock majorant.  These kernels stream voxel arrays and are bound by
-// HBM bandwidth: coalesced grid-stride loops sized to the SM count.
+// Woodcock majorant.  These kernels stream voxel arrays in coalesced
+// grid-stride loops sized to the SM count; the folds are bound by the FP64
+// pipe before HBM.
 #include <algorithm>
 #include <cstring>
 
@@ -280,7 +281,7 @@ __device__ __forceinline__ void batch_tallies(const SimParams& P, size_t V, size
 }
 
 // Voxels with dose, gathered by the threads of a CTA so that the FP64 work
-// per voxel (weights, mean, 1/mass, square root: about 30 operations) runs
+// per voxel (weights, mean, 1/density, square root: about 16 operations) runs
 // with full warps however few of a warp's voxels hold dose.
 struct FoldItem {
     double v[4];      // sums over the long batches (e, e^2) and over the short ones, or the tallies

@@ -17,9 +17,10 @@
 // A lane whose particle waits or has ended takes another from the stack, which
 // is refilled from the phase's input (freshly generated primaries, then the
 // queue of banked particles), so warps stay full until the input is drained.
-// Tables live in shared memory (Sec. 2.2.2 reads them by linear
-// interpolation); random numbers come from Philox4x32-10 keyed per history
-// and particle, so results do not depend on scheduling.
+// Tables live in shared memory (but the electrons' largest where it would
+// crowd out warps, kFarWarps) and are read by linear interpolation (Sec.
+// 2.2.2); random numbers come from Philox4x32-10 keyed per history and
+// particle, so results do not depend on scheduling.
 #include <algorithm>
 #include <cfloat>
 
@@ -34,9 +35,9 @@ constexpr uint32_t kFull = 0xffffffffu;
 
 // CTA shape each phase kernel is compiled for: threads per CTA and the
 // resident CTAs per SM that fix its register budget.  A warp's stack takes
-// 4.6 KB (photons) or 6.0 KB (electrons) of shared memory, so one CTA stages
+// 4.6 KB (photons) or 7.0 KB (electrons) of shared memory, so one CTA stages
 // the tables once and leaves the L1 what it can.  Photons: 896 threads and 72
-// registers, which wide phases fill (narrow_threads for the others); 1e8 CT
+// registers, which wide phases fill (kNarrowThreads for the others); 1e8 CT
 // histories take 16.8 ms of photon phases instead of 17.9 at 768 and 17.1 at
 // 1024 (64 registers), the lung slab's 2.5e8 25.2 instead of 27.0 and 24.8.
 // Electrons at 896 lose 5-8 %, at 640 4 %.
@@ -718,8 +719,8 @@ __device__ __forceinline__ int walk_stretch(const SimParams& P, Electron& p, ElS
 // not give up the warp.
 constexpr int kDrainedStretches = 16;
 
-// A lane's round: set up a step when none is in progress (`starts`, with the
-// draw x), walk, and at the step's end escape, be absorbed, or wait for the
+// A lane's round: set up a step when none is in progress (with the draw x in
+// the start voxel's material `mat`), walk, and at the step's end escape, be absorbed, or wait for the
 // hard-event candidate.
 template <int GEN, bool FAR>
 __device__ __forceinline__ Round electron_round(const SimParams& P, const ElSmem& S, Electron& p, ElStep& st,
@@ -1196,8 +1197,8 @@ constexpr uint32_t kElReady = 32, kElWait = 32, kElStack = kElReady + kElWait + 
 struct ElStack {
     uint4 a[kElStack], b[kElStack], c[kElStack], d[kElStack];
     Slots held[2];      // the warp's queue reservations, used only by event rounds
-    // What a lane needs once a round or a step, kept out of its registers (24
-    // instead of 72 bytes of spills): history, id and draw counter of its
+    // What a lane needs once a round or a step, kept out of its registers (no
+    // spills instead of 72 bytes): history, id and draw counter of its
     // electron; direction after the hinge and mass thickness of leg 2.  1e8 CT
     // histories: electron phases 24.0 -> 23.3 ms, lung slab 47.1 -> 46.2.  The
     // KB a warp leaves room for 24 warps beside 58 KB of tables (4 materials
@@ -1941,7 +1942,7 @@ int launch_phase(gdpm_ctx* ctx, Runner& r, cudaStream_t st, int particle, const 
     // This phase's CTAs may start and stage their tables while the last ones of
     // the kernel before it run, except beside other requests, which then find
     // those SMs free.  A start costs some 5 us otherwise: 1e4 pencil photons (4
-    // phases) 0.20 -> 0.18 ms, a 1e5 beamlet (8) 0.83 -> 0.79.
+    // phases) 0.195 -> 0.170 ms, a 1e5 beamlet (8) 0.83 -> 0.77.
     cudaLaunchAttribute early{};
     early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     early.val.programmaticStreamSerializationAllowed = 1;
